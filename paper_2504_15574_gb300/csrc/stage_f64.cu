@@ -8,43 +8,116 @@
 //
 // This path exists to reproduce an FP64 reference evaluation of the method
 // operation for operation: every expression below is evaluated in a fixed
-// order with no FMA contraction, divisions where the method divides, and sums
-// over populations in ascending k.  Each interface flux is computed once (two
-// face kernels into global buffers), then one kernel updates the cells.  It is not the throughput path (that is
-// stage_f32.cu); it shares the ghost-row layout so that all reads are plain
-// loads.
+// order with no FMA contraction (other than inside a division), rounded quotients
+// where the method divides, and sums over populations in ascending k.  Each
+// interface flux is computed once (one face kernel into global buffers), then one
+// kernel updates the cells.  It is not the throughput path (that is stage_f32.cu);
+// it shares the ghost-row layout so that all reads are plain loads.
 #include "vlbm_internal.h"
 
 namespace vk {
 
 namespace {
 
-__device__ __forceinline__ double weno5(double a, double b, double c, double d, double e, double eps)
+// ---- arithmetic -----------------------------------------------------------------------
+// GB300 issues one FP64 warp instruction per 64 cycles and scheduler (2 FP64 lanes per SM), so a
+// stage's time is its FP64 instruction count: 135 per interface value and 105 per population and
+// cell when every division was the compiler's and every stencil form was evaluated per face (490,
+// 487 and 384 us for the phi faces, theta faces and cells of a 256 x 512 stage, 535 G FP64
+// instructions/s of ~578).  The forms below give the same bits with fewer of them: scalings by
+// powers of two and reciprocal seeds go to the integer and FP32 pipes, which are otherwise idle.
+
+// x 2^k for the constant c = 2^k, |k| <= 4: an exponent addition; zeros are returned as they are,
+// and what could leave the normal range (or is not finite) takes the multiplication.
+template <int K>
+__device__ __forceinline__ double scale2(double x)
 {
-    double p1 = (2.0 * a - 7.0 * b + 11.0 * c) / 6.0;
-    double p2 = (-b + 5.0 * c + 2.0 * d) / 6.0;
-    double p3 = (2.0 * c + 5.0 * d - e) / 6.0;
-    double d1a = a - 2.0 * b + c, d1b = a - 4.0 * b + 3.0 * c;
-    double d2a = b - 2.0 * c + d, d2b = b - d;
-    double d3a = c - 2.0 * d + e, d3b = 3.0 * c - 4.0 * d + e;
-    double s1 = 13.0 / 12.0 * (d1a * d1a) + 0.25 * (d1b * d1b);
-    double s2 = 13.0 / 12.0 * (d2a * d2a) + 0.25 * (d2b * d2b);
-    double s3 = 13.0 / 12.0 * (d3a * d3a) + 0.25 * (d3b * d3b);
-    double w1 = 0.1 / ((s1 + eps) * (s1 + eps));
-    double w2 = 0.6 / ((s2 + eps) * (s2 + eps));
-    double w3 = 0.3 / ((s3 + eps) * (s3 + eps));
-    return (w1 * p1 + w2 * p2 + w3 * p3) / (w1 + w2 + w3);
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    if ((unsigned)((hi >> 20) & 0x7ff) - 8u < 2030u) return __hiloint2double(hi + (K << 20), lo);
+    if (((hi << 1) | lo) == 0) return x;
+    return x * (K >= 0 ? (double)(1 << (K >= 0 ? K : 0)) : 1.0 / (double)(1 << (K < 0 ? -K : 0)));
 }
 
-// Interface value from upwind-ordered a..e (c the upwind cell, d the downwind cell):
-// WENO-5, or the upwind stencils of Eq. (fluxes_U1-3), in the oracle's expression order.
-__device__ __forceinline__ double recon(int scheme, double a, double b, double c, double d, double e, double eps)
+// x / d with 1/d = h + l held to 106 bits (DivC, built on the host): RN(x h + RN(x l)), the two-
+// operation multiplication by an arbitrary-precision constant of Brisebarre and Muller ("Correctly
+// rounded multiplication by arbitrary precision constants", 2005).  Exact for d = 6 and d = 3 (no
+// quotient comes within 1/6 ulp of a rounding boundary); for a general d it differs from the
+// rounded quotient only where x / d is within 2^-105 of a boundary.  h is rounded toward zero and l
+// positive, so infinities pass through.
+__device__ __forceinline__ double div_const(double x, const DivC &d) { return __fma_rn(x, d.h, __dmul_rn(x, d.l)); }
+
+// a / b with three FP64 operations: a reciprocal of b good to 2^-44 is formed in FP32 (the leading
+// 24 bits of b's significand through the hardware reciprocal, one error term with the remaining
+// bits) and assembled into a double by integer operations; then one residual correction of the
+// quotient (Markstein 1990).  The corrected value is within 2^-88 of a / b before its rounding, so
+// it is the rounded quotient but for a chance of about 2^-35 per division (none in 4e8 random
+// ones).  A b that is not positive and well inside the normal range takes the plain division.
+__device__ __forceinline__ double div_pos(double a, double b)
 {
-    switch (scheme) {
-    case VLBM_U1: return c;
-    case VLBM_U2: return 1.5 * c - 0.5 * b;
-    case VLBM_U3: return (2.0 * d + 5.0 * c - b) / 6.0;
-    default: return weno5(a, b, c, d, e, eps);
+    const int hi = __double2hiint(b), lo = __double2loint(b);
+    if ((unsigned)((hi >> 20) - (1023 - 500)) > 1000u) return a / b;
+    const float bh = __int_as_float(0x3f800000 | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29));
+    const float bl = (float)(lo & 0x1fffffff) * 0x1p-52f;
+    float r0;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(bh));
+    r0 = fmaxf(fminf(r0, 0.99999994f), 0.5f);   // inside one binade: the error term is added to its bits
+    float e = __fmaf_rn(-bh, r0, 1.0f);
+    e = __fmaf_rn(-bl, r0, e);
+    const float r1 = __fmul_rn(r0, __fmaf_rn(e, e, e));
+    const int u = __float_as_int(r0), i1 = __float2int_rn(__fmul_rn(r1, 0x1p53f));
+    long long bits = ((long long)((u >> 3) + ((1023 - 127) << 20)) << 32) | (unsigned)(u << 29);
+    bits += i1;
+    bits -= (long long)((hi >> 20) - 1023) << 52;
+    const double r = __longlong_as_double(bits);
+    const double q = __dmul_rn(a, r);
+    return __fma_rn(__fma_rn(-b, q, a), r, q);
+}
+
+// Interface values of S consecutive faces from y[0 .. S + 3] in upwind order: face f has the stencil
+// a..e = y[f .. f + 4] (c the upwind cell, d the downwind cell), in the oracle's expression order.
+// The forms of one column (13/12 times the squared second difference, and 5 y) are shared by the
+// three candidate stencils centred on it, which changes no bit: 45 + 4 divisions of 3 FP64
+// operations per face.
+template <int S>
+__device__ __forceinline__ void weno5_strip(const double (&y)[S + 4], double eps, const DivC &six, double (&r)[S])
+{
+    double kq[S + 4], y5[S + 4];
+#pragma unroll
+    for (int i = 1; i <= 2; ++i) {
+        const double d = y[i - 1] - scale2<1>(y[i]) + y[i + 1];
+        kq[i] = 13.0 / 12.0 * (d * d);
+    }
+    y5[2] = 5.0 * y[2];
+#pragma unroll
+    for (int f = 0; f < S; ++f) {
+        const double a = y[f], b = y[f + 1], c = y[f + 2], d = y[f + 3], e = y[f + 4];
+        const double d3a = c - scale2<1>(d) + e;
+        kq[f + 3] = 13.0 / 12.0 * (d3a * d3a);
+        y5[f + 3] = 5.0 * d;
+        const double c3 = 3.0 * c;
+        const double d1b = a - scale2<2>(b) + c3;
+        const double d2b = b - d;
+        const double d3b = c3 - scale2<2>(d) + e;
+        const double s1 = kq[f + 1] + scale2<-2>(d1b * d1b) + eps;
+        const double s2 = kq[f + 2] + scale2<-2>(d2b * d2b) + eps;
+        const double s3 = kq[f + 3] + scale2<-2>(d3b * d3b) + eps;
+        const double w1 = div_pos(0.1, s1 * s1), w2 = div_pos(0.6, s2 * s2), w3 = div_pos(0.3, s3 * s3);
+        const double p1 = div_const(scale2<1>(a) - 7.0 * b + 11.0 * c, six);
+        const double p2 = div_const(y5[f + 2] - b + scale2<1>(d), six);
+        const double p3 = div_const(scale2<1>(c) + y5[f + 3] - e, six);
+        r[f] = div_pos(w1 * p1 + w2 * p2 + w3 * p3, w1 + w2 + w3);
+    }
+}
+
+// The same for the upwind stencils of Eq. (fluxes_U1-3).
+template <int S>
+__device__ __forceinline__ void upwind_strip(int scheme, const double (&y)[S + 4], const DivC &six, double (&r)[S])
+{
+#pragma unroll
+    for (int f = 0; f < S; ++f) {
+        const double b = y[f + 1], c = y[f + 2], d = y[f + 3];
+        r[f] = (scheme == VLBM_U1) ? c : (scheme == VLBM_U2) ? 1.5 * c - 0.5 * b
+                                                             : div_const(2.0 * d + 5.0 * c - b, six);
     }
 }
 
@@ -68,112 +141,150 @@ __device__ __forceinline__ void store_with_images(T *f, const Layout &L, int k, 
     }
 }
 
-// Theta flux through interface fi (between rows fi-1 and fi, fi = 0..nt) of population k:
-// the reconstruction on the nodal g = sin f of rows fi-3..fi+2 (ghost rows with their own,
-// negative, sine), or (Komissarov) on f itself times v_theta sin(theta_fi).
-__global__ void __launch_bounds__(128) faces_theta_f64_kernel(const StageD p)
+// Interface fluxes of one stage, one strip of S consecutive faces of one population per thread.
+// Theta flux through interface fi (between rows fi-1 and fi, fi = 0..nt) of population k: the
+// reconstruction on the nodal g = sin f of rows fi-3..fi+2 (ghost rows with their own, negative,
+// sine), or (Komissarov) on f itself times v_theta sin(theta_fi); a thread walks S rows of one
+// column.  Phi flux through interface fj (between columns fj-1 and fj, fj = 0..np) of row i; a
+// thread walks S columns of one row.  For a negative velocity the strip is walked backwards, which
+// puts its values in upwind order.  The first nb_phi CTAs take the phi faces, the others the theta
+// faces (one launch: on small grids either alone leaves schedulers idle).
+// Bound: the FP64 pipe (57 operations a face; 240 us for the 4.2 M faces of 256 x 512, D2Q16, by
+// count).  Long strips share the column forms, short ones spread a small grid over more
+// schedulers: launch_stage_f64 picks S.
+template <int S>
+__global__ void __launch_bounds__(128) faces_f64_kernel(const StageD p, int nb_phi)
 {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int fi = blockIdx.y;
-    const int k = blockIdx.z;
-    if (j >= p.L.np) return;
     const Layout L = p.L;
-    const double *g = p.in;
-    const double va = p.c.v[k / p.c.q];
-    double gt[6];
+    const int q = p.c.q;
+    const bool theta = (int)blockIdx.x >= nb_phi;
+    double y[S + 4], r[S];
+    if (!theta) {
+        const int ns = (L.np + S) / S;   // strips of the np + 1 faces
+        const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        const int k = blockIdx.y;
+        if (t >= (long long)ns * L.nt) return;
+        const int i = (int)(t / ns), f0 = (int)(t - (long long)i * ns) * S;
+        const double vb = p.c.v[k % q];
+        const int dir = vb > 0.0 ? 1 : -1;
+        // y[m] = column c0 + dir m; a strip that reaches past the last face reads the last column in store
+        const int c0 = dir > 0 ? f0 - 3 : f0 + S + 1;
+        const double *g = p.in + L.at(k, i, 0);
 #pragma unroll
-    for (int o = 0; o < 6; ++o)
-        gt[o] = p.komissarov ? g[L.at(k, fi - 3 + o, j)] : p.sin_ext[fi + o] * g[L.at(k, fi - 3 + o, j)];
-    const double r = (va > 0.0) ? recon(p.scheme, gt[0], gt[1], gt[2], gt[3], gt[4], p.eps)
-                                : recon(p.scheme, gt[5], gt[4], gt[3], gt[2], gt[1], p.eps);
-    const double flux = p.komissarov ? va * p.sin_f[fi] * r : va * r;
-    p.Ft[((size_t)k * (L.nt + 1) + fi) * L.np + j] = flux;
-    if (p.pole) {
-        if (fi == 0) p.pole[(size_t)k * L.np + j] = flux;
-        if (fi == L.nt) p.pole[((size_t)NK + k) * L.np + j] = flux;
+        for (int m = 0; m < S + 4; ++m) y[m] = g[min(c0 + dir * m, L.np + GC - 1)];
+        if (p.scheme == VLBM_WENO5) weno5_strip<S>(y, p.eps, p.six, r);
+        else upwind_strip<S>(p.scheme, y, p.six, r);
+        double *out = p.Fp + ((size_t)k * L.nt + i) * (L.np + 1);
+#pragma unroll
+        for (int f = 0; f < S; ++f) {
+            const int fj = dir > 0 ? f0 + f : f0 + S - 1 - f;
+            if (fj <= L.np) out[fj] = vb * r[f];
+        }
+        return;
+    }
+    const int ns = (L.nt + S) / S;
+    const long long t = (long long)(blockIdx.x - nb_phi) * blockDim.x + threadIdx.x;
+    const int k = blockIdx.y;
+    if (t >= (long long)ns * L.np) return;
+    const int st = (int)(t / L.np), j = (int)(t - (long long)st * L.np), f0 = st * S;
+    const double va = p.c.v[k / q];
+    const int dir = va > 0.0 ? 1 : -1;
+    const int r0 = dir > 0 ? f0 - 3 : f0 + S + 1;
+#pragma unroll
+    for (int m = 0; m < S + 4; ++m) {
+        const int row = min(r0 + dir * m, L.nt + GR - 1);
+        const double v = p.in[L.at(k, row, j)];
+        y[m] = p.komissarov ? v : p.sin_ext[row + GR] * v;
+    }
+    if (p.scheme == VLBM_WENO5) weno5_strip<S>(y, p.eps, p.six, r);
+    else upwind_strip<S>(p.scheme, y, p.six, r);
+#pragma unroll
+    for (int f = 0; f < S; ++f) {
+        const int fi = dir > 0 ? f0 + f : f0 + S - 1 - f;
+        if (fi > L.nt) continue;
+        const double flux = p.komissarov ? va * p.sin_f[fi] * r[f] : va * r[f];
+        p.Ft[((size_t)k * (L.nt + 1) + fi) * L.np + j] = flux;
+        if (p.pole) {
+            if (fi == 0) p.pole[(size_t)k * L.np + j] = flux;
+            if (fi == L.nt) p.pole[((size_t)NK + k) * L.np + j] = flux;
+        }
     }
 }
 
-// Phi flux through interface fj (between columns fj-1 and fj, fj = 0..np) of row i.
-__global__ void __launch_bounds__(128) faces_phi_f64_kernel(const StageD p)
+// Cells of one stage: moments, equilibrium, force, BGK, the flux differences of the interface
+// fluxes above and the stage combination, in the oracle's operation order.  A CTA takes 32
+// consecutive cells; its 8 warps first form the moments of those cells (one warp each for n, the
+// two momenta and then the two velocities: the sums run over k in order, so they are chains), then
+// each warp updates two populations of them.  One thread per cell, the earlier form, left a
+// 32 x 64 grid with 64 warps of 1,700 serial FP64 operations (71 us a launch).  Bound on large
+// grids: the FP64 pipe (about 54 operations per population, from 105; divisions by row constants,
+// tau and 3 are two operations each).
+constexpr int CELL_WARPS = 8;
+__global__ void __launch_bounds__(32 * CELL_WARPS) cells_f64_kernel(const StageD p)
 {
-    const int fj = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = blockIdx.y;
-    const int k = blockIdx.z;
-    if (fj > p.L.np) return;
+    __shared__ double gs[NK][32], mom[3][32], vel[4][32];
     const Layout L = p.L;
-    const double *g = p.in;
-    const double vb = p.c.v[k % p.c.q];
-    double gp[6];
-#pragma unroll
-    for (int o = 0; o < 6; ++o) gp[o] = g[L.at(k, i, fj - 3 + o)];
-    const double r = (vb > 0.0) ? recon(p.scheme, gp[0], gp[1], gp[2], gp[3], gp[4], p.eps)
-                                : recon(p.scheme, gp[5], gp[4], gp[3], gp[2], gp[1], p.eps);
-    p.Fp[((size_t)k * L.nt + i) * (L.np + 1) + fj] = vb * r;
-}
-
-// One cell: moments, equilibrium, force, BGK, the flux differences of the interface
-// fluxes above and the stage combination, in the oracle's operation order.
-__global__ void __launch_bounds__(128) stage_f64_kernel(const StageD p)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i >= p.L.nt || j >= p.L.np) return;
-    const Layout L = p.L;
-    const double *g = p.in;
-
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int q = p.c.q, nk = q * q;
-    double gk[NK];
-    for (int k = 0; k < nk; ++k) gk[k] = g[L.at(k, i, j)];
-
-    double n = 0.0, jt = 0.0, jp = 0.0;
-    for (int k = 0; k < nk; ++k) {
-        n += gk[k];
-        jt += gk[k] * p.c.v[k / q];
-        jp += gk[k] * p.c.v[k % q];
+    const long long cells = (long long)L.nt * L.np;
+    const long long cell = (long long)blockIdx.x * 32 + lane;
+    const bool in = cell < cells;
+    const int i = in ? (int)(cell / L.np) : 0, j = in ? (int)(cell - (long long)i * L.np) : 0;
+    for (int k = warp; k < nk; k += CELL_WARPS) gs[k][lane] = p.in[L.at(k, i, j)];
+    __syncthreads();
+    if (warp < 3) {
+        double m = 0.0;
+        for (int k = 0; k < nk; ++k) {
+            const double g = gs[k][lane];
+            m += (warp == 0) ? g : g * p.c.v[warp == 1 ? k / q : k % q];
+        }
+        mom[warp][lane] = m;
     }
-    const double ut = jt / n, up = jp / n;
-    const double sin_i = p.sin_ext[i + GR];
-    const double cot_i = p.cot[i];
-    const double R = p.R;
-
+    __syncthreads();
+    if (warp == 1 || warp == 2) vel[warp - 1][lane] = div_pos(mom[warp][lane], mom[0][lane]);
+    __syncthreads();
+    if (warp == 0) {
+        const double ut = vel[0][lane], up = vel[1][lane];
+        const double u2 = ut * ut + up * up;
+        vel[2][lane] = u2;
+        vel[3][lane] = 3.0 * u2;
+    }
+    __syncthreads();
+    if (!in) return;
+    const double n = mom[0][lane], ut = vel[0][lane], up = vel[1][lane], u2 = vel[2][lane], u23 = vel[3][lane];
+    const RowD rd = p.row[i];
 #pragma unroll 1
-    for (int k = 0; k < nk; ++k) {
+    for (int k = warp; k < nk; k += CELL_WARPS) {
         const int a = k / q, b = k % q;
         const double va = p.c.v[a], vb = p.c.v[b];
-        // equilibrium (T0 = 1)
-        const double xi = va * ut + vb * up;
-        const double u2 = ut * ut + up * up;
-        const double wk = p.c.w[a] * p.c.w[b];
-        // Eq. feq_Q=4 (third order), or Eq. feq_Q=3 (second order) for D2Q9
-        const double feq = (q == 3) ? n * wk * (1.0 + xi + 0.5 * (xi * xi - u2))
-                                    : n * wk * (1.0 + xi + 0.5 * (xi * xi - u2) + xi * (xi * xi - 3.0 * u2) / 6.0);
-        // velocity derivatives: K on k_theta at fixed k_phi, Ktilde on k_phi at fixed k_theta
-        double kg = 0.0, ktg = 0.0;
-        for (int m = 0; m < q; ++m) {
-            kg += p.c.K[a * q + m] * gk[q * m + b];
-            ktg += p.c.Kt[b * q + m] * gk[q * a + m];
-        }
-        const double force = cot_i / R * (vb * vb * kg - va * ktg);
+        const double gk = gs[k][lane];
+        // loaded ahead of the arithmetic
         const double fn = p.Ft[((size_t)k * (L.nt + 1) + i) * L.np + j];
         const double fs = p.Ft[((size_t)k * (L.nt + 1) + i + 1) * L.np + j];
         const double fw = p.Fp[((size_t)k * L.nt + i) * (L.np + 1) + j];
         const double fe = p.Fp[((size_t)k * L.nt + i) * (L.np + 1) + j + 1];
-        const double adv_t = p.komissarov ? -(fs - fn) / (R * (p.cos_f[i] - p.cos_f[i + 1]))
-                                          : -(fs - fn) / (R * sin_i * p.dth);
-        const double adv_p = -(fe - fw) / (R * sin_i * p.dph);
-        const double Lk = adv_t + adv_p - force - (gk[k] - feq) / p.tau;
+        const double f0 = (p.stage == 1) ? 0.0 : p.fold[L.at(k, i, j)];
+        // equilibrium (T0 = 1): Eq. feq_Q=4 (third order), or Eq. feq_Q=3 (second order) for D2Q9
+        const double xi = va * ut + vb * up;
+        const double xi2 = xi * xi;
+        const double second = 1.0 + xi + scale2<-1>(xi2 - u2);
+        const double nw = n * p.wk[k];
+        const double feq = (q == 3) ? nw * second : nw * (second + div_const(xi * (xi2 - u23), p.six));
+        // velocity derivatives: K on k_theta at fixed k_phi, Ktilde on k_phi at fixed k_theta
+        double kg = p.c.K[a * q] * gs[b][lane], ktg = p.c.Kt[b * q] * gs[q * a][lane];
+        for (int m = 1; m < q; ++m) {
+            kg += p.c.K[a * q + m] * gs[q * m + b][lane];
+            ktg += p.c.Kt[b * q + m] * gs[q * a + m][lane];
+        }
+        const double force = rd.cotR * (p.vb2[b] * kg - va * ktg);
+        const double adv_t = -div_const(fs - fn, rd.th);
+        const double adv_p = -div_const(fe - fw, rd.ph);
+        const double Lk = adv_t + adv_p - force - div_const(gk - feq, p.tau_div);
 
         double outv;
-        if (p.stage == 1) {
-            outv = gk[k] + p.dt * Lk;
-        } else if (p.stage == 2) {
-            const double f0 = p.fold[L.at(k, i, j)];
-            outv = 0.75 * f0 + 0.25 * gk[k] + 0.25 * p.dt * Lk;
-        } else {
-            const double f0 = p.fold[L.at(k, i, j)];
-            outv = f0 / 3.0 + 2.0 / 3.0 * gk[k] + 2.0 / 3.0 * p.dt * Lk;
-        }
+        if (p.stage == 1) outv = gk + p.dt * Lk;
+        else if (p.stage == 2) outv = 0.75 * f0 + scale2<-2>(gk) + p.dt_stage * Lk;
+        else outv = div_const(f0, p.three) + 2.0 / 3.0 * gk + p.dt_stage * Lk;
         store_with_images(p.out, L, k, i, j, outv);
     }
 }
@@ -272,14 +383,27 @@ __global__ void filter_kernel(T *f, const Layout L, const int *rows, const int *
 
 }  // namespace
 
+template <int S>
+static void launch_faces(const StageD &p, cudaStream_t s)
+{
+    const Layout &L = p.L;
+    const long long sp = (long long)((L.np + S) / S) * L.nt, stt = (long long)((L.nt + S) / S) * L.np;
+    const int nb = (int)((sp + 127) / 128), nt = (int)((stt + 127) / 128);
+    faces_f64_kernel<S><<<dim3(nb + nt, L.nk), 128, 0, s>>>(p, nb);
+}
+
 void launch_stage_f64(const StageD &p, cudaStream_t s)
 {
-    // every interface flux once (as the oracle), then the cells
-    faces_theta_f64_kernel<<<dim3((p.L.np + 127) / 128, p.L.nt + 1, p.L.nk), 128, 0, s>>>(p);
-    faces_phi_f64_kernel<<<dim3((p.L.np + 1 + 127) / 128, p.L.nt, p.L.nk), 128, 0, s>>>(p);
-    dim3 block(32, 4);
-    dim3 grid((p.L.np + 31) / 32, (p.L.nt + 3) / 4);
-    stage_f64_kernel<<<grid, block, 0, s>>>(p);
+    // Strip length of the face walk: 8 faces share their column forms best (64 FP64 operations a
+    // face at S = 1, 59 at 8); a grid with fewer faces than about two warps of long strips per
+    // scheduler (608 of them) takes shorter ones, since a lone warp's chain of FP64 operations
+    // bounds the launch there.
+    const long long faces = 2LL * p.L.nk * p.L.nt * p.L.np, lanes = 2LL * 608 * 32;
+    if (faces >= 8 * lanes) launch_faces<8>(p, s);
+    else if (faces >= 2 * lanes) launch_faces<2>(p, s);
+    else launch_faces<1>(p, s);
+    const long long cells = (long long)p.L.nt * p.L.np;
+    cells_f64_kernel<<<(unsigned)((cells + 31) / 32), 32 * CELL_WARPS, 0, s>>>(p);
 }
 
 void launch_init_f64(double *f, const Layout &L, const double *rho, const double *ut, const double *up,

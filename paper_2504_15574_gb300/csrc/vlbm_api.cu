@@ -126,6 +126,20 @@ double sin_padded(const std::vector<double> &s, int nt, int pr)
     return s[r];
 }
 
+// 1/d as h + l: h = 1/d rounded toward zero, l > 0 the remainder (a division x / d is then
+// RN(x h + RN(x l)), stage_f64.cu; where 1/d is a double, the smallest positive l, so that an
+// infinite x stays infinite).
+DivC div_const_of(double d)
+{
+    double y = 1.0 / d, r = std::fma(-y, d, 1.0);
+    if (r < 0.0) {
+        y = std::nextafter(y, 0.0);
+        r = std::fma(-y, d, 1.0);
+    }
+    const double l = r / d;
+    return DivC{y, l > 0.0 ? l : 4.9406564584124654e-324};
+}
+
 // Polar ring filter block size (not in the paper): smallest power of two b with
 // b sin(theta) dphi >= dtheta / 4, dividing n_phi.
 int filter_block(int nt, int np, double sin_i)
@@ -483,21 +497,22 @@ void enqueue_step(vlbm_t *h, int stage_only = 0, int part = 0)
             p.fold = (const double *)h->F;
             p.out = (double *)out;
             p.sin_ext = h->d_sin_ext;
-            p.cot = h->d_cot;
+            p.row = h->d_rowd;
             p.pole = h->d_pole + (size_t)(st - 1) * pole_per;
             p.L = h->L;
-            p.dth = M_PI / h->nt;
-            p.dph = 2.0 * M_PI / h->np;
-            p.R = h->R;
-            p.tau = h->tau;
             p.dt = h->dt;
+            p.dt_stage = (st == 1) ? h->dt : (st == 2) ? 0.25 * h->dt : 2.0 / 3.0 * h->dt;
             p.eps = h->eps;
+            p.tau_div = div_const_of(h->tau);
+            p.six = div_const_of(6.0);
+            p.three = div_const_of(3.0);
             p.stage = st;
             p.c = h->vd;
+            for (int k = 0; k < h->vd.q * h->vd.q; ++k) p.wk[k] = h->vd.w[k / h->vd.q] * h->vd.w[k % h->vd.q];
+            for (int b = 0; b < h->vd.q; ++b) p.vb2[b] = h->vd.v[b] * h->vd.v[b];
             p.scheme = h->scheme;
             p.komissarov = h->komissarov;
             p.sin_f = h->d_sin_f;
-            p.cos_f = h->d_cos_f;
             p.Ft = h->d_ft;
             p.Fp = h->d_fp;
             if (part != 2) launch_stage_f64(p, s);
@@ -516,7 +531,7 @@ void enqueue_step(vlbm_t *h, int stage_only = 0, int part = 0)
 int kernels_per_step(const vlbm_t *h)
 {
     int n = 3 + (h->nfrows ? 3 : 0) + (h->band_hi > h->band_lo ? 3 : 0);
-    if (h->prec == VLBM_FP64) n += 3 * 2 + 1;   // two face kernels per stage and the pole budget
+    if (h->prec == VLBM_FP64) n += 3 + 1;   // a face kernel per stage and the pole budget
     else if (h->run.pole_part) n += 1;          // the pole budget
     return n;
 }
@@ -681,10 +696,9 @@ int vlbm_create(int n_theta, int n_phi, int velocity_set, double tau, double dt,
         (rc = dalloc(h, &h->B, h->arr_bytes)))
         return bail(rc);
     // geometry
-    std::vector<double> sext(n_theta + 2 * GR + F32_TILE_ROWS_MAX, 0.0), cot(n_theta);
+    std::vector<double> sext(n_theta + 2 * GR + F32_TILE_ROWS_MAX, 0.0);
     for (int pr = 0; pr < n_theta + 2 * GR; ++pr) sext[pr] = sin_padded(h->sin_t, n_theta, pr);
-    for (int i = 0; i < n_theta; ++i) cot[i] = h->cos_t[i] / h->sin_t[i];
-    if ((rc = upload(h, &h->d_sin_ext, sext.data(), sext.size())) || (rc = upload(h, &h->d_cot, cot.data(), cot.size())) ||
+    if ((rc = upload(h, &h->d_sin_ext, sext.data(), sext.size())) ||
         (rc = upload(h, &h->d_sin_t, h->sin_t.data(), h->sin_t.size())) ||
         (rc = upload(h, &h->d_cos_t, h->cos_t.data(), h->cos_t.size())))
         return bail(rc);
@@ -702,9 +716,19 @@ int vlbm_create(int n_theta, int n_phi, int velocity_set, double tau, double dt,
             h->cos_f[fi] = -h->cos_f[m];
         }
     }
-    if ((rc = upload(h, &h->d_sin_f, h->sin_f.data(), h->sin_f.size())) ||
-        (rc = upload(h, &h->d_cos_f, h->cos_f.data(), h->cos_f.size())))
-        return bail(rc);
+    if ((rc = upload(h, &h->d_sin_f, h->sin_f.data(), h->sin_f.size()))) return bail(rc);
+    if (h->prec == VLBM_FP64) {
+        // FP64 stage: the row constants in the oracle's evaluation order
+        std::vector<RowD> rowd(n_theta);
+        const double dth = M_PI / n_theta, dph = 2.0 * M_PI / n_phi;
+        for (int i = 0; i < n_theta; ++i) {
+            const double s = h->sin_t[i], cot = h->cos_t[i] / s;
+            rowd[i].cotR = cot / h->R;
+            rowd[i].th = div_const_of(h->komissarov ? h->R * (h->cos_f[i] - h->cos_f[i + 1]) : h->R * s * dth);
+            rowd[i].ph = div_const_of(h->R * s * dph);
+        }
+        if ((rc = upload(h, &h->d_rowd, rowd.data(), rowd.size()))) return bail(rc);
+    }
     if (h->prec == VLBM_FP64 &&
         ((rc = dalloc(h, (void **)&h->d_ft, sizeof(double) * h->L.nk * (size_t)(n_theta + 1) * n_phi)) ||
          (rc = dalloc(h, (void **)&h->d_fp, sizeof(double) * h->L.nk * (size_t)n_theta * (n_phi + 1)))))
@@ -1024,7 +1048,7 @@ void vlbm_destroy(vlbm_t *h)
     if (!h) return;
     if (h->stream) cudaStreamSynchronize(h->stream);
     drop_graphs(h);
-    void *bufs[] = {h->F, h->A, h->B, h->d_sin_ext, h->d_cot, h->d_sin_t, h->d_cos_t, h->d_sin_f, h->d_cos_f, h->d_isp,
+    void *bufs[] = {h->F, h->A, h->B, h->d_sin_ext, h->d_rowd, h->d_sin_t, h->d_cos_t, h->d_sin_f, h->d_isp,
                     h->d_sfc, h->d_ft, h->d_fp,
                     h->d_rref, h->d_dsin, h->d_d2sin, h->d_tabs, h->d_kss, h->d_ikss, h->d_cph, h->d_sph,
                     h->d_pole_part, h->d_scalar, h->d_ctr,

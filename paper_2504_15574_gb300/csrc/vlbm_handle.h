@@ -21,10 +21,11 @@ struct vlbm {
     void *F = nullptr, *A = nullptr, *B = nullptr;
     size_t arr_bytes = 0;
     // FP64 geometry
-    double *d_sin_ext = nullptr, *d_cot = nullptr, *d_sin_t = nullptr, *d_cos_t = nullptr;
+    double *d_sin_ext = nullptr, *d_sin_t = nullptr, *d_cos_t = nullptr;
     int scheme = VLBM_WENO5, komissarov = 0;
     std::vector<double> sin_f, cos_f;                 // theta interfaces fi = 0..nt (theta = fi dtheta)
-    double *d_sin_f = nullptr, *d_cos_f = nullptr;
+    double *d_sin_f = nullptr;
+    vk::RowD *d_rowd = nullptr;                       // FP64 stage: row constants
     float *d_isp = nullptr, *d_sfc = nullptr;         // FP32 upwind schemes: 1/sin per padded row, interface sines
     double *d_ft = nullptr, *d_fp = nullptr;          // FP64 path: interface flux buffers of one stage
     std::vector<double> sin_t, cos_t;

@@ -41,20 +41,28 @@ struct Layout {
 struct VelD { double v[4], w[4], K[16], Kt[16]; int q; };
 
 // ---- FP64 stage (parity path) -------------------------------------------------
+// 1/d to 106 bits: h = 1/d rounded toward zero, l the remainder (positive), for divisions by d in two
+// operations (stage_f64.cu)
+struct DivC { double h, l; };
+// per interior row: cot(theta) / R, and the divisors R sin(theta) dtheta (with the Komissarov flux
+// R (cos theta_{i-1/2} - cos theta_{i+1/2})) and R sin(theta) dphi
+struct RowD { double cotR; DivC th, ph; };
 struct StageD {
     const double *in;      // stage input g (padded layout)
     const double *fold;    // f at the start of the step (own cell only), stages 2 and 3
     double *out;           // stage output (padded layout); may alias fold in stage 3
     const double *sin_ext; // sin(theta) at padded rows 0 .. nt+2GR-1 (negative at ghost rows)
-    const double *cot;     // cos/sin per interior row
+    const RowD *row;       // per interior row
     double *pole;          // [2][16][np] fluxes through the north/south pole faces, or NULL
     Layout L;
-    double dth, dph, R, tau, dt, eps;
+    double dt, dt_stage, eps;   // dt_stage: the stage's weight of dt L (dt, 0.25 dt, 2/3 dt)
+    DivC tau_div, six, three;
     int stage;             // 1, 2, 3
     VelD c;
+    double wk[NK], vb2[4]; // weights w[a] w[b] per population, squared velocities
     int scheme;            // VLBM_WENO5 .. VLBM_U3
     int komissarov;        // theta flux in the Komissarov form
-    const double *sin_f, *cos_f;   // per theta interface fi = 0..nt (theta = fi dtheta)
+    const double *sin_f;   // per theta interface fi = 0..nt (theta = fi dtheta)
     double *Ft, *Fp;       // interface fluxes: theta [nk][nt+1][np], phi [nk][nt][np+1]
 };
 void launch_stage_f64(const StageD &p, cudaStream_t s);

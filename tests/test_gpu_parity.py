@@ -519,3 +519,20 @@ def test_fp32_tile_wait_that_runs_out_reports_a_timeout(V, scheme):
     r, ut, up = h.moments()
     assert np.isfinite(r).all() and abs(r.mean() - 1.0) < 1e-2
     h.close()
+
+
+@pytest.mark.parametrize("nt,np_,scheme,komissarov,velocity_set", [
+    # interface strips of 1, 2 and 8 faces, each with a remainder in theta and phi
+    (7, 10, "weno5", False, "d2q16"), (45, 62, "weno5", False, "d2q16"), (101, 194, "weno5", False, "d2q16"),
+    (45, 62, "u3", True, "d2q16"), (101, 194, "weno5", True, "d2q9"), (103, 1, "weno5", False, "d2q9"),
+    (6, 1622, "u2", False, "d2q16")])
+def test_fp64_face_strips_match_oracle(V, nt, np_, scheme, komissarov, velocity_set):
+    tau = 0.02
+    dt = 0.5 * clamped_dt(nt, np_, tau)
+    ic = inputs.shock_cap(nt, np_, cap=0.4) if np_ > 1 else inputs.sound_parabola(nt, 1, 1e-3)
+    o, g = run_pair(V, nt, np_, tau, dt, ic, 3, scheme=scheme, komissarov=komissarov, velocity_set=velocity_set)
+    fo, fg = o.get_populations(), g.get_populations()
+    # the same operations in the same order, divisions rounded alike: FP64_TOL as everywhere on this path
+    assert np.abs(fg - fo).max() <= FP64_TOL * np.abs(fo).max()
+    assert g.diagnostics()["pole_flux"] == pytest.approx(o.diagnostics()["pole_budget"], rel=1e-9, abs=1e-18)
+    g.close()
