@@ -10,13 +10,13 @@
 // into the library instead of memory from cudaMalloc.
 //
 // The scratch is a file-scope __device__ array of VLBM_NOALLOC_MAX_ROWS x 6
-// doubles (768 KiB); every GPU that loads the library holds it until the
+// doubles (768 KiB, six partial sums per CTA of at most VLBM_NOALLOC_MAX_ROWS); every GPU that loads the library holds it until the
 // process exits.  Host code cannot use the array's name as a device address, so
 // the first call on each device looks its address up with cudaGetSymbolAddress
 // (with that device current) and caches it; that first call should therefore
 // come before any stream capture, and the cached address does not survive a
 // cudaDeviceReset of that device.  All calls share the one array: calls whose
-// kernels overlap on the GPU (on different streams) race on it.  The per-row
+// kernels overlap on the GPU (on different streams) race on it.  The per-CTA
 // partial sums are fully rewritten by every call, so nothing in the scratch has
 // to start at zero.
 #include <mutex>
@@ -27,7 +27,7 @@
 
 namespace {
 
-constexpr int NOALLOC_THREADS = 256;
+constexpr int NOALLOC_THREADS = 128;
 constexpr int NQ = 6;   // mass, momentum x/y/z, energy, non-finite count
 constexpr int MAX_DEVICES = 64;
 
@@ -37,67 +37,123 @@ std::mutex g_mu;
 double *g_scratch_ptr[MAX_DEVICES] = {};
 thread_local std::string g_noalloc_error;
 
-struct VelNA { double v[4], w[4]; };
+struct VelNA { double v2, v3; };   // the positive velocities (v[2], v[3]); v[0] = -v[3], v[1] = -v[2]
 
-// One block per row of a dense [16][nt][np] FP64 population array.
-__global__ void noalloc_rows_kernel(const double *f, int nt, int np, double radius, VelNA c, double *part)
+// Sums of a dense [16][nt][np] FP64 population array.  Bound: GB300's FP64 pipe (one warp
+// instruction per 64 cycles and scheduler), so the work per cell is kept to 40 FP64 instructions:
+// the sums of each k_theta row and k_phi column of the 4 x 4 populations (24 additions) give
+// density, momenta (the velocities come in +- pairs) and energy, a thread keeps one column for all
+// its rows so that cos(phi), sin(phi) enter once per column, and the row factors are formed once per
+// CTA.  (One thread per cell with its own sincos took 170 FP64 instructions a cell: 177 us for
+// 512 x 1024.)  Non-finite values are found on the exponent bits in the integer pipe.
+// Thread: column 32 chunk + lane, rows blockIdx.y rows .. + rows - 1; a CTA's four warps take
+// consecutive column chunks.
+constexpr int NA_ROWS_MAX = 64;
+
+__device__ __forceinline__ void na_load(const double *f, size_t plane, size_t cell, double (&v)[16])
 {
-    const int i = blockIdx.x;
-    const double pi = 3.14159265358979323846;
-    const double dth = pi / nt, dph = 2.0 * pi / np;
-    const int m = nt - 1 - i;
-    const double st = sin(((i <= m ? i : m) + 0.5) * dth);
-    const double ct = (i == m) ? 0.0 : (i < m ? 1.0 : -1.0) * cos(((i <= m ? i : m) + 0.5) * dth);
-    const double area = radius * radius * dth * dph;
-    double acc[NQ] = {0, 0, 0, 0, 0, 0};
-    for (int j = threadIdx.x; j < np; j += NOALLOC_THREADS) {
-        double sp, cp;
-        sincos((j + 0.5) * dph, &sp, &cp);
-        double n = 0.0, jt = 0.0, jp = 0.0, e = 0.0, bad = 0.0;
-        for (int k = 0; k < 16; ++k) {
-            const double va = c.v[k / 4], vb = c.v[k % 4];
-            const double fk = f[((size_t)k * nt + i) * np + j];
-            if (!isfinite(fk)) bad = 1.0;
-            n += fk;
-            jt += fk * va;
-            jp += fk * vb;
-            e += fk * (va * va + vb * vb);
-        }
-        const double dA = st * area;
-        acc[0] += n * dA;
-        acc[1] += (jt * ct * cp - jp * sp) * dA;
-        acc[2] += (jt * ct * sp + jp * cp) * dA;
-        acc[3] += (-jt * st) * dA;
-        acc[4] += 0.5 * e * dA;
-        acc[5] += bad;   // one per cell holding a NaN or Inf population
-    }
-    __shared__ double red[NQ][NOALLOC_THREADS];
-    for (int q = 0; q < NQ; ++q) red[q][threadIdx.x] = acc[q];
-    __syncthreads();
-    for (int w = NOALLOC_THREADS / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w)
-            for (int q = 0; q < NQ; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0)
-        for (int q = 0; q < NQ; ++q) part[(size_t)q * nt + i] = red[q][0];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = __ldg(f + k * plane + cell);
 }
 
-__global__ void noalloc_final_kernel(const double *part, int nrows, double *out)
+__global__ void __launch_bounds__(NOALLOC_THREADS) noalloc_sums_kernel(const double *f, int nt, int np, double radius,
+                                                                        VelNA c, int rows, double *part)
 {
-    __shared__ double red[NQ][NOALLOC_THREADS];
-    double acc[NQ] = {0, 0, 0, 0, 0, 0};
-    for (int i = threadIdx.x; i < nrows; i += NOALLOC_THREADS)
-        for (int q = 0; q < NQ; ++q) acc[q] += part[(size_t)q * nrows + i];
-    for (int q = 0; q < NQ; ++q) red[q][threadIdx.x] = acc[q];
-    __syncthreads();
-    for (int w = NOALLOC_THREADS / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w)
-            for (int q = 0; q < NQ; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + w];
-        __syncthreads();
+    __shared__ double rs[NA_ROWS_MAX], rc[NA_ROWS_MAX];   // area sin(theta), area sin(theta) cos(theta)
+    __shared__ double red[NQ][NOALLOC_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i0 = blockIdx.y * rows, n = min(rows, nt - i0);
+    const double pi = 3.14159265358979323846;
+    const double area = radius * radius * (pi / nt) * (2.0 * pi / np);
+    if ((int)threadIdx.x < n) {
+        const int i = i0 + threadIdx.x, m = nt - 1 - i;
+        double st, ct;
+        sincospi(((i <= m ? i : m) + 0.5) / nt, &st, &ct);
+        if (i == m) ct = 0.0;
+        if (i > m) ct = -ct;
+        rs[threadIdx.x] = st;
+        rc[threadIdx.x] = ct;
     }
-    if (threadIdx.x == 0)
-        for (int q = 0; q < NQ; ++q) out[q] = red[q][0];
+    __syncthreads();
+    const size_t plane = (size_t)nt * np;
+    const int chunks = (np + 31) / 32;
+    double acc[NQ] = {0, 0, 0, 0, 0, 0};
+    int bad = 0;
+    for (int ch = blockIdx.x * (NOALLOC_THREADS / 32) + warp; ch < chunks; ch += gridDim.x * (NOALLOC_THREADS / 32)) {
+        const int j = 32 * ch + lane;
+        const bool in = j < np;
+        const size_t cell0 = (size_t)i0 * np + (in ? j : np - 1);
+        // sums over the rows, weighted by the row's sine: populations of |v_theta| = v[3] and v[2], of
+        // |v_phi| = v[3], j_theta cos(theta), j_phi, j_theta sin(theta)
+        double so = 0.0, si = 0.0, sp = 0.0, a = 0.0, b = 0.0, z = 0.0;
+        double v[16];
+        na_load(f, plane, cell0, v);
+        for (int r = 0; r < n; ++r) {
+            double w[16];
+            if (r + 1 < n) na_load(f, plane, cell0 + (size_t)(r + 1) * np, w);
+            int top = 0;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) top = max(top, __double2hiint(v[k]) & 0x7fffffff);
+            if (in && top >= 0x7ff00000) ++bad;
+            double R[4], C[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                R[m] = (v[4 * m] + v[4 * m + 1]) + (v[4 * m + 2] + v[4 * m + 3]);
+                C[m] = (v[m] + v[m + 4]) + (v[m + 8] + v[m + 12]);
+            }
+            const double jt = fma(c.v3, R[3] - R[0], c.v2 * (R[2] - R[1]));
+            const double jp = fma(c.v3, C[3] - C[0], c.v2 * (C[2] - C[1]));
+            const double s = rs[r], sj = s * jt;
+            so = fma(s, R[0] + R[3], so);
+            si = fma(s, R[1] + R[2], si);
+            sp = fma(s, C[0] + C[3], sp);
+            a = fma(rc[r], sj, a);
+            b = fma(s, jp, b);
+            z = fma(s, sj, z);
+            if (r + 1 < n) {
+#pragma unroll
+                for (int k = 0; k < 16; ++k) v[k] = w[k];
+            }
+        }
+        if (!in) continue;
+        double sph, cph;
+        sincospi((2.0 * j + 1.0) / np, &sph, &cph);
+        // sum |v|^2 f = v3^2 (so + sp) + v2^2 (si + the populations of |v_phi| = v[2])
+        const double mass = so + si;
+        acc[0] += mass;
+        acc[1] += fma(a, cph, -(b * sph));
+        acc[2] += fma(a, sph, b * cph);
+        acc[3] -= z;
+        acc[4] += fma(c.v3 * c.v3, so + sp, c.v2 * c.v2 * (si + (mass - sp)));
+    }
+    acc[5] = bad;
+    // warps by shuffles, then the four warps in order
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], m);
+        if (lane == 0) red[q][warp] = acc[q];
+    }
+    __syncthreads();
+    if (threadIdx.x < NQ) {
+        const int q = threadIdx.x;
+        double t = red[q][0];
+        for (int w = 1; w < NOALLOC_THREADS / 32; ++w) t += red[q][w];
+        const double scale = (q < 4) ? area : (q == 4 ? 0.5 * area : 1.0);
+        part[(size_t)q * gridDim.x * gridDim.y + (size_t)blockIdx.y * gridDim.x + blockIdx.x] = t * scale;
+    }
+}
+
+// One warp per quantity adds the n CTA partials in a fixed order.
+__global__ void __launch_bounds__(32 * NQ) noalloc_final_kernel(const double *part, int n, double *out)
+{
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    double t = 0.0;
+#pragma unroll 4
+    for (int b = lane; b < n; b += 32) t += part[(size_t)q * n + b];
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) t += __shfl_xor_sync(0xffffffffu, t, m);
+    if (lane == 0) out[q] = t;
 }
 
 int na_fail(int code, const std::string &m)
@@ -140,20 +196,16 @@ int vlbm_diagnostics_noalloc(const double *f_dev, int n_theta, int n_phi, double
     double *part = nullptr;
     int rc = scratch_for_current_device(&part);
     if (rc) return rc;
-    VelNA c;
-    const double big = sqrt(3.0 + sqrt(6.0)), small = sqrt(3.0 - sqrt(6.0));
-    c.v[0] = -big;
-    c.v[1] = -small;
-    c.v[2] = small;
-    c.v[3] = big;
-    for (int a = 0; a < 4; ++a) {
-        const double x = c.v[a];
-        const double h5 = x * x * x * x * x - 10.0 * x * x * x + 15.0 * x;   // He_5
-        c.w[a] = 24.0 / (h5 * h5);
-    }
+    const VelNA c{sqrt(3.0 - sqrt(6.0)), sqrt(3.0 + sqrt(6.0))};
     cudaStream_t s = (cudaStream_t)stream;
-    noalloc_rows_kernel<<<n_theta, NOALLOC_THREADS, 0, s>>>(f_dev, n_theta, n_phi, radius, c, part);
-    noalloc_final_kernel<<<1, NOALLOC_THREADS, 0, s>>>(part, n_theta, out_dev);
+    // rows per CTA: two warps per scheduler (608 of them) where the grid is large enough, which
+    // saturates the FP64 pipe; within the shared row tables and the scratch's count of CTAs
+    const int chunks = (n_phi + 31) / 32, cx = (chunks + NOALLOC_THREADS / 32 - 1) / (NOALLOC_THREADS / 32);
+    const long long want = ((long long)n_theta * chunks + 1215) / 1216;
+    const int rows = (int)(want < 1 ? 1 : want > NA_ROWS_MAX ? NA_ROWS_MAX : want);
+    const int gy = (n_theta + rows - 1) / rows, gx = cx < VLBM_NOALLOC_MAX_ROWS / gy ? cx : VLBM_NOALLOC_MAX_ROWS / gy;
+    noalloc_sums_kernel<<<dim3(gx, gy), NOALLOC_THREADS, 0, s>>>(f_dev, n_theta, n_phi, radius, c, rows, part);
+    noalloc_final_kernel<<<1, 32 * NQ, 0, s>>>(part, gx * gy, out_dev);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return na_fail(VLBM_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
     return VLBM_OK;

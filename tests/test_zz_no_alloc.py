@@ -79,3 +79,30 @@ def test_noalloc_counts_the_cells_holding_a_nonfinite_population():
                                       torch.cuda.current_stream().cuda_stream)
         torch.cuda.synchronize()
         assert out[5].item() == 3.0, (call, out[5].item())
+
+
+@pytest.mark.parametrize("nt,np_", [(1, 1), (5, 4099), (300, 70), (1001, 2), (640, 1300)])
+def test_noalloc_sums_match_numpy(nt, np_):
+    """Column chunks of 32 with a remainder, one and many rows per CTA, a last CTA with fewer rows."""
+    require_gpu()
+    import torch
+
+    from paper_2504_15574_gb300 import vlbm
+    vlbm.load()
+    rng = np.random.default_rng(nt)
+    f = rng.uniform(0.5, 1.5, (16, nt, np_))
+    th, ph = (np.arange(nt) + 0.5) * np.pi / nt, (np.arange(np_) + 0.5) * 2 * np.pi / np_
+    v = np.array([-np.sqrt(3 + np.sqrt(6)), -np.sqrt(3 - np.sqrt(6)), np.sqrt(3 - np.sqrt(6)), np.sqrt(3 + np.sqrt(6))])
+    va, vb = np.repeat(v, 4), np.tile(v, 4)
+    area = 1.3**2 * np.sin(th)[:, None] * (np.pi / nt) * (2 * np.pi / np_)
+    jt, jp = np.tensordot(va, f, 1), np.tensordot(vb, f, 1)
+    st, ct, sp, cp = np.sin(th)[:, None], np.cos(th)[:, None], np.sin(ph)[None], np.cos(ph)[None]
+    ref = [(f.sum(0) * area).sum(), ((jt * ct * cp - jp * sp) * area).sum(), ((jt * ct * sp + jp * cp) * area).sum(),
+           (-jt * st * area).sum(), (0.5 * np.tensordot(va**2 + vb**2, f, 1) * area).sum(), 0.0]
+    out = torch.full((6,), float("nan"), dtype=torch.float64, device="cuda")
+    f_dev = torch.from_numpy(f).to("cuda")
+    vlbm.vlbm_diagnostics_noalloc(f_dev.data_ptr(), nt, np_, 1.3, out.data_ptr(),
+                                  torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    # FP64 sums in another order: rounding of sums of positive terms; momenta cancel, so on the mass's scale
+    np.testing.assert_allclose(out.cpu().numpy(), ref, rtol=1e-12, atol=1e-12 * ref[0])
