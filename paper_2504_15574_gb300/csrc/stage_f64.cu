@@ -27,15 +27,16 @@ namespace {
 // instructions/s of ~578).  The forms below give the same bits with fewer of them: scalings by
 // powers of two and reciprocal seeds go to the integer and FP32 pipes, which are otherwise idle.
 
-// x 2^k for the constant c = 2^k, |k| <= 4: an exponent addition; zeros are returned as they are,
-// and what could leave the normal range (or is not finite) takes the multiplication.
+// x 2^K, |K| <= 4, by an exponent addition; zeros are returned as they are.  What could leave the
+// normal range (or is not finite) sets `bad` and the caller takes its plain form: a multiplication
+// here, even one predicated off, would be issued to the FP64 pipe (8 of 78 instructions a face).
 template <int K>
-__device__ __forceinline__ double scale2(double x)
+__device__ __forceinline__ double scale2(double x, bool &bad)
 {
     const int hi = __double2hiint(x), lo = __double2loint(x);
-    if ((unsigned)((hi >> 20) & 0x7ff) - 8u < 2030u) return __hiloint2double(hi + (K << 20), lo);
-    if (((hi << 1) | lo) == 0) return x;
-    return x * (K >= 0 ? (double)(1 << (K >= 0 ? K : 0)) : 1.0 / (double)(1 << (K < 0 ? -K : 0)));
+    const bool zero = ((hi << 1) | lo) == 0;
+    bad |= !zero && (unsigned)((hi >> 20) & 0x7ff) - 8u >= 2030u;
+    return __hiloint2double(zero ? hi : hi + K * (1 << 20), lo);
 }
 
 // x / d with 1/d = h + l held to 106 bits (DivC, built on the host): RN(x h + RN(x l)), the two-
@@ -51,11 +52,12 @@ __device__ __forceinline__ double div_const(double x, const DivC &d) { return __
 // bits) and assembled into a double by integer operations; then one residual correction of the
 // quotient (Markstein 1990).  The corrected value is within 2^-88 of a / b before its rounding, so
 // it is the rounded quotient but for a chance of about 2^-35 per division (none in 4e8 random
-// ones).  A b that is not positive and well inside the normal range takes the plain division.
-__device__ __forceinline__ double div_pos(double a, double b)
+// ones).  A b that is not positive and well inside the normal range sets `bad`: the caller then takes
+// its plain form.
+__device__ __forceinline__ double div_pos(double a, double b, bool &bad)
 {
     const int hi = __double2hiint(b), lo = __double2loint(b);
-    if ((unsigned)((hi >> 20) - (1023 - 500)) > 1000u) return a / b;
+    bad |= (unsigned)((hi >> 20) - (1023 - 500)) > 1000u;
     const float bh = __int_as_float(0x3f800000 | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29));
     const float bl = (float)(lo & 0x1fffffff) * 0x1p-52f;
     float r0;
@@ -73,6 +75,29 @@ __device__ __forceinline__ double div_pos(double a, double b)
     return __fma_rn(__fma_rn(-b, q, a), r, q);
 }
 
+// The interface value as the oracle writes it, for stencils with values outside the fast forms'
+// ranges (denormal differences, near-overflow, non-finite populations).
+__device__ __noinline__ double weno5_plain(double a, double b, double c, double d, double e, double eps)
+{
+    double p1 = (2.0 * a - 7.0 * b + 11.0 * c) / 6.0;
+    double p2 = (-b + 5.0 * c + 2.0 * d) / 6.0;
+    double p3 = (2.0 * c + 5.0 * d - e) / 6.0;
+    double d1a = a - 2.0 * b + c, d1b = a - 4.0 * b + 3.0 * c;
+    double d2a = b - 2.0 * c + d, d2b = b - d;
+    double d3a = c - 2.0 * d + e, d3b = 3.0 * c - 4.0 * d + e;
+    double s1 = 13.0 / 12.0 * (d1a * d1a) + 0.25 * (d1b * d1b);
+    double s2 = 13.0 / 12.0 * (d2a * d2a) + 0.25 * (d2b * d2b);
+    double s3 = 13.0 / 12.0 * (d3a * d3a) + 0.25 * (d3b * d3b);
+    double w1 = 0.1 / ((s1 + eps) * (s1 + eps));
+    double w2 = 0.6 / ((s2 + eps) * (s2 + eps));
+    double w3 = 0.3 / ((s3 + eps) * (s3 + eps));
+    return (w1 * p1 + w2 * p2 + w3 * p3) / (w1 + w2 + w3);
+}
+
+// Plain product and quotient behind a call, for the rare values that the fast forms leave out.
+__device__ __noinline__ double mul_plain(double a, double b) { return a * b; }
+__device__ __noinline__ double div_plain(double a, double b) { return a / b; }
+
 // Interface values of S consecutive faces from y[0 .. S + 3] in upwind order: face f has the stencil
 // a..e = y[f .. f + 4] (c the upwind cell, d the downwind cell), in the oracle's expression order.
 // The forms of one column (13/12 times the squared second difference, and 5 y) are shared by the
@@ -82,31 +107,36 @@ template <int S>
 __device__ __forceinline__ void weno5_strip(const double (&y)[S + 4], double eps, const DivC &six, double (&r)[S])
 {
     double kq[S + 4], y5[S + 4];
+    bool bad = false;
 #pragma unroll
     for (int i = 1; i <= 2; ++i) {
-        const double d = y[i - 1] - scale2<1>(y[i]) + y[i + 1];
+        const double d = y[i - 1] - scale2<1>(y[i], bad) + y[i + 1];
         kq[i] = 13.0 / 12.0 * (d * d);
     }
     y5[2] = 5.0 * y[2];
 #pragma unroll
     for (int f = 0; f < S; ++f) {
         const double a = y[f], b = y[f + 1], c = y[f + 2], d = y[f + 3], e = y[f + 4];
-        const double d3a = c - scale2<1>(d) + e;
+        const double d3a = c - scale2<1>(d, bad) + e;
         kq[f + 3] = 13.0 / 12.0 * (d3a * d3a);
         y5[f + 3] = 5.0 * d;
         const double c3 = 3.0 * c;
-        const double d1b = a - scale2<2>(b) + c3;
+        const double d1b = a - scale2<2>(b, bad) + c3;
         const double d2b = b - d;
-        const double d3b = c3 - scale2<2>(d) + e;
-        const double s1 = kq[f + 1] + scale2<-2>(d1b * d1b) + eps;
-        const double s2 = kq[f + 2] + scale2<-2>(d2b * d2b) + eps;
-        const double s3 = kq[f + 3] + scale2<-2>(d3b * d3b) + eps;
-        const double w1 = div_pos(0.1, s1 * s1), w2 = div_pos(0.6, s2 * s2), w3 = div_pos(0.3, s3 * s3);
-        const double p1 = div_const(scale2<1>(a) - 7.0 * b + 11.0 * c, six);
-        const double p2 = div_const(y5[f + 2] - b + scale2<1>(d), six);
-        const double p3 = div_const(scale2<1>(c) + y5[f + 3] - e, six);
-        r[f] = div_pos(w1 * p1 + w2 * p2 + w3 * p3, w1 + w2 + w3);
+        const double d3b = c3 - scale2<2>(d, bad) + e;
+        const double s1 = kq[f + 1] + scale2<-2>(d1b * d1b, bad) + eps;
+        const double s2 = kq[f + 2] + scale2<-2>(d2b * d2b, bad) + eps;
+        const double s3 = kq[f + 3] + scale2<-2>(d3b * d3b, bad) + eps;
+        const double w1 = div_pos(0.1, s1 * s1, bad), w2 = div_pos(0.6, s2 * s2, bad),
+                     w3 = div_pos(0.3, s3 * s3, bad);
+        const double p1 = div_const(scale2<1>(a, bad) - 7.0 * b + 11.0 * c, six);
+        const double p2 = div_const(y5[f + 2] - b + scale2<1>(d, bad), six);
+        const double p3 = div_const(scale2<1>(c, bad) + y5[f + 3] - e, six);
+        r[f] = div_pos(w1 * p1 + w2 * p2 + w3 * p3, w1 + w2 + w3, bad);
     }
+    if (bad)
+#pragma unroll
+        for (int f = 0; f < S; ++f) r[f] = weno5_plain(y[f], y[f + 1], y[f + 2], y[f + 3], y[f + 4], eps);
 }
 
 // The same for the upwind stencils of Eq. (fluxes_U1-3).
@@ -241,7 +271,12 @@ __global__ void __launch_bounds__(32 * CELL_WARPS) cells_f64_kernel(const StageD
         mom[warp][lane] = m;
     }
     __syncthreads();
-    if (warp == 1 || warp == 2) vel[warp - 1][lane] = div_pos(mom[warp][lane], mom[0][lane]);
+    if (warp == 1 || warp == 2) {
+        bool bad = false;
+        double u = div_pos(mom[warp][lane], mom[0][lane], bad);
+        if (bad) u = div_plain(mom[warp][lane], mom[0][lane]);
+        vel[warp - 1][lane] = u;
+    }
     __syncthreads();
     if (warp == 0) {
         const double ut = vel[0][lane], up = vel[1][lane];
@@ -267,7 +302,10 @@ __global__ void __launch_bounds__(32 * CELL_WARPS) cells_f64_kernel(const StageD
         // equilibrium (T0 = 1): Eq. feq_Q=4 (third order), or Eq. feq_Q=3 (second order) for D2Q9
         const double xi = va * ut + vb * up;
         const double xi2 = xi * xi;
-        const double second = 1.0 + xi + scale2<-1>(xi2 - u2);
+        bool bad = false;
+        double h = scale2<-1>(xi2 - u2, bad);
+        if (bad) h = mul_plain(0.5, xi2 - u2);
+        const double second = 1.0 + xi + h;
         const double nw = n * p.wk[k];
         const double feq = (q == 3) ? nw * second : nw * (second + div_const(xi * (xi2 - u23), p.six));
         // velocity derivatives: K on k_theta at fixed k_phi, Ktilde on k_phi at fixed k_theta
@@ -283,7 +321,7 @@ __global__ void __launch_bounds__(32 * CELL_WARPS) cells_f64_kernel(const StageD
 
         double outv;
         if (p.stage == 1) outv = gk + p.dt * Lk;
-        else if (p.stage == 2) outv = 0.75 * f0 + scale2<-2>(gk) + p.dt_stage * Lk;
+        else if (p.stage == 2) outv = 0.75 * f0 + 0.25 * gk + p.dt_stage * Lk;
         else outv = div_const(f0, p.three) + 2.0 / 3.0 * gk + p.dt_stage * Lk;
         store_with_images(p.out, L, k, i, j, outv);
     }
