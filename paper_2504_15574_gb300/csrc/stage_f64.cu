@@ -14,6 +14,7 @@
 // kernel updates the cells.  It is not the throughput path (that is stage_f32.cu);
 // it shares the ghost-row layout so that all reads are plain loads.
 #include "vlbm_internal.h"
+#include "f64_int.cuh"
 
 namespace vk {
 
@@ -24,20 +25,9 @@ namespace {
 // stage's time is its FP64 instruction count: 135 per interface value and 105 per population and
 // cell when every division was the compiler's and every stencil form was evaluated per face (490,
 // 487 and 384 us for the phi faces, theta faces and cells of a 256 x 512 stage, 535 G FP64
-// instructions/s of ~578).  The forms below give the same bits with fewer of them: scalings by
-// powers of two and reciprocal seeds go to the integer and FP32 pipes, which are otherwise idle.
-
-// x 2^K, |K| <= 4, by an exponent addition; zeros are returned as they are.  What could leave the
-// normal range (or is not finite) sets `bad` and the caller takes its plain form: a multiplication
-// here, even one predicated off, would be issued to the FP64 pipe (8 of 78 instructions a face).
-template <int K>
-__device__ __forceinline__ double scale2(double x, bool &bad)
-{
-    const int hi = __double2hiint(x), lo = __double2loint(x);
-    const bool zero = ((hi << 1) | lo) == 0;
-    bad |= !zero && (unsigned)((hi >> 20) & 0x7ff) - 8u >= 2030u;
-    return __hiloint2double(zero ? hi : hi + K * (1 << 20), lo);
-}
+// instructions/s of ~610).  The forms below give the same bits with fewer of them: most products go
+// to the integer pipe (f64_int.cuh; issue slots were 11 % used), scalings by powers of two become
+// exponent additions, and reciprocal seeds come from the FP32 pipe.
 
 // x / d with 1/d = h + l held to 106 bits (DivC, built on the host): RN(x h + RN(x l)), the two-
 // operation multiplication by an arbitrary-precision constant of Brisebarre and Muller ("Correctly
@@ -47,17 +37,18 @@ __device__ __forceinline__ double scale2(double x, bool &bad)
 // positive, so infinities pass through.
 __device__ __forceinline__ double div_const(double x, const DivC &d) { return __fma_rn(x, d.h, __dmul_rn(x, d.l)); }
 
-// a / b with three FP64 operations: a reciprocal of b good to 2^-44 is formed in FP32 (the leading
-// 24 bits of b's significand through the hardware reciprocal, one error term with the remaining
-// bits) and assembled into a double by integer operations; then one residual correction of the
-// quotient (Markstein 1990).  The corrected value is within 2^-88 of a / b before its rounding, so
-// it is the rounded quotient but for a chance of about 2^-35 per division (none in 4e8 random
-// ones).  A b that is not positive and well inside the normal range sets `bad`: the caller then takes
-// its plain form.
-__device__ __forceinline__ double div_pos(double a, double b, bool &bad)
+// The same with the product by l on the integer pipe; x zero or well inside the normal range.
+__device__ __forceinline__ double div_const_int(double x, const DivC &d)
+{
+    return __fma_rn(x, d.h, mul_int_z(x, d.l));
+}
+
+// 1 / b to 2^-44 for a positive b in [2^-500, 2^500]: the leading 24 bits of b's significand through
+// the hardware's FP32 reciprocal, one error term with the remaining bits, assembled into a double by
+// integer operations.
+__device__ __forceinline__ double recip_seed(double b)
 {
     const int hi = __double2hiint(b), lo = __double2loint(b);
-    bad |= (unsigned)((hi >> 20) - (1023 - 500)) > 1000u;
     const float bh = __int_as_float(0x3f800000 | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29));
     const float bl = (float)(lo & 0x1fffffff) * 0x1p-52f;
     float r0;
@@ -70,14 +61,22 @@ __device__ __forceinline__ double div_pos(double a, double b, bool &bad)
     long long bits = ((long long)((u >> 3) + ((1023 - 127) << 20)) << 32) | (unsigned)(u << 29);
     bits += i1;
     bits -= (long long)((hi >> 20) - 1023) << 52;
-    const double r = __longlong_as_double(bits);
-    const double q = __dmul_rn(a, r);
+    return __longlong_as_double(bits);
+}
+
+// a / b for such a b: the product with the seed on the integer pipe (a zero or well inside the normal
+// range), then one residual correction in two FP64 operations (Markstein 1990).  The corrected
+// value is within 2^-88 of a / b before its rounding, so it is the rounded quotient but for a chance
+// of about 2^-35 per division (none in 4e8 random ones).
+__device__ __forceinline__ double div_pos(double a, double b)
+{
+    const double r = recip_seed(b), q = mul_int_z(a, r);
     return __fma_rn(__fma_rn(-b, q, a), r, q);
 }
 
-// The interface value as the oracle writes it, for stencils with values outside the fast forms'
-// ranges (denormal differences, near-overflow, non-finite populations).
-__device__ __noinline__ double weno5_plain(double a, double b, double c, double d, double e, double eps)
+// Interface flux v r of a stencil with values outside the fast forms' range (beyond [2^-400, 2^100)
+// and not zero, or not finite), with the interface value r as the oracle writes it.
+__device__ __noinline__ double weno5_plain(double a, double b, double c, double d, double e, double eps, double v)
 {
     double p1 = (2.0 * a - 7.0 * b + 11.0 * c) / 6.0;
     double p2 = (-b + 5.0 * c + 2.0 * d) / 6.0;
@@ -91,63 +90,79 @@ __device__ __noinline__ double weno5_plain(double a, double b, double c, double 
     double w1 = 0.1 / ((s1 + eps) * (s1 + eps));
     double w2 = 0.6 / ((s2 + eps) * (s2 + eps));
     double w3 = 0.3 / ((s3 + eps) * (s3 + eps));
-    return (w1 * p1 + w2 * p2 + w3 * p3) / (w1 + w2 + w3);
+    return v * ((w1 * p1 + w2 * p2 + w3 * p3) / (w1 + w2 + w3));
 }
 
-// Plain product and quotient behind a call, for the rare values that the fast forms leave out.
-__device__ __noinline__ double mul_plain(double a, double b) { return a * b; }
-__device__ __noinline__ double div_plain(double a, double b) { return a / b; }
-
-// Interface values of S consecutive faces from y[0 .. S + 3] in upwind order: face f has the stencil
-// a..e = y[f .. f + 4] (c the upwind cell, d the downwind cell), in the oracle's expression order.
-// The forms of one column (13/12 times the squared second difference, and 5 y) are shared by the
-// three candidate stencils centred on it, which changes no bit: 45 + 4 divisions of 3 FP64
-// operations per face.
-template <int S>
-__device__ __forceinline__ void weno5_strip(const double (&y)[S + 4], double eps, const DivC &six, double (&r)[S])
+// Walks n consecutive WENO-5 faces from the values load(0), load(1), ... in upwind order: face f has the
+// stencil a..e = values f .. f + 4 (c the upwind cell, d the downwind cell), in the oracle's
+// expression order, and gives its flux to store(f, flux), v times the interface value (store_r: the
+// value itself, for the Komissarov factor).  The forms of one column (13/12 times the squared second
+// difference, and 5 y) are shared by the three candidate stencils centred on it, which changes no
+// bit.  34 FP64 instructions a face: with every value zero or in [2^-400, 2^100), differences are
+// zero or multiples of the smallest ulp, so no product leaves the normal range.
+template <class Load, class Store>
+__device__ __forceinline__ void weno5_walk(int n, bool plain, double eps, double v, const DivC &six, Load load,
+                                           Store store)
 {
-    double kq[S + 4], y5[S + 4];
-    bool bad = false;
-#pragma unroll
-    for (int i = 1; i <= 2; ++i) {
-        const double d = y[i - 1] - scale2<1>(y[i], bad) + y[i + 1];
-        kq[i] = 13.0 / 12.0 * (d * d);
-    }
-    y5[2] = 5.0 * y[2];
-#pragma unroll
-    for (int f = 0; f < S; ++f) {
-        const double a = y[f], b = y[f + 1], c = y[f + 2], d = y[f + 3], e = y[f + 4];
-        const double d3a = c - scale2<1>(d, bad) + e;
-        kq[f + 3] = 13.0 / 12.0 * (d3a * d3a);
-        y5[f + 3] = 5.0 * d;
-        const double c3 = 3.0 * c;
-        const double d1b = a - scale2<2>(b, bad) + c3;
+    double a = load(0), b = load(1), c = load(2), d = load(3), e = load(4);
+    const double vb = a - scale2<1>(b) + c, vc = b - scale2<1>(c) + d;
+    const double c1312 = 13.0 / 12.0;
+    double k1 = mul_int_z(sq_int(vb), c1312), k2 = mul_int_z(sq_int(vc), c1312), c5 = mul_small<5>(c);
+    // values still to be walked over that are outside the range keep the next faces on the plain form
+    int out = 0;
+    if (!(f64_within<400, 100>(a))) out = 1;
+    if (!(f64_within<400, 100>(b))) out = 2;
+    if (!(f64_within<400, 100>(c))) out = 3;
+    if (!(f64_within<400, 100>(d))) out = 4;
+#pragma unroll 1
+    for (int f = 0; f < n; ++f) {
+        const double next = load(min(f + 5, n + 3));
+        if (!(f64_within<400, 100>(e))) out = 5;
+        const double d3a = c - scale2<1>(d) + e;
+        const double k3 = mul_int_z(sq_int(d3a), c1312);
+        const double d5 = mul_small<5>(d), c3 = mul_small<3>(c);
+        const double d1b = a - scale2<2>(b) + c3;
         const double d2b = b - d;
-        const double d3b = c3 - scale2<2>(d, bad) + e;
-        const double s1 = kq[f + 1] + scale2<-2>(d1b * d1b, bad) + eps;
-        const double s2 = kq[f + 2] + scale2<-2>(d2b * d2b, bad) + eps;
-        const double s3 = kq[f + 3] + scale2<-2>(d3b * d3b, bad) + eps;
-        const double w1 = div_pos(0.1, s1 * s1, bad), w2 = div_pos(0.6, s2 * s2, bad),
-                     w3 = div_pos(0.3, s3 * s3, bad);
-        const double p1 = div_const(scale2<1>(a, bad) - 7.0 * b + 11.0 * c, six);
-        const double p2 = div_const(y5[f + 2] - b + scale2<1>(d, bad), six);
-        const double p3 = div_const(scale2<1>(c, bad) + y5[f + 3] - e, six);
-        r[f] = div_pos(w1 * p1 + w2 * p2 + w3 * p3, w1 + w2 + w3, bad);
+        const double d3b = c3 - scale2<2>(d) + e;
+        const double s1 = k1 + scale2<-2>(sq_int(d1b)) + eps;
+        const double s2 = k2 + scale2<-2>(sq_int(d2b)) + eps;
+        const double s3 = k3 + scale2<-2>(sq_int(d3b)) + eps;
+        const double w1 = div_pos(0.1, mul_int(s1, s1)), w2 = div_pos(0.6, mul_int(s2, s2)),
+                     w3 = div_pos(0.3, mul_int(s3, s3));
+        const double p1 = div_const_int(scale2<1>(a) - mul_small<7>(b) + mul_small<11>(c), six);
+        const double p2 = div_const_int(c5 - b + scale2<1>(d), six);
+        const double p3 = div_const_int(scale2<1>(c) + d5 - e, six);
+        const double num = mul_int_z(p1, w1) + mul_int_z(p2, w2) + mul_int_z(p3, w3);
+        const double r = div_pos(num, w1 + w2 + w3);
+        double flux = mul_int_zz(r, v);   // (v = 0: a D2Q9 population at rest along the axis)
+        if (plain || out > 0 || !f64_within<500, 500>(num)) flux = weno5_plain(a, b, c, d, e, eps, v);
+        store(f, flux);
+        --out;
+        a = b;
+        b = c;
+        c = d;
+        d = e;
+        e = next;
+        k1 = k2;
+        k2 = k3;
+        c5 = d5;
     }
-    if (bad)
-#pragma unroll
-        for (int f = 0; f < S; ++f) r[f] = weno5_plain(y[f], y[f + 1], y[f + 2], y[f + 3], y[f + 4], eps);
 }
 
 // The same for the upwind stencils of Eq. (fluxes_U1-3).
-template <int S>
-__device__ __forceinline__ void upwind_strip(int scheme, const double (&y)[S + 4], const DivC &six, double (&r)[S])
+template <class Load, class Store>
+__device__ __forceinline__ void upwind_walk(int n, int scheme, double v, const DivC &six, Load load, Store store)
 {
-#pragma unroll
-    for (int f = 0; f < S; ++f) {
-        const double b = y[f + 1], c = y[f + 2], d = y[f + 3];
-        r[f] = (scheme == VLBM_U1) ? c : (scheme == VLBM_U2) ? 1.5 * c - 0.5 * b
-                                                             : div_const(2.0 * d + 5.0 * c - b, six);
+    double b = load(1), c = load(2), d = load(3);
+#pragma unroll 1
+    for (int f = 0; f < n; ++f) {
+        const double next = load(min(f + 4, n + 3));
+        const double r = (scheme == VLBM_U1) ? c : (scheme == VLBM_U2) ? 1.5 * c - 0.5 * b
+                                                                       : div_const(2.0 * d + 5.0 * c - b, six);
+        store(f, v * r);
+        b = c;
+        c = d;
+        d = next;
     }
 }
 
@@ -178,67 +193,105 @@ __device__ __forceinline__ void store_with_images(T *f, const Layout &L, int k, 
 // column.  Phi flux through interface fj (between columns fj-1 and fj, fj = 0..np) of row i; a
 // thread walks S columns of one row.  For a negative velocity the strip is walked backwards, which
 // puts its values in upwind order.  The first nb_phi CTAs take the phi faces, the others the theta
-// faces (one launch: on small grids either alone leaves schedulers idle).
-// Bound: the FP64 pipe (57 operations a face; 240 us for the 4.2 M faces of 256 x 512, D2Q16, by
-// count).  Long strips share the column forms, short ones spread a small grid over more
-// schedulers: launch_stage_f64 picks S.
-template <int S>
-__global__ void __launch_bounds__(128) faces_f64_kernel(const StageD p, int nb_phi)
+// faces (one launch: on small grids either alone leaves schedulers idle).  The walk is a rolled
+// loop: unrolled, its 1,000 instructions a face would not stay in the instruction cache.
+__global__ void __launch_bounds__(128) faces_f64_kernel(const StageD p, int nb_phi, int S)
 {
     const Layout L = p.L;
-    const int q = p.c.q;
-    const bool theta = (int)blockIdx.x >= nb_phi;
-    double y[S + 4], r[S];
-    if (!theta) {
+    const int q = p.c.q, k = blockIdx.y;
+    if ((int)blockIdx.x < nb_phi) {
         const int ns = (L.np + S) / S;   // strips of the np + 1 faces
         const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-        const int k = blockIdx.y;
         if (t >= (long long)ns * L.nt) return;
-        const int i = (int)(t / ns), f0 = (int)(t - (long long)i * ns) * S;
+        const int i = (int)(t / ns), f0 = (int)(t - (long long)i * ns) * S, n = min(S, L.np + 1 - f0);
         const double vb = p.c.v[k % q];
         const int dir = vb > 0.0 ? 1 : -1;
-        // y[m] = column c0 + dir m; a strip that reaches past the last face reads the last column in store
-        const int c0 = dir > 0 ? f0 - 3 : f0 + S + 1;
-        const double *g = p.in + L.at(k, i, 0);
-#pragma unroll
-        for (int m = 0; m < S + 4; ++m) y[m] = g[min(c0 + dir * m, L.np + GC - 1)];
-        if (p.scheme == VLBM_WENO5) weno5_strip<S>(y, p.eps, p.six, r);
-        else upwind_strip<S>(p.scheme, y, p.six, r);
-        double *out = p.Fp + ((size_t)k * L.nt + i) * (L.np + 1);
-#pragma unroll
-        for (int f = 0; f < S; ++f) {
-            const int fj = dir > 0 ? f0 + f : f0 + S - 1 - f;
-            if (fj <= L.np) out[fj] = vb * r[f];
-        }
+        // value m is column f0 - 3 + m, or (backwards) column f0 + n + 1 - m
+        const double *g = p.in + L.at(k, i, dir > 0 ? f0 - 3 : f0 + n + 1);
+        double *out = p.Fp + ((size_t)k * L.nt + i) * (L.np + 1) + (dir > 0 ? f0 : f0 + n - 1);
+        auto load = [&](int m) { return g[dir * m]; };
+        auto store = [&](int f, double flux) { out[dir * f] = flux; };
+        if (p.scheme == VLBM_WENO5) weno5_walk(n, p.plain, p.eps, vb, p.six, load, store);
+        else upwind_walk(n, p.scheme, vb, p.six, load, store);
         return;
     }
     const int ns = (L.nt + S) / S;
     const long long t = (long long)(blockIdx.x - nb_phi) * blockDim.x + threadIdx.x;
-    const int k = blockIdx.y;
     if (t >= (long long)ns * L.np) return;
-    const int st = (int)(t / L.np), j = (int)(t - (long long)st * L.np), f0 = st * S;
+    const int st = (int)(t / L.np), j = (int)(t - (long long)st * L.np), f0 = st * S, n = min(S, L.nt + 1 - f0);
     const double va = p.c.v[k / q];
     const int dir = va > 0.0 ? 1 : -1;
-    const int r0 = dir > 0 ? f0 - 3 : f0 + S + 1;
-#pragma unroll
-    for (int m = 0; m < S + 4; ++m) {
-        const int row = min(r0 + dir * m, L.nt + GR - 1);
-        const double v = p.in[L.at(k, row, j)];
-        y[m] = p.komissarov ? v : p.sin_ext[row + GR] * v;
-    }
-    if (p.scheme == VLBM_WENO5) weno5_strip<S>(y, p.eps, p.six, r);
-    else upwind_strip<S>(p.scheme, y, p.six, r);
-#pragma unroll
-    for (int f = 0; f < S; ++f) {
-        const int fi = dir > 0 ? f0 + f : f0 + S - 1 - f;
-        if (fi > L.nt) continue;
-        const double flux = p.komissarov ? va * p.sin_f[fi] * r[f] : va * r[f];
+    const int r0 = dir > 0 ? f0 - 3 : f0 + n + 1;
+    auto load = [&](int m) {
+        const int row = r0 + dir * m;
+        const double x = p.in[L.at(k, row, j)];
+        return p.komissarov ? x : p.sin_ext[row + GR] * x;
+    };
+    auto store = [&](int f, double flux) {
+        const int fi = dir > 0 ? f0 + f : f0 + n - 1 - f;
         p.Ft[((size_t)k * (L.nt + 1) + fi) * L.np + j] = flux;
         if (p.pole) {
             if (fi == 0) p.pole[(size_t)k * L.np + j] = flux;
             if (fi == L.nt) p.pole[((size_t)NK + k) * L.np + j] = flux;
         }
+    };
+    // (Komissarov: the walk gives the value itself, the flux is v_theta sin(theta_fi) times it)
+    auto store_kom = [&](int f, double r) {
+        const int fi = dir > 0 ? f0 + f : f0 + n - 1 - f;
+        store(f, va * p.sin_f[fi] * r);
+    };
+    if (p.scheme == VLBM_WENO5) {
+        if (p.komissarov) weno5_walk(n, p.plain, p.eps, 1.0, p.six, load, store_kom);
+        else weno5_walk(n, p.plain, p.eps, va, p.six, load, store);
+    } else if (p.komissarov) {
+        upwind_walk(n, p.scheme, 1.0, p.six, load, store_kom);
+    } else {
+        upwind_walk(n, p.scheme, va, p.six, load, store);
     }
+}
+
+// One population's update of one cell.  FAST: products on the integer pipe, for populations that are
+// zero or in [2^-40, 2^100) and a positive density (then every product here is zero or normal).
+template <bool FAST>
+__device__ __forceinline__ void cell_update(const StageD &p, const Layout &L, const RowD &rd,
+                                            const double (*gs)[32], int lane, int i, int j, int k, double n,
+                                            double ut, double up, double u2, double u23)
+{
+    auto mul = [](double a, double b) { return FAST ? mul_int_zz(a, b) : a * b; };
+    auto divc = [](double a, const DivC &d) { return FAST ? div_const_int(a, d) : div_const(a, d); };
+    const int q = p.c.q, a = k / q, b = k % q;
+    const double va = p.c.v[a], vb = p.c.v[b];
+    const double gk = gs[k][lane];
+    // loaded ahead of the arithmetic
+    const double fn = p.Ft[((size_t)k * (L.nt + 1) + i) * L.np + j];
+    const double fs = p.Ft[((size_t)k * (L.nt + 1) + i + 1) * L.np + j];
+    const double fw = p.Fp[((size_t)k * L.nt + i) * (L.np + 1) + j];
+    const double fe = p.Fp[((size_t)k * L.nt + i) * (L.np + 1) + j + 1];
+    const double f0 = (p.stage == 1) ? 0.0 : p.fold[L.at(k, i, j)];
+    // equilibrium (T0 = 1): Eq. feq_Q=4 (third order), or Eq. feq_Q=3 (second order) for D2Q9
+    const double xi = mul(va, ut) + mul(vb, up);
+    const double xi2 = mul(xi, xi);
+    const double half = xi2 - u2;
+    const double second = 1.0 + xi + (FAST ? scale2<-1>(half) : 0.5 * half);
+    const double nw = mul(n, p.wk[k]);
+    const double feq = (q == 3) ? mul(nw, second) : mul(nw, second + divc(mul(xi, xi2 - u23), p.six));
+    // velocity derivatives: K on k_theta at fixed k_phi, Ktilde on k_phi at fixed k_theta
+    double kg = mul(p.c.K[a * q], gs[b][lane]), ktg = mul(p.c.Kt[b * q], gs[q * a][lane]);
+#pragma unroll 1
+    for (int m = 1; m < q; ++m) {
+        kg += mul(p.c.K[a * q + m], gs[q * m + b][lane]);
+        ktg += mul(p.c.Kt[b * q + m], gs[q * a + m][lane]);
+    }
+    const double force = mul(rd.cotR, mul(p.vb2[b], kg) - mul(va, ktg));
+    const double adv_t = -div_const(fs - fn, rd.th);
+    const double adv_p = -div_const(fe - fw, rd.ph);
+    const double Lk = adv_t + adv_p - force - divc(gk - feq, p.tau_div);
+
+    double outv;
+    if (p.stage == 1) outv = gk + p.dt * Lk;
+    else if (p.stage == 2) outv = 0.75 * f0 + (FAST ? scale2<-2>(gk) : 0.25 * gk) + p.dt_stage * Lk;
+    else outv = div_const(f0, p.three) + mul(2.0 / 3.0, gk) + p.dt_stage * Lk;
+    store_with_images(p.out, L, k, i, j, outv);
 }
 
 // Cells of one stage: moments, equilibrium, force, BGK, the flux differences of the interface
@@ -260,23 +313,30 @@ __global__ void __launch_bounds__(32 * CELL_WARPS) cells_f64_kernel(const StageD
     const long long cell = (long long)blockIdx.x * 32 + lane;
     const bool in = cell < cells;
     const int i = in ? (int)(cell / L.np) : 0, j = in ? (int)(cell - (long long)i * L.np) : 0;
-    for (int k = warp; k < nk; k += CELL_WARPS) gs[k][lane] = p.in[L.at(k, i, j)];
-    __syncthreads();
+    bool out = p.plain;
+    for (int k = warp; k < nk; k += CELL_WARPS) {
+        const double g = p.in[L.at(k, i, j)];
+        out |= !f64_within<40, 100>(g);
+        gs[k][lane] = g;
+    }
+    const bool plain = __syncthreads_or(out);
     if (warp < 3) {
         double m = 0.0;
-        for (int k = 0; k < nk; ++k) {
-            const double g = gs[k][lane];
-            m += (warp == 0) ? g : g * p.c.v[warp == 1 ? k / q : k % q];
+        if (warp == 0) {
+            for (int k = 0; k < nk; ++k) m += gs[k][lane];
+        } else {
+            for (int k = 0; k < nk; ++k) {
+                const double g = gs[k][lane], v = p.c.v[warp == 1 ? k / q : k % q];
+                m += plain ? g * v : mul_int_zz(g, v);
+            }
         }
         mom[warp][lane] = m;
     }
     __syncthreads();
-    if (warp == 1 || warp == 2) {
-        bool bad = false;
-        double u = div_pos(mom[warp][lane], mom[0][lane], bad);
-        if (bad) u = div_plain(mom[warp][lane], mom[0][lane]);
-        vel[warp - 1][lane] = u;
-    }
+    // (a density that is not positive takes the plain forms: its velocities may be of any size)
+    const double n = mom[0][lane];
+    const bool slow = plain || !(n > 0.0) || !f64_within<110, 110>(n);
+    if (warp == 1 || warp == 2) vel[warp - 1][lane] = slow ? mom[warp][lane] / n : div_pos(mom[warp][lane], n);
     __syncthreads();
     if (warp == 0) {
         const double ut = vel[0][lane], up = vel[1][lane];
@@ -286,44 +346,12 @@ __global__ void __launch_bounds__(32 * CELL_WARPS) cells_f64_kernel(const StageD
     }
     __syncthreads();
     if (!in) return;
-    const double n = mom[0][lane], ut = vel[0][lane], up = vel[1][lane], u2 = vel[2][lane], u23 = vel[3][lane];
+    const double ut = vel[0][lane], up = vel[1][lane], u2 = vel[2][lane], u23 = vel[3][lane];
     const RowD rd = p.row[i];
 #pragma unroll 1
     for (int k = warp; k < nk; k += CELL_WARPS) {
-        const int a = k / q, b = k % q;
-        const double va = p.c.v[a], vb = p.c.v[b];
-        const double gk = gs[k][lane];
-        // loaded ahead of the arithmetic
-        const double fn = p.Ft[((size_t)k * (L.nt + 1) + i) * L.np + j];
-        const double fs = p.Ft[((size_t)k * (L.nt + 1) + i + 1) * L.np + j];
-        const double fw = p.Fp[((size_t)k * L.nt + i) * (L.np + 1) + j];
-        const double fe = p.Fp[((size_t)k * L.nt + i) * (L.np + 1) + j + 1];
-        const double f0 = (p.stage == 1) ? 0.0 : p.fold[L.at(k, i, j)];
-        // equilibrium (T0 = 1): Eq. feq_Q=4 (third order), or Eq. feq_Q=3 (second order) for D2Q9
-        const double xi = va * ut + vb * up;
-        const double xi2 = xi * xi;
-        bool bad = false;
-        double h = scale2<-1>(xi2 - u2, bad);
-        if (bad) h = mul_plain(0.5, xi2 - u2);
-        const double second = 1.0 + xi + h;
-        const double nw = n * p.wk[k];
-        const double feq = (q == 3) ? nw * second : nw * (second + div_const(xi * (xi2 - u23), p.six));
-        // velocity derivatives: K on k_theta at fixed k_phi, Ktilde on k_phi at fixed k_theta
-        double kg = p.c.K[a * q] * gs[b][lane], ktg = p.c.Kt[b * q] * gs[q * a][lane];
-        for (int m = 1; m < q; ++m) {
-            kg += p.c.K[a * q + m] * gs[q * m + b][lane];
-            ktg += p.c.Kt[b * q + m] * gs[q * a + m][lane];
-        }
-        const double force = rd.cotR * (p.vb2[b] * kg - va * ktg);
-        const double adv_t = -div_const(fs - fn, rd.th);
-        const double adv_p = -div_const(fe - fw, rd.ph);
-        const double Lk = adv_t + adv_p - force - div_const(gk - feq, p.tau_div);
-
-        double outv;
-        if (p.stage == 1) outv = gk + p.dt * Lk;
-        else if (p.stage == 2) outv = 0.75 * f0 + 0.25 * gk + p.dt_stage * Lk;
-        else outv = div_const(f0, p.three) + 2.0 / 3.0 * gk + p.dt_stage * Lk;
-        store_with_images(p.out, L, k, i, j, outv);
+        if (slow) cell_update<false>(p, L, rd, gs, lane, i, j, k, n, ut, up, u2, u23);
+        else cell_update<true>(p, L, rd, gs, lane, i, j, k, n, ut, up, u2, u23);
     }
 }
 
@@ -421,25 +449,18 @@ __global__ void filter_kernel(T *f, const Layout L, const int *rows, const int *
 
 }  // namespace
 
-template <int S>
-static void launch_faces(const StageD &p, cudaStream_t s)
-{
-    const Layout &L = p.L;
-    const long long sp = (long long)((L.np + S) / S) * L.nt, stt = (long long)((L.nt + S) / S) * L.np;
-    const int nb = (int)((sp + 127) / 128), nt = (int)((stt + 127) / 128);
-    faces_f64_kernel<S><<<dim3(nb + nt, L.nk), 128, 0, s>>>(p, nb);
-}
-
 void launch_stage_f64(const StageD &p, cudaStream_t s)
 {
-    // Strip length of the face walk: 8 faces share their column forms best (64 FP64 operations a
-    // face at S = 1, 59 at 8); a grid with fewer faces than about two warps of long strips per
-    // scheduler (608 of them) takes shorter ones, since a lone warp's chain of FP64 operations
-    // bounds the launch there.
-    const long long faces = 2LL * p.L.nk * p.L.nt * p.L.np, lanes = 2LL * 608 * 32;
-    if (faces >= 8 * lanes) launch_faces<8>(p, s);
-    else if (faces >= 2 * lanes) launch_faces<2>(p, s);
-    else launch_faces<1>(p, s);
+    // Strip length of the face walk: long strips share their column forms best (the first face of a
+    // strip forms two columns more); a grid with fewer faces than about two warps of long strips per
+    // scheduler (608 of them) takes shorter ones, since a lone warp's chain of operations bounds
+    // the launch there.
+    const Layout &L = p.L;
+    const long long faces = 2LL * L.nk * L.nt * L.np, lanes = 2LL * 608 * 32;
+    const int S = faces >= 16 * lanes ? 16 : faces >= 8 * lanes ? 8 : faces >= 4 * lanes ? 4 : faces >= 2 * lanes ? 2 : 1;
+    const long long sp = (long long)((L.np + S) / S) * L.nt, stt = (long long)((L.nt + S) / S) * L.np;
+    const int nb = (int)((sp + 127) / 128), nt = (int)((stt + 127) / 128);
+    faces_f64_kernel<<<dim3(nb + nt, L.nk), 128, 0, s>>>(p, nb, S);
     const long long cells = (long long)p.L.nt * p.L.np;
     cells_f64_kernel<<<(unsigned)((cells + 31) / 32), 32 * CELL_WARPS, 0, s>>>(p);
 }

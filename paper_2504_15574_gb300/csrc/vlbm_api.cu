@@ -504,6 +504,8 @@ void enqueue_step(vlbm_t *h, int stage_only = 0, int part = 0)
             p.dt_stage = (st == 1) ? h->dt : (st == 2) ? 0.25 * h->dt : 2.0 / 3.0 * h->dt;
             p.eps = h->eps;
             p.tau_div = div_const_of(h->tau);
+            // the fast forms bound every factor by the populations' range: options far outside take plain ones
+            p.plain = !(h->eps > 1e-60 && h->eps < 1e30 && h->tau > 1e-30 && h->tau < 1e30 && h->R > 1e-30 && h->R < 1e30);
             p.six = div_const_of(6.0);
             p.three = div_const_of(3.0);
             p.stage = st;

@@ -59,6 +59,7 @@ struct StageD {
     DivC tau_div, six, three;
     int stage;             // 1, 2, 3
     VelD c;
+    int plain;             // 1: an option outside the fast forms' ranges (stage_f64.cu): plain arithmetic
     double wk[NK], vb2[4]; // weights w[a] w[b] per population, squared velocities
     int scheme;            // VLBM_WENO5 .. VLBM_U3
     int komissarov;        // theta flux in the Komissarov form

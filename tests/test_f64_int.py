@@ -1,0 +1,58 @@
+"""The integer-pipe FP64 products of the FP64 stage (csrc/f64_int.cuh), compiled for the host, against the
+hardware's products: bit for bit over random significands, rounding ties, powers of two and zeros."""
+import os
+import subprocess
+
+from conftest import ROOT
+
+HARNESS = r"""
+#include "f64_int.cuh"
+#include <cmath>
+#include <cstdio>
+#include <random>
+using namespace vk;
+static double of(uint64_t u) { double x; memcpy(&x, &u, 8); return x; }
+int main()
+{
+    std::mt19937_64 g(11);
+    auto value = [&]() {
+        const uint64_t r = g();
+        uint64_t m = r & 0xfffffffffffffull;
+        switch ((r >> 53) % 8) {
+        case 0: m = 0; break;                                     // a power of two
+        case 1: m = 0xfffffffffffffull - (r & 7); break;          // just below one
+        case 2: m &= 0xffffffc000000ull; break;                   // 26 bits: exact products and ties
+        case 3: m = r & 7; break;
+        }
+        return of((r & 0x8000000000000000ull) | ((uint64_t)(1023 - 450 + g() % 900) << 52) | m);
+    };
+    long bad = 0;
+    for (long t = 0; t < 3000000; ++t) {
+        double a = value(), b = value();
+        if (t % 100 == 0) a = t % 200 ? 0.0 : -0.0;
+        if (t % 100 == 1) b = 0.0;
+        const double p = a * b;
+        bad += mul_int_zz(a, b) != p || (p != 0.0 && f64_bits(mul_int_zz(a, b)) != f64_bits(p));
+        if (b != 0.0) bad += mul_int_z(a, b) != p;
+        bad += sq_int(a) != a * a;
+        bad += mul_small<3>(a) != 3.0 * a || mul_small<5>(a) != 5.0 * a || mul_small<7>(a) != 7.0 * a ||
+               mul_small<11>(a) != 11.0 * a;
+        bad += scale2<1>(a) != 2.0 * a || scale2<2>(a) != 4.0 * a || scale2<-1>(a) != 0.5 * a ||
+               scale2<-2>(a) != 0.25 * a;
+        const bool in = a == 0.0 || (std::fabs(a) >= 0x1p-400 && std::fabs(a) < 0x1p100);
+        bad += f64_within<400, 100>(a) != in;
+    }
+    for (double x : {(double)INFINITY, -(double)INFINITY, (double)NAN, 5e-324, 1e300})
+        bad += f64_within<400, 100>(x);
+    std::printf("%ld\n", bad);
+}
+"""
+
+
+def test_integer_products_equal_the_hardware_products(tmp_path):
+    src = tmp_path / "f64_int.cpp"
+    src.write_text(HARNESS)
+    exe = tmp_path / "f64_int"
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-I",
+                    os.path.join(ROOT, "paper_2504_15574_gb300", "csrc"), str(src), "-o", str(exe)], check=True)
+    assert int(subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout) == 0

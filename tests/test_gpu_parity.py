@@ -536,3 +536,17 @@ def test_fp64_face_strips_match_oracle(V, nt, np_, scheme, komissarov, velocity_
     assert np.abs(fg - fo).max() <= FP64_TOL * np.abs(fo).max()
     assert g.diagnostics()["pole_flux"] == pytest.approx(o.diagnostics()["pole_budget"], rel=1e-9, abs=1e-18)
     g.close()
+
+
+@pytest.mark.parametrize("scale,step_cells", [(1e-14, False), (1e31, False), (1.0, True)])
+def test_fp64_values_outside_the_fast_forms_range_match_oracle(V, scale, step_cells):
+    """Populations below 2^-40 or above 2^100, everywhere and in single cells, take the plain arithmetic."""
+    nt, np_ = 12, 20
+    rho, ut, up, _ = inputs.gaussian_vortices(nt, np_, 3)
+    rho = scale * rho
+    if step_cells:
+        rho[2, 3], rho[8, 15] = 1e-13, 1e31
+    o, g = run_pair(V, nt, np_, 0.02, 1e-4, (rho, ut, up, None), 2)
+    fo, fg = o.get_populations(), g.get_populations()
+    assert np.abs(fg - fo).max() <= FP64_TOL * np.abs(fo).max()
+    g.close()
