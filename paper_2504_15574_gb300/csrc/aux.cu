@@ -136,30 +136,6 @@ __global__ void guard_kernel(const T *f, size_t total, unsigned *flag)
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1u);
 }
 
-// budget += dt * (m1/6 + m2/6 + 2 m3/3), m_s = -R dph sum_{k,j} (F_south - F_north)
-__global__ void pole_budget_kernel(const double *pole3, int np, double R, double dph, double dt, double *budget)
-{
-    __shared__ double red[3][DIAG_THREADS];
-    const size_t per = (size_t)NK * np;
-    double acc[3] = {0, 0, 0};
-    for (int s = 0; s < 3; ++s) {
-        const double *pn = pole3 + (size_t)s * 2 * per;
-        const double *ps = pn + per;
-        for (size_t x = threadIdx.x; x < per; x += DIAG_THREADS) acc[s] += ps[x] - pn[x];
-    }
-    for (int s = 0; s < 3; ++s) red[s][threadIdx.x] = acc[s];
-    __syncthreads();
-    for (int w = DIAG_THREADS / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w)
-            for (int s = 0; s < 3; ++s) red[s][threadIdx.x] += red[s][threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const double m1 = -R * dph * red[0][0], m2 = -R * dph * red[1][0], m3 = -R * dph * red[2][0];
-        *budget += dt * (m1 / 6.0 + m2 / 6.0 + 2.0 * m3 / 3.0);
-    }
-}
-
 }  // namespace
 
 void launch_fill_ghosts_f64(double *f, const Layout &L, cudaStream_t s)
@@ -202,12 +178,6 @@ void launch_guard_f64(const double *f, size_t n, unsigned *flag, cudaStream_t s)
 void launch_guard_f32(const float *f, size_t n, unsigned *flag, cudaStream_t s)
 {
     guard_kernel<float><<<152 * 8, 256, 0, s>>>(f, n, flag);
-}
-
-void launch_pole_budget(const double *pole3, int np, double R, double dph, double dt, double *budget,
-                        cudaStream_t s)
-{
-    pole_budget_kernel<<<1, DIAG_THREADS, 0, s>>>(pole3, np, R, dph, dt, budget);
 }
 
 }  // namespace vk

@@ -252,9 +252,9 @@ __global__ void __launch_bounds__(128) faces_f64_kernel(const StageD p, int nb_p
 
 // One population's update of one cell.  FAST: products on the integer pipe, for populations that are
 // zero or in [2^-40, 2^100) and a positive density (then every product here is zero or normal).
-template <bool FAST>
+template <bool FAST, int CELLS>
 __device__ __forceinline__ void cell_update(const StageD &p, const Layout &L, const RowD &rd,
-                                            const double (*gs)[32], int lane, int i, int j, int k, double n,
+                                            const double (*gs)[CELLS], int lane, int i, int j, int k, double n,
                                             double ut, double up, double u2, double u23)
 {
     auto mul = [](double a, double b) { return FAST ? mul_int_zz(a, b) : a * b; };
@@ -294,64 +294,94 @@ __device__ __forceinline__ void cell_update(const StageD &p, const Layout &L, co
     store_with_images(p.out, L, k, i, j, outv);
 }
 
-// Cells of one stage: moments, equilibrium, force, BGK, the flux differences of the interface
-// fluxes above and the stage combination, in the oracle's operation order.  A CTA takes 32
-// consecutive cells; its 8 warps first form the moments of those cells (one warp each for n, the
-// two momenta and then the two velocities: the sums run over k in order, so they are chains), then
-// each warp updates two populations of them.  One thread per cell, the earlier form, left a
-// 32 x 64 grid with 64 warps of 1,700 serial FP64 operations (71 us a launch).  Bound on large
-// grids: the FP64 pipe (about 54 operations per population, from 105; divisions by row constants,
-// tau and 3 are two operations each).
-constexpr int CELL_WARPS = 8;
-__global__ void __launch_bounds__(32 * CELL_WARPS) cells_f64_kernel(const StageD p)
+// Pole mass-flux budget of one step, by the threads of one CTA: budget += dt (m1/6 + m2/6 + 2 m3/3),
+// m_s = -R dph sum_{k,j} (F_south - F_north) of stage s.
+__device__ __forceinline__ void pole_budget_f64(const StageD &p)
 {
-    __shared__ double gs[NK][32], mom[3][32], vel[4][32];
+    constexpr int NT = 256;
+    __shared__ double red[3][NT];
+    const int np = p.L.np;
+    const size_t per = (size_t)NK * np;
+    double acc[3] = {0, 0, 0};
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const double *pn = p.pole_all + (size_t)s * 2 * per, *ps = pn + per;
+#pragma unroll 4
+        for (size_t x = threadIdx.x; x < per; x += NT) acc[s] += ps[x] - pn[x];
+    }
+    for (int s = 0; s < 3; ++s) red[s][threadIdx.x] = acc[s];
+    __syncthreads();
+    for (int w = NT / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w)
+            for (int s = 0; s < 3; ++s) red[s][threadIdx.x] += red[s][threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const double m1 = -p.R * p.dph * red[0][0], m2 = -p.R * p.dph * red[1][0], m3 = -p.R * p.dph * red[2][0];
+        *p.budget += p.dt * (m1 / 6.0 + m2 / 6.0 + 2.0 * m3 / 3.0);
+    }
+}
+
+// Cells of one stage: moments, equilibrium, force, BGK, the flux differences of the interface
+// fluxes above and the stage combination, in the oracle's operation order.  A CTA of 256 threads
+// takes CELLS consecutive cells (32 or 16): thread = cell and slot.  Slots 0, 1, 2 first form the
+// moments (the sums run over k in order, so they are chains), 1 and 2 then the velocities; then
+// each slot updates the populations slot, slot + 256 / CELLS, ....  One thread per cell, the earlier
+// form, left a 32 x 64 grid with 64 warps of 1,700 serial FP64 operations (71 us a launch).  Bound
+// on large grids: the FP64 pipe (37 instructions per population, from 105).  16 cells per CTA where
+// 32 would leave SMs without one.  In stage 3 one more CTA adds the step's pole budget (a launch
+// of its own was 3-10 us a step).
+template <int CELLS>
+__global__ void __launch_bounds__(256) cells_f64_kernel(const StageD p, int nblocks)
+{
+    constexpr int SLOTS = 256 / CELLS;
+    __shared__ double gs[NK][CELLS], mom[3][CELLS], vel[4][CELLS];
+    if ((int)blockIdx.x == nblocks) {
+        pole_budget_f64(p);
+        return;
+    }
     const Layout L = p.L;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = threadIdx.x % CELLS, slot = threadIdx.x / CELLS;
     const int q = p.c.q, nk = q * q;
     const long long cells = (long long)L.nt * L.np;
-    const long long cell = (long long)blockIdx.x * 32 + lane;
+    const long long cell = (long long)blockIdx.x * CELLS + c;
     const bool in = cell < cells;
     const int i = in ? (int)(cell / L.np) : 0, j = in ? (int)(cell - (long long)i * L.np) : 0;
     bool out = p.plain;
-    for (int k = warp; k < nk; k += CELL_WARPS) {
+    for (int k = slot; k < nk; k += SLOTS) {
         const double g = p.in[L.at(k, i, j)];
         out |= !f64_within<40, 100>(g);
-        gs[k][lane] = g;
+        gs[k][c] = g;
     }
     const bool plain = __syncthreads_or(out);
-    if (warp < 3) {
+    if (slot < 3) {
         double m = 0.0;
-        if (warp == 0) {
-            for (int k = 0; k < nk; ++k) m += gs[k][lane];
-        } else {
-            for (int k = 0; k < nk; ++k) {
-                const double g = gs[k][lane], v = p.c.v[warp == 1 ? k / q : k % q];
-                m += plain ? g * v : mul_int_zz(g, v);
-            }
+        for (int k = 0; k < nk; ++k) {
+            const double g = gs[k][c], v = slot == 0 ? 1.0 : p.c.v[slot == 1 ? k / q : k % q];
+            m += plain ? g * v : mul_int_zz(g, v);
         }
-        mom[warp][lane] = m;
+        mom[slot][c] = m;
     }
     __syncthreads();
     // (a density that is not positive takes the plain forms: its velocities may be of any size)
-    const double n = mom[0][lane];
+    const double n = mom[0][c];
     const bool slow = plain || !(n > 0.0) || !f64_within<110, 110>(n);
-    if (warp == 1 || warp == 2) vel[warp - 1][lane] = slow ? mom[warp][lane] / n : div_pos(mom[warp][lane], n);
+    if (slot == 1 || slot == 2) vel[slot - 1][c] = slow ? mom[slot][c] / n : div_pos(mom[slot][c], n);
     __syncthreads();
-    if (warp == 0) {
-        const double ut = vel[0][lane], up = vel[1][lane];
+    if (slot == 0) {
+        const double ut = vel[0][c], up = vel[1][c];
         const double u2 = ut * ut + up * up;
-        vel[2][lane] = u2;
-        vel[3][lane] = 3.0 * u2;
+        vel[2][c] = u2;
+        vel[3][c] = 3.0 * u2;
     }
     __syncthreads();
     if (!in) return;
-    const double ut = vel[0][lane], up = vel[1][lane], u2 = vel[2][lane], u23 = vel[3][lane];
+    const double ut = vel[0][c], up = vel[1][c], u2 = vel[2][c], u23 = vel[3][c];
     const RowD rd = p.row[i];
 #pragma unroll 1
-    for (int k = warp; k < nk; k += CELL_WARPS) {
-        if (slow) cell_update<false>(p, L, rd, gs, lane, i, j, k, n, ut, up, u2, u23);
-        else cell_update<true>(p, L, rd, gs, lane, i, j, k, n, ut, up, u2, u23);
+    for (int k = slot; k < nk; k += SLOTS) {
+        if (slow) cell_update<false, CELLS>(p, L, rd, gs, c, i, j, k, n, ut, up, u2, u23);
+        else cell_update<true, CELLS>(p, L, rd, gs, c, i, j, k, n, ut, up, u2, u23);
     }
 }
 
@@ -462,7 +492,14 @@ void launch_stage_f64(const StageD &p, cudaStream_t s)
     const int nb = (int)((sp + 127) / 128), nt = (int)((stt + 127) / 128);
     faces_f64_kernel<<<dim3(nb + nt, L.nk), 128, 0, s>>>(p, nb, S);
     const long long cells = (long long)p.L.nt * p.L.np;
-    cells_f64_kernel<<<(unsigned)((cells + 31) / 32), 32 * CELL_WARPS, 0, s>>>(p);
+    const int extra = (p.stage == 3 && p.budget) ? 1 : 0;
+    if (cells <= 32LL * 152 * 2) {   // 32 cells per CTA: fewer than two CTAs per SM
+        const unsigned nb = (unsigned)((cells + 15) / 16);
+        cells_f64_kernel<16><<<nb + extra, 256, 0, s>>>(p, (int)nb);
+    } else {
+        const unsigned nb = (unsigned)((cells + 31) / 32);
+        cells_f64_kernel<32><<<nb + extra, 256, 0, s>>>(p, (int)nb);
+    }
 }
 
 void launch_init_f64(double *f, const Layout &L, const double *rho, const double *ut, const double *up,

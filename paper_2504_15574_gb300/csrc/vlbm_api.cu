@@ -499,6 +499,10 @@ void enqueue_step(vlbm_t *h, int stage_only = 0, int part = 0)
             p.sin_ext = h->d_sin_ext;
             p.row = h->d_rowd;
             p.pole = h->d_pole + (size_t)(st - 1) * pole_per;
+            p.pole_all = h->d_pole;
+            p.budget = h->d_budget;
+            p.R = h->R;
+            p.dph = 2.0 * M_PI / h->np;
             p.L = h->L;
             p.dt = h->dt;
             p.dt_stage = (st == 1) ? h->dt : (st == 2) ? 0.25 * h->dt : 2.0 / 3.0 * h->dt;
@@ -525,15 +529,13 @@ void enqueue_step(vlbm_t *h, int stage_only = 0, int part = 0)
                 launch_filter_f32((float2 *)out, h->L, h->vd.q, h->d_frows, h->d_fblocks, h->nfrows, s);
         }
     }
-    if (!stage_only && h->prec == VLBM_FP64)
-        launch_pole_budget(h->d_pole, h->np, h->R, 2.0 * M_PI / h->np, h->dt, h->d_budget, s);
     if (!stage_only && h->prec == VLBM_FP32 && h->run.pole_part) launch_budget_f32(h, s);
 }
 
 int kernels_per_step(const vlbm_t *h)
 {
     int n = 3 + (h->nfrows ? 3 : 0) + (h->band_hi > h->band_lo ? 3 : 0);
-    if (h->prec == VLBM_FP64) n += 3 + 1;   // a face kernel per stage and the pole budget
+    if (h->prec == VLBM_FP64) n += 3;   // a face kernel per stage
     else if (h->run.pole_part) n += 1;          // the pole budget
     return n;
 }
@@ -1016,11 +1018,8 @@ int vlbm_profile_step(vlbm_t *h, int n, double *ms_per_stage, int *launches)
             acc[st - 1] += ms;
             acc[st + 2] += h->nfrows ? mf : 0.0f;
         }
-        // the step's pole budget, outside the timed launches
-        if (h->prec == VLBM_FP64)
-            launch_pole_budget(h->d_pole, h->np, h->R, 2.0 * M_PI / h->np, h->dt, h->d_budget, h->stream);
-        else if (h->run.pole_part)
-            launch_budget_f32(h, h->stream);
+        // the step's pole budget (FP32), outside the timed launches
+        if (h->prec == VLBM_FP32 && h->run.pole_part) launch_budget_f32(h, h->stream);
     }
     CK(h, cudaGetLastError());
     h->steps += n;

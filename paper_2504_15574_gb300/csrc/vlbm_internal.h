@@ -54,6 +54,9 @@ struct StageD {
     const double *sin_ext; // sin(theta) at padded rows 0 .. nt+2GR-1 (negative at ghost rows)
     const RowD *row;       // per interior row
     double *pole;          // [2][16][np] fluxes through the north/south pole faces, or NULL
+    const double *pole_all;   // [3][2][16][np]: those of all three stages
+    double *budget;        // pole mass-flux budget, updated by stage 3 (NULL: left alone)
+    double R, dph;
     Layout L;
     double dt, dt_stage, eps;   // dt_stage: the stage's weight of dt L (dt, 0.25 dt, 2/3 dt)
     DivC tau_div, six, three;
@@ -265,8 +268,5 @@ void launch_diag_final(const double *part, int nrows, double *out, cudaStream_t 
 // Non-finite guard over a whole array of n floats / doubles: sets *flag to 1 on NaN/Inf.
 void launch_guard_f64(const double *f, size_t n, unsigned *flag, cudaStream_t s);
 void launch_guard_f32(const float *f, size_t n, unsigned *flag, cudaStream_t s);
-// Pole mass-flux budget: budget += dt * (m1/6 + m2/6 + 2 m3/3), m_s = -R dph sum (F_south - F_north).
-void launch_pole_budget(const double *pole3, int np, double R, double dph, double dt, double *budget,
-                        cudaStream_t s);
 
 }  // namespace vk
