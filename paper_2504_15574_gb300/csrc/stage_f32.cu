@@ -650,12 +650,12 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
     const TabT<TY, NPQ> &tab = S.tab[tb];
     // the tile's pole-face partials (the face phase's per-pair sums, added in pair order)
     if (R.pole_part != nullptr && tid == 0) {
-        const size_t base = (size_t)(stage - 1) * 2 * R.tiles_x + bx;
         for (int pole = 0; pole < 2; ++pole) {
             if (pole == 0 ? i0 != 0 : i0 + TY < L.nt) continue;
             double sum = 0.0;
             for (int q = 0; q < NFQ; ++q) sum += S.polew[pole][q];
-            R.pole_part[base + (size_t)pole * R.tiles_x] = sum;
+            // (this element's only addition of the launch: an atomic because it does not wait for the old value)
+            atomicAdd(&R.pole_part[bx + (size_t)pole * R.tiles_x], sum * (stage == 3 ? 2.0 / 3.0 : 1.0 / 6.0));
         }
     }
     // ---- one cell per thread: warp = cell row, lane = column
@@ -840,6 +840,7 @@ __device__ __forceinline__ bool stage_tile(const RunF &R, const typename VelOf<Q
     const float dte = stage_dte(stage, R.dt);
 
     if (tid == 0) {
+        pdl_wait();   // (returns at once but for the first tile of a launch_after launch)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&S.bar[0])),
                      "r"(stage == 1 ? TILE_BYTES : TILE_BYTES + CORE_BYTES)
@@ -859,8 +860,10 @@ __device__ __forceinline__ bool stage_tile(const RunF &R, const typename VelOf<Q
                 "r"(smem_u32(&S.bar[0]))
                 : "memory");
     }
-    // per-tile tables while the tile is in flight
+    // per-tile tables while the tile is in flight (or the previous kernel still runs)
     fill_tab<TY, NPQ, LIN || KW>(S.tab[0], R, i0, dte);
+    pdl_wait();
+    pdl_trigger();
     // (the barrier of the load wait also publishes the tables; the caller has made the
     // mbarrier's initialisation visible to every thread before this tile began)
     const bool ok = __syncthreads_and(wait_phase(&S.bar[0], parity, R.wait_ns));
@@ -978,6 +981,8 @@ __global__ void __launch_bounds__(256, 3)
     // leaves last (counted in ctr[1]) resets both counters for the next launch of this slot.
     __shared__ int next_tile;
     int t = (int)blockIdx.x;
+    pdl_wait();
+    pdl_trigger();
     if (tid == 0 && t < total) {
         issue_box(t, 0);
         if (stage != 1) issue_f(t);
@@ -1410,7 +1415,10 @@ __device__ __forceinline__ void filter_row_f32(f2 *f, const Layout &L, int vq, i
 __global__ void __launch_bounds__(FILT_THREADS) filter_f32_kernel(f2 *f, const Layout L, int vq, const int *rows,
                                                                    const int *blocks)
 {
-    filter_row_f32(f, L, vq, rows[blockIdx.x], blocks[blockIdx.x], blockIdx.y);
+    const int row = rows[blockIdx.x], block = blocks[blockIdx.x];
+    pdl_wait();
+    pdl_trigger();
+    filter_row_f32(f, L, vq, row, block, blockIdx.y);
 }
 
 // One CTA per (run, filtered row) item of a batch and pair plane: the row of the
@@ -1421,11 +1429,12 @@ __global__ void __launch_bounds__(FILT_THREADS) batch_filter_f32_kernel(const Ru
     const int4 it = items[blockIdx.x];   // (run, row, block size, unused)
     const RunF &R = runs[it.x];
     f2 *out = (stage == 1) ? R.A : (stage == 2) ? R.B : R.F;
+    pdl_wait();
+    pdl_trigger();
     filter_row_f32(out, R.L, vq, it.y, it.z, blockIdx.y);
 }
 
 constexpr int DIAG_THREADS = 256;
-constexpr int NDIAG = 6;
 
 // FP64 diagnostics of the FP32 state, one CTA per row: the density deviations of every cell are
 // summed in FP64 (each stored value converted once; mass = area (rho_ref sin(theta) n_phi +
@@ -1492,32 +1501,6 @@ __global__ void diag_rows_f32_kernel(const f2 *f, const Layout L, const double *
         part[4 * (size_t)L.nt + i] = 0.5 * fma(2.0 * rho_ref * st * L.np, area, red[6][0] * ik);
         part[5 * (size_t)L.nt + i] = red[7][0];
     }
-}
-
-// Pole mass-flux budget of one FP32 step: m_s = -R dphi (F_south - F_north) per stage with
-// F = sum over columns and populations of v_theta times the pole face's reconstruction
-// (part / k for the deviations plus the reference state's ref_n, ref_s), then
-// budget += dt (m1/6 + m2/6 + 2 m3/3) (the SSP-RK3 weights of the stages' tendencies, Sec. 3.7).
-// One warp; the tile partials are added in column order.
-__global__ void pole_budget_f32_kernel(const double *part, int ntx, double ref_n, double ref_s, double inv_ks,
-                                       double R, double dph, double dt, double *budget)
-{
-    // the six partial rows (stage, pole) are loaded together and reduced side by side: one memory
-    // round trip and six independent shuffle chains (each row summed in the same order as alone)
-    double x[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < ntx; b += 32) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) x[k] += part[(size_t)k * ntx + b];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) x[k] += __shfl_xor_sync(0xffffffffu, x[k], o);
-    }
-    double m[3];
-#pragma unroll
-    for (int st = 0; st < 3; ++st) m[st] = -R * dph * ((x[2 * st + 1] * inv_ks + ref_s) - (x[2 * st] * inv_ks + ref_n));
-    if (threadIdx.x == 0) *budget += dt * (m[0] / 6.0 + m[1] / 6.0 + 2.0 * m[2] / 3.0);
 }
 
 // Reference density of the FP32 storage on the device: the area-weighted mean of rho,
@@ -1704,6 +1687,8 @@ static void launch_persist_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out
                              const RunF &run, const typename VelOf<Q>::type &c, int stage, bool lin, TileRows rows,
                              const void *tabs, unsigned *err, unsigned *ctr, cudaStream_t s)
 {
+    // a launch of some of the tile rows waits on two streams (enqueue_split_step): plain edges there
+    const bool early = rows.count < 0;
     if (rows.count < 0) rows = TileRows{0, (run.L.nt + 7) / 8, 1 << 30, 0};
     if (rows.count == 0) return;
     typedef TabT<8, (Q == 3 ? 5 : NP2)> Tab;
@@ -1713,10 +1698,10 @@ static void launch_persist_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out
     const size_t smem = persist_smem<Q>();
     if (lin) {
         const int grid = std::min(total, persist_grid<true, Q>());
-        stage_f32_persist_kernel<true, Q><<<grid, 256, smem, s>>>(tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
+        launch_after(early, stage_f32_persist_kernel<true, Q>, grid, 256, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
     } else {
         const int grid = std::min(total, persist_grid<false, Q>());
-        stage_f32_persist_kernel<false, Q><<<grid, 256, smem, s>>>(tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
+        launch_after(early, stage_f32_persist_kernel<false, Q>, grid, 256, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
     }
 }
 
@@ -1739,20 +1724,21 @@ static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, 
                            const RunF &run, const typename VelOf<Q>::type &c, int stage, int ty, bool lin,
                            TileRows rows, unsigned *err, cudaStream_t s)
 {
+    const bool early = rows.count < 0;   // (as launch_persist_q)
     if (rows.count < 0) rows = TileRows{0, (run.L.nt + ty - 1) / ty, 1 << 30, 0};
     if (rows.count == 0) return;
     const dim3 grid((run.L.np + TX - 1) / TX, rows.count);
     if (!lin && run.komissarov) {   // WENO-5 with the Komissarov theta flux
-        if (ty == 4) stage_f32_kernel<4, false, Q, true><<<grid, 128, smem_bytes<4, Q>(), s>>>(tm_in, tm_out, tm_f, run, c, stage, rows, err);
-        else stage_f32_kernel<8, false, Q, true><<<grid, 256, smem_bytes<8, Q>(), s>>>(tm_in, tm_out, tm_f, run, c, stage, rows, err);
+        if (ty == 4) launch_after(early, stage_f32_kernel<4, false, Q, true>, grid, 128, smem_bytes<4, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+        else launch_after(early, stage_f32_kernel<8, false, Q, true>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
         return;
     }
     if (ty == 4) {
-        if (lin) stage_f32_kernel<4, true, Q><<<grid, 128, smem_bytes<4, Q>(), s>>>(tm_in, tm_out, tm_f, run, c, stage, rows, err);
-        else stage_f32_kernel<4, false, Q><<<grid, 128, smem_bytes<4, Q>(), s>>>(tm_in, tm_out, tm_f, run, c, stage, rows, err);
+        if (lin) launch_after(early, stage_f32_kernel<4, true, Q>, grid, 128, smem_bytes<4, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+        else launch_after(early, stage_f32_kernel<4, false, Q>, grid, 128, smem_bytes<4, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
     } else {
-        if (lin) stage_f32_kernel<8, true, Q><<<grid, 256, smem_bytes<8, Q>(), s>>>(tm_in, tm_out, tm_f, run, c, stage, rows, err);
-        else stage_f32_kernel<8, false, Q><<<grid, 256, smem_bytes<8, Q>(), s>>>(tm_in, tm_out, tm_f, run, c, stage, rows, err);
+        if (lin) launch_after(early, stage_f32_kernel<8, true, Q>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+        else launch_after(early, stage_f32_kernel<8, false, Q>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
     }
 }
 
@@ -1775,11 +1761,11 @@ static void launch_batch_q(const RunF *runs, const CUtensorMap *tms, const int2 
                            cudaStream_t s)
 {
     if (ty == 4) {
-        if (lin) batch_stage_f32_kernel<4, true, Q><<<ctas, 128, smem_bytes<4, Q>(), s>>>(runs, tms, work, ntiles, c, stage, err);
-        else batch_stage_f32_kernel<4, false, Q><<<ctas, 128, smem_bytes<4, Q>(), s>>>(runs, tms, work, ntiles, c, stage, err);
+        if (lin) launch_after(true, batch_stage_f32_kernel<4, true, Q>, ctas, 128, smem_bytes<4, Q>(), s, runs, tms, work, ntiles, c, stage, err);
+        else launch_after(true, batch_stage_f32_kernel<4, false, Q>, ctas, 128, smem_bytes<4, Q>(), s, runs, tms, work, ntiles, c, stage, err);
     } else {
-        if (lin) batch_stage_f32_kernel<8, true, Q><<<ctas, 256, smem_bytes<8, Q>(), s>>>(runs, tms, work, ntiles, c, stage, err);
-        else batch_stage_f32_kernel<8, false, Q><<<ctas, 256, smem_bytes<8, Q>(), s>>>(runs, tms, work, ntiles, c, stage, err);
+        if (lin) launch_after(true, batch_stage_f32_kernel<8, true, Q>, ctas, 256, smem_bytes<8, Q>(), s, runs, tms, work, ntiles, c, stage, err);
+        else launch_after(true, batch_stage_f32_kernel<8, false, Q>, ctas, 256, smem_bytes<8, Q>(), s, runs, tms, work, ntiles, c, stage, err);
     }
 }
 
@@ -1831,12 +1817,6 @@ void launch_moments_f32(const float2 *f, const Layout &L, double *rho, double *u
     moments_f32_kernel<<<grid, 128, 0, s>>>(f, L, rho, ut, up, T, vel_f32(c), rho_ref, inv_ks_s);
 }
 
-void launch_pole_budget_f32(const double *part, int ntx, double ref_n, double ref_s, double ks, double R, double dph,
-                            double dt, double *budget, cudaStream_t s)
-{
-    pole_budget_f32_kernel<<<1, 32, 0, s>>>(part, ntx, ref_n, ref_s, 1.0 / ks, R, dph, dt, budget);
-}
-
 void launch_rho_ref(const double *rho, int nt, int np, const double *sin_t, double *rowsum, double *out,
                     cudaStream_t s)
 {
@@ -1872,15 +1852,15 @@ void launch_fill_ghosts_f32(float2 *f, const Layout &L, int q, cudaStream_t s)
 void launch_batch_filter_f32(const RunF *runs, const int4 *items, int nitems, int q, int stage, cudaStream_t s)
 {
     if (nitems <= 0) return;
-    batch_filter_f32_kernel<<<dim3(nitems, f32_pairs(q)), FILT_THREADS, 0, s>>>(runs, items, q, stage);
+    launch_after(true, batch_filter_f32_kernel, dim3(nitems, f32_pairs(q)), FILT_THREADS, 0, s, runs, items, q, stage);
 }
 
 void launch_filter_f32(float2 *f, const Layout &L, int q, const int *rows, const int *blocks, int nrows,
-                       cudaStream_t s)
+                       cudaStream_t s, bool early)
 {
     if (nrows <= 0) return;
     dim3 grid(nrows, f32_pairs(q));
-    filter_f32_kernel<<<grid, FILT_THREADS, 0, s>>>(f, L, q, rows, blocks);
+    launch_after(early, filter_f32_kernel, grid, FILT_THREADS, 0, s, f, L, q, rows, blocks);
 }
 
 void launch_diagnostics_f32(const float2 *f, const Layout &L, const double *sin_t, const double *cos_t,

@@ -437,13 +437,6 @@ void launch_stage_f32_any(vlbm_t *h, int st, cudaStream_t s, TileRows rows = Til
     else launch_stage_f32(tm, tmo, h->tmFc, h->run, h->vc, st, h->ty, lin, h->d_flags, s, rows);
 }
 
-// The FP32 step's pole mass-flux budget from the stage kernels' pole partials
-void launch_budget_f32(vlbm_t *h, cudaStream_t s)
-{
-    launch_pole_budget_f32(h->d_pole_part, h->run.tiles_x, h->pole_ref[0], h->pole_ref[1], h->kscale, h->R,
-                           2.0 * M_PI / h->np, h->dt, h->d_budget, s);
-}
-
 // One FP32 RK3 step with the polar filter.  The tile rows touching a filtered row and the filter
 // run on stream2, created with the highest priority so that their CTAs go first; the tile rows
 // clear of the filtered rows run on the handle's stream.  A stage's interior launch reads rows
@@ -465,13 +458,11 @@ void enqueue_split_step(vlbm_t *h)
         if (st > 1) cudaStreamWaitEvent(s2, evI[st - 2], 0);
         launch_stage_f32_any(h, st, s2, polar, 1);
         cudaEventRecord(evP[st - 1], s2);
-        launch_filter_f32((float2 *)out, h->L, h->vd.q, h->d_frows, h->d_fblocks, h->nfrows, s2);
+        launch_filter_f32((float2 *)out, h->L, h->vd.q, h->d_frows, h->d_fblocks, h->nfrows, s2, false);
         if (st > 1) cudaStreamWaitEvent(s, evP[st - 2], 0);
         launch_stage_f32_any(h, st, s, inner, 2);
         cudaEventRecord(evI[st - 1], s);
     }
-    // the step's pole budget: its partials come from the polar launches, all on stream2
-    if (h->run.pole_part) launch_budget_f32(h, s2);
     cudaEventRecord(h->evs[0], s2);
     cudaStreamWaitEvent(s, h->evs[0], 0);
 }
@@ -526,17 +517,15 @@ void enqueue_step(vlbm_t *h, int stage_only = 0, int part = 0)
         } else {
             if (part != 2) launch_stage_f32_any(h, st, s);
             if (h->nfrows && part != 1)
-                launch_filter_f32((float2 *)out, h->L, h->vd.q, h->d_frows, h->d_fblocks, h->nfrows, s);
+                launch_filter_f32((float2 *)out, h->L, h->vd.q, h->d_frows, h->d_fblocks, h->nfrows, s, true);
         }
     }
-    if (!stage_only && h->prec == VLBM_FP32 && h->run.pole_part) launch_budget_f32(h, s);
 }
 
 int kernels_per_step(const vlbm_t *h)
 {
     int n = 3 + (h->nfrows ? 3 : 0) + (h->band_hi > h->band_lo ? 3 : 0);
     if (h->prec == VLBM_FP64) n += 3;   // a face kernel per stage
-    else if (h->run.pole_part) n += 1;          // the pole budget
     return n;
 }
 
@@ -573,6 +562,7 @@ int after_reset(vlbm_t *h)
     if (h->prec == VLBM_FP64) launch_fill_ghosts_f64((double *)h->F, h->L, h->stream);
     else launch_fill_ghosts_f32((float2 *)h->F, h->L, h->vd.q, h->stream);
     CK(h, cudaMemsetAsync(h->d_budget, 0, sizeof(double), h->stream));
+    if (h->d_pole_part) CK(h, cudaMemsetAsync(h->d_pole_part, 0, sizeof(double) * 2 * h->run.tiles_x, h->stream));
     CK(h, cudaMemsetAsync(h->d_flags, 0, sizeof(unsigned) * 4, h->stream));
     CK(h, cudaGetLastError());
     h->steps = 0;
@@ -793,7 +783,7 @@ int vlbm_create(int n_theta, int n_phi, int velocity_set, double tau, double dt,
         }
         const int ntx = (n_phi + F32_TILE_COLS - 1) / F32_TILE_COLS;
         if ((rc = upload(h, &h->d_cph, cph.data(), cph.size())) || (rc = upload(h, &h->d_sph, sph.data(), sph.size())) ||
-            (rc = dalloc(h, (void **)&h->d_pole_part, sizeof(double) * 3 * 2 * (size_t)ntx)) ||
+            (rc = dalloc(h, (void **)&h->d_pole_part, sizeof(double) * 2 * (size_t)ntx)) ||
             (rc = dalloc(h, (void **)&h->d_ctr, sizeof(unsigned) * 6)) ||
             (rc = dalloc(h, (void **)&h->d_scalar, sizeof(double) * 8)))
             return bail(rc);
@@ -970,7 +960,22 @@ int vlbm_diagnostics(vlbm_t *h, vlbm_diag *out)
     double v[8];
     CK(h, cudaMemcpyAsync(v, h->d_diag, 6 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaMemcpyAsync(v + 6, h->d_budget, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    std::vector<double> pole;
+    if (h->prec == VLBM_FP32 && h->run.pole_part) {
+        pole.resize(2 * (size_t)h->run.tiles_x);
+        CK(h, cudaMemcpyAsync(pole.data(), h->d_pole_part, sizeof(double) * pole.size(), cudaMemcpyDeviceToHost,
+                              h->stream));
+    }
     CK(h, cudaStreamSynchronize(h->stream));
+    if (!pole.empty()) {
+        // -dt R dphi times the stage-weighted flux out of the south minus the north pole: the deviations'
+        // sums, and the reference state's constant flux of every step taken
+        double sum[2] = {0.0, 0.0};
+        for (int k = 0; k < 2; ++k)
+            for (int b = 0; b < h->run.tiles_x; ++b) sum[k] += pole[(size_t)k * h->run.tiles_x + b];
+        const double dev = (sum[1] - sum[0]) / h->kscale, ref = (h->pole_ref[1] - h->pole_ref[0]) * (double)h->steps;
+        v[6] = -h->dt * h->R * (2.0 * M_PI / h->np) * (dev + ref);
+    }
     out->time = (double)h->steps * h->dt;
     out->steps = h->steps;
     out->mass = v[0];
@@ -1018,8 +1023,6 @@ int vlbm_profile_step(vlbm_t *h, int n, double *ms_per_stage, int *launches)
             acc[st - 1] += ms;
             acc[st + 2] += h->nfrows ? mf : 0.0f;
         }
-        // the step's pole budget (FP32), outside the timed launches
-        if (h->prec == VLBM_FP32 && h->run.pole_part) launch_budget_f32(h, h->stream);
     }
     CK(h, cudaGetLastError());
     h->steps += n;

@@ -23,6 +23,36 @@
 
 namespace vk {
 
+// Programmatic dependent launch.  A kernel launched with launch_after may start while the kernel before it
+// in its stream is still running, once every CTA of that one has called pdl_trigger (or has ended): its
+// prologue (barrier set-up, tables, weights: nothing that a kernel writes) then overlaps the other's
+// tail and the launch latency.  pdl_wait returns when the kernels before have completed and their
+// writes are visible; every read of, and write to, what other kernels touch comes after it.  Kernels call
+// pdl_trigger after pdl_wait: called before it, several later kernels start as well, fill the SMs that
+// happen to be free, and run there two and three CTAs to an SM beside idle ones (128 x 256 steps
+// measured 7 % slower than plain launches that way).  (Kernels
+// launched with <<<>>>, or with early = false, wait for everything before them as ever.)
+#if defined(__CUDACC__)
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+inline void launch_after(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                         A &&...args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
+
 constexpr int NK = 16;   // D2Q16 populations
 constexpr int GR = 3;    // ghost rows per pole (WENO-5 half-width)
 constexpr int GC = 4;    // ghost columns per side (3 needed, 4 keeps TMA x-coordinates 16-byte aligned)
@@ -97,9 +127,10 @@ struct RunF {
     int komissarov;            // theta flux in the Komissarov form (upwind schemes)
     const float *isp;          // [nt + 2GR + 8] 1/sin at padded row pr (negative at ghost rows)
     const float *sfc;          // [nt + 1 + 8] sin(fi dtheta) of theta interface fi (0 at both poles)
-    // pole mass-flux budget (NULL: not recorded): per stage, pole (north, south) and tile column, the
-    // sum over the tile's columns and populations of v_theta times the theta-face value of dg on the
-    // pole face, [3][2][tiles_x]
+    // pole mass-flux budget (NULL: not recorded): per pole (north, south) and tile column, [2][tiles_x],
+    // the sum over the stages run, each by its weight in the step (1/6, 1/6, 2/3), and over the tile's
+    // columns and populations of v_theta times the theta-face value of dg on the pole face.  Every
+    // element is added to by one CTA per stage launch, so the sums need no launch of their own.
     double *pole_part;
     // limit of the stage kernels' first wait for a tile's copies (ns; the second, after which
     // the CTA leaves, is always 1 s)
@@ -229,8 +260,9 @@ void launch_unpack_f32(const double *dense, const Layout &L, float2 *f, const Ve
                        const double *sin_t, double ks, cudaStream_t s);
 // (q: the velocity set's order, which fixes the pair planes and the pole images of the slots)
 void launch_fill_ghosts_f32(float2 *f, const Layout &L, int q, cudaStream_t s);
+// (early: launch_after's)
 void launch_filter_f32(float2 *f, const Layout &L, int q, const int *rows, const int *blocks, int nrows,
-                       cudaStream_t s);
+                       cudaStream_t s, bool early);
 // Polar filter of every (run, row, block size) item of a batch on the output array of `stage`.
 void launch_batch_filter_f32(const RunF *runs, const int4 *items, int nitems, int q, int stage, cudaStream_t s);
 // FP64 diagnostics of an FP32 state (cph, sph: cos and sin of the column angles, FP64 [np]); out as
@@ -238,11 +270,6 @@ void launch_batch_filter_f32(const RunF *runs, const int4 *items, int nitems, in
 void launch_diagnostics_f32(const float2 *f, const Layout &L, const double *sin_t, const double *cos_t,
                             const double *cph, const double *sph, const VelD &c, double area, double rho_ref,
                             double ks, double *part, double *out, cudaStream_t s);
-// Pole mass-flux budget of one FP32 step from the stage kernels' pole partials ([3][2][ntx], RunF.pole_part):
-// budget += dt (m1/6 + m2/6 + 2 m3/3), m_s = -R dphi ((S_south / ks + ref_s) - (S_north / ks + ref_n)) with
-// ref_n, ref_s the reference state's v_theta-weighted pole fluxes summed over the columns.
-void launch_pole_budget_f32(const double *part, int ntx, double ref_n, double ref_s, double ks, double R, double dph,
-                            double dt, double *budget, cudaStream_t s);
 // Area-weighted mean of a device density field (rowsum: nt doubles of scratch; out: one double).
 void launch_rho_ref(const double *rho, int nt, int np, const double *sin_t, double *rowsum, double *out,
                     cudaStream_t s);
