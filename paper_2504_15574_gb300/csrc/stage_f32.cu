@@ -134,6 +134,116 @@ __device__ __forceinline__ f2 sub2(f2 a, f2 b)
 __device__ __forceinline__ f2 splat(float x) { return make_float2(x, x); }
 __device__ __forceinline__ f2 swap2(f2 a) { return make_float2(a.y, a.x); }
 
+// ---- polar ring filter: block means -------------------------------------------------
+// Block sums are compensated: every addition is Knuth's error-free TwoSum, so a partial sum is an
+// unevaluated pair hi + lo of floats that carries the exact sum of its inputs up to the rounding of the
+// small lo parts (relative error ~2^-46).  Every form adds the columns of a block along the same binary
+// tree (neighbours, pairs of neighbours, ..., the lower partial first), so the stage kernels' means
+// and the filter kernel's agree bit for bit.  The block mean is the pair scaled by the exact 1/b and
+// rounded once to FP32, which is the value of an FP64 accumulation (to ~2^-46) at FP32-pipe cost:
+// GB300's FP64 rate is 1/64 of its FP32 rate.
+struct FF { f2 hi, lo; };   // a float-float pair per member
+
+__device__ __forceinline__ void two_sum(f2 a, f2 b, f2 &s, f2 &e)
+{
+    s = add2(a, b);
+    const f2 v = sub2(s, a);
+    e = add2(sub2(a, sub2(s, v)), sub2(b, v));
+}
+
+// (a.hi + a.lo) + (b.hi + b.lo) as a renormalised pair; a is the lower-index partial
+__device__ __forceinline__ FF ff_add(FF a, FF b)
+{
+    f2 s, e, hi, lo;
+    two_sum(a.hi, b.hi, s, e);
+    e = add2(e, add2(a.lo, b.lo));
+    two_sum(s, e, hi, lo);
+    return FF{hi, lo};
+}
+
+__device__ __forceinline__ FF ff_shfl_xor(FF a, int m, unsigned mask = 0xffffffffu)
+{
+    FF r;
+    r.hi.x = __shfl_xor_sync(mask, a.hi.x, m);
+    r.hi.y = __shfl_xor_sync(mask, a.hi.y, m);
+    r.lo.x = __shfl_xor_sync(mask, a.lo.x, m);
+    r.lo.y = __shfl_xor_sync(mask, a.lo.y, m);
+    return r;
+}
+
+// mean of the block whose sum is a.hi + a.lo: with r = 1/b exact (b a power of two),
+// lo r is exact and fma(hi, r, lo r) rounds hi r + lo r once, so the result is the
+// correctly rounded mean of the pair (the value an FP64 total scaled and rounded to
+// FP32 would give, without the FP64 pipe)
+__device__ __forceinline__ f2 ff_mean(FF a, float inv_b)
+{
+    return make_float2(fmaf(a.hi.x, inv_b, a.lo.x * inv_b), fmaf(a.hi.y, inv_b, a.lo.y * inv_b));
+}
+
+// Replaces v[q], q < 8, of every lane by the mean over its aligned block of b lanes (2 .. 32, a power of
+// two; mask: the lanes in the call).  A butterfly in which each of the first three steps also halves
+// the number of pairs a lane sums (the partner sums the other half), and which hands the means back the
+// same way: 9 pair additions instead of the 40 of eight plain butterflies, whose extra work on the
+// filtered rows cost more than the separate filter launch had.
+__device__ __forceinline__ void ring_means(f2 (&v)[8], int b, unsigned mask)
+{
+    const int lane = threadIdx.x & 31;
+    const float inv_b = __int_as_float((254 << 23) - __float_as_int((float)b));   // 1/b of a power of two
+    const f2 zero = make_float2(0.0f, 0.0f);
+    auto pick = [](bool up, f2 lo, f2 hi) { return make_float2(up ? hi.x : lo.x, up ? hi.y : lo.y); };
+    auto shfl = [&](f2 x, int m) {
+        return make_float2(__shfl_xor_sync(mask, x.x, m), __shfl_xor_sync(mask, x.y, m));
+    };
+    auto add = [&](bool up, FF mine, FF other) { return up ? ff_add(other, mine) : ff_add(mine, other); };
+    const bool u1 = lane & 1, u2 = lane & 2, u4 = lane & 4;
+    // step 1: pairs q (even lanes) or 4 + q (odd lanes), q < 4
+    FF p[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const f2 keep = pick(u1, v[q], v[q + 4]), got = shfl(pick(u1, v[q + 4], v[q]), 1);
+        p[q] = add(u1, FF{keep, zero}, FF{got, zero});
+    }
+    f2 r[4];
+    if (b == 2) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) r[q] = ff_mean(p[q], inv_b);
+    } else {
+        FF h[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const FF keep{pick(u2, p[q].hi, p[q + 2].hi), pick(u2, p[q].lo, p[q + 2].lo)};
+            const FF send{pick(u2, p[q + 2].hi, p[q].hi), pick(u2, p[q + 2].lo, p[q].lo)};
+            h[q] = add(u2, keep, FF{shfl(send.hi, 2), shfl(send.lo, 2)});
+        }
+        f2 t[2];
+        if (b == 4) {
+            t[0] = ff_mean(h[0], inv_b);
+            t[1] = ff_mean(h[1], inv_b);
+        } else {
+            const FF keep{pick(u4, h[0].hi, h[1].hi), pick(u4, h[0].lo, h[1].lo)};
+            const FF send{pick(u4, h[1].hi, h[0].hi), pick(u4, h[1].lo, h[0].lo)};
+            FF s = add(u4, keep, FF{shfl(send.hi, 4), shfl(send.lo, 4)});
+#pragma unroll 1
+            for (int m = 8; m < b; m <<= 1) s = add(lane & m, s, FF{shfl(s.hi, m), shfl(s.lo, m)});
+            const f2 mine = ff_mean(s, inv_b), other = shfl(mine, 4);
+            t[0] = pick(u4, mine, other);
+            t[1] = pick(u4, other, mine);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const f2 other = shfl(t[q], 2);
+            r[q] = pick(u2, t[q], other);
+            r[q + 2] = pick(u2, other, t[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const f2 other = shfl(r[q], 1);
+        v[q] = pick(u1, r[q], other);
+        v[q + 4] = pick(u1, other, r[q]);
+    }
+}
+
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float r;
@@ -789,6 +899,16 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
     // the output tile is staged in shared memory and leaves with one TMA store; the issuing
     // thread waits until the store has read it
     const bool core = (i0 >= GR && i0 + TY <= L.nt - GR && q0 >= GC && q0 + TX <= L.np - GC);
+    if (rc.ring > 1) {   // polar ring filter of this row (a row is a warp: uniform)
+        const int nv = L.np - q0;
+        const unsigned mask = nv >= 32 ? 0xffffffffu : (1u << nv) - 1u;
+        f2 v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = q < NPQ ? o[q < NPQ ? q : 0] : splat(0.0f);
+        ring_means(v, rc.ring, mask);
+#pragma unroll
+        for (int q = 0; q < NPQ; ++q) o[q] = v[q];
+    }
     if (core) {
         f2 *ob = &S.ob[0][0][0];
 #pragma unroll
@@ -1236,57 +1356,13 @@ __global__ void fill_ghosts_f32_kernel(f2 *f, const Layout L, int vq)
 
 // Polar ring filter, one CTA per (filtered row, pair plane).  The row is walked in
 // windows of 2048 columns; each of the 256 threads owns 8 consecutive columns.
-// Block sums are compensated: every addition is Knuth's error-free TwoSum, so a
-// partial sum is an unevaluated pair hi + lo of floats that carries the exact sum
-// of its inputs up to the rounding of the small lo parts (relative error ~2^-46).
 // Partials are combined across the threads of an aligned block by xor shuffles
 // (the lower lane's partial always first, so both partners form the same pair)
-// and, for blocks wider than a warp, through shared memory in warp order.  The
-// block mean is the pair scaled by the exact 1/b and rounded once to FP32, which is
-// the value of an FP64 accumulation (to ~2^-46) at FP32-pipe cost: GB300's FP64
-// rate is 1/64 of its FP32 rate.  Blocks wider than a window (b > 2048, only for
+// and, for blocks wider than a warp, through shared memory in warp order.  Blocks wider than a window (b > 2048, only for
 // n_phi above ~25000) take the slice path below.
 constexpr int FILT_THREADS = 256;
 constexpr int FILT_COLS = 8;
 constexpr int FILT_WIN = FILT_THREADS * FILT_COLS;
-
-struct FF { f2 hi, lo; };   // a float-float pair per member
-
-__device__ __forceinline__ void two_sum(f2 a, f2 b, f2 &s, f2 &e)
-{
-    s = add2(a, b);
-    const f2 v = sub2(s, a);
-    e = add2(sub2(a, sub2(s, v)), sub2(b, v));
-}
-
-// (a.hi + a.lo) + (b.hi + b.lo) as a renormalised pair; a is the lower-index partial
-__device__ __forceinline__ FF ff_add(FF a, FF b)
-{
-    f2 s, e, hi, lo;
-    two_sum(a.hi, b.hi, s, e);
-    e = add2(e, add2(a.lo, b.lo));
-    two_sum(s, e, hi, lo);
-    return FF{hi, lo};
-}
-
-__device__ __forceinline__ FF ff_shfl_xor(FF a, int m)
-{
-    FF r;
-    r.hi.x = __shfl_xor_sync(0xffffffffu, a.hi.x, m);
-    r.hi.y = __shfl_xor_sync(0xffffffffu, a.hi.y, m);
-    r.lo.x = __shfl_xor_sync(0xffffffffu, a.lo.x, m);
-    r.lo.y = __shfl_xor_sync(0xffffffffu, a.lo.y, m);
-    return r;
-}
-
-// mean of the block whose sum is a.hi + a.lo: with r = 1/b exact (b a power of two),
-// lo r is exact and fma(hi, r, lo r) rounds hi r + lo r once, so the result is the
-// correctly rounded mean of the pair (the value an FP64 total scaled and rounded to
-// FP32 would give, without the FP64 pipe)
-__device__ __forceinline__ f2 ff_mean(FF a, float inv_b)
-{
-    return make_float2(fmaf(a.hi.x, inv_b, a.lo.x * inv_b), fmaf(a.hi.y, inv_b, a.lo.y * inv_b));
-}
 
 // ghost images of cell (p, i, j): periodic columns and, on the first/last GR rows, the pole image
 __device__ __forceinline__ void store_ghosts(f2 *f, const Layout &L, int vq, int p, int i, int j, f2 v)
@@ -1296,6 +1372,14 @@ __device__ __forceinline__ void store_ghosts(f2 *f, const Layout &L, int vq, int
     if (i < GR || i >= L.nt - GR) store_pole_image(f, L, vq, p, i, j, v);
 }
 
+// the sum of the B columns v[j0], v[j0 + 1], ... along the binary tree
+template <int B>
+__device__ __forceinline__ FF ff_tree(const f2 (&v)[FILT_COLS], int j0)
+{
+    if constexpr (B == 1) return FF{v[j0], splat(0.0f)};
+    else return ff_add(ff_tree<B / 2>(v, j0), ff_tree<B / 2>(v, j0 + B / 2));
+}
+
 // means of the aligned blocks of B columns within one thread's FILT_COLS columns (n valid)
 template <int B>
 __device__ __forceinline__ void thread_block_means(f2 (&v)[FILT_COLS], int n, float inv_b)
@@ -1303,14 +1387,7 @@ __device__ __forceinline__ void thread_block_means(f2 (&v)[FILT_COLS], int n, fl
 #pragma unroll
     for (int j0 = 0; j0 < FILT_COLS; j0 += B) {
         if (j0 >= n) break;
-        FF a{v[j0], splat(0.0f)};
-#pragma unroll
-        for (int m = 1; m < B; ++m) {
-            f2 e;
-            two_sum(a.hi, v[j0 + m], a.hi, e);
-            a.lo = add2(a.lo, e);
-        }
-        const f2 mean = ff_mean(a, inv_b);
+        const f2 mean = ff_mean(ff_tree<B>(v, j0), inv_b);
 #pragma unroll
         for (int m = 0; m < B; ++m) v[j0 + m] = mean;
     }
@@ -1348,13 +1425,7 @@ __device__ __forceinline__ void filter_row_f32(f2 *f, const Layout &L, int vq, i
                 if (b == 2) thread_block_means<2>(v, n, inv_b);
                 else thread_block_means<4>(v, n, inv_b);
             } else {
-                FF a{v[0], splat(0.0f)};
-#pragma unroll
-                for (int m = 1; m < FILT_COLS; ++m) {
-                    f2 e;
-                    two_sum(a.hi, v[m], a.hi, e);
-                    a.lo = add2(a.lo, e);
-                }
+                FF a = ff_tree<FILT_COLS>(v, 0);
                 const int per = b / FILT_COLS;   // threads per block (a power of two)
                 const int wl = min(per, 32);
                 for (int m = 1; m < wl; m <<= 1) {

@@ -304,7 +304,9 @@ int build_f32_tables(vlbm_t *h)
         rc.cotR = (float)(cot / R);
         rc.ephi = (float)(4.0 * h->eps * s * s * ks * ks);
         rc.kth = (float)(s / (R * (h->cos_f[i] - h->cos_f[i + 1])));
-        rc.pad1 = rc.pad2 = 0.0f;
+        const int block = h->filter ? filter_block(nt, h->np, s) : 1;
+        rc.ring = (h->ring_in_stage && block <= F32_RING_MAX) ? block : 0;
+        rc.pad = 0;
         row[i] = rc;
         double rk[NK];
         for (int k = 0; k < q * q; ++k) {
@@ -732,7 +734,7 @@ int vlbm_create(int n_theta, int n_phi, int velocity_set, double tau, double dt,
         std::vector<int> rows, blocks;
         for (int i = 0; i < n_theta; ++i) {
             const int b = filter_block(n_theta, n_phi, h->sin_t[i]);
-            if (b > 1) {
+            if (b > (h->prec == VLBM_FP32 ? F32_RING_MAX : 1)) {
                 rows.push_back(i);
                 blocks.push_back(b);
             }
@@ -742,7 +744,7 @@ int vlbm_create(int n_theta, int n_phi, int velocity_set, double tau, double dt,
             ((rc = upload(h, &h->d_frows, rows.data(), rows.size())) || (rc = upload(h, &h->d_fblocks, blocks.data(), blocks.size()))))
             return bail(rc);
         // FP32: the tile rows whose stage input box (GR rows beyond the tile on each side)
-        // touches no filtered row
+        // touches no row of the filter kernel
         int iN = -1, iS = n_theta;
         for (int i : rows) {
             if (2 * i < n_theta) iN = std::max(iN, i);
@@ -1158,7 +1160,7 @@ int batch_refresh(vlbm_batch_t *b)
         if (!h->filter) continue;
         for (int i = 0; i < h->nt; ++i) {
             const int bs = filter_block(h->nt, h->np, h->sin_t[i]);
-            if (bs > 1) fitems.push_back(make_int4(r, i, bs, 0));
+            if (bs > (h->ring_in_stage ? F32_RING_MAX : 1)) fitems.push_back(make_int4(r, i, bs, 0));
         }
     }
     b->nfitems = (int)fitems.size();
@@ -1343,6 +1345,11 @@ int vlbm_batch_create(int nruns, const int *n_theta, const int *n_phi, const dou
         h->band_lo = h->band_hi = 0;
         b->runs.push_back(h);
     }
+    // the members' polar filter: in the stage kernels, and one filter launch per stage for the rows with
+    // blocks too wide for a tile; a batch without such rows keeps all of it in that launch
+    bool wide = false;
+    for (const vlbm_t *h : b->runs) wide = wide || h->nfrows > 0;
+    for (vlbm_t *h : b->runs) h->ring_in_stage = wide;
     if (cudaMalloc(&b->d_flags, 4 * sizeof(unsigned)) != cudaSuccess ||
         cudaMemset(b->d_flags, 0, 4 * sizeof(unsigned)) != cudaSuccess ||
         cudaMallocHost(&b->h_flags, 4 * sizeof(unsigned)) != cudaSuccess ||

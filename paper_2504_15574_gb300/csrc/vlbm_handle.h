@@ -43,7 +43,8 @@ struct vlbm {
     unsigned long long wait_ns = 1000000000ull;       // FP32 stage kernels: first wait limit on a tile's copies
     // polar filter
     int *d_frows = nullptr, *d_fblocks = nullptr;
-    int nfrows = 0;
+    int nfrows = 0;         // rows of the filter kernel (FP32: those the stage kernels do not filter themselves)
+    bool ring_in_stage = true;   // FP32: the stage kernels filter rows of blocks up to F32_RING_MAX
     // diagnostics, budget, I/O scratch
     double *d_pole = nullptr, *d_budget = nullptr, *d_mom = nullptr, *d_dense = nullptr;
     double *d_part = nullptr, *d_diag = nullptr;

@@ -109,7 +109,8 @@ void launch_stage_f64(const StageD &p, cudaStream_t s);
 // Per interior row: k s (s = sin(theta)), 1/(k s), 1/(R s dphi), cot(theta)/R, the phi WENO
 // regulariser ephi = 4 eps s^2 k^2 (the WENO on f has eps; on dg = k s f its forms carry k s),
 // and for the Komissarov theta flux kth = s / (R (cos theta_{i-1/2} - cos theta_{i+1/2})).
-struct RowF { float s, inv_s, inv_dph, cotR, ephi, kth, pad1, pad2; };
+// ring: block size of the polar filter if the stage kernel applies it (2 .. F32_RING_MAX; 0 or 1: not).
+struct RowF { float s, inv_s, inv_dph, cotR, ephi, kth; int ring, pad; };
 // Per-run parameters of the FP32 stage: one solver, or one member of a batch.
 struct RunF {
     float2 *F, *A, *B;         // dg at the step start, after stage 1, after stage 2 (pair layout)
@@ -202,6 +203,10 @@ constexpr int F32_TILE_COLS = 32;
 // different bank groups (21 r mod 8 is a permutation), which the phi-face walk relies on.
 constexpr int F32_BOX_COLS = F32_TILE_COLS + 2 * GC + 2;
 constexpr int F32_TILE_ROWS_MAX = 8;
+// Widest ring block that the stage kernels average themselves, in the cell phase: such blocks lie within
+// one row of a tile.  Wider ones (the few rows next to a pole of a grid with more than 400 columns) are
+// left to the filter kernel.
+constexpr int F32_RING_MAX = F32_TILE_COLS;
 // One stage of one run, tile rows ty (4 or 8).  tm_in is the box map (F32_BOX_COLS x (ty + 2 GR)
 // x 8) of the stage input array; tm_out and tm_f are the tile-core maps (F32_TILE_COLS x ty x 8)
 // of the stage output array and of F (the step's start values).

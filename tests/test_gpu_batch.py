@@ -153,3 +153,22 @@ def test_batch_refuses_weno_with_komissarov(V):
     with pytest.raises(V.VlbmError) as ex:
         V.Batch(GRIDS, TAU, 1e-4, komissarov=True)
     assert ex.value.code == V.VLBM_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("nt,np_,velocity_set", [(40, 100, "d2q16"), (48, 96, "d2q16"), (126, 384, "d2q16"),
+                                                  (13, 10, "d2q9"), (64, 160, "d2q9")])
+def test_ring_blocks_in_the_stage_kernels_equal_the_filter_kernel_bitwise(V, nt, np_, velocity_set):
+    """A solver's stage kernels average ring blocks of up to 32 columns themselves; a batch without wider
+    blocks leaves them to the filter kernel.  Both add along the same tree, so the states are the same
+    bits: ragged last tiles, blocks of 2 to 32 columns, rows with and without ghost images."""
+    dt = 0.5 * V.vlbm_max_stable_dt(nt, np_, TAU, polar_filter=True)
+    ic = inputs.gaussian_vortices(nt, np_, 3, umax=0.08)
+    s = V.Solver(nt, np_, TAU, dt, precision="fp32", polar_filter=True, velocity_set=velocity_set)
+    s.init_moments(*ic[:3])
+    b = V.Batch([(nt, np_)], TAU, dt, polar_filter=True, velocity_set=velocity_set)
+    b.init_moments(0, *ic[:3])
+    s.step(12)
+    b.step(12)
+    assert np.array_equal(s.get_populations(), b.get_populations(0))
+    s.close()
+    b.close()
