@@ -45,6 +45,7 @@
 #include <cstring>
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 namespace vk {
 
@@ -52,6 +53,7 @@ namespace {
 
 constexpr int TX = F32_TILE_COLS;
 constexpr int NP2 = 8;                 // population pairs of D2Q16
+constexpr int WIDE_TILES = 2 * 152;    // most tiles of a launch of the 512-thread form
 constexpr int SC = F32_BOX_COLS;       // tile columns in shared memory (TX + 2 GC + 2)
 
 // Per-tile tables of one stage, for the tile's rows: the sine differences (FP64-derived) and the
@@ -78,7 +80,8 @@ struct __align__(128) BoxT {
 
 // NPP pair planes: 8 for D2Q16, 5 for D2Q9.  NBUF box buffers and NTAB table buffers: one each for
 // the one-tile CTAs; the persistent stage kernel alternates two table buffers.
-template <int TY, int NPP = NP2, int NBUF = 1, int NTAB = NBUF>
+// WIDE: two threads per cell (D2Q16), with theirs in advT.
+template <int TY, int NPP = NP2, int NBUF = 1, int NTAB = NBUF, bool WIDE = false>
 struct __align__(128) SmemT {
     BoxT<TY, NPP> tile[NBUF];           // TMA destinations (must stay first)
     float2 adv[NPP][TY][TX + 1];        // per cell and pair: dte (flux differences + s rref); row
@@ -86,9 +89,10 @@ struct __align__(128) SmemT {
     __align__(128) float2 ob[NPP][TY][TX];   // stages 2, 3: the tile of F (TMA load); then the output
                                              // tile staged for the TMA store (TMA wants 128-byte
                                              // aligned shared memory)
-    // D2Q9 with 8 warps: the theta walkers' flux differences of the four flux pairs, written
+    // D2Q9 with 8 warps, D2Q16 with 16: the theta walkers' flux differences of the flux pairs, written
     // beside adv by other warps than the phi walkers' (one element otherwise)
-    float2 advT[NPP == 5 ? 4 : 1][NPP == 5 ? TY : 1][NPP == 5 ? TX + 1 : 1];
+    static constexpr int NAT = WIDE ? 8 : NPP == 5 ? 4 : 1;
+    float2 advT[NAT][NAT > 1 ? TY : 1][NAT > 1 ? TX + 1 : 1];
     TabT<TY, NPP> tab[NTAB];
     double polew[2][NPP];               // pole faces of the tile (north, south): per pair, v_theta-weighted
                                         // face values summed over the tile's columns
@@ -104,6 +108,9 @@ typedef SmemT<8, 5> Smem8q3;
 typedef SmemT<4, 5> Smem4q3;
 typedef SmemT<8, NP2, 1, 2> SmemQ8;
 typedef SmemT<8, 5, 1, 2> SmemQ8q3;
+typedef SmemT<8, NP2, 1, 1, true> Smem8w;
+static_assert(offsetof(Smem8w, tile) == 0 && offsetof(Smem8w, ob) % 128 == 0, "as below");
+static_assert(2 * (sizeof(Smem8w) + 128 + 1024) <= 228 * 1024, "two wide tiles per SM");
 static_assert(offsetof(Smem8, tile) == 0 && offsetof(Smem8, ob) % 128 == 0 && offsetof(Smem4, ob) % 128 == 0 &&
                   offsetof(Smem8q3, ob) % 128 == 0 && offsetof(Smem4q3, ob) % 128 == 0 &&
                   offsetof(SmemQ8, ob) % 128 == 0 && offsetof(SmemQ8q3, ob) % 128 == 0 &&
@@ -180,67 +187,53 @@ __device__ __forceinline__ f2 ff_mean(FF a, float inv_b)
     return make_float2(fmaf(a.hi.x, inv_b, a.lo.x * inv_b), fmaf(a.hi.y, inv_b, a.lo.y * inv_b));
 }
 
-// Replaces v[q], q < 8, of every lane by the mean over its aligned block of b lanes (2 .. 32, a power of
-// two; mask: the lanes in the call).  A butterfly in which each of the first three steps also halves
-// the number of pairs a lane sums (the partner sums the other half), and which hands the means back the
-// same way: 9 pair additions instead of the 40 of eight plain butterflies, whose extra work on the
+// out[k] = the mean, over this lane's aligned block of b lanes (2 .. 32, a power of two; mask: the lanes in
+// the call), of the a[k] of the block's lanes, the sums over m lanes being formed already (m = 1: a[k].lo
+// is zero).  A butterfly in which a step with N > 1 values also halves the number of values that a
+// lane sums (the partner, lane ^ m, sums the other half) and hands the means back the same way: for
+// eight pairs 9 pair additions instead of the 40 of eight plain butterflies, whose extra work on the
 // filtered rows cost more than the separate filter launch had.
-__device__ __forceinline__ void ring_means(f2 (&v)[8], int b, unsigned mask)
+template <int N, int M>
+__device__ __forceinline__ void ring_means(const FF (&a)[N], f2 (&out)[N], int b, unsigned mask)
 {
-    const int lane = threadIdx.x & 31;
     const float inv_b = __int_as_float((254 << 23) - __float_as_int((float)b));   // 1/b of a power of two
-    const f2 zero = make_float2(0.0f, 0.0f);
     auto pick = [](bool up, f2 lo, f2 hi) { return make_float2(up ? hi.x : lo.x, up ? hi.y : lo.y); };
     auto shfl = [&](f2 x, int m) {
         return make_float2(__shfl_xor_sync(mask, x.x, m), __shfl_xor_sync(mask, x.y, m));
     };
-    auto add = [&](bool up, FF mine, FF other) { return up ? ff_add(other, mine) : ff_add(mine, other); };
-    const bool u1 = lane & 1, u2 = lane & 2, u4 = lane & 4;
-    // step 1: pairs q (even lanes) or 4 + q (odd lanes), q < 4
-    FF p[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const f2 keep = pick(u1, v[q], v[q + 4]), got = shfl(pick(u1, v[q + 4], v[q]), 1);
-        p[q] = add(u1, FF{keep, zero}, FF{got, zero});
-    }
-    f2 r[4];
-    if (b == 2) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) r[q] = ff_mean(p[q], inv_b);
-    } else {
-        FF h[2];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const FF keep{pick(u2, p[q].hi, p[q + 2].hi), pick(u2, p[q].lo, p[q + 2].lo)};
-            const FF send{pick(u2, p[q + 2].hi, p[q].hi), pick(u2, p[q + 2].lo, p[q].lo)};
-            h[q] = add(u2, keep, FF{shfl(send.hi, 2), shfl(send.lo, 2)});
-        }
-        f2 t[2];
-        if (b == 4) {
-            t[0] = ff_mean(h[0], inv_b);
-            t[1] = ff_mean(h[1], inv_b);
-        } else {
-            const FF keep{pick(u4, h[0].hi, h[1].hi), pick(u4, h[0].lo, h[1].lo)};
-            const FF send{pick(u4, h[1].hi, h[0].hi), pick(u4, h[1].lo, h[0].lo)};
-            FF s = add(u4, keep, FF{shfl(send.hi, 4), shfl(send.lo, 4)});
+    if constexpr (N == 1) {
+        FF s = a[0];
 #pragma unroll 1
-            for (int m = 8; m < b; m <<= 1) s = add(lane & m, s, FF{shfl(s.hi, m), shfl(s.lo, m)});
-            const f2 mine = ff_mean(s, inv_b), other = shfl(mine, 4);
-            t[0] = pick(u4, mine, other);
-            t[1] = pick(u4, other, mine);
+        for (int m = M; m < b; m <<= 1) {
+            const FF o{shfl(s.hi, m), shfl(s.lo, m)};
+            s = (threadIdx.x & m) ? ff_add(o, s) : ff_add(s, o);
         }
+        out[0] = ff_mean(s, inv_b);
+    } else {
+        if (b == M) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const f2 other = shfl(t[q], 2);
-            r[q] = pick(u2, t[q], other);
-            r[q + 2] = pick(u2, other, t[q]);
+            for (int k = 0; k < N; ++k) out[k] = ff_mean(a[k], inv_b);
+            return;
         }
-    }
+        const bool up = threadIdx.x & M;
+        FF h[N / 2];
+        f2 r[N / 2];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const f2 other = shfl(r[q], 1);
-        v[q] = pick(u1, r[q], other);
-        v[q + 4] = pick(u1, other, r[q]);
+        for (int k = 0; k < N / 2; ++k) {
+            FF keep{pick(up, a[k].hi, a[k + N / 2].hi), a[k].lo}, got{shfl(pick(up, a[k + N / 2].hi, a[k].hi), M), a[k].lo};
+            if constexpr (M > 1) {
+                keep.lo = pick(up, a[k].lo, a[k + N / 2].lo);
+                got.lo = shfl(pick(up, a[k + N / 2].lo, a[k].lo), M);
+            }
+            h[k] = up ? ff_add(got, keep) : ff_add(keep, got);
+        }
+        ring_means<N / 2, 2 * M>(h, r, b, mask);
+#pragma unroll
+        for (int k = 0; k < N / 2; ++k) {
+            const f2 other = shfl(r[k], M);
+            out[k] = pick(up, r[k], other);
+            out[k + N / 2] = pick(up, other, r[k]);
+        }
     }
 }
 
@@ -524,19 +517,19 @@ __device__ __forceinline__ f2 theta_face_value(const RunF &R, const VC &c, const
 // Face phase of one stage of one TY x TX tile (q0 = bx TX, i0 = by TY) whose input box and
 // tables are in tile buffer b of S: the phi and theta faces of every pair into S.adv (and S.advT).
 // Ends without a barrier.
-template <int TY, bool LIN, int Q, bool KW = false, class Sm>
+template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false, class Sm>
 __device__ __forceinline__ void tile_faces(const RunF &R, const typename VelOf<Q>::type &c, float dte, Sm &S,
                                            int b, int tb, int bx, int by)
 {
     constexpr int NPQ = (Q == 3) ? 5 : NP2;   // pair planes
     constexpr int NFQ = (Q == 3) ? 4 : NP2;   // pairs with fluxes (D2Q9's fifth: the rest population)
     constexpr int SR = TY + 2 * GR;
-    constexpr int NT = TY * 32;
-    constexpr int NW = NT / 32;
+    constexpr int NW = WIDE ? 2 * TY : TY;
     // warps of the face phases: D2Q16 and 4-warp D2Q9 tiles walk a pair's phi faces and then its
-    // theta faces on one warp (pairs warp, warp + NW, ...); 8-warp D2Q9 tiles walk the four
-    // pairs' phi faces on warps 0-3 and their theta faces on warps 4-7, into advT
-    constexpr bool SPLIT = (Q == 3) && (NW == 2 * NFQ);
+    // theta faces on one warp (pairs warp, warp + NW, ...); 8-warp D2Q9 and 16-warp (WIDE) D2Q16
+    // tiles walk the pairs' phi faces on the first half of the warps and their theta faces on the
+    // second, into advT
+    constexpr bool SPLIT = NW == 2 * NFQ;
     constexpr int FSTEP = SPLIT ? NFQ : NW;
     (void)SR; (void)NFQ; (void)FSTEP; (void)SPLIT;
     const int tid = threadIdx.x;
@@ -611,7 +604,8 @@ __device__ __forceinline__ void tile_faces(const RunF &R, const typename VelOf<Q
                 if (fy > 0) {
                     const int cy = fy - 1;
                     const f2 idth = splat(kom ? tab.rowc[cy].kth : R.inv_dth);
-                    if constexpr (SPLIT) S.advT[q][cy][lane] = mul2(sub2(prev, fl), idth);
+                    if constexpr (WIDE) S.advT[q][cy][lane] = sub2(prev, fl);   // (the cell phase applies idth)
+                    else if constexpr (SPLIT) S.advT[q][cy][lane] = mul2(sub2(prev, fl), idth);
                     else S.adv[q][cy][lane] = fma2(sub2(prev, fl), idth, S.adv[q][cy][lane]);
                 }
                 prev = fl;
@@ -692,7 +686,8 @@ __device__ __forceinline__ void tile_faces(const RunF &R, const typename VelOf<Q
                 if (fy > 0) {
                     const int cy = fy - 1;
                     const f2 vk = KW ? mul2(vt, splat(tab.rowc[cy].kth)) : vt;
-                    if constexpr (SPLIT) S.advT[q][cy][lane] = mul2(vk, sub2(prev, v));
+                    if constexpr (WIDE) S.advT[q][cy][lane] = sub2(prev, v);   // (the cell phase applies vk)
+                    else if constexpr (SPLIT) S.advT[q][cy][lane] = mul2(vk, sub2(prev, v));
                     else S.adv[q][cy][lane] = fma2(vk, sub2(prev, v), S.adv[q][cy][lane]);
                 }
                 prev = v;
@@ -723,7 +718,7 @@ __device__ __forceinline__ void tile_faces(const RunF &R, const typename VelOf<Q
 template <int TY, int NPQ, class Sm>
 __device__ __forceinline__ void load_cell_g(const Sm &S, int b, f2 *G)
 {
-    const int cy = threadIdx.x >> 5, cx = threadIdx.x & 31;
+    const int cy = (threadIdx.x >> 5) & (TY - 1), cx = threadIdx.x & 31;
 #pragma unroll
     for (int q = 0; q < NPQ; ++q) G[q] = S.tile[b].v[q][cy + GR][cx + GC];
 }
@@ -733,7 +728,9 @@ __device__ __forceinline__ void load_cell_g(const Sm &S, int b, f2 *G)
 // the tile (one TMA store through tmo from S.ob for tiles clear of every ghost image, with a
 // barrier inside; per cell with its images otherwise).  In stages 2 and 3, S.ob holds the tile
 // of F when this begins.  Threads of cells outside the grid return early.
-template <int TY, bool LIN, int Q, class Sm>
+// WIDE: two threads per cell, the warps of its row in the two halves of the CTA, each of which updates
+// the pairs of one k_theta half (both form the moments).
+template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false, class Sm>
 __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q>::type &c, int stage, float dte,
                                            const CUtensorMap *tmo, int bx, int by, Sm &S, int b, int tb,
                                            const f2 *Gin)
@@ -741,12 +738,12 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
     constexpr int NPQ = (Q == 3) ? 5 : NP2;   // pair planes
     constexpr int NFQ = (Q == 3) ? 4 : NP2;   // pairs with fluxes (D2Q9's fifth: the rest population)
     constexpr int SR = TY + 2 * GR;
-    constexpr int NT = TY * 32;
-    constexpr int NW = NT / 32;
+    constexpr int NW = WIDE ? 2 * TY : TY;
     // warps of the face phases: D2Q16 and 4-warp D2Q9 tiles walk a pair's phi faces and then its
-    // theta faces on one warp (pairs warp, warp + NW, ...); 8-warp D2Q9 tiles walk the four
-    // pairs' phi faces on warps 0-3 and their theta faces on warps 4-7, into advT
-    constexpr bool SPLIT = (Q == 3) && (NW == 2 * NFQ);
+    // theta faces on one warp (pairs warp, warp + NW, ...); 8-warp D2Q9 and 16-warp (WIDE) D2Q16
+    // tiles walk the pairs' phi faces on the first half of the warps and their theta faces on the
+    // second, into advT
+    constexpr bool SPLIT = NW == 2 * NFQ;
     constexpr int FSTEP = SPLIT ? NFQ : NW;
     (void)SR; (void)NFQ; (void)FSTEP; (void)SPLIT;
     const int tid = threadIdx.x;
@@ -768,16 +765,17 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
             atomicAdd(&R.pole_part[bx + (size_t)pole * R.tiles_x], sum * (stage == 3 ? 2.0 / 3.0 : 1.0 / 6.0));
         }
     }
-    // ---- one cell per thread: warp = cell row, lane = column
-    const int cy = warp, cx = lane;
+    // ---- one cell per thread (WIDE: two): warp = cell row, lane = column
+    constexpr int NO = WIDE ? NPQ / 2 : NPQ;   // pairs that a thread updates, from pair oq on
+    const int cy = warp & (TY - 1), cx = lane, oq = WIDE ? NO * (warp / TY) : 0;
     const int i = i0 + cy, j = q0 + cx;
     if (i >= L.nt || j >= L.np) return;
     // the step's start values of this cell (stages 2, 3; the slots this thread's output
     // overwrites below)
-    f2 F0[NPQ];
+    f2 F0[NO];
     if (stage != 1) {
 #pragma unroll
-        for (int q = 0; q < NPQ; ++q) F0[q] = S.ob[q][cy][cx];
+        for (int q = 0; q < NO; ++q) F0[q] = S.ob[oq + q][cy][cx];
     }
     const RowF rc = tab.rowc[cy];
     f2 G[NPQ];
@@ -860,40 +858,66 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
     const f2 cG = splat(cgv);
     const f2 cF = splat((stage == 2) ? 0.75f : __fsub_rn(1.0f, 2.0f / 3.0f));
 
-    f2 o[NPQ];
+    // the theta walkers' factor of a face difference (WIDE: applied here)
+    const f2 idth = splat(LIN ? (R.komissarov != 0 ? rc.kth : R.inv_dth) : 0.0f);
+    const f2 vth = splat(KW ? dte : __fmul_rn(dte, R.inv_dth)), kth = splat(rc.kth);
+    f2 o[NO];
+    auto update = [&](auto first) {
+        constexpr int Q0 = decltype(first)::value;
 #pragma unroll
-    for (int q = 0; q < NPQ; ++q) {
-        // xi = v . u; the equilibrium deviation times sc s, without w
-        f2 xi, feq, fb;
-        if constexpr (Q == 4) {
-            const int g = q >> 2, b = q & 3;
-            xi = fma2(c.vth[g], ut2, mul2(c.vphi2[b], up2));
-            feq = fma2(xi, fma2(xi, fma2(xi, e3, e2), e1), e0);
-            // force bracket on dg: K along k_theta (pairs (0,b),(1,b) with swapped partners), Ktilde
-            // along k_phi (pairs (g,0..3)), the velocity factors folded into the coefficients
-            const f2 P0 = G[b], P1 = G[4 + b];
-            const f2 *Gg = G + 4 * g;
-            fb = mul2(c.kf[q][0], P0);
-            fb = fma2(c.kf[q][1], swap2(P0), fb);
-            fb = fma2(c.kf[q][2], P1, fb);
-            fb = fma2(c.kf[q][3], swap2(P1), fb);
+        for (int k = 0; k < NO; ++k) {
+            const int q = Q0 + k;
+            // xi = v . u; the equilibrium deviation times sc s, without w
+            f2 xi, feq, fb;
+            if constexpr (Q == 4) {
+                const int g = q >> 2, b = q & 3;
+                xi = fma2(c.vth[g], ut2, mul2(c.vphi2[b], up2));
+                feq = fma2(xi, fma2(xi, fma2(xi, e3, e2), e1), e0);
+                // force bracket on dg: K along k_theta (pairs (0,b),(1,b) with swapped partners), Ktilde
+                // along k_phi (pairs (g,0..3)), the velocity factors folded into the coefficients
+                const f2 P0 = G[b], P1 = G[4 + b];
+                const f2 *Gg = G + 4 * g;
+                fb = mul2(c.kf[q][0], P0);
+                fb = fma2(c.kf[q][1], swap2(P0), fb);
+                fb = fma2(c.kf[q][2], P1, fb);
+                fb = fma2(c.kf[q][3], swap2(P1), fb);
 #pragma unroll
-            for (int m = 0; m < 4; ++m) fb = fma2(c.ktf[q][m], Gg[m], fb);
-        } else {
-            xi = fma2(c.vt2[q], ut2, mul2(c.vb2[q], up2));
-            feq = fma2(xi, fma2(xi, e2, e1), e0);
-            fb = make_float2(fbs[2 * q], fbs[2 * q + 1]);
+                for (int m = 0; m < 4; ++m) fb = fma2(c.ktf[q][m], Gg[m], fb);
+            } else {
+                xi = fma2(c.vt2[q], ut2, mul2(c.vb2[q], up2));
+                feq = fma2(xi, fma2(xi, e2, e1), e0);
+                fb = make_float2(fbs[2 * q], fbs[2 * q + 1]);
+            }
+            // dte times: flux differences + s rref - force + s feq_dev / tau (the rest population
+            // of D2Q9 has no flux: its share is the reference tendency alone)
+            f2 a;
+            if (q >= NFQ) {
+                a = tab.rr[cy][q];
+            } else {
+                a = S.adv[q][cy][cx];
+                if constexpr (WIDE) {   // (as the theta walker of the same warp adds its difference)
+                    if constexpr (LIN) {
+                        a = fma2(S.advT[q][cy][cx], idth, a);
+                    } else {
+                        const f2 vt = mul2(pair_vth(c, q), vth);
+                        a = fma2(KW ? mul2(vt, kth) : vt, S.advT[q][cy][cx], a);
+                    }
+                } else if constexpr (SPLIT) {
+                    a = add2(a, S.advT[q][cy][cx]);
+                }
+            }
+            a = fma2(ncot, fb, a);
+            a = fma2(c.w2[q], feq, a);
+            o[k] = fma2(cG, G[q], a);
+            if (stage != 1) o[k] = fma2(cF, F0[k], o[k]);
         }
-        // dte times: flux differences + s rref - force + s feq_dev / tau (the rest population
-        // of D2Q9 has no flux: its share is the reference tendency alone)
-        f2 a;
-        if (q >= NFQ) a = tab.rr[cy][q];
-        else if constexpr (SPLIT) a = add2(S.adv[q][cy][cx], S.advT[q][cy][cx]);
-        else a = S.adv[q][cy][cx];
-        a = fma2(ncot, fb, a);
-        a = fma2(c.w2[q], feq, a);
-        o[q] = fma2(cG, G[q], a);
-        if (stage != 1) o[q] = fma2(cF, F0[q], o[q]);
+    };
+    (void)idth; (void)vth; (void)kth;
+    if constexpr (WIDE) {
+        if (oq == 0) update(std::integral_constant<int, 0>());
+        else update(std::integral_constant<int, NO>());
+    } else {
+        update(std::integral_constant<int, 0>());
     }
     // tiles clear of the ghost images (no pole-row or seam image to write, no ragged edge):
     // the output tile is staged in shared memory and leaves with one TMA store; the issuing
@@ -902,17 +926,19 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
     if (rc.ring > 1) {   // polar ring filter of this row (a row is a warp: uniform)
         const int nv = L.np - q0;
         const unsigned mask = nv >= 32 ? 0xffffffffu : (1u << nv) - 1u;
-        f2 v[8];
+        constexpr int NR = WIDE ? 4 : 8;
+        FF v[NR];
+        f2 m[NR];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = q < NPQ ? o[q < NPQ ? q : 0] : splat(0.0f);
-        ring_means(v, rc.ring, mask);
+        for (int q = 0; q < NR; ++q) v[q] = FF{q < NO ? o[q < NO ? q : 0] : splat(0.0f), splat(0.0f)};
+        ring_means<NR, 1>(v, m, rc.ring, mask);
 #pragma unroll
-        for (int q = 0; q < NPQ; ++q) o[q] = v[q];
+        for (int q = 0; q < NO; ++q) o[q] = m[q];
     }
     if (core) {
         f2 *ob = &S.ob[0][0][0];
 #pragma unroll
-        for (int q = 0; q < NPQ; ++q) ob[(q * TY + cy) * TX + cx] = o[q];
+        for (int q = 0; q < NO; ++q) ob[((oq + q) * TY + cy) * TX + cx] = o[q];
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
         if (tid == 0) {
@@ -928,10 +954,10 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
     const bool plain = (i >= GR && i < L.nt - GR && j >= GC && j < L.np - GC);
     if (plain) {
 #pragma unroll
-        for (int q = 0; q < NPQ; ++q) out[L.at(q, i, j)] = o[q];
+        for (int q = 0; q < NO; ++q) out[L.at(oq + q, i, j)] = o[q];
     } else {
 #pragma unroll
-        for (int q = 0; q < NPQ; ++q) store_images(out, L, Q, q, i, j, o[q]);
+        for (int q = 0; q < NO; ++q) store_images(out, L, Q, oq + q, i, j, o[q]);
     }
 }
 
@@ -945,10 +971,10 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
 // LIN: the upwind schemes U1-U3 (Eq. fluxes_U1-3, optionally with the Komissarov theta flux)
 // instead of WENO-5.
 // Q: the velocity set (4: D2Q16, 3: D2Q9 in five pairs).
-template <int TY, bool LIN, int Q, bool KW = false>
+template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false>
 __device__ __forceinline__ bool stage_tile(const RunF &R, const typename VelOf<Q>::type &c, int stage,
                                            const CUtensorMap *tm, const CUtensorMap *tmo, const CUtensorMap *tmf,
-                                           int bx, int by, SmemT<TY, (Q == 3 ? 5 : NP2)> &S, unsigned parity,
+                                           int bx, int by, SmemT<TY, (Q == 3 ? 5 : NP2), 1, 1, WIDE> &S, unsigned parity,
                                            unsigned *err)
 {
     constexpr int NPQ = (Q == 3) ? 5 : NP2;
@@ -994,22 +1020,30 @@ __device__ __forceinline__ bool stage_tile(const RunF &R, const typename VelOf<Q
         wait_phase(&S.bar[0], parity, 1000000000ull);
         return false;
     }
-    tile_faces<TY, LIN, Q, KW>(R, c, dte, S, 0, 0, bx, by);
+    tile_faces<TY, LIN, Q, KW, WIDE>(R, c, dte, S, 0, 0, bx, by);
     __syncthreads();
     f2 G[NPQ];
     load_cell_g<TY, NPQ>(S, 0, G);
-    tile_cells<TY, LIN, Q>(R, c, stage, dte, tmo, bx, by, S, 0, 0, G);
+    tile_cells<TY, LIN, Q, KW, WIDE>(R, c, stage, dte, tmo, bx, by, S, 0, 0, G);
     return true;
 }
 
-template <int TY, bool LIN, int Q, bool KW = false>
-__global__ void __launch_bounds__(TY * 32, (Q == 3 ? 32 : 24) / TY) stage_f32_kernel(const __grid_constant__ CUtensorMap tm,
+// WIDE (D2Q16, TY = 8): 512 threads, the phi and theta faces on different warps and two threads per
+// cell, for grids of at most two tiles per SM: a tile alone on its SM is a chain of its warps' walks,
+// which this halves.  Measured per step against the 256-thread form (U3: the persistent kernel):
+// 128 x 256 17.1 against 18.0 us, 181 x 384 23.8 against 28.5; U3 + Komissarov 12.1 against 17.9 and
+// 16.5 against 24.6; at three tiles per SM it loses (216 x 400: 31.5 against 29.7), since two CTAs of
+// 64 registers fit where three of 80 do, and beside another launch too (the polar part of the split
+// schedule: 256 x 512 with the filter 48.4 against 44.0).  The same operations on every value, so the
+// same bits.
+template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false>
+__global__ void __launch_bounds__(TY * (WIDE ? 64 : 32), WIDE ? 2 : (Q == 3 ? 32 : 24) / TY) stage_f32_kernel(const __grid_constant__ CUtensorMap tm,
                                                                       const __grid_constant__ CUtensorMap tmo,
                                                                       const __grid_constant__ CUtensorMap tmf,
                                                                       const RunF R, const typename VelOf<Q>::type c,
                                                                       int stage, const TileRows rows, unsigned *err)
 {
-    typedef SmemT<TY, (Q == 3 ? 5 : NP2)> Smem;
+    typedef SmemT<TY, (Q == 3 ? 5 : NP2), 1, 1, WIDE> Smem;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
     if (threadIdx.x == 0) {
@@ -1018,7 +1052,7 @@ __global__ void __launch_bounds__(TY * 32, (Q == 3 ? 32 : 24) / TY) stage_f32_ke
     }
     __syncthreads();   // no thread may poll the barrier before its initialisation is visible
     const int by = rows.first + (int)blockIdx.y + ((int)blockIdx.y >= rows.split ? rows.skip : 0);
-    stage_tile<TY, LIN, Q, KW>(R, c, stage, &tm, &tmo, &tmf, blockIdx.x, by, S, 0u, err);
+    stage_tile<TY, LIN, Q, KW, WIDE>(R, c, stage, &tm, &tmo, &tmf, blockIdx.x, by, S, 0u, err);
 }
 
 // Persistent stage kernel (8 tile rows, three CTAs per SM): CTA b takes the launch's tiles
@@ -1628,6 +1662,8 @@ __global__ void density_of_populations_kernel(const double *dense, int nk, size_
 template <int TY, int Q = 4>
 static size_t smem_bytes() { return sizeof(SmemT<TY, (Q == 3 ? 5 : NP2)>) + 128; }
 
+static size_t wide_smem() { return sizeof(Smem8w) + 128; }
+
 // Shared memory of the persistent stage kernel
 template <int Q>
 static size_t persist_smem() { return sizeof(SmemT<8, (Q == 3 ? 5 : NP2), 1, 2>) + 128; }
@@ -1661,6 +1697,13 @@ static cudaError_t prepare_persist()
     return persist_grid<LIN, Q>() > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
+template <bool LIN, bool KW>
+static cudaError_t prepare_wide()
+{
+    return cudaFuncSetAttribute(stage_f32_kernel<8, LIN, 4, KW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)wide_smem());
+}
+
 template <int TY, bool LIN>
 cudaError_t prepare_one()
 {
@@ -1690,6 +1733,8 @@ cudaError_t prepare_stage_f32()
     cudaError_t e;
     if ((e = prepare_one<8, false>()) || (e = prepare_one<4, false>()) || (e = prepare_one<8, true>()) ||
         (e = prepare_one<4, true>()))
+        return e;
+    if ((e = prepare_wide<false, false>()) || (e = prepare_wide<true, false>()) || (e = prepare_wide<false, true>()))
         return e;
     if ((e = prepare_persist<false, 4>()) || (e = prepare_persist<true, 4>()) || (e = prepare_persist<false, 3>()))
         return e;
@@ -1790,6 +1835,8 @@ void launch_stage_f32_persist_q3(const CUtensorMap &tm_in, const CUtensorMap &tm
     launch_persist_q<3>(tm_in, tm_out, tm_f, run, c, stage, lin, rows, tabs, err, ctr, s);
 }
 
+bool stage_f32_wide(const Layout &L) { return (long long)((L.np + TX - 1) / TX) * ((L.nt + 7) / 8) <= WIDE_TILES; }
+
 template <int Q>
 static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f,
                            const RunF &run, const typename VelOf<Q>::type &c, int stage, int ty, bool lin,
@@ -1799,6 +1846,14 @@ static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, 
     if (rows.count < 0) rows = TileRows{0, (run.L.nt + ty - 1) / ty, 1 << 30, 0};
     if (rows.count == 0) return;
     const dim3 grid((run.L.np + TX - 1) / TX, rows.count);
+    if constexpr (Q == 4) {
+        if (ty == 8 && early && stage_f32_wide(run.L)) {
+            if (lin) launch_after(early, stage_f32_kernel<8, true, 4, false, true>, grid, 512, wide_smem(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+            else if (run.komissarov) launch_after(early, stage_f32_kernel<8, false, 4, true, true>, grid, 512, wide_smem(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+            else launch_after(early, stage_f32_kernel<8, false, 4, false, true>, grid, 512, wide_smem(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+            return;
+        }
+    }
     if (!lin && run.komissarov) {   // WENO-5 with the Komissarov theta flux
         if (ty == 4) launch_after(early, stage_f32_kernel<4, false, Q, true>, grid, 128, smem_bytes<4, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
         else launch_after(early, stage_f32_kernel<8, false, Q, true>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);

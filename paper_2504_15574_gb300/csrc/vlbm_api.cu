@@ -423,7 +423,8 @@ void launch_stage_f32_any(vlbm_t *h, int st, cudaStream_t s, TileRows rows = Til
     const CUtensorMap &tm = (st == 1) ? h->tmF : (st == 2) ? h->tmA : h->tmB;
     const CUtensorMap &tmo = (st == 1) ? h->tmAc : (st == 2) ? h->tmBc : h->tmFc;
     const bool lin = h->scheme != VLBM_WENO5;
-    if (h->ty == 8 && lin) {
+    const bool wide = h->vd.q == 4 && rows.count < 0 && stage_f32_wide(h->L);
+    if (h->ty == 8 && lin && !wide) {
         // the upwind schemes: the persistent kernel, whose next tile's copies are in flight during
         // the cell phase (their lighter faces leave the one-tile kernel's loads exposed; for WENO-5
         // the one-tile kernel with three resident CTAs per SM measured faster)

@@ -217,6 +217,8 @@ struct TileRows { int first, count, split, skip; };
 void launch_stage_f32(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f, const RunF &run,
                       const VelC &c, int stage, int ty, bool lin, unsigned *err, cudaStream_t s,
                       TileRows rows = TileRows{0, -1, 0, 0});
+// Whether a D2Q16 launch of all 8-row tiles of a grid takes the stage kernel's 512-thread form.
+bool stage_f32_wide(const Layout &L);
 // The same for D2Q9 (five pair planes; tensor maps of depth 5).
 void launch_stage_f32_q3(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f,
                          const RunF &run, const VelC3 &c, int stage, int ty, bool lin, unsigned *err, cudaStream_t s,

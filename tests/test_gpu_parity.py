@@ -550,3 +550,26 @@ def test_fp64_values_outside_the_fast_forms_range_match_oracle(V, scale, step_ce
     fo, fg = o.get_populations(), g.get_populations()
     assert np.abs(fg - fo).max() <= FP64_TOL * np.abs(fo).max()
     g.close()
+
+
+@pytest.mark.parametrize("nt,np_,scheme,komissarov,filt", [
+    (45, 100, "weno5", False, False), (16, 64, "weno5", True, False), (45, 100, "u3", True, False),
+    (9, 34, "u2", False, False), (48, 96, "weno5", False, True), (48, 96, "u3", True, True)])
+def test_fp32_two_threads_per_cell_equal_four_row_tiles(V, nt, np_, scheme, komissarov, filt):
+    """Small grids take the 512-thread form of the 8-row stage kernel, tile_rows = 4 never does: the same
+    operations, so the same bits (WENO-5 with the Komissarov flux: the stated bound of two tile heights)."""
+    ic = inputs.gaussian_vortices(nt, np_, 5, umax=0.08)
+    dt = literal_dt(nt) / 2 if filt else clamped_dt(nt, np_, 0.02)
+    out = []
+    for rows in (8, 4):
+        s = V.Solver(nt, np_, 0.02, dt, precision="fp32", polar_filter=filt, scheme=scheme, komissarov=komissarov,
+                     tile_rows=rows)
+        s.init_moments(*ic)
+        s.step(20)
+        out.append((s.get_populations(), s.diagnostics()["pole_flux"]))
+        s.close()
+    if scheme == "weno5" and komissarov:
+        assert np.abs(out[0][0] - out[1][0]).max() <= W5K_TILE_ROWS_TOL * np.abs(out[1][0]).max()
+    else:
+        assert np.array_equal(out[0][0], out[1][0])
+        assert out[0][1] == out[1][1]
