@@ -10,13 +10,15 @@
 //
 // Arithmetic: activations and weights in BF16, products accumulated in FP32 on
 // the tensor cores (mma.sync m16n8k16, BF16 in, FP32 out); master weights, Adam
-// moments, losses and gradients of the weights in FP32.  Every convolution,
-// forward and backward, is a "valid" 3x3 convolution over an explicitly padded
-// channels-last tensor [rows][cols][channels]:
-//   forward:        Y  = conv(pad(X), W)
-//   backward data:  dP = conv(zero-pad-2(dY), W flipped and transposed), then the
-//                   adjoint of pad() folds ghost gradients onto their sources;
+// moments, losses and gradients of the weights in FP32.  Channels-last tensors
+// [rows][cols][channels]; dY is the gradient at a layer's pre-activation (BF16):
+//   forward:         Y  = "valid" 3x3 convolution of the explicitly padded pad(X) with W;
+//   backward data:   dX = 3x3 convolution of dY with W flipped and transposed, its halo
+//                    the adjoint of pad() (conv_bwd_kernel), masked by the ReLU below;
 //   backward weight: dW[co][tap][ci] = sum_p dY[p][co] pad(X)[p + tap][ci].
+// At the sizes of a coarse grid every launch is bound by latency, not by the tensor
+// rate: the kernels are launched early (launch_after), fetch what no kernel before
+// them writes (weights) ahead of their wait, and a backward pass is nine launches.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -36,12 +38,24 @@ __device__ __forceinline__ unsigned pack_bf16(float lo, float hi)
     return *reinterpret_cast<unsigned *>(&v);
 }
 
-__device__ __forceinline__ unsigned pack_raw(__nv_bfloat16 lo, __nv_bfloat16 hi)
+// four (two) 8x8 matrices of 16-bit elements; lane l gives the address of row l % 8 of matrix l / 8
+__device__ __forceinline__ void ldsm4(unsigned (&r)[4], const void *p)
 {
-    __nv_bfloat162 v;
-    v.x = lo;
-    v.y = hi;
-    return *reinterpret_cast<unsigned *>(&v);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+__device__ __forceinline__ void ldsm4_trans(unsigned (&r)[4], const void *p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+__device__ __forceinline__ void ldsm2(unsigned (&r)[2], const void *p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
+                 : "=r"(r[0]), "=r"(r[1])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
 }
 
 // D = A (16x16 bf16, row) * B (16x8 bf16, col) + C, FP32 accumulate
@@ -76,288 +90,449 @@ __device__ __forceinline__ void for_padded_positions(int H, int W, int y, int x,
     }
 }
 
-// adjoint of pad_kernel: dX[y][x] = dXp[y+1][x+1] + ghost copies that read (y, x)
-__global__ void unpad_kernel(const float *dXp, int H, int W, int C, unsigned negmask, float *dX)
+// ---- 3x3 convolutions on the tensor cores -------------------------------------------
+// CTA: 4 output rows x 64 columns, 16 warps of 16 pixels of one row, so that 128 x 256 is one CTA per SM:
+// at these sizes a layer is bound by what its CTAs read from L2 (with one row and 4 warps per CTA 16 MB
+// for 32 -> 32 channels, mostly the weights once per CTA: 6 us a layer; 6.6 MB now), then by the latency of
+// one such read.  Fragments come by ldmatrix, outputs leave by 16-byte stores through shared memory.
+constexpr int CONV_PIX = 64, CONV_ROWS = 4;
+constexpr int CONV_THREADS = CONV_ROWS * CONV_PIX * 2;
+
+// 16 bytes from global to shared memory without a register in between (zeros with in = false): a staging
+// loop then keeps all its loads in flight.
+__device__ __forceinline__ void copy16(void *dst, const void *src, bool in = true)
 {
-    const int c = threadIdx.x;
-    const int x = blockIdx.x, y = blockIdx.y;
-    if (c >= C) return;
-    const int Wp = W + 2;
-    auto at = [&](int yp, int xp) { return dXp[((size_t)yp * Wp + xp) * C + c]; };
-    float s = at(y + 1, x + 1);
-    // ghost columns (xp = 0 reads x = W-1, xp = W+1 reads x = 0), in the interior rows
-    if (x == W - 1) s += at(y + 1, 0);
-    if (x == 0) s += at(y + 1, W + 1);
-    // ghost rows: row yp = 0 (or H+1), column xp reads row 0 (or H-1) at column xp-1+W/2 (mod W)
-    const float sg = ((negmask >> c) & 1u) ? -1.0f : 1.0f;
-    for (int pole = 0; pole < 2; ++pole) {
-        const int yrow = pole ? H - 1 : 0;
-        if (y != yrow) continue;
-        const int yp = pole ? H + 1 : 0;
-        for (int xp = 0; xp < Wp; ++xp) {
-            int xs = (xp - 1 + W / 2) % W;
-            if (xs < 0) xs += W;
-            if (xs == x) s += sg * at(yp, xp);
-        }
-    }
-    dX[((size_t)y * W + x) * C + c] = s;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(in ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Shared memory: the input rows of the CTA and the weights (+ 8 channels a pixel or output: bank spread)
+template <int CI, int CO>
+struct ConvSmem {
+    __nv_bfloat16 x[CONV_ROWS + 2][CONV_PIX + 2][CI + 8];
+    __nv_bfloat16 w[CO][9 * CI + 8];
+};
+// the outputs of one warp on their way out (in the place of the inputs)
+struct ConvOut { __nv_bfloat16 v[16][LC_HID + 8]; };
+
+// the weights [CO][9][CI] into shared memory
+template <int CI, int CO>
+__device__ __forceinline__ void stage_weights(ConvSmem<CI, CO> &S, const __nv_bfloat16 *Wt)
+{
+    constexpr int WV = 9 * CI / 8;
+#pragma unroll
+    for (int e = threadIdx.x; e < CO * WV; e += CONV_THREADS) copy16(&S.w[e / WV][8 * (e % WV)], Wt + 8 * e);
 }
 
-// ---- valid 3x3 convolution on the tensor cores --------------------------------------
-// Xp [Hp][Wp][Ci] bf16 (Ci multiple of 16), Wt [Co][9][Ci] bf16 (Co multiple of 8, <= 32),
-// out [Hp-2][Wp-2][Co]: Yf (fp32, optional) and Yb (bf16, optional, after ReLU if relu).
-// CTA: one output row, 64 consecutive output columns, 4 warps of 16 pixels.
-constexpr int CONV_PIX = 64;
-
+// acc += the products of this warp's 16 pixels (from column p0 of its staged rows) with tap `wt`'s weights,
+// staged input row xr, column offset dx
 template <int CI, int CO>
-// part0 (optional): per CTA (index blockIdx.y gridDim.x + blockIdx.x) the sum over its pixels of
-// sin_t[row] times output channel 0 (the direct form's drho before its scale; FP64)
-__global__ void __launch_bounds__(128) conv3x3_kernel(const __nv_bfloat16 *Xp, int Hp, int Wp,
-                                                       const __nv_bfloat16 *Wt, const float *bias, float *Yf,
-                                                       __nv_bfloat16 *Yb, __nv_bfloat16 *Ypad, int relu,
-                                                       double *part0, const double *sin_t)
+__device__ __forceinline__ void conv_tap(float (&acc)[CO / 8][4], const ConvSmem<CI, CO> &S, int p0, int xr, int dx,
+                                         int wt)
 {
-    constexpr int XS = CI + 8;           // padded channel stride in shared memory (bank spread)
-    constexpr int WS = 9 * CI + 8;
-    __shared__ __align__(16) __nv_bfloat16 xs[3][CONV_PIX + 2][XS];
-    __shared__ __align__(16) __nv_bfloat16 ws[CO][WS];
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int kc = 0; kc < CI / 16; ++kc) {
+        unsigned a[4];
+        ldsm4(a, &S.x[xr][p0 + (lane & 15) + dx][kc * 16 + (lane >> 4) * 8]);
+        if constexpr (CO == 8) {
+            unsigned b[2];
+            ldsm2(b, &S.w[lane & 7][wt * CI + kc * 16 + ((lane >> 3) & 1) * 8]);
+            mma_bf16(acc[0], a, b);
+        } else {
+#pragma unroll
+            for (int nb = 0; nb < CO / 8; nb += 2) {
+                unsigned b[4];
+                ldsm4(b, &S.w[nb * 8 + (lane & 7) + (lane >> 4) * 8][wt * CI + kc * 16 + ((lane >> 3) & 1) * 8]);
+                mma_bf16(acc[nb], a, b);
+                mma_bf16(acc[nb + 1], a, b + 2);
+            }
+        }
+    }
+}
+
+// Forward layer.  Xp [Hp][Wp][CI] bf16 (CI multiple of 16), Wt [CO][9][CI] bf16, out [Hp-2][Wp-2][CO].  Hidden
+// layers (CO = 32): after the ReLU into Ypad (the next layer's padded input) and Yb (optional).  Last layer
+// (CO = 8): Yf in FP32, and part0 (optional): per CTA (index blockIdx.y gridDim.x + blockIdx.x) the sum over
+// its pixels of sin_t[row] times output channel 0 (the direct form's drho before its scale; FP64).
+template <int CI, int CO>
+__global__ void __launch_bounds__(CONV_THREADS) conv3x3_kernel(const __nv_bfloat16 *Xp, int Hp, int Wp,
+                                                                const __nv_bfloat16 *Wt, const float *bias, float *Yf,
+                                                                __nv_bfloat16 *Yb, __nv_bfloat16 *Ypad,
+                                                                double *part0, const double *sin_t)
+{
+    extern __shared__ __align__(16) unsigned char conv_smem_raw[];
+    ConvSmem<CI, CO> &S = *reinterpret_cast<ConvSmem<CI, CO> *>(conv_smem_raw);
     const int Ho = Hp - 2, Wo = Wp - 2;
-    const int y = blockIdx.y, x0 = blockIdx.x * CONV_PIX;
+    const int y0 = blockIdx.y * CONV_ROWS, x0 = blockIdx.x * CONV_PIX;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // stage the input rows y..y+2, columns x0..x0+65 (zero beyond Wp) and the weights, 16 bytes
-    // (8 channels) per access: CI, XS and WS are multiples of 8
+    // weights and biases were written at least two launches before this one (features_kernel and, with
+    // new weights, the kernel that makes its input come between)
+    stage_weights<CI, CO>(S, Wt);
+    pdl_wait();
+    pdl_trigger();
+    // the input rows y0 .. y0 + 5, columns x0 .. x0 + 65 (zero beyond Wp)
     constexpr int CV = CI / 8;
-    for (int e = tid; e < 3 * (CONV_PIX + 2) * CV; e += blockDim.x) {
+#pragma unroll
+    for (int e = tid; e < (CONV_ROWS + 2) * (CONV_PIX + 2) * CV; e += CONV_THREADS) {
         const int cv = e % CV, rest = e / CV, xx = rest % (CONV_PIX + 2), r = rest / (CONV_PIX + 2);
         const int gx = x0 + xx;
-        const uint4 v = (gx < Wp) ? *reinterpret_cast<const uint4 *>(Xp + ((size_t)(y + r) * Wp + gx) * CI + 8 * cv)
-                                  : make_uint4(0u, 0u, 0u, 0u);
-        *reinterpret_cast<uint4 *>(&xs[r][xx][8 * cv]) = v;
+        copy16(&S.x[r][xx][8 * cv], Xp + ((size_t)min(y0 + r, Hp - 1) * Wp + min(gx, Wp - 1)) * CI + 8 * cv, gx < Wp);
     }
-    constexpr int WV = 9 * CI / 8;
-    for (int e = tid; e < CO * WV; e += blockDim.x)
-        *reinterpret_cast<uint4 *>(&ws[e / WV][8 * (e % WV)]) = *reinterpret_cast<const uint4 *>(Wt + 8 * e);
+    copy_commit();
+    copy_wait<0>();
     __syncthreads();
 
-    const int g = lane >> 2, t = lane & 3;
+    const int g = lane >> 2, t = lane & 3, wr = warp / 4, y = y0 + wr, p0 = (warp % 4) * 16;
     float acc[CO / 8][4];
 #pragma unroll
     for (int nb = 0; nb < CO / 8; ++nb)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[nb][q] = 0.0f;
-    const int pbase = warp * 16;        // this warp's first pixel within the CTA tile
 #pragma unroll
-    for (int tap = 0; tap < 9; ++tap) {
-        const int dy = tap / 3, dx = tap % 3;
+    for (int tap = 0; tap < 9; ++tap) conv_tap<CI, CO>(acc, S, p0, wr + tap / 3, tap % 3, tap);
+    // accumulators: pixels g and g + 8 of the warp, channels 2 t, 2 t + 1 of each block of 8
+    if constexpr (CO == 8) {
+        double s = 0.0;
 #pragma unroll
-        for (int kc = 0; kc < CI / 16; ++kc) {
-            const int k0 = kc * 16 + 2 * t;
-            unsigned a[4];
-            a[0] = *reinterpret_cast<const unsigned *>(&xs[dy][pbase + g + dx][k0]);
-            a[1] = *reinterpret_cast<const unsigned *>(&xs[dy][pbase + g + 8 + dx][k0]);
-            a[2] = *reinterpret_cast<const unsigned *>(&xs[dy][pbase + g + dx][k0 + 8]);
-            a[3] = *reinterpret_cast<const unsigned *>(&xs[dy][pbase + g + 8 + dx][k0 + 8]);
+        for (int half = 0; half < 2; ++half) {
+            const int x = x0 + p0 + g + 8 * half;
+            if (x >= Wo || y >= Ho) continue;
+            const float v0 = acc[0][2 * half] + bias[2 * t], v1 = acc[0][2 * half + 1] + bias[2 * t + 1];
+            if (t == 0) s += (double)v0;
+            *reinterpret_cast<float2 *>(Yf + ((size_t)y * Wo + x) * CO + 2 * t) = make_float2(v0, v1);
+        }
+        if (part0) {   // (uniform over the CTA)
+            __shared__ double red[CONV_THREADS / 32];
+            s *= y < Ho ? sin_t[y] : 0.0;
+#pragma unroll
+            for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+            if (lane == 0) red[warp] = s;
+            __syncthreads();
+            if (tid == 0) {
+                for (int k = 1; k < CONV_THREADS / 32; ++k) s += red[k];
+                part0[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = s;
+            }
+        }
+    } else {
+        __syncthreads();   // every warp is done with the inputs
+        ConvOut &O = reinterpret_cast<ConvOut *>(conv_smem_raw)[warp];
+#pragma unroll
+        for (int half = 0; half < 2; ++half)
 #pragma unroll
             for (int nb = 0; nb < CO / 8; ++nb) {
-                unsigned b[2];
-                b[0] = *reinterpret_cast<const unsigned *>(&ws[nb * 8 + g][tap * CI + k0]);
-                b[1] = *reinterpret_cast<const unsigned *>(&ws[nb * 8 + g][tap * CI + k0 + 8]);
-                mma_bf16(acc[nb], a, b);
+                const int co = nb * 8 + 2 * t;
+                *reinterpret_cast<__nv_bfloat162 *>(&O.v[g + 8 * half][co]) =
+                    __floats2bfloat162_rn(fmaxf(acc[nb][2 * half] + bias[co], 0.0f),
+                                          fmaxf(acc[nb][2 * half + 1] + bias[co + 1], 0.0f));
             }
-        }
-    }
-    // epilogue: rows g and g+8 of the warp tile, columns 2t, 2t+1 of each n-block
-    double p0 = 0.0;
+        __syncwarp();
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-        const int x = x0 + pbase + g + 8 * half;
-        if (x >= Wo) continue;
-        if (part0 && t == 0) p0 += (double)(acc[0][2 * half] + (bias ? bias[0] : 0.0f));
-        const size_t o = ((size_t)y * Wo + x) * CO;
-#pragma unroll
-        for (int nb = 0; nb < CO / 8; ++nb) {
-            const int co = nb * 8 + 2 * t;
-            float v0 = acc[nb][2 * half] + (bias ? bias[co] : 0.0f);
-            float v1 = acc[nb][2 * half + 1] + (bias ? bias[co + 1] : 0.0f);
-            if (Yf) {
-                Yf[o + co] = v0;
-                Yf[o + co + 1] = v1;
-            }
-            if (relu) {
-                v0 = fmaxf(v0, 0.0f);
-                v1 = fmaxf(v1, 0.0f);
-            }
-            const __nv_bfloat162 pr = __floats2bfloat162_rn(v0, v1);
-            if (Yb) *reinterpret_cast<__nv_bfloat162 *>(Yb + o + co) = pr;
+        for (int k = 0; k < 2; ++k) {
+            const int px = lane / 4 + 8 * k, c8 = (lane % 4) * 8, x = x0 + p0 + px;
+            if (x >= Wo || y >= Ho) continue;
+            const uint4 v = *reinterpret_cast<const uint4 *>(&O.v[px][c8]);
+            if (Yb) *reinterpret_cast<uint4 *>(Yb + ((size_t)y * Wo + x) * CO + c8) = v;
             // hidden activations carry no sign flip across the poles
-            if (Ypad)
-                for_padded_positions(Ho, Wo, y, x, [&](int prow, int pcol, bool) {
-                    *reinterpret_cast<__nv_bfloat162 *>(Ypad + ((size_t)prow * (Wo + 2) + pcol) * CO + co) = pr;
-                });
+            for_padded_positions(Ho, Wo, y, x, [&](int prow, int pcol, bool) {
+                *reinterpret_cast<uint4 *>(Ypad + ((size_t)prow * (Wo + 2) + pcol) * CO + c8) = v;
+            });
         }
-    }
-    if (part0) {   // (uniform over the CTA)
-        __shared__ double red[128];
-        red[tid] = p0 * sin_t[y];
-        __syncthreads();
-        for (int k = 64; k > 0; k >>= 1) {
-            if (tid < k) red[tid] += red[tid + k];
-            __syncthreads();
-        }
-        if (tid == 0) part0[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = red[0];
     }
 }
 
-// ---- weight gradient on the tensor cores ---------------------------------------------
-// dY [H][W][CO] bf16 (gradient at the pre-activation), Xp [H+2][W+2][CI] bf16.
-// One CTA per output row: part[row][9][CO][CI] and partb[row][CO] (bias) in FP32.
-template <int CI, int CO>
-__global__ void __launch_bounds__(128) wgrad_kernel(const __nv_bfloat16 *dY, const __nv_bfloat16 *Xp, int H, int W,
-                                                     float *part, float *partb)
+// Backward data of layer l >= 1: the gradient dYin [H][W][32] (BF16) at the pre-activation of layer l - 1 from
+// dY [H][W][CI] at that of layer l, with Wt [32][9][CI] (taps flipped, channels swapped) and the ReLU mask
+// of act [H][W][32].  Columns wrap.  Beyond a pole, pad() has the row on the opposite meridian, so the
+// pole row's gradient gets, in the place of the missing row's taps, the opposite meridian's gradients
+// through the taps that reach across: row 0 through the taps of the row below it (r = 2), row H - 1
+// through those of r = 0.  (Unfused, with a zero-padded copy of dY, the gradient at the padded
+// positions in FP32 and a kernel to fold it back: 29 + 59 + 112 + 24 us for the three layers of
+// 128 x 256; 37 us of each fold was one row's serial search for its ghosts.)
+template <int CI>
+__global__ void __launch_bounds__(CONV_THREADS) conv_bwd_kernel(const __nv_bfloat16 *dY, int H, int W,
+                                                                 const __nv_bfloat16 *Wt, const __nv_bfloat16 *act,
+                                                                 __nv_bfloat16 *dYin)
 {
-    constexpr int NPIX = 64;
-    __shared__ __align__(16) __nv_bfloat16 dys[NPIX][CO + 8];
-    __shared__ __align__(16) __nv_bfloat16 xs[3][NPIX + 2][CI + 8];
-    const int y = blockIdx.x;
+    constexpr int CO = LC_HID;
+    extern __shared__ __align__(16) unsigned char conv_smem_raw[];
+    ConvSmem<CI, CO> &S = *reinterpret_cast<ConvSmem<CI, CO> *>(conv_smem_raw);
+    const int y0 = blockIdx.y * CONV_ROWS, x0 = blockIdx.x * CONV_PIX;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int g = lane >> 2, t = lane & 3;
-    // warp w: taps w, w+4, w+8 (<9); each tap: (CO/16) x (CI/8) accumulator tiles
-    float acc[3][CO / 16][CI / 8][4];
+    stage_weights<CI, CO>(S, Wt);   // (written by an earlier step)
+    pdl_wait();
+    pdl_trigger();
+    constexpr int CV = CI / 8;
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+    for (int e = tid; e < (CONV_ROWS + 2) * (CONV_PIX + 2) * CV; e += CONV_THREADS) {
+        const int cv = e % CV, rest = e / CV, xx = rest % (CONV_PIX + 2), r = rest / (CONV_PIX + 2);
+        // rows -1 and H: the pole rows, half way round (rows beyond them belong to no output)
+        const int row = min(max(y0 - 1 + r, 0), H - 1);
+        int gx = x0 + xx - 1 + (row != y0 - 1 + r ? W / 2 : 0);
+        gx %= W;
+        if (gx < 0) gx += W;
+        copy16(&S.x[r][xx][8 * cv], dY + ((size_t)row * W + gx) * CI + 8 * cv);
+    }
+    copy_commit();
+    copy_wait<0>();
+    __syncthreads();
+    const int g = lane >> 2, t = lane & 3, wr = warp / 4, y = y0 + wr, p0 = (warp % 4) * 16;
+    float acc[CO / 8][4];
 #pragma unroll
-        for (int m = 0; m < CO / 16; ++m)
+    for (int nb = 0; nb < CO / 8; ++nb)
 #pragma unroll
-            for (int n = 0; n < CI / 8; ++n)
+        for (int q = 0; q < 4; ++q) acc[nb][q] = 0.0f;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[a][m][n][q] = 0.0f;
+    for (int r = 0; r < 3; ++r) {
+        const int tr = (r == 0 && y == 0) ? 2 : (r == 2 && y == H - 1) ? 0 : r;
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) conv_tap<CI, CO>(acc, S, p0, wr + r, dx, 3 * tr + dx);
+    }
+    __syncthreads();   // every warp is done with the inputs
+    ConvOut &O = reinterpret_cast<ConvOut *>(conv_smem_raw)[warp];
+#pragma unroll
+    for (int half = 0; half < 2; ++half)
+#pragma unroll
+        for (int nb = 0; nb < CO / 8; ++nb)
+            *reinterpret_cast<__nv_bfloat162 *>(&O.v[g + 8 * half][nb * 8 + 2 * t]) =
+                __floats2bfloat162_rn(acc[nb][2 * half], acc[nb][2 * half + 1]);
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int px = lane / 4 + 8 * k, c8 = (lane % 4) * 8, x = x0 + p0 + px;
+        if (x >= W || y >= H) continue;
+        const size_t o = ((size_t)y * W + x) * CO + c8;
+        uint4 v = *reinterpret_cast<const uint4 *>(&O.v[px][c8]);
+        const uint4 z = *reinterpret_cast<const uint4 *>(act + o);
+        __nv_bfloat16 *vp = reinterpret_cast<__nv_bfloat16 *>(&v);
+        const __nv_bfloat16 *zp = reinterpret_cast<const __nv_bfloat16 *>(&z);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (__bfloat162float(zp[c]) <= 0.0f) vp[c] = __float2bfloat16(0.0f);
+        *reinterpret_cast<uint4 *>(dYin + o) = v;
+    }
+}
+
+// ---- weight gradients on the tensor cores --------------------------------------------
+// All layers in one launch: layer blockIdx.y from dY [H][W][CO] bf16 (gradient at the pre-activation) and
+// Xp [H+2][W+2][CI] bf16; CTA blockIdx.x takes `rows` output rows and writes its sums part[cta][9][CO][CI]
+// and partb[cta][CO] (bias) in FP32.  One warp per tap: pixels are the k index of the product, so both
+// operands are read from their pixel-major staging by transposing ldmatrix (two-byte gathers were 45 us
+// a layer at 128 x 256).  rows: about two CTAs per SM over the four layers, so that few partial sums
+// are written and read again.
+constexpr int WG_PIX = 64;
+constexpr int WG_THREADS = 9 * 32;
+
+template <int CI, int CO>
+__device__ __forceinline__ void wgrad_layer(const LcWgradLayer &l, int H, int W, int rows, unsigned char *smem)
+{
+    constexpr int DS = CO + 8, XS = CI + 8;
+    // two buffers, the copies of the next 64 pixels in flight during one's products: per buffer dY
+    // [WG_PIX][DS] and the input rows [3][WG_PIX + 2][XS]
+    constexpr int BUF = WG_PIX * DS + 3 * (WG_PIX + 2) * XS;
+    __nv_bfloat16 *buf = reinterpret_cast<__nv_bfloat16 *>(smem);
+    const int tid = threadIdx.x, lane = tid & 31, tap = tid >> 5;
+    const int dy = tap / 3, dx = tap % 3;
+    float acc[CO / 16][CI / 8][4];
+#pragma unroll
+    for (int m = 0; m < CO / 16; ++m)
+#pragma unroll
+        for (int n = 0; n < CI / 8; ++n)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[m][n][q] = 0.0f;
+    // bias: thread = channel tid % CO, pixels tid / CO, + BS, ...
+    constexpr int BS = 256 / CO;
     float bsum = 0.0f;
-    for (int x0 = 0; x0 < W; x0 += NPIX) {
-        __syncthreads();
-        for (int e = tid; e < NPIX * CO; e += blockDim.x) {
-            const int p = e / CO, c = e % CO;
-            dys[p][c] = (x0 + p < W) ? dY[((size_t)y * W + x0 + p) * CO + c] : __float2bfloat16(0.0f);
+    const int y0 = blockIdx.x * rows, nx = (W + WG_PIX - 1) / WG_PIX, nt = (min(y0 + rows, H) - y0) * nx;
+    auto fetch = [&](int c) {
+        const int y = y0 + c / nx, x0 = (c % nx) * WG_PIX;
+        __nv_bfloat16 *dys = buf + (c & 1) * BUF, *xs = dys + WG_PIX * DS;
+#pragma unroll
+        for (int e = tid; e < WG_PIX * (CO / 8); e += WG_THREADS) {
+            const int cv = e % (CO / 8), px = e / (CO / 8);
+            copy16(dys + px * DS + 8 * cv, l.dY + ((size_t)y * W + min(x0 + px, W - 1)) * CO + 8 * cv, x0 + px < W);
         }
-        for (int e = tid; e < 3 * (NPIX + 2) * CI; e += blockDim.x) {
-            const int c = e % CI, rest = e / CI, xx = rest % (NPIX + 2), r = rest / (NPIX + 2);
-            const int gx = x0 + xx;
-            xs[r][xx][c] = (gx < W + 2) ? Xp[((size_t)(y + r) * (W + 2) + gx) * CI + c] : __float2bfloat16(0.0f);
+#pragma unroll
+        for (int e = tid; e < 3 * (WG_PIX + 2) * (CI / 8); e += WG_THREADS) {
+            const int cv = e % (CI / 8), rest = e / (CI / 8), xx = rest % (WG_PIX + 2), r = rest / (WG_PIX + 2);
+            copy16(xs + (r * (WG_PIX + 2) + xx) * XS + 8 * cv,
+                   l.Xp + ((size_t)(y + r) * (W + 2) + min(x0 + xx, W + 1)) * CI + 8 * cv, x0 + xx < W + 2);
         }
-        __syncthreads();
-        if (tid < CO)
-            for (int p = 0; p < NPIX; ++p) bsum += __bfloat162float(dys[p][tid]);
+        copy_commit();
+    };
+    fetch(0);
+    for (int c = 0; c < nt; ++c) {
+        const __nv_bfloat16 *dys = buf + (c & 1) * BUF, *xs = dys + WG_PIX * DS;
+        {
+            if (c + 1 < nt) {
+                fetch(c + 1);
+                copy_wait<1>();
+            } else {
+                copy_wait<0>();
+            }
+            __syncthreads();
+            if (tid < 256)
+                for (int px = tid / CO; px < WG_PIX; px += BS) bsum += __bfloat162float(dys[px * DS + tid % CO]);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const int tap = warp + 4 * a;
-            if (tap >= 9) break;
-            const int dy = tap / 3, dx = tap % 3;
+            for (int ks = 0; ks < WG_PIX / 16; ++ks) {
+                // A[co][pixel] = dY[pixel][co]: rows of the staging are pixels (k), hence the transposition;
+                // matrices (co, k), (co + 8, k), (co, k + 8), (co + 8, k + 8)
+                unsigned a[CO / 16][4];
 #pragma unroll
-            for (int ks = 0; ks < NPIX / 16; ++ks) {
-                const int p0 = ks * 16 + 2 * t;   // k = pixel
+                for (int m = 0; m < CO / 16; ++m)
+                    ldsm4_trans(a[m], dys + (ks * 16 + (lane & 7) + (lane >> 4) * 8) * DS + m * 16 + ((lane >> 3) & 1) * 8);
 #pragma unroll
-                for (int m = 0; m < CO / 16; ++m) {
-                    // A[m = co][k = pixel] = dY[pixel][co]
-                    unsigned av[4];
-                    const int co0 = m * 16 + g;
-                    av[0] = pack_raw(dys[p0][co0], dys[p0 + 1][co0]);
-                    av[1] = pack_raw(dys[p0][co0 + 8], dys[p0 + 1][co0 + 8]);
-                    av[2] = pack_raw(dys[p0 + 8][co0], dys[p0 + 9][co0]);
-                    av[3] = pack_raw(dys[p0 + 8][co0 + 8], dys[p0 + 9][co0 + 8]);
+                for (int n = 0; n < CI / 8; n += 2) {
+                    // B[pixel][ci] = Xp[y + dy][pixel + dx][ci]: matrices (k, ci), (k + 8, ci), (k, ci + 8), (k + 8, ci + 8)
+                    unsigned b[4];
+                    ldsm4_trans(b, xs + (dy * (WG_PIX + 2) + ks * 16 + (lane & 15) + dx) * XS + n * 8 + (lane >> 4) * 8);
 #pragma unroll
-                    for (int n = 0; n < CI / 8; ++n) {
-                        // B[k = pixel][n = ci] = Xp[y + dy][pixel + dx][ci]
-                        const int ci = n * 8 + g;
-                        unsigned bv[2];
-                        bv[0] = pack_raw(xs[dy][p0 + dx][ci], xs[dy][p0 + 1 + dx][ci]);
-                        bv[1] = pack_raw(xs[dy][p0 + 8 + dx][ci], xs[dy][p0 + 9 + dx][ci]);
-                        mma_bf16(acc[a][m][n], av, bv);
+                    for (int m = 0; m < CO / 16; ++m) {
+                        mma_bf16(acc[m][n], a[m], b);
+                        mma_bf16(acc[m][n + 1], a[m], b + 2);
                     }
                 }
             }
+            __syncthreads();   // the buffer may be fetched into again
         }
     }
+    const int g = lane >> 2, t = lane & 3;
+    float *part = l.part + ((size_t)blockIdx.x * 9 + tap) * CO * CI;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int tap = warp + 4 * a;
-        if (tap >= 9) break;
+    for (int m = 0; m < CO / 16; ++m)
 #pragma unroll
-        for (int m = 0; m < CO / 16; ++m)
+        for (int n = 0; n < CI / 8; ++n)
 #pragma unroll
-            for (int n = 0; n < CI / 8; ++n)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int co = m * 16 + g + 8 * (q >> 1);
-                    const int ci = n * 8 + 2 * t + (q & 1);
-                    part[(((size_t)y * 9 + tap) * CO + co) * CI + ci] = acc[a][m][n][q];
-                }
+            for (int h = 0; h < 2; ++h)
+                *reinterpret_cast<float2 *>(part + (size_t)(m * 16 + g + 8 * h) * CI + n * 8 + 2 * t) =
+                    make_float2(acc[m][n][2 * h], acc[m][n][2 * h + 1]);
+    __syncthreads();
+    float *red = reinterpret_cast<float *>(smem);
+    if (tid < 256) red[tid] = bsum;
+    __syncthreads();
+    if (tid < CO) {
+        float b = 0.0f;
+        for (int k = 0; k < BS; ++k) b += red[k * CO + tid];
+        l.partb[(size_t)blockIdx.x * CO + tid] = b;
     }
-    if (tid < CO) partb[(size_t)y * CO + tid] = bsum;
 }
 
-// sums partials over rows in order: out[i] = sum_r part[r][i]
-__global__ void reduce_rows_kernel(const float *part, int rows, int n, float *out)
+__global__ void __launch_bounds__(WG_THREADS) wgrad_kernel(const LcBackward p, int rows)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    __shared__ __align__(16) unsigned char smem[2 * (WG_PIX * (LC_HID + 8) + 3 * (WG_PIX + 2) * (LC_HID + 8)) * 2];
+    pdl_wait();
+    pdl_trigger();
+    const LcWgradLayer &l = p.w[blockIdx.y];
+    if (blockIdx.y == 0) wgrad_layer<LC_CIN, LC_HID>(l, p.H, p.W, rows, smem);
+    else if (blockIdx.y < LC_LAYERS - 1) wgrad_layer<LC_HID, LC_HID>(l, p.H, p.W, rows, smem);
+    else wgrad_layer<LC_HID, LC_COUTP2>(l, p.H, p.W, rows, smem);
+}
+
+// The gradient of every parameter from the CTAs' partial sums (added in order) into g, in the master layout
+// (per layer W[co][ci][3][3], b[co]); with adam set, one Adam step (bias-corrected) on the FP32 master
+// weights and their BF16 copies: forward [COp][9][CIp] and backward data [CIp][9][COp2] (taps flipped,
+// channels swapped; the copies' padding channels stay zero).  Thread: one element of a layer's partial
+// sums [9][COp2][CIp] or one bias, and a quarter of the CTAs' partial sums; the quarters are added through
+// shared memory.  The last CTA adds the loss's partial sums.  (Per layer two reductions, a layout pass, a
+// copy, then Adam and a pass per layer over the copies: 26 launches, 110 us at 128 x 256.)
+constexpr int UPD_ELEMS = 64;
+__global__ void __launch_bounds__(4 * UPD_ELEMS) update_kernel(const LcBackward p, const LcAdam a, const double *lpart,
+                                                                int nl, double *loss)
+{
+    __shared__ double red[256];
+    pdl_wait();
+    pdl_trigger();
+    if (blockIdx.x == gridDim.x - 1) {
+        double s = 0.0;
+        for (int i = threadIdx.x; i < nl; i += 256) s += lpart[i];
+        red[threadIdx.x] = s;
+        __syncthreads();
+        for (int k = 128; k > 0; k >>= 1) {
+            if ((int)threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) *loss = red[0];
+        return;
+    }
+    int e = blockIdx.x * UPD_ELEMS + threadIdx.x % UPD_ELEMS, l = 0;
+    const int quarter = threadIdx.x / UPD_ELEMS, per = (p.ctas + 3) / 4;
+    for (; l < LC_LAYERS; ++l) {
+        const int total = 9 * p.w[l].cop2 * p.w[l].cip + p.w[l].cop2;
+        if (e < total) break;
+        e -= total;
+    }
+    const bool in = l < LC_LAYERS;
+    const LcWgradLayer &w = p.w[in ? l : 0];
+    const int n = 9 * w.cop2 * w.cip;
+    const bool bias = e >= n;
     float s = 0.0f;
-    for (int r = 0; r < rows; ++r) s += part[(size_t)r * n + i];
-    out[i] = s;
+    if (in) {
+        const int stride = bias ? w.cop2 : n;
+        const float *src = bias ? w.partb + (e - n) : w.part + e;
+        const int r1 = min((quarter + 1) * per, p.ctas);
+#pragma unroll 16
+        for (int r = quarter * per; r < r1; ++r) s += src[(size_t)r * stride];
+    }
+    float *sum = reinterpret_cast<float *>(red);
+    sum[threadIdx.x] = s;
+    __syncthreads();
+    if (!in || quarter) return;
+    for (int k = 1; k < 4; ++k) s += sum[k * UPD_ELEMS + threadIdx.x];
+    const int ci = e % w.cip, co = bias ? e - n : (e / w.cip) % w.cop2, tap = e / (w.cip * w.cop2);
+    if (co >= w.co || (!bias && ci >= w.ci)) return;
+    const size_t i = bias ? w.boff + co : w.woff + ((size_t)co * w.ci + ci) * 9 + tap;
+    a.g[i] = s;
+    if (!a.step) return;
+    const float mi = a.b1 * a.m[i] + (1.0f - a.b1) * s;
+    const float vi = a.b2 * a.v[i] + (1.0f - a.b2) * s * s;
+    a.m[i] = mi;
+    a.v[i] = vi;
+    const float x = a.w[i] - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+    a.w[i] = x;
+    if (bias) return;
+    const __nv_bfloat16 h = __float2bfloat16(x);
+    w.wf[((size_t)co * 9 + tap) * w.cip + ci] = h;
+    if (w.wb) w.wb[((size_t)ci * 9 + 8 - tap) * w.cop2 + co] = h;
 }
 
 // ---- elementwise pieces -------------------------------------------------------------
-// dP (bf16, zero-padded by 2 on rows and columns, channel count CP >= C) from the
-// FP32 gradient at a layer output and the ReLU mask of that output (mask NULL: none).
-__global__ void grad_pad2_kernel(const float *dY, const __nv_bfloat16 *act, int H, int W, int C, int CP,
-                                 __nv_bfloat16 *dP)
-{
-    const int c = threadIdx.x;
-    const int xp = blockIdx.x, yp = blockIdx.y;
-    if (c >= CP) return;
-    const int y = yp - 2, x = xp - 2;
-    float v = 0.0f;
-    if (c < C && y >= 0 && y < H && x >= 0 && x < W) {
-        const size_t i = ((size_t)y * W + x) * C + c;
-        v = dY[i];
-        if (act && __bfloat162float(act[i]) <= 0.0f) v = 0.0f;
-    }
-    dP[((size_t)yp * (W + 4) + xp) * CP + c] = __float2bfloat16(v);
-}
-
-// the un-padded gradient at the pre-activation (bf16), for the weight gradient
-__global__ void grad_pre_kernel(const float *dY, const __nv_bfloat16 *act, int n, int C, int CP,
-                                __nv_bfloat16 *dPre)
+// the gradient at the network's output [HW][CO] (FP32) as the last layer's dY [HW][CP] (BF16, zero-padded)
+__global__ void grad_pre_kernel(const float *dY, int n, int C, int CP, __nv_bfloat16 *dPre)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n * CP) return;
     const int c = i % CP, p = i / CP;
-    float v = 0.0f;
-    if (c < C) {
-        v = dY[(size_t)p * C + c];
-        if (act && __bfloat162float(act[(size_t)p * C + c]) <= 0.0f) v = 0.0f;
-    }
-    dPre[i] = __float2bfloat16(v);
+    dPre[i] = __float2bfloat16(c < C ? dY[(size_t)p * C + c] : 0.0f);
 }
 
-// area-weighted mean-square loss against targets [3][H][W] (scaled), gradient into dY [H][W][CO]
+// area-weighted mean-square loss against targets [3][H][W] (scaled), its gradient as the last layer's dY
+// [H][W][LC_COUTP2] (BF16, zero beyond the three outputs)
 __global__ void loss_kernel(const float *Y, int CO, const double *target, const double *sin_t, int H, int W,
-                            float3 inv_scale, double wsum, float *dY, double *part)
+                            float3 inv_scale, double inv_w3, __nv_bfloat16 *dY, double *part)
 {
+    pdl_wait();
+    pdl_trigger();
     __shared__ double red[256];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     double l = 0.0;
     if (i < H * W) {
         const int y = i / W;
-        const double w = sin_t[y] / wsum;
+        const double w3 = sin_t[y] * inv_w3;   // sin(theta) / (3 wsum)
         const float sc[3] = {inv_scale.x, inv_scale.y, inv_scale.z};
-        for (int c = 0; c < CO; ++c) {
-            float g = 0.0f;
-            if (c < 3) {
-                const double d = (double)Y[(size_t)i * CO + c] - target[(size_t)c * H * W + i] * sc[c];
-                l += w * d * d / 3.0;
-                g = (float)(2.0 * w * d / 3.0);
-            }
-            dY[(size_t)i * CO + c] = g;
+        float g[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double d = (double)Y[(size_t)i * CO + c] - target[(size_t)c * H * W + i] * sc[c];
+            l += w3 * d * d;
+            g[c] = (float)(2.0 * w3 * d);
         }
+        uint4 *dst = reinterpret_cast<uint4 *>(dY + (size_t)i * LC_COUTP2);
+        dst[0] = make_uint4(pack_bf16(g[0], g[1]), pack_bf16(g[2], 0.0f), 0u, 0u);
+        dst[1] = make_uint4(0u, 0u, 0u, 0u);
     }
     red[threadIdx.x] = l;
     __syncthreads();
@@ -382,20 +557,6 @@ __global__ void sum_kernel(const double *part, int n, double *out)
     if (threadIdx.x == 0) *out = red[0];
 }
 
-// Adam on FP32 master weights (bias-corrected), then the bf16 copies.
-__global__ void adam_kernel(float *w, const float *g, float *m, float *v, int n, float lr, float b1, float b2,
-                            float eps, float c1, float c2)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
-
 // bf16 weight layouts of one layer from its FP32 master [CO][CI][3][3]:
 //   fwd [COp][9][CIp] and bwd-data [CIp2][9][COp2] (taps flipped, channels swapped)
 __global__ void weights_bf16_kernel(const float *w, int CO, int CI, int COp, int CIp, __nv_bfloat16 *fwd, int CIp2,
@@ -411,15 +572,6 @@ __global__ void weights_bf16_kernel(const float *w, int CO, int CI, int COp, int
         const int ftap = 8 - tap;
         bwd[i] = __float2bfloat16((co < CO && ci < CI) ? w[((size_t)co * CI + ci) * 9 + ftap] : 0.0f);
     }
-}
-
-// weight gradient from [9][CO][CI] into the master layout [CO][CI][3][3]
-__global__ void wgrad_layout_kernel(const float *g9, int CO, int CI, int COp, int CIp, float *g)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= CO * CI * 9) return;
-    const int tap = i % 9, ci = (i / 9) % CI, co = i / (9 * CI);
-    g[i] = g9[((size_t)tap * COp + co) * CIp + ci];
 }
 
 // Value of a moment field at grid point (r, c) for -3 <= r < H + 3: columns wrap; a
@@ -456,6 +608,8 @@ __device__ __forceinline__ void lc_differences(const float *a, int H, int W, int
 __global__ void dev_of_moments_kernel(const double *in4, int n, float *dev)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
     if (c >= n) return;
     dev[c] = (float)(in4[c] - 1.0);
     dev[(size_t)n + c] = (float)in4[(size_t)n + c];
@@ -475,8 +629,11 @@ __global__ void features_kernel(const float *dev, int H, int W, const double *si
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t HW = (size_t)H * W;
-    if (i >= H * W) return;
     const int r = i / W, c = i - r * W;
+    const float cos_r = i < H * W ? (float)cos_t[r] : 0.0f, sin_r = i < H * W ? (float)sin_t[r] : 0.0f;
+    pdl_wait();
+    pdl_trigger();
+    if (i >= H * W) return;
     const float *drho = dev, *ut = dev + HW, *up = dev + 2 * HW;
     float raw[LC_NSCALE];
     raw[0] = drho[i];
@@ -506,8 +663,8 @@ __global__ void features_kernel(const float *dev, int H, int W, const double *si
         const float x = raw[q] * sc.inv[q];
         v[q < 4 ? q : q + 2] = fminf(fmaxf(x, -LC_CLAMP), LC_CLAMP);
     }
-    v[4] = (float)cos_t[r];
-    v[5] = (float)sin_t[r];
+    v[4] = cos_r;
+    v[5] = sin_r;
     // the padded input of layer 0 at all positions of (r, c); pole images negate LC_NEGMASK
     uint4 plain[2], image[2];
     __nv_bfloat16 *pb = reinterpret_cast<__nv_bfloat16 *>(plain), *ib = reinterpret_cast<__nv_bfloat16 *>(image);
@@ -849,14 +1006,17 @@ __global__ void vort_grad_kernel(const double *u, int H, int W, int CO, const do
 // Moments (rho, u^theta, u^phi, T) of the FP32 pair layout (dg = ks s (f - w rho_ref)) in FP32
 // arithmetic on the deviations: n = rho_ref + sum dg / s, j = sum v dg / s (the reference
 // state carries no momentum), and T - 1 = (rho_ref |u|^2 + sum df |v - u|^2 - 2 dn) / (2 n),
-// using sum_k w_k |v_k|^2 = 2 (T0 = 1); stored as FP64 for the feature kernel.
-__global__ void lc_moments_kernel(const float2 *f, const Layout L, const VelD c, double rho_ref,
-                                  const double *sin_t, double ks, float *dev)
+// using sum_k w_k |v_k|^2 = 2 (T0 = 1).  FP32 velocities and row factors (inv_ks_s = 1 / (ks s)) from
+// the host: converting them here was a dozen instructions on the FP64 pipe.
+struct VelM { float v[4], rho_ref, drho_ref; };   // drho_ref = rho_ref - 1
+__global__ void lc_moments_kernel(const float2 *f, const Layout L, const VelM c, const float *inv_ks_s, float *dev)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = blockIdx.y;
+    const float inv_s = inv_ks_s[i];
+    pdl_wait();
+    pdl_trigger();
     if (j >= L.np) return;
-    const float inv_s = (float)(1.0 / (ks * sin_t[i]));
     float2 g[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) g[q] = f[L.at(q, i, j)];
@@ -864,25 +1024,25 @@ __global__ void lc_moments_kernel(const float2 *f, const Layout L, const VelD c,
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const int gq = q >> 2, b = q & 3;
-        const float va0 = (float)c.v[2 * gq], va1 = (float)c.v[2 * gq + 1], vb = (float)c.v[b];
+        const float va0 = c.v[2 * gq], va1 = c.v[2 * gq + 1], vb = c.v[b];
         dn += g[q].x + g[q].y;
         jt += va0 * g[q].x + va1 * g[q].y;
         jp += vb * (g[q].x + g[q].y);
     }
     dn *= inv_s;
-    const float n = (float)rho_ref + dn;
+    const float n = c.rho_ref + dn;
     const float ut = jt * inv_s / n, up = jp * inv_s / n;
     float e = 0.0f;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const int gq = q >> 2, b = q & 3;
-        const float va0 = (float)c.v[2 * gq] - ut, va1 = (float)c.v[2 * gq + 1] - ut, vb = (float)c.v[b] - up;
+        const float va0 = c.v[2 * gq] - ut, va1 = c.v[2 * gq + 1] - ut, vb = c.v[b] - up;
         e += g[q].x * (va0 * va0 + vb * vb) + g[q].y * (va1 * va1 + vb * vb);
     }
     e *= inv_s;
-    const float tm1 = ((float)rho_ref * (ut * ut + up * up) + e - 2.0f * dn) / (2.0f * n);
+    const float tm1 = (c.rho_ref * (ut * ut + up * up) + e - 2.0f * dn) / (2.0f * n);
     const size_t HW = (size_t)L.nt * L.np, cell = (size_t)i * L.np + j;
-    dev[cell] = (float)(rho_ref - 1.0) + dn;   // rho - 1 at the resolution of the deviation
+    dev[cell] = c.drho_ref + dn;   // rho - 1 at the resolution of the deviation
     dev[HW + cell] = ut;
     dev[2 * HW + cell] = up;
     dev[3 * HW + cell] = tm1;
@@ -932,58 +1092,69 @@ __device__ __forceinline__ void nudge_cell(float2 *f, const Layout &L, const flo
 }
 
 __global__ void nudge_kernel(float2 *f, const Layout L, const float *dev, const double *delta, const double *mean,
-                             double wsum, const VelN c, const double *sin_t, double ks)
+                             double wsum, const VelN c, const float *ks_s)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = blockIdx.y;
+    const float s = ks_s[i];
+    pdl_wait();
+    pdl_trigger();
     if (j >= L.np) return;
     const size_t n = (size_t)L.nt * L.np, cell = (size_t)i * L.np + j;
     const float drho = (float)(delta[cell] - (*mean) / wsum), dut = (float)delta[n + cell],
                 dup = (float)delta[2 * n + cell];
-    nudge_cell(f, L, dev, i, j, drho, dut, dup, c, (float)(ks * sin_t[i]));
+    nudge_cell(f, L, dev, i, j, drho, dut, dup, c, s);
 }
 
 // The direct form's nudge straight from the net output Y [H][W][CO] (scaled by sc) and the last
 // convolution's nparts partial sums of sin(theta) Y_0: each block reduces the partials to the area
 // mean of drho itself, so neither an outputs pass nor a separate reduction runs.
 __global__ void nudge_direct_kernel(float2 *f, const Layout L, const float *dev, const float *Y, int CO, float3 sc,
-                                    const double *part0, int nparts, double wsum, const VelN c,
-                                    const double *sin_t, double ks)
+                                    const double *part0, int nparts, double wsum, const VelN c, const float *ks_s)
 {
     __shared__ double red[128];
+    const float s = ks_s[blockIdx.y];
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.y;
+    const size_t cell = (size_t)i * L.np + min(j, L.np - 1);
+    pdl_wait();
+    pdl_trigger();
+    // (the cell's output is on its way during the reduction)
+    const float y0 = Y[cell * CO], y1 = Y[cell * CO + 1], y2 = Y[cell * CO + 2];
     double t = 0.0;
-    for (int b = threadIdx.x; b < nparts; b += blockDim.x) t += part0[b];
+#pragma unroll 4
+    for (int b = threadIdx.x; b < nparts; b += 128) t += part0[b];
     red[threadIdx.x] = t;
     __syncthreads();
     for (int k = 64; k > 0; k >>= 1) {
         if ((int)threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
         __syncthreads();
     }
-    const double mean = red[0] * (double)sc.x / wsum;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = blockIdx.y;
     if (j >= L.np) return;
-    const size_t cell = (size_t)i * L.np + j;
-    const float drho = (float)((double)Y[cell * CO] * (double)sc.x - mean);
-    const float dut = (float)((double)Y[cell * CO + 1] * (double)sc.y);
-    const float dup = (float)((double)Y[cell * CO + 2] * (double)sc.z);
-    nudge_cell(f, L, dev, i, j, drho, dut, dup, c, (float)(ks * sin_t[i]));
+    const double mean = red[0] * (double)sc.x / wsum;
+    const float drho = (float)((double)y0 * (double)sc.x - mean);
+    const float dut = (float)((double)y1 * (double)sc.y);
+    const float dup = (float)((double)y2 * (double)sc.z);
+    nudge_cell(f, L, dev, i, j, drho, dut, dup, c, s);
 }
+
+template <int CI, int CO>
+size_t conv_smem(dim3 grid)
+{
+    const size_t in = sizeof(ConvSmem<CI, CO>), out = CO == 8 ? 0 : sizeof(ConvOut) * (CONV_THREADS / 32);
+    return spread_smem((long long)grid.x * grid.y, in > out ? in : out);
+}
+
+dim3 conv_grid(int H, int W) { return dim3((W + CONV_PIX - 1) / CONV_PIX, (H + CONV_ROWS - 1) / CONV_ROWS); }
 
 template <int CI, int CO>
 void conv_launch(const __nv_bfloat16 *Xp, int Hp, int Wp, const __nv_bfloat16 *Wt, const float *bias, float *Yf,
-                 __nv_bfloat16 *Yb, __nv_bfloat16 *Ypad, int relu, cudaStream_t s, double *part0 = nullptr,
+                 __nv_bfloat16 *Yb, __nv_bfloat16 *Ypad, cudaStream_t s, double *part0 = nullptr,
                  const double *sin_t = nullptr)
 {
-    dim3 grid((Wp - 2 + CONV_PIX - 1) / CONV_PIX, Hp - 2);
-    conv3x3_kernel<CI, CO><<<grid, 128, 0, s>>>(Xp, Hp, Wp, Wt, bias, Yf, Yb, Ypad, relu, part0, sin_t);
-}
-
-template <int CI, int CO>
-void wgrad_launch(const __nv_bfloat16 *dY, const __nv_bfloat16 *Xp, int H, int W, float *part, float *partb,
-                  cudaStream_t s)
-{
-    wgrad_kernel<CI, CO><<<H, 128, 0, s>>>(dY, Xp, H, W, part, partb);
+    const dim3 grid = conv_grid(Hp - 2, Wp - 2);
+    launch_after(true, conv3x3_kernel<CI, CO>, grid, CONV_THREADS, conv_smem<CI, CO>(grid), s, Xp, Hp, Wp, Wt, bias, Yf, Yb,
+                 Ypad, part0, sin_t);
 }
 
 }  // namespace
@@ -991,67 +1162,65 @@ void wgrad_launch(const __nv_bfloat16 *dY, const __nv_bfloat16 *Xp, int H, int W
 // ---- the network ----------------------------------------------------------------------
 // Layer l: CI_l -> CO_l; padded channel counts: input 16 (4 used), hidden 32, output 8 (3 used).
 void lc_conv(int layer, const __nv_bfloat16 *Xp, int Hp, int Wp, const __nv_bfloat16 *Wt, const float *bias,
-             float *Yf, __nv_bfloat16 *Yb, __nv_bfloat16 *Ypad, int relu, cudaStream_t s, double *part0,
-             const double *sin_t)
+             float *Yf, __nv_bfloat16 *Yb, __nv_bfloat16 *Ypad, cudaStream_t s, double *part0, const double *sin_t)
 {
-    if (layer == 0) conv_launch<LC_CIN, LC_HID>(Xp, Hp, Wp, Wt, bias, Yf, Yb, Ypad, relu, s);
-    else if (layer < LC_LAYERS - 1) conv_launch<LC_HID, LC_HID>(Xp, Hp, Wp, Wt, bias, Yf, Yb, Ypad, relu, s);
-    else conv_launch<LC_HID, LC_COUT>(Xp, Hp, Wp, Wt, bias, Yf, Yb, Ypad, relu, s, part0, sin_t);
+    if (layer == 0) conv_launch<LC_CIN, LC_HID>(Xp, Hp, Wp, Wt, bias, Yf, Yb, Ypad, s);
+    else if (layer < LC_LAYERS - 1) conv_launch<LC_HID, LC_HID>(Xp, Hp, Wp, Wt, bias, Yf, Yb, Ypad, s);
+    else conv_launch<LC_HID, LC_COUT>(Xp, Hp, Wp, Wt, bias, Yf, Yb, Ypad, s, part0, sin_t);
 }
 
-int lc_conv_ctas(int H, int W) { return ((W + CONV_PIX - 1) / CONV_PIX) * H; }
+int lc_conv_ctas(int H, int W) { return (int)(conv_grid(H, W).x * conv_grid(H, W).y); }
 
-// backward-data convolution of layer l >= 1: input dP [H+4][W+4][COp2], output dXp [H+2][W+2][CI_l]
-void lc_conv_bwd(int layer, const __nv_bfloat16 *dP, int H, int W, const __nv_bfloat16 *Wb, float *dXp, cudaStream_t s)
+cudaError_t lc_prepare_conv()
 {
-    if (layer < LC_LAYERS - 1) conv_launch<LC_HID, LC_HID>(dP, H + 4, W + 4, Wb, nullptr, dXp, nullptr, nullptr, 0, s);
-    else conv_launch<LC_COUTP2, LC_HID>(dP, H + 4, W + 4, Wb, nullptr, dXp, nullptr, nullptr, 0, s);
+    auto set = [](auto *kernel) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SPREAD_SMEM);
+    };
+    cudaError_t e = set(conv3x3_kernel<LC_CIN, LC_HID>);
+    if (e == cudaSuccess) e = set(conv3x3_kernel<LC_HID, LC_HID>);
+    if (e == cudaSuccess) e = set(conv3x3_kernel<LC_HID, LC_COUT>);
+    if (e == cudaSuccess) e = set(conv_bwd_kernel<LC_HID>);
+    if (e == cudaSuccess) e = set(conv_bwd_kernel<LC_COUTP2>);
+    return e;
 }
 
-void lc_wgrad(int layer, const __nv_bfloat16 *dPre, const __nv_bfloat16 *Xp, int H, int W, float *part, float *partb,
-              cudaStream_t s)
+void lc_backward(const LcBackward &p, const LcAdam &adam, const double *loss_part, int nl, double *loss, cudaStream_t s)
 {
-    if (layer == 0) wgrad_launch<LC_CIN, LC_HID>(dPre, Xp, H, W, part, partb, s);
-    else if (layer < LC_LAYERS - 1) wgrad_launch<LC_HID, LC_HID>(dPre, Xp, H, W, part, partb, s);
-    else wgrad_launch<LC_HID, LC_COUTP2>(dPre, Xp, H, W, part, partb, s);
+    const dim3 grid = conv_grid(p.H, p.W);
+    for (int l = LC_LAYERS - 1; l > 0; --l) {
+        const LcWgradLayer &w = p.w[l], &in = p.w[l - 1];
+        if (l == LC_LAYERS - 1) launch_after(true, conv_bwd_kernel<LC_COUTP2>, grid, CONV_THREADS, conv_smem<LC_COUTP2, LC_HID>(grid), s, w.dY, p.H, p.W, w.wb, w.act, in.dY);
+        else launch_after(true, conv_bwd_kernel<LC_HID>, grid, CONV_THREADS, conv_smem<LC_HID, LC_HID>(grid), s, w.dY, p.H, p.W, w.wb, w.act, in.dY);
+    }
+    launch_after(true, wgrad_kernel, dim3(p.ctas, LC_LAYERS), WG_THREADS, 0, s, p, lc_wgrad_rows(p.H));
+    int n = 0;
+    for (int l = 0; l < LC_LAYERS; ++l) n += 9 * p.w[l].cop2 * p.w[l].cip + p.w[l].cop2;
+    launch_after(true, update_kernel, (n + UPD_ELEMS - 1) / UPD_ELEMS + 1, 4 * UPD_ELEMS, 0, s, p, adam, loss_part, nl, loss);
 }
 
-void lc_unpad(const float *dXp, int H, int W, int C, unsigned negmask, float *dX, cudaStream_t s)
-{
-    unpad_kernel<<<dim3(W, H), C, 0, s>>>(dXp, H, W, C, negmask, dX);
-}
+// output rows per CTA of the weight gradients, and the CTAs per layer
+int lc_wgrad_rows(int H) { return (LC_LAYERS * H + 303) / 304; }
+int lc_wgrad_ctas(int H) { return (H + lc_wgrad_rows(H) - 1) / lc_wgrad_rows(H); }
 
-void lc_grad_pad2(const float *dY, const __nv_bfloat16 *act, int H, int W, int C, int CP, __nv_bfloat16 *dP,
-                  cudaStream_t s)
-{
-    grad_pad2_kernel<<<dim3(W + 4, H + 4), CP, 0, s>>>(dY, act, H, W, C, CP, dP);
-}
+int lc_loss_parts(int H, int W) { return (H * W + 255) / 256; }
 
-void lc_grad_pre(const float *dY, const __nv_bfloat16 *act, int n, int C, int CP, __nv_bfloat16 *dPre, cudaStream_t s)
+void lc_grad_pre(const float *dY, int n, int C, int CP, __nv_bfloat16 *dPre, cudaStream_t s)
 {
-    grad_pre_kernel<<<(n * CP + 255) / 256, 256, 0, s>>>(dY, act, n, C, CP, dPre);
-}
-
-void lc_reduce_rows(const float *part, int rows, int n, float *out, cudaStream_t s)
-{
-    reduce_rows_kernel<<<(n + 255) / 256, 256, 0, s>>>(part, rows, n, out);
+    grad_pre_kernel<<<(n * CP + 255) / 256, 256, 0, s>>>(dY, n, C, CP, dPre);
 }
 
 void lc_loss(const float *Y, int CO, const double *target, const double *sin_t, int H, int W, float3 inv_scale,
-             double wsum, float *dY, double *part, double *loss, cudaStream_t s)
+             double wsum, __nv_bfloat16 *dY, double *part, cudaStream_t s)
 {
-    const int nb = (H * W + 255) / 256;
-    loss_kernel<<<nb, 256, 0, s>>>(Y, CO, target, sin_t, H, W, inv_scale, wsum, dY, part);
-    sum_kernel<<<1, 256, 0, s>>>(part, nb, loss);
+    launch_after(true, loss_kernel, (H * W + 255) / 256, 256, 0, s, Y, CO, target, sin_t, H, W, inv_scale,
+                 1.0 / (3.0 * wsum), dY, part);
 }
 
 void lc_stream_loss(const float *Y, int CO, const double *target, const double *sin_t, const LcStream &g,
-                    double inv_s1, double inv_s2, double wsum, double *gv, float *dY, double *part, double *loss,
-                    cudaStream_t s)
+                    double inv_s1, double inv_s2, double wsum, double *gv, float *dY, double *part, cudaStream_t s)
 {
     const int nb = (g.H * g.W + 255) / 256;
     stream_loss_kernel<float><<<nb, 256, 0, s>>>(Y, CO, target, sin_t, g, inv_s1, inv_s2, wsum, gv, part);
-    sum_kernel<<<1, 256, 0, s>>>(part, nb, loss);
     stream_adjoint_kernel<float><<<nb, 256, 0, s>>>(gv, CO, g, sin_t, dY);
 }
 
@@ -1080,14 +1249,13 @@ static void poisson(const double *x, int inv_sin, int nb, double *psi, const LcP
 
 void lc_vort_loss(const float *Y, int CO, const double *target, const double *sin_t, const LcStream &g,
                   const LcPoisson &P, double inv_s1, double inv_s2, double wsum, double *gv, float *dY, double *part,
-                  double *loss, cudaStream_t s)
+                  cudaStream_t s)
 {
     const int n = g.H * g.W, nb = (n + 255) / 256;
     const LcStream g1{g.H, g.W, 1.0, g.R, g.dth, g.dph};
     vort_in_kernel<<<nb, 256, 0, s>>>(Y, CO, n, g.W, g.s0, sin_t, P.w, P.part);
     poisson(P.w, 0, nb, P.psi, P, sin_t, s);
     stream_loss_kernel<double><<<nb, 256, 0, s>>>(P.psi, 1, target, sin_t, g1, inv_s1, inv_s2, wsum, gv, part);
-    sum_kernel<<<1, 256, 0, s>>>(part, nb, loss);
     // backward: the curl's adjoint, the solve's adjoint S P S^-1 and the mean removal's
     stream_adjoint_kernel<double><<<nb, 256, 0, s>>>(gv, 1, g1, sin_t, P.w);
     cell_sums_kernel<<<nb, 256, 0, s>>>(P.w, n, P.W, sin_t, 0, P.part);
@@ -1158,12 +1326,6 @@ int lc_poisson_tables(int H, int W, float *dev)
     return cudaMemcpy(dev, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice) == cudaSuccess ? 0 : -1;
 }
 
-void lc_adam(float *w, const float *g, float *m, float *v, int n, float lr, float b1, float b2, float eps, float c1,
-             float c2, cudaStream_t s)
-{
-    adam_kernel<<<(n + 255) / 256, 256, 0, s>>>(w, g, m, v, n, lr, b1, b2, eps, c1, c2);
-}
-
 void lc_weights_bf16(const float *w, int CO, int CI, int COp, int CIp, __nv_bfloat16 *fwd, int CIp2, int COp2,
                      __nv_bfloat16 *bwd, cudaStream_t s)
 {
@@ -1171,21 +1333,15 @@ void lc_weights_bf16(const float *w, int CO, int CI, int COp, int CIp, __nv_bflo
     weights_bf16_kernel<<<(n + 255) / 256, 256, 0, s>>>(w, CO, CI, COp, CIp, fwd, CIp2, COp2, bwd);
 }
 
-void lc_wgrad_layout(const float *g9, int CO, int CI, int COp, int CIp, float *g, cudaStream_t s)
-{
-    const int n = CO * CI * 9;
-    wgrad_layout_kernel<<<(n + 255) / 256, 256, 0, s>>>(g9, CO, CI, COp, CIp, g);
-}
-
 void lc_features(const float *dev, int H, int W, const double *sin_t, const double *cos_t,
                  const LcInScale &inv_scale, __nv_bfloat16 *Xp, cudaStream_t s)
 {
-    features_kernel<<<(H * W + 255) / 256, 256, 0, s>>>(dev, H, W, sin_t, cos_t, inv_scale, Xp);
+    launch_after(true, features_kernel, (H * W + 127) / 128, 128, 0, s, dev, H, W, sin_t, cos_t, inv_scale, Xp);
 }
 
 void lc_dev_of_moments(const double *in4, int H, int W, float *dev, cudaStream_t s)
 {
-    dev_of_moments_kernel<<<(H * W + 255) / 256, 256, 0, s>>>(in4, H * W, dev);
+    launch_after(true, dev_of_moments_kernel, (H * W + 255) / 256, 256, 0, s, in4, H * W, dev);
 }
 
 void lc_outputs(const float *Y, int CO, int H, int W, float3 scale, const double *sin_t, double *out, double *part,
@@ -1196,34 +1352,36 @@ void lc_outputs(const float *Y, int CO, int H, int W, float3 scale, const double
     sum_kernel<<<1, 256, 0, s>>>(part, nb, mean);
 }
 
-void lc_moments(const float2 *f, const Layout &L, const VelD &c, double rho_ref, const double *sin_t, double ks,
-                float *dev, cudaStream_t s)
+void lc_moments(const float2 *f, const Layout &L, const VelD &c, double rho_ref, const float *inv_ks_s, float *dev,
+                cudaStream_t s)
 {
-    dim3 grid((L.np + 127) / 128, L.nt);
-    lc_moments_kernel<<<grid, 128, 0, s>>>(f, L, c, rho_ref, sin_t, ks, dev);
+    VelM cm;
+    for (int a = 0; a < 4; ++a) cm.v[a] = (float)c.v[a];
+    cm.rho_ref = (float)rho_ref;
+    cm.drho_ref = (float)(rho_ref - 1.0);
+    launch_after(true, lc_moments_kernel, dim3((L.np + 127) / 128, L.nt), 128, 0, s, f, L, cm, inv_ks_s, dev);
 }
 
 void lc_nudge(float2 *f, const Layout &L, const float *dev, const double *delta, const double *mean, double wsum,
-              const VelD &c, const double *sin_t, double ks, cudaStream_t s)
+              const VelD &c, const float *ks_s, cudaStream_t s)
 {
     VelN cn;
     for (int a = 0; a < 4; ++a) cn.v[a] = (float)c.v[a];
     for (int a = 0; a < 4; ++a)
         for (int b = 0; b < 4; ++b) cn.w[4 * a + b] = (float)(c.w[a] * c.w[b]);
     dim3 grid((L.np + 127) / 128, L.nt);
-    nudge_kernel<<<grid, 128, 0, s>>>(f, L, dev, delta, mean, wsum, cn, sin_t, ks);
+    launch_after(true, nudge_kernel, grid, 128, 0, s, f, L, dev, delta, mean, wsum, cn, ks_s);
 }
 
 void lc_nudge_direct(float2 *f, const Layout &L, const float *dev, const float *Y, int CO, float3 scale,
-                     const double *part0, int nparts, double wsum, const VelD &c, const double *sin_t, double ks,
-                     cudaStream_t s)
+                     const double *part0, int nparts, double wsum, const VelD &c, const float *ks_s, cudaStream_t s)
 {
     VelN cn;
     for (int a = 0; a < 4; ++a) cn.v[a] = (float)c.v[a];
     for (int a = 0; a < 4; ++a)
         for (int b = 0; b < 4; ++b) cn.w[4 * a + b] = (float)(c.w[a] * c.w[b]);
     dim3 grid((L.np + 127) / 128, L.nt);
-    nudge_direct_kernel<<<grid, 128, 0, s>>>(f, L, dev, Y, CO, scale, part0, nparts, wsum, cn, sin_t, ks);
+    launch_after(true, nudge_direct_kernel, grid, 128, 0, s, f, L, dev, Y, CO, scale, part0, nparts, wsum, cn, ks_s);
 }
 
 }  // namespace vk

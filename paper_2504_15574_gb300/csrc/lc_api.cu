@@ -28,11 +28,11 @@ struct vlbm_lc {
     __nv_bfloat16 *d_wf[LC_LAYERS] = {}, *d_wb[LC_LAYERS] = {};
     double *d_sin = nullptr, *d_cos = nullptr, *d_in = nullptr, *d_tg = nullptr, *d_out = nullptr, *d_part = nullptr, *d_scal = nullptr;
     __nv_bfloat16 *d_xp[LC_LAYERS] = {}, *d_z[LC_LAYERS] = {};
-    float *d_y = nullptr, *d_dy = nullptr, *d_dxp = nullptr, *d_dx = nullptr;
+    float *d_y = nullptr, *d_dy = nullptr;
     float *d_dev = nullptr;      // the network's moment deviations (rho - 1, u^theta, u^phi, T - 1) [4][H][W]
     double *d_cpart = nullptr;   // direct-form correction: the last layer's per-CTA sums of sin(theta) output 0
-    __nv_bfloat16 *d_dp = nullptr, *d_dpre = nullptr;
-    float *d_wpart = nullptr, *d_bpart = nullptr, *d_g9 = nullptr;
+    __nv_bfloat16 *d_dpre[LC_LAYERS] = {};   // gradients at the pre-activations [H][W][cop2]
+    float *d_wpart[LC_LAYERS] = {}, *d_bpart[LC_LAYERS] = {};   // their weight gradients' partial sums per CTA
     double wsum = 0.0;
     float in_scale[LC_NSCALE] = {1e-3f, 1e-2f, 1e-2f, 1e-3f, 1e-6f, 1e-6f, 1e-5f, 1e-5f, 1e-5f,
                                  1e-5f, 1e-5f, 1e-5f, 1e-5f, 1e-5f};
@@ -47,12 +47,23 @@ struct vlbm_lc {
     bool vort_ok = false;        // the vorticity form's mode solve fits this grid
     long long t = 0;
     std::vector<void *> bufs;
-    cudaGraphExec_t g_exec = nullptr;   // vlbm_lc_rollout: one corrected step of solver g_solver
+    // vlbm_lc_rollout: one corrected step of solver g_solver, and ROLL_STEPS of them (within a graph the
+    // launches of consecutive steps overlap; between graphs they do not)
+    cudaGraphExec_t g_exec = nullptr, g_many = nullptr;
     vlbm_t *g_solver = nullptr;
     unsigned long long g_gen = 0;       // the solver's step generation when g_exec was captured
 };
 
 namespace {
+
+constexpr int ROLL_STEPS = 8;
+
+void drop_rollout(vlbm_lc_t *n)
+{
+    if (n->g_exec) cudaGraphExecDestroy(n->g_exec);
+    if (n->g_many) cudaGraphExecDestroy(n->g_many);
+    n->g_exec = n->g_many = nullptr;
+}
 
 int lfail(vlbm_lc_t *n, int code, const std::string &m)
 {
@@ -109,8 +120,8 @@ int forward(vlbm_lc_t *n, const float *dev, cudaStream_t s, bool keep = true, do
     for (int l = 0; l < LC_LAYERS; ++l) {
         const bool last = (l == LC_LAYERS - 1);
         lc_conv(l, n->d_xp[l], H + 2, W + 2, n->d_wf[l], n->d_w + n->boff[l], last ? n->d_y : nullptr,
-                (last || !keep) ? nullptr : n->d_z[l], last ? nullptr : n->d_xp[l + 1], last ? 0 : 1, s,
-                last ? part0 : nullptr, n->d_sin);
+                (last || !keep) ? nullptr : n->d_z[l], last ? nullptr : n->d_xp[l + 1], s, last ? part0 : nullptr,
+                n->d_sin);
     }
     LCK(n, cudaGetLastError());
     return VLBM_OK;
@@ -145,36 +156,34 @@ void enqueue_outputs(vlbm_lc_t *n, cudaStream_t s)
     }
 }
 
-// loss and gradient of every parameter into d_g; loss into d_scal[0]
-int backward(vlbm_lc_t *n)
+// loss and gradient of every parameter into d_g; loss into d_scal[0]; with lr > 0 the Adam step t too
+int backward(vlbm_lc_t *n, float lr = 0.0f)
 {
     const int H = n->H, W = n->W, HW = H * W;
-    if (n->form == VLBM_LC_VORTICITY) {
-        lc_vort_loss(n->d_y, LC_COUT, n->d_tg, n->d_sin, stream_geometry(n), poisson_work(n), 1.0 / n->out_scale[1],
-                     1.0 / n->out_scale[2], n->wsum, n->d_gv, n->d_dy, n->d_part, n->d_scal, n->stream);
-    } else if (n->form == VLBM_LC_STREAM) {
-        lc_stream_loss(n->d_y, LC_COUT, n->d_tg, n->d_sin, stream_geometry(n), 1.0 / n->out_scale[1],
-                       1.0 / n->out_scale[2], n->wsum, n->d_gv, n->d_dy, n->d_part, n->d_scal, n->stream);
-    } else {
+    if (n->form == VLBM_LC_DIRECT) {
         const float3 ios = make_float3(1.0f / n->out_scale[0], 1.0f / n->out_scale[1], 1.0f / n->out_scale[2]);
-        lc_loss(n->d_y, LC_COUT, n->d_tg, n->d_sin, H, W, ios, n->wsum, n->d_dy, n->d_part, n->d_scal, n->stream);
+        lc_loss(n->d_y, LC_COUT, n->d_tg, n->d_sin, H, W, ios, n->wsum, n->d_dpre[LC_LAYERS - 1], n->d_part, n->stream);
+    } else {
+        if (n->form == VLBM_LC_VORTICITY)
+            lc_vort_loss(n->d_y, LC_COUT, n->d_tg, n->d_sin, stream_geometry(n), poisson_work(n),
+                         1.0 / n->out_scale[1], 1.0 / n->out_scale[2], n->wsum, n->d_gv, n->d_dy, n->d_part, n->stream);
+        else
+            lc_stream_loss(n->d_y, LC_COUT, n->d_tg, n->d_sin, stream_geometry(n), 1.0 / n->out_scale[1],
+                           1.0 / n->out_scale[2], n->wsum, n->d_gv, n->d_dy, n->d_part, n->stream);
+        lc_grad_pre(n->d_dy, HW, LC_COUT, LC_COUTP2, n->d_dpre[LC_LAYERS - 1], n->stream);
     }
-    // gradient at the output of layer l lives in d_dy with cop[l] channels
-    for (int l = LC_LAYERS - 1; l >= 0; --l) {
-        const int C = n->cop[l], CP = n->cop2[l];
-        const __nv_bfloat16 *act = (l == LC_LAYERS - 1) ? nullptr : n->d_z[l];
-        lc_grad_pre(n->d_dy, act, HW, C, CP, n->d_dpre, n->stream);
-        lc_wgrad(l, n->d_dpre, n->d_xp[l], H, W, n->d_wpart, n->d_bpart, n->stream);
-        lc_reduce_rows(n->d_wpart, H, 9 * n->cop2[l] * n->cip[l], n->d_g9, n->stream);
-        lc_wgrad_layout(n->d_g9, n->co[l], n->ci[l], n->cop2[l], n->cip[l], n->d_g + n->woff[l], n->stream);
-        lc_reduce_rows(n->d_bpart, H, n->cop2[l], n->d_dx, n->stream);   // bias gradient (first co entries)
-        LCK(n, cudaMemcpyAsync(n->d_g + n->boff[l], n->d_dx, sizeof(float) * n->co[l], cudaMemcpyDeviceToDevice,
-                               n->stream));
-        if (l == 0) break;
-        lc_grad_pad2(n->d_dy, act, H, W, C, CP, n->d_dp, n->stream);
-        lc_conv_bwd(l, n->d_dp, H, W, n->d_wb[l], n->d_dxp, n->stream);
-        lc_unpad(n->d_dxp, H, W, LC_HID, 0u, n->d_dy, n->stream);      // gradient at the output of layer l-1
-    }
+    LcBackward p;
+    p.H = H;
+    p.W = W;
+    p.ctas = lc_wgrad_ctas(H);
+    for (int l = 0; l < LC_LAYERS; ++l)
+        p.w[l] = LcWgradLayer{n->d_dpre[l], n->d_xp[l], l ? n->d_z[l - 1] : nullptr, n->d_wf[l],
+                              l ? n->d_wb[l] : nullptr, n->d_wpart[l], n->d_bpart[l], n->ci[l], n->co[l], n->cip[l],
+                              n->cop2[l], n->woff[l], n->boff[l]};
+    const float b1 = 0.9f, b2 = 0.999f;
+    const float c1 = 1.0f - std::pow(b1, (float)n->t), c2 = 1.0f - std::pow(b2, (float)n->t);
+    const LcAdam adam{lr > 0.0f, n->d_g, n->d_w, n->d_m, n->d_v, lr, b1, b2, 1e-8f, c1, c2};
+    lc_backward(p, adam, n->d_part, lc_loss_parts(H, W), n->d_scal, n->stream);
     LCK(n, cudaGetLastError());
     return VLBM_OK;
 }
@@ -194,21 +203,43 @@ int check_solver(vlbm_lc_t *n, vlbm_t *h)
 // cell's ghost images).
 int enqueue_correction(vlbm_lc_t *n, vlbm_t *h, cudaStream_t s)
 {
-    lc_moments((const float2 *)h->F, h->L, h->vd, h->rho_ref, h->d_sin_t, h->kscale, n->d_dev, s);
+    lc_moments((const float2 *)h->F, h->L, h->vd, h->rho_ref, h->d_ikss, n->d_dev, s);
     int rc;
     if (n->form == VLBM_LC_DIRECT) {
         // the output scaling and the area mean of drho ride on the last convolution and the nudge
         if ((rc = forward(n, n->d_dev, s, false, n->d_cpart))) return rc;
         const float3 sc = make_float3(n->out_scale[0], n->out_scale[1], n->out_scale[2]);
         lc_nudge_direct((float2 *)h->F, h->L, n->d_dev, n->d_y, LC_COUT, sc, n->d_cpart, lc_conv_ctas(n->H, n->W),
-                        n->wsum, h->vd, n->d_sin, h->kscale, s);
+                        n->wsum, h->vd, h->d_kss, s);
         LCK(n, cudaGetLastError());
         return VLBM_OK;
     }
     if ((rc = forward(n, n->d_dev, s, false))) return rc;
     enqueue_outputs(n, s);
-    lc_nudge((float2 *)h->F, h->L, n->d_dev, n->d_out, n->d_scal + 1, n->wsum, h->vd, n->d_sin, h->kscale, s);
+    lc_nudge((float2 *)h->F, h->L, n->d_dev, n->d_out, n->d_scal + 1, n->wsum, h->vd, h->d_kss, s);
     LCK(n, cudaGetLastError());
+    return VLBM_OK;
+}
+
+// `steps` corrected coarse steps (the solver's RK3 step, then the correction) as a graph
+int capture_rollout(vlbm_lc_t *n, vlbm_t *h, int steps, cudaGraphExec_t *exec)
+{
+    cudaGraph_t g = nullptr;
+    LCK(n, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
+    int rc = VLBM_OK;
+    for (int q = 0; q < steps && !rc; ++q) {
+        solver_enqueue_step(h);
+        rc = enqueue_correction(n, h, h->stream);
+    }
+    cudaError_t e = cudaStreamEndCapture(h->stream, &g);
+    if (rc) {
+        if (g) cudaGraphDestroy(g);
+        return rc;
+    }
+    if (e != cudaSuccess) return lfail(n, VLBM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+    e = cudaGraphInstantiate(exec, g, cudaGraphInstantiateFlagUseNodePriority);
+    cudaGraphDestroy(g);
+    if (e != cudaSuccess) return lfail(n, VLBM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
     return VLBM_OK;
 }
 
@@ -262,8 +293,7 @@ int vlbm_lc_create(int n_theta, int n_phi, unsigned long long seed, vlbm_lc_t **
         for (size_t q = 0; q < (size_t)co[l] * ci[l] * 9; ++q)
             w[n->woff[l] + q] = (float)(a * (2.0 * ((smix(s) >> 11) * (1.0 / 9007199254740992.0)) - 1.0));
     }
-    const size_t HW = (size_t)n_theta * n_phi, HWp = (size_t)(n_theta + 2) * (n_phi + 2),
-                 HWp2 = (size_t)(n_theta + 4) * (n_phi + 4);
+    const size_t HW = (size_t)n_theta * n_phi, HWp = (size_t)(n_theta + 2) * (n_phi + 2);
     int rc = 0;
     auto A = [&](auto **p, size_t c) {
         if (!rc) rc = lalloc(n, p, c);
@@ -277,6 +307,9 @@ int vlbm_lc_create(int n_theta, int n_phi, unsigned long long seed, vlbm_lc_t **
         A(&n->d_wb[l], (size_t)n->cip[l] * 9 * n->cop2[l]);
         A(&n->d_xp[l], HWp * n->cip[l]);
         A(&n->d_z[l], HW * LC_HID);
+        A(&n->d_dpre[l], HW * n->cop2[l]);
+        A(&n->d_wpart[l], (size_t)lc_wgrad_ctas(n_theta) * 9 * n->cop2[l] * n->cip[l]);
+        A(&n->d_bpart[l], (size_t)lc_wgrad_ctas(n_theta) * n->cop2[l]);
     }
     A(&n->d_sin, (size_t)n_theta);
     A(&n->d_cos, (size_t)n_theta);
@@ -288,14 +321,7 @@ int vlbm_lc_create(int n_theta, int n_phi, unsigned long long seed, vlbm_lc_t **
     A(&n->d_part, HW / 256 + 2);
     A(&n->d_scal, 4);
     A(&n->d_y, HW * LC_COUT);
-    A(&n->d_dy, HW * LC_HID);
-    A(&n->d_dxp, HWp * LC_HID);
-    A(&n->d_dx, HW * LC_HID);
-    A(&n->d_dp, HWp2 * LC_HID);
-    A(&n->d_dpre, HW * LC_HID);
-    A(&n->d_wpart, (size_t)n_theta * 9 * LC_HID * LC_HID);
-    A(&n->d_bpart, (size_t)n_theta * LC_HID);
-    A(&n->d_g9, (size_t)9 * LC_HID * LC_HID);
+    A(&n->d_dy, HW * LC_COUT);
     A(&n->d_gv, 2 * HW);
     const size_t M = (size_t)n_phi / 2 + 1;
     A(&n->d_ptabs, lc_poisson_table_floats(n_theta, n_phi));
@@ -320,7 +346,7 @@ int vlbm_lc_create(int n_theta, int n_phi, unsigned long long seed, vlbm_lc_t **
     if (cudaMemcpy(n->d_sin, sn.data(), sizeof(double) * n_theta, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(n->d_cos, cs.data(), sizeof(double) * n_theta, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(n->d_w, w.data(), sizeof(float) * off, cudaMemcpyHostToDevice) != cudaSuccess ||
-        lc_poisson_tables(n_theta, n_phi, n->d_ptabs) != 0 ||
+        lc_poisson_tables(n_theta, n_phi, n->d_ptabs) != 0 || lc_prepare_conv() != cudaSuccess ||
         refresh_bf16(n) != VLBM_OK || cudaStreamSynchronize(n->stream) != cudaSuccess) {
         vlbm_lc_destroy(n);
         return VLBM_ERR_CUDA;
@@ -365,10 +391,7 @@ int vlbm_lc_set_scales(vlbm_lc_t *n, const double *in_scale, const double *out_s
         if (!(out_scale[q] >= 0.0) || !std::isfinite(out_scale[q]))
             return lfail(n, VLBM_ERR_ARG, "output scales must be >= 0");
     for (int q = 0; q < LC_NSCALE; ++q) n->in_scale[q] = (float)in_scale[q];
-    if (n->g_exec) {   // the scales are kernel arguments of the captured rollout step
-        cudaGraphExecDestroy(n->g_exec);
-        n->g_exec = nullptr;
-    }
+    drop_rollout(n);   // the scales are kernel arguments of the captured rollout step
     for (int q = 0; q < 3; ++q) n->out_scale[q] = (float)out_scale[q];
     return VLBM_OK;
 }
@@ -381,10 +404,7 @@ int vlbm_lc_set_output_form(vlbm_lc_t *n, int form, double radius)
     if (form == VLBM_LC_VORTICITY && !n->vort_ok)
         return lfail(n, VLBM_ERR_UNSUPPORTED, "the vorticity form's mode solve does not fit this many rows");
     if (!(radius > 0.0) || !std::isfinite(radius)) return lfail(n, VLBM_ERR_ARG, "radius must be > 0");
-    if (n->g_exec) {   // the form is part of the captured rollout step
-        cudaGraphExecDestroy(n->g_exec);
-        n->g_exec = nullptr;
-    }
+    drop_rollout(n);   // the form is part of the captured rollout step
     n->form = form;
     n->radius = radius;
     return VLBM_OK;
@@ -426,12 +446,9 @@ int vlbm_lc_train_step(vlbm_lc_t *n, const double *inputs, const double *targets
     if (!n || !inputs || !targets || !(lr > 0.0f)) return VLBM_ERR_ARG;
     if (int rc0 = check_trainable(n)) return rc0;
     int rc;
-    if ((rc = upload_io(n, inputs, targets)) || (rc = forward(n, n->d_dev, n->stream)) || (rc = backward(n))) return rc;
+    if ((rc = upload_io(n, inputs, targets)) || (rc = forward(n, n->d_dev, n->stream))) return rc;
     n->t += 1;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.0f - std::pow(b1, (float)n->t), c2 = 1.0f - std::pow(b2, (float)n->t);
-    lc_adam(n->d_w, n->d_g, n->d_m, n->d_v, n->nparam, lr, b1, b2, 1e-8f, c1, c2, n->stream);
-    if ((rc = refresh_bf16(n))) return rc;
+    if ((rc = backward(n, lr))) return rc;
     if (loss) LCK(n, cudaMemcpyAsync(loss, n->d_scal, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
     LCK(n, cudaStreamSynchronize(n->stream));
     return VLBM_OK;
@@ -454,29 +471,14 @@ int vlbm_lc_rollout(vlbm_lc_t *n, vlbm_t *h, int steps)
     if (!h->d_row) return lfail(n, VLBM_ERR_ARG, "FP32 state not initialised");
     // the captured step holds the solver's launch parameters (its FP32 reference density among
     // them): rebuild for another solver or once the solver has renewed them
-    if (n->g_exec && (n->g_solver != h || n->g_gen != h->step_gen)) {
-        cudaGraphExecDestroy(n->g_exec);
-        n->g_exec = nullptr;
-    }
-    if (!n->g_exec) {
-        // one corrected coarse step (the solver's RK3 step, then the correction) as a graph
-        cudaGraph_t g = nullptr;
-        LCK(n, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-        solver_enqueue_step(h);
-        rc = enqueue_correction(n, h, h->stream);
-        cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-        if (rc) {
-            if (g) cudaGraphDestroy(g);
-            return rc;
-        }
-        if (e != cudaSuccess) return lfail(n, VLBM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-        e = cudaGraphInstantiate(&n->g_exec, g, cudaGraphInstantiateFlagUseNodePriority);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) return lfail(n, VLBM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-        n->g_solver = h;
-        n->g_gen = h->step_gen;
-    }
-    for (int q = 0; q < steps; ++q) LCK(n, cudaGraphLaunch(n->g_exec, h->stream));
+    if (n->g_exec && (n->g_solver != h || n->g_gen != h->step_gen)) drop_rollout(n);
+    if (!n->g_exec && (rc = capture_rollout(n, h, 1, &n->g_exec))) return rc;
+    if (steps >= ROLL_STEPS && !n->g_many && (rc = capture_rollout(n, h, ROLL_STEPS, &n->g_many))) return rc;
+    n->g_solver = h;
+    n->g_gen = h->step_gen;
+    int left = steps;
+    for (; left >= ROLL_STEPS; left -= ROLL_STEPS) LCK(n, cudaGraphLaunch(n->g_many, h->stream));
+    for (; left > 0; --left) LCK(n, cudaGraphLaunch(n->g_exec, h->stream));
     solver_count_steps(h, steps);
     if ((rc = vlbm_sync(h))) return lfail(n, rc, vlbm_last_error(h));
     return VLBM_OK;
@@ -488,7 +490,7 @@ void vlbm_lc_destroy(vlbm_lc_t *n)
 {
     if (!n) return;
     if (n->stream) cudaStreamSynchronize(n->stream);
-    if (n->g_exec) cudaGraphExecDestroy(n->g_exec);
+    drop_rollout(n);
     for (void *p : n->bufs) cudaFree(p);
     if (n->stream) cudaStreamDestroy(n->stream);
     delete n;

@@ -24,48 +24,70 @@ constexpr float LC_CLAMP = 8.0f;   // bound of every scaled input feature
 constexpr unsigned LC_NEGMASK = (1u << 1) | (1u << 2) | (1u << 5) | (0xFFu << 8);
 struct LcInScale { float inv[LC_NSCALE]; };
 
-// Layer `layer` on the padded input Xp: FP32 pre-activations Yf, BF16 (ReLU) outputs Yb
-// [H][W][CO] and / or the next layer's padded input Ypad [H+2][W+2][CO] (any may be NULL).
-// part0 (last layer only; optional): per CTA of the launch (lc_conv_ctas of them) the sum over its
-// pixels of sin_t[row] times output 0.
+// Layer `layer` on the padded input Xp.  Hidden layers: after the ReLU the BF16 outputs Yb [H][W][CO] (may be
+// NULL) and the next layer's padded input Ypad [H+2][W+2][CO].  Last layer: FP32 outputs Yf, and part0
+// (optional): per CTA of the launch (lc_conv_ctas of them) the sum over its pixels of sin_t[row] times
+// output 0.
 void lc_conv(int layer, const __nv_bfloat16 *Xp, int Hp, int Wp, const __nv_bfloat16 *Wt, const float *bias,
-             float *Yf, __nv_bfloat16 *Yb, __nv_bfloat16 *Ypad, int relu, cudaStream_t s,
-             double *part0 = nullptr, const double *sin_t = nullptr);
+             float *Yf, __nv_bfloat16 *Yb, __nv_bfloat16 *Ypad, cudaStream_t s, double *part0 = nullptr,
+             const double *sin_t = nullptr);
+// Raises the convolutions' shared-memory limits (call outside any stream capture).
+cudaError_t lc_prepare_conv();
 int lc_conv_ctas(int H, int W);
-void lc_conv_bwd(int layer, const __nv_bfloat16 *dP, int H, int W, const __nv_bfloat16 *Wb, float *dXp, cudaStream_t s);
-void lc_wgrad(int layer, const __nv_bfloat16 *dPre, const __nv_bfloat16 *Xp, int H, int W, float *part, float *partb,
-              cudaStream_t s);
-void lc_unpad(const float *dXp, int H, int W, int C, unsigned negmask, float *dX, cudaStream_t s);
-void lc_grad_pad2(const float *dY, const __nv_bfloat16 *act, int H, int W, int C, int CP, __nv_bfloat16 *dP,
-                  cudaStream_t s);
-void lc_grad_pre(const float *dY, const __nv_bfloat16 *act, int n, int C, int CP, __nv_bfloat16 *dPre, cudaStream_t s);
-void lc_reduce_rows(const float *part, int rows, int n, float *out, cudaStream_t s);
+// One layer of the backward pass: its gradient dY at the pre-activation [H][W][cop2] (BF16), its padded
+// input Xp [H+2][W+2][cip], the activations act [H][W][32] that its input was (the ReLU mask of the layer
+// below; NULL for layer 0), BF16 weights (forward wf, backward data wb; NULL for layer 0), partial sums of
+// its weight and bias gradients per CTA, channel counts and master offsets.
+struct LcWgradLayer {
+    __nv_bfloat16 *dY;
+    const __nv_bfloat16 *Xp, *act;
+    __nv_bfloat16 *wf, *wb;
+    float *part, *partb;
+    int ci, co, cip, cop2;
+    size_t woff, boff;
+};
+struct LcBackward {
+    int H, W, ctas;   // ctas: lc_wgrad_ctas(H)
+    LcWgradLayer w[LC_LAYERS];
+};
+// Gradient output g and, with step set, the Adam step of the master weights w (m, v: moments; c1, c2: bias
+// corrections).
+struct LcAdam {
+    int step;
+    float *g, *w, *m, *v;
+    float lr, b1, b2, eps, c1, c2;
+};
+int lc_wgrad_rows(int H);
+int lc_wgrad_ctas(int H);
+// The backward pass from the last layer's dY, the update, and the loss from its nl partial sums.
+void lc_backward(const LcBackward &p, const LcAdam &adam, const double *loss_part, int nl, double *loss,
+                 cudaStream_t s);
+// The loss's partial sums (lc_loss_parts of them) and the last layer's dY (direct form) or the gradient at
+// the network's output (the other forms, for lc_grad_pre).
+int lc_loss_parts(int H, int W);
 void lc_loss(const float *Y, int CO, const double *target, const double *sin_t, int H, int W, float3 inv_scale,
-             double wsum, float *dY, double *part, double *loss, cudaStream_t s);
-void lc_adam(float *w, const float *g, float *m, float *v, int n, float lr, float b1, float b2, float eps, float c1,
-             float c2, cudaStream_t s);
+             double wsum, __nv_bfloat16 *dY, double *part, cudaStream_t s);
+void lc_grad_pre(const float *dY, int n, int C, int CP, __nv_bfloat16 *dPre, cudaStream_t s);
 void lc_weights_bf16(const float *w, int CO, int CI, int COp, int CIp, __nv_bfloat16 *fwd, int CIp2, int COp2,
                      __nv_bfloat16 *bwd, cudaStream_t s);
-void lc_wgrad_layout(const float *g9, int CO, int CI, int COp, int CIp, float *g, cudaStream_t s);
 // The padded layer-0 input from the moment deviations dev = (rho - 1, u^theta, u^phi, T - 1)
 // [4][H][W] (FP32).
 void lc_features(const float *dev, int H, int W, const double *sin_t, const double *cos_t,
                  const LcInScale &inv_scale, __nv_bfloat16 *Xp, cudaStream_t s);
 // The deviations dev [4][H][W] (FP32) of FP64 moments (rho, u^theta, u^phi, T) [4][H][W].
 void lc_dev_of_moments(const double *in4, int H, int W, float *dev, cudaStream_t s);
-// The deviations (rho - 1, u^theta, u^phi, T - 1) [4][H][W] of a solver's FP32 state (state scale
-// ks), FP32 arithmetic on the stored deviations.
-void lc_moments(const float2 *f, const Layout &L, const VelD &c, double rho_ref, const double *sin_t, double ks,
-                float *dev, cudaStream_t s);
+// The deviations (rho - 1, u^theta, u^phi, T - 1) [4][H][W] of a solver's FP32 state (inv_ks_s: its
+// 1 / (k sin theta) per row), FP32 arithmetic on the stored deviations.
+void lc_moments(const float2 *f, const Layout &L, const VelD &c, double rho_ref, const float *inv_ks_s, float *dev,
+                cudaStream_t s);
 void lc_outputs(const float *Y, int CO, int H, int W, float3 scale, const double *sin_t, double *out, double *part,
                 double *mean, cudaStream_t s);
 void lc_nudge(float2 *f, const Layout &L, const float *dev, const double *delta, const double *mean, double wsum,
-              const VelD &c, const double *sin_t, double ks, cudaStream_t s);
+              const VelD &c, const float *ks_s, cudaStream_t s);   // ks_s: the solver's k sin(theta) per row
 // The direct form's nudge from the net output Y [H][W][CO] (times scale) and the last layer's
 // nparts partial sums of sin(theta) output 0 (the area mean of drho is removed).
 void lc_nudge_direct(float2 *f, const Layout &L, const float *dev, const float *Y, int CO, float3 scale,
-                     const double *part0, int nparts, double wsum, const VelD &c, const double *sin_t, double ks,
-                     cudaStream_t s);
+                     const double *part0, int nparts, double wsum, const VelD &c, const float *ks_s, cudaStream_t s);
 // Stream-function output form: output 0 times s0 is a stream function psi on the H x W cell grid
 // of a sphere of radius R (dth = pi / H, dph = 2 pi / W), the correction its centred curl
 // (0, d_phi psi / (R sin theta), -d_theta psi / R), psi continued across a pole as a scalar.
@@ -73,8 +95,7 @@ struct LcStream { int H, W; double s0, R, dth, dph; };
 // Loss of the stream form against the velocity targets (channels 1, 2 of target [3][H][W]) scaled
 // by inv_s1, inv_s2; the gradient at the net output into dY [H][W][CO] (gv: [2][H][W] scratch).
 void lc_stream_loss(const float *Y, int CO, const double *target, const double *sin_t, const LcStream &g,
-                    double inv_s1, double inv_s2, double wsum, double *gv, float *dY, double *part, double *loss,
-                    cudaStream_t s);
+                    double inv_s1, double inv_s2, double wsum, double *gv, float *dY, double *part, cudaStream_t s);
 // The stream form's correction (0, du^theta, du^phi) [3][H][W]; *mean (the drho area sum) = 0.
 void lc_stream_outputs(const float *Y, int CO, const LcStream &g, const double *sin_t, double *out, double *part,
                        double *mean, cudaStream_t s);
@@ -93,7 +114,7 @@ struct LcPoisson {
 };
 void lc_vort_loss(const float *Y, int CO, const double *target, const double *sin_t, const LcStream &g,
                   const LcPoisson &P, double inv_s1, double inv_s2, double wsum, double *gv, float *dY, double *part,
-                  double *loss, cudaStream_t s);
+                  cudaStream_t s);
 void lc_vort_outputs(const float *Y, int CO, const LcStream &g, const LcPoisson &P, const double *sin_t, double *out,
                      double *part, double *mean, cudaStream_t s);
 // The tables of an H x W grid (R = 1): their size in floats, and a blocking fill of a device array

@@ -1701,7 +1701,7 @@ template <bool LIN, bool KW>
 static cudaError_t prepare_wide()
 {
     return cudaFuncSetAttribute(stage_f32_kernel<8, LIN, 4, KW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)wide_smem());
+                                SPREAD_SMEM);
 }
 
 template <int TY, bool LIN>
@@ -1848,9 +1848,10 @@ static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, 
     const dim3 grid((run.L.np + TX - 1) / TX, rows.count);
     if constexpr (Q == 4) {
         if (ty == 8 && early && stage_f32_wide(run.L)) {
-            if (lin) launch_after(early, stage_f32_kernel<8, true, 4, false, true>, grid, 512, wide_smem(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
-            else if (run.komissarov) launch_after(early, stage_f32_kernel<8, false, 4, true, true>, grid, 512, wide_smem(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
-            else launch_after(early, stage_f32_kernel<8, false, 4, false, true>, grid, 512, wide_smem(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+            const size_t smem = spread_smem((long long)grid.x * grid.y, wide_smem());
+            if (lin) launch_after(early, stage_f32_kernel<8, true, 4, false, true>, grid, 512, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+            else if (run.komissarov) launch_after(early, stage_f32_kernel<8, false, 4, true, true>, grid, 512, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+            else launch_after(early, stage_f32_kernel<8, false, 4, false, true>, grid, 512, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
             return;
         }
     }

@@ -35,6 +35,11 @@ namespace vk {
 #if defined(__CUDACC__)
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A grid of at most one CTA per SM asks for more shared memory than half an SM has (spread_smem): of two
+// launches in a row the second's CTAs would otherwise start on the SMs that the first leaves idle, two to
+// four to an SM, and run there after the others have long become free.
+constexpr int SPREAD_SMEM = 116 * 1024;
+inline size_t spread_smem(long long ctas, size_t need) { return ctas <= 152 && need < SPREAD_SMEM ? SPREAD_SMEM : need; }
 template <class... P, class... A>
 inline void launch_after(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                          A &&...args)

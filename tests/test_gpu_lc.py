@@ -412,3 +412,41 @@ def test_vorticity_form_is_refused_where_its_mode_solve_does_not_fit(V):
     net.set_output_form("stream", 1.0)
     net.set_output_form("direct", 1.0)
     net.close()
+
+
+@pytest.mark.parametrize("H,W", [(4, 8), (5, 66), (6, 130), (13, 64), (33, 20)])
+def test_network_at_the_edges_of_its_tiles(V, H, W):
+    """Convolution tiles of 4 rows and 64 columns with remainders in both, grids of one tile, more rows than
+    a weight-gradient CTA takes: forward, loss and gradients against the FP64 reference with the stated
+    bounds of the 16 x 32 case; the rollout in graphs of one and of eight steps against step and apply."""
+    scale = _in_scale(H, W)
+    net = V.LearnedCorrection(H, W, seed=7, in_scale=scale, out_scale=OUT_SCALE)
+    p = net.get_weights().astype(np.float64)
+    p[-3:] = [0.3, -0.2, 0.1]
+    net.set_weights(p)
+    x, t = _sample(H, W, 11)
+    pw = _bf16_weights(p)
+    y_ref, _ = L.forward(pw, x, scale, quantize=_bf16)
+    y = net.predict(x) / np.asarray(OUT_SCALE)[:, None, None]
+    assert np.abs(y - y_ref).max() <= 3e-2 * np.abs(y_ref).max()
+    loss, g = net.gradients(x, t)
+    loss_ref, g_ref = L.loss_and_grad(pw, x, t, scale, OUT_SCALE, quantize=_bf16)
+    assert loss == pytest.approx(loss_ref, rel=3e-2)
+    o = 0
+    for ci, co in L.LAYERS:
+        for n in (co * ci * 9, co):
+            a, b = g[o:o + n], g_ref[o:o + n]
+            assert np.linalg.norm(a - b) <= (8e-2 if n > co else 3e-2) * np.linalg.norm(b), (o, n)
+            o += n
+    if H < 6:
+        return
+    a, b = (V.Solver(H, W, 2e-3, 1e-5, precision="fp32", guard=False) for _ in range(2))
+    for s in (a, b):
+        s.init_moments(*inputs.gaussian_vortices(H, W, run=6))
+    net.rollout(a, 10)
+    for _ in range(10):
+        b.step(1)
+        net.apply(b)
+    assert np.array_equal(a.get_populations(), b.get_populations())
+    a.close()
+    b.close()
