@@ -59,20 +59,27 @@ __device__ __forceinline__ void na_load(const double *f, size_t plane, size_t ce
 __global__ void __launch_bounds__(NOALLOC_THREADS) noalloc_sums_kernel(const double *f, int nt, int np, double radius,
                                                                         VelNA c, int rows, double *part)
 {
-    __shared__ double rs[NA_ROWS_MAX], rc[NA_ROWS_MAX];   // area sin(theta), area sin(theta) cos(theta)
+    __shared__ double rs[NA_ROWS_MAX], rc[NA_ROWS_MAX];   // sin(theta), cos(theta) of the CTA's rows
+    __shared__ double ls[32], lc[32];                      // sin, cos of a lane's offset in its chunk of columns
+    __shared__ double bs[NOALLOC_THREADS / 32], bc[NOALLOC_THREADS / 32];   // ... of the warps' first chunks
     __shared__ double red[NQ][NOALLOC_THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i0 = blockIdx.y * rows, n = min(rows, nt - i0);
     const double pi = 3.14159265358979323846;
     const double area = radius * radius * (pi / nt) * (2.0 * pi / np);
-    if ((int)threadIdx.x < n) {
-        const int i = i0 + threadIdx.x, m = nt - 1 - i;
+    // one sincos per thread, in warps of their own: the rows (threads 0 .. 63), the lane offsets and the chunks
+    if ((int)threadIdx.x < NA_ROWS_MAX) {
+        const int i = i0 + min((int)threadIdx.x, n - 1), m = nt - 1 - i;
         double st, ct;
         sincospi(((i <= m ? i : m) + 0.5) / nt, &st, &ct);
         if (i == m) ct = 0.0;
         if (i > m) ct = -ct;
         rs[threadIdx.x] = st;
         rc[threadIdx.x] = ct;
+    } else if (warp == 2) {
+        sincospi((2.0 * lane + 1.0) / np, &ls[lane], &lc[lane]);
+    } else if (lane < NOALLOC_THREADS / 32) {
+        sincospi(64.0 * (blockIdx.x * (NOALLOC_THREADS / 32) + lane) / np, &bs[lane], &bc[lane]);
     }
     __syncthreads();
     const size_t plane = (size_t)nt * np;
@@ -116,8 +123,10 @@ __global__ void __launch_bounds__(NOALLOC_THREADS) noalloc_sums_kernel(const dou
             }
         }
         if (!in) continue;
-        double sph, cph;
-        sincospi((2.0 * j + 1.0) / np, &sph, &cph);
+        // phi_j = 2 pi (32 ch) / np + (2 lane + 1) pi / np
+        double sb = bs[warp], cb = bc[warp];
+        if (ch >= (int)(gridDim.x * (NOALLOC_THREADS / 32))) sincospi(64.0 * ch / np, &sb, &cb);
+        const double sph = fma(sb, lc[lane], cb * ls[lane]), cph = fma(cb, lc[lane], -(sb * ls[lane]));
         // sum |v|^2 f = v3^2 (so + sp) + v2^2 (si + the populations of |v_phi| = v[2])
         const double mass = so + si;
         acc[0] += mass;
@@ -127,13 +136,22 @@ __global__ void __launch_bounds__(NOALLOC_THREADS) noalloc_sums_kernel(const dou
         acc[4] += fma(c.v3 * c.v3, so + sp, c.v2 * c.v2 * (si + (mass - sp)));
     }
     acc[5] = bad;
-    // warps by shuffles, then the four warps in order
+    // warps by a butterfly whose first steps also halve the sums that a lane carries (9 additions, not 30):
+    // after them lane l has sum l / 4 of its group of 8 quantities, over all lanes
+    double h4[4], h2[2];
+    const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4;
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-#pragma unroll
-        for (int m = 16; m > 0; m >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], m);
-        if (lane == 0) red[q][warp] = acc[q];
+    for (int q = 0; q < 4; ++q) {
+        const double up = q + 4 < NQ ? acc[q + 4 < NQ ? q + 4 : 0] : 0.0;
+        h4[q] = (u16 ? up : acc[q]) + __shfl_xor_sync(0xffffffffu, u16 ? acc[q] : up, 16);
     }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+        h2[q] = (u8 ? h4[q + 2] : h4[q]) + __shfl_xor_sync(0xffffffffu, u8 ? h4[q] : h4[q + 2], 8);
+    double h = (u4 ? h2[1] : h2[0]) + __shfl_xor_sync(0xffffffffu, u4 ? h2[0] : h2[1], 4);
+    h += __shfl_xor_sync(0xffffffffu, h, 2);
+    h += __shfl_xor_sync(0xffffffffu, h, 1);
+    if ((lane & 3) == 0 && lane / 4 < NQ) red[lane / 4][warp] = h;
     __syncthreads();
     if (threadIdx.x < NQ) {
         const int q = threadIdx.x;
