@@ -13,12 +13,16 @@
 // moments, losses and gradients of the weights in FP32.  Channels-last tensors
 // [rows][cols][channels]; dY is the gradient at a layer's pre-activation (BF16):
 //   forward:         Y  = "valid" 3x3 convolution of the explicitly padded pad(X) with W;
-//   backward data:   dX = 3x3 convolution of dY with W flipped and transposed, its halo
-//                    the adjoint of pad() (conv_bwd_kernel), masked by the ReLU below;
+//   backward data:   dX at the padded positions = 3x3 convolution of dY (zero outside the grid)
+//                    with W flipped and transposed; the adjoint of pad() folds the ghost
+//                    positions' values onto their sources; the ReLU below masks it;
 //   backward weight: dW[co][tap][ci] = sum_p dY[p][co] pad(X)[p + tap][ci].
 // At the sizes of a coarse grid every launch is bound by latency, not by the tensor
 // rate: the kernels are launched early (launch_after), fetch what no kernel before
-// them writes (weights) ahead of their wait, and a backward pass is nine launches.
+// them writes (weights) ahead of their wait, and a backward pass is twelve launches.
+// Every sum runs in a fixed order that does not depend on the launch shapes (products along the taps,
+// the ghosts of a pixel one after the other, rows in order): training is a chain of thousands of steps
+// through BF16 roundings, so another order of a sum gives another network in the end.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -245,23 +249,22 @@ __global__ void __launch_bounds__(CONV_THREADS) conv3x3_kernel(const __nv_bfloat
     }
 }
 
-// Backward data of layer l >= 1: the gradient dYin [H][W][32] (BF16) at the pre-activation of layer l - 1 from
-// dY [H][W][CI] at that of layer l, with Wt [32][9][CI] (taps flipped, channels swapped) and the ReLU mask
-// of act [H][W][32].  Columns wrap.  Beyond a pole, pad() has the row on the opposite meridian, so the
-// pole row's gradient gets, in the place of the missing row's taps, the opposite meridian's gradients
-// through the taps that reach across: row 0 through the taps of the row below it (r = 2), row H - 1
-// through those of r = 0.  (Unfused, with a zero-padded copy of dY, the gradient at the padded
-// positions in FP32 and a kernel to fold it back: 29 + 59 + 112 + 24 us for the three layers of
-// 128 x 256; 37 us of each fold was one row's serial search for its ghosts.)
+// Backward data of layer l >= 1, over the padded positions [H+2][W+2] of the layer's input: the 3x3 convolution
+// of dY [H][W][CI] (zero outside the grid) with Wt [32][9][CI] (taps flipped, channels swapped).  Positions
+// that no ghost folds onto are finished here: the ReLU mask of act [H][W][32], then dYin (BF16), the
+// gradient at the pre-activation of layer l - 1.  The others, the grid's edge and the ghosts around it, go
+// to dXp [H+2][W+2][32] in FP32 for fold_edge_kernel.  (With a zero-padded copy of dY, all of dXp in FP32,
+// a fold over all pixels that searched a pole row's ghosts serially, and a masking pass: 29 + 59 + 112 +
+// 24 us for the three layers of 128 x 256.)
 template <int CI>
 __global__ void __launch_bounds__(CONV_THREADS) conv_bwd_kernel(const __nv_bfloat16 *dY, int H, int W,
                                                                  const __nv_bfloat16 *Wt, const __nv_bfloat16 *act,
-                                                                 __nv_bfloat16 *dYin)
+                                                                 __nv_bfloat16 *dYin, float *dXp)
 {
     constexpr int CO = LC_HID;
     extern __shared__ __align__(16) unsigned char conv_smem_raw[];
     ConvSmem<CI, CO> &S = *reinterpret_cast<ConvSmem<CI, CO> *>(conv_smem_raw);
-    const int y0 = blockIdx.y * CONV_ROWS, x0 = blockIdx.x * CONV_PIX;
+    const int y0 = blockIdx.y * CONV_ROWS - 1, x0 = blockIdx.x * CONV_PIX - 1;   // first output position
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     stage_weights<CI, CO>(S, Wt);   // (written by an earlier step)
     pdl_wait();
@@ -270,12 +273,10 @@ __global__ void __launch_bounds__(CONV_THREADS) conv_bwd_kernel(const __nv_bfloa
 #pragma unroll
     for (int e = tid; e < (CONV_ROWS + 2) * (CONV_PIX + 2) * CV; e += CONV_THREADS) {
         const int cv = e % CV, rest = e / CV, xx = rest % (CONV_PIX + 2), r = rest / (CONV_PIX + 2);
-        // rows -1 and H: the pole rows, half way round (rows beyond them belong to no output)
-        const int row = min(max(y0 - 1 + r, 0), H - 1);
-        int gx = x0 + xx - 1 + (row != y0 - 1 + r ? W / 2 : 0);
-        gx %= W;
-        if (gx < 0) gx += W;
-        copy16(&S.x[r][xx][8 * cv], dY + ((size_t)row * W + gx) * CI + 8 * cv);
+        const int gy = y0 - 1 + r, gx = x0 - 1 + xx;
+        copy16(&S.x[r][xx][8 * cv],
+               dY + ((size_t)min(max(gy, 0), H - 1) * W + min(max(gx, 0), W - 1)) * CI + 8 * cv,
+               gy >= 0 && gy < H && gx >= 0 && gx < W);
     }
     copy_commit();
     copy_wait<0>();
@@ -287,24 +288,28 @@ __global__ void __launch_bounds__(CONV_THREADS) conv_bwd_kernel(const __nv_bfloa
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[nb][q] = 0.0f;
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        const int tr = (r == 0 && y == 0) ? 2 : (r == 2 && y == H - 1) ? 0 : r;
-#pragma unroll
-        for (int dx = 0; dx < 3; ++dx) conv_tap<CI, CO>(acc, S, p0, wr + r, dx, 3 * tr + dx);
-    }
+    for (int tap = 0; tap < 9; ++tap) conv_tap<CI, CO>(acc, S, p0, wr + tap / 3, tap % 3, tap);
     __syncthreads();   // every warp is done with the inputs
     ConvOut &O = reinterpret_cast<ConvOut *>(conv_smem_raw)[warp];
 #pragma unroll
-    for (int half = 0; half < 2; ++half)
+    for (int half = 0; half < 2; ++half) {
+        const int x = x0 + p0 + g + 8 * half;
+        const bool edge = y <= 0 || y >= H - 1 || x <= 0 || x >= W - 1;
 #pragma unroll
-        for (int nb = 0; nb < CO / 8; ++nb)
-            *reinterpret_cast<__nv_bfloat162 *>(&O.v[g + 8 * half][nb * 8 + 2 * t]) =
+        for (int nb = 0; nb < CO / 8; ++nb) {
+            const int co = nb * 8 + 2 * t;
+            *reinterpret_cast<__nv_bfloat162 *>(&O.v[g + 8 * half][co]) =
                 __floats2bfloat162_rn(acc[nb][2 * half], acc[nb][2 * half + 1]);
+            if (edge && y <= H && x <= W)
+                *reinterpret_cast<float2 *>(dXp + ((size_t)(y + 1) * (W + 2) + x + 1) * CO + co) =
+                    make_float2(acc[nb][2 * half], acc[nb][2 * half + 1]);
+        }
+    }
     __syncwarp();
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int px = lane / 4 + 8 * k, c8 = (lane % 4) * 8, x = x0 + p0 + px;
-        if (x >= W || y >= H) continue;
+        if (y <= 0 || y >= H - 1 || x <= 0 || x >= W - 1) continue;
         const size_t o = ((size_t)y * W + x) * CO + c8;
         uint4 v = *reinterpret_cast<const uint4 *>(&O.v[px][c8]);
         const uint4 z = *reinterpret_cast<const uint4 *>(act + o);
@@ -317,18 +322,55 @@ __global__ void __launch_bounds__(CONV_THREADS) conv_bwd_kernel(const __nv_bfloa
     }
 }
 
+// The edge pixels of conv_bwd_kernel: a pixel's own value, then its ghosts one after the other (the columns
+// that wrap, then the pole row's copies on the opposite meridian in the order of their columns), masked and
+// rounded.  Thread: pixel blockIdx.x blockDim.y + threadIdx.y of the edge (rows 0 and H - 1, then columns 0
+// and W - 1 of the rows between), channel threadIdx.x.
+__global__ void __launch_bounds__(LC_HID * 8) fold_edge_kernel(const float *dXp, int H, int W, const __nv_bfloat16 *act,
+                                                                __nv_bfloat16 *dYin)
+{
+    pdl_wait();
+    pdl_trigger();
+    const int c = threadIdx.x, Wp = W + 2;
+    int e = blockIdx.x * blockDim.y + threadIdx.y, y, x;
+    if (e >= 2 * W + 2 * (H - 2)) return;
+    if (e < 2 * W) {
+        y = e < W ? 0 : H - 1;
+        x = e < W ? e : e - W;
+    } else {
+        e -= 2 * W;
+        y = 1 + e / 2;
+        x = e % 2 ? W - 1 : 0;
+    }
+    auto at = [&](int yp, int xp) { return dXp[((size_t)yp * Wp + xp) * LC_HID + c]; };
+    float s = at(y + 1, x + 1);
+    if (x == W - 1) s += at(y + 1, 0);
+    if (x == 0) s += at(y + 1, W + 1);
+    // padded column xp of a ghost row reads column (xp - 1 + W/2) mod W of its pole row
+    const int xp = (x - W / 2 + W) % W + 1;
+    for (int pole = 0; pole < 2; ++pole) {
+        if (y != (pole ? H - 1 : 0)) continue;
+        const int yp = pole ? H + 1 : 0;
+        if (xp == W) s += at(yp, 0);
+        s += at(yp, xp);
+        if (xp == 1) s += at(yp, W + 1);
+    }
+    const size_t o = ((size_t)y * W + x) * LC_HID + c;
+    dYin[o] = __float2bfloat16(__bfloat162float(act[o]) <= 0.0f ? 0.0f : s);
+}
+
 // ---- weight gradients on the tensor cores --------------------------------------------
 // All layers in one launch: layer blockIdx.y from dY [H][W][CO] bf16 (gradient at the pre-activation) and
-// Xp [H+2][W+2][CI] bf16; CTA blockIdx.x takes `rows` output rows and writes its sums part[cta][9][CO][CI]
-// and partb[cta][CO] (bias) in FP32.  One warp per tap: pixels are the k index of the product, so both
+// Xp [H+2][W+2][CI] bf16; CTA blockIdx.x takes one output row and writes its sums part[row][9][CO][CI] and
+// partb[row][CO] (bias) in FP32.  One warp per tap: pixels are the k index of the product, so both
 // operands are read from their pixel-major staging by transposing ldmatrix (two-byte gathers were 45 us
-// a layer at 128 x 256).  rows: about two CTAs per SM over the four layers, so that few partial sums
-// are written and read again.
+// a layer at 128 x 256).  (Two rows per CTA would halve the partial sums, 3 us less in all, in another
+// order of the sums.)
 constexpr int WG_PIX = 64;
 constexpr int WG_THREADS = 9 * 32;
 
 template <int CI, int CO>
-__device__ __forceinline__ void wgrad_layer(const LcWgradLayer &l, int H, int W, int rows, unsigned char *smem)
+__device__ __forceinline__ void wgrad_layer(const LcWgradLayer &l, int W, unsigned char *smem)
 {
     constexpr int DS = CO + 8, XS = CI + 8;
     // two buffers, the copies of the next 64 pixels in flight during one's products: per buffer dY
@@ -344,12 +386,10 @@ __device__ __forceinline__ void wgrad_layer(const LcWgradLayer &l, int H, int W,
         for (int n = 0; n < CI / 8; ++n)
 #pragma unroll
             for (int q = 0; q < 4; ++q) acc[m][n][q] = 0.0f;
-    // bias: thread = channel tid % CO, pixels tid / CO, + BS, ...
-    constexpr int BS = 256 / CO;
-    float bsum = 0.0f;
-    const int y0 = blockIdx.x * rows, nx = (W + WG_PIX - 1) / WG_PIX, nt = (min(y0 + rows, H) - y0) * nx;
+    float bsum = 0.0f;   // bias: thread = channel
+    const int y = blockIdx.x, nt = (W + WG_PIX - 1) / WG_PIX;
     auto fetch = [&](int c) {
-        const int y = y0 + c / nx, x0 = (c % nx) * WG_PIX;
+        const int x0 = c * WG_PIX;
         __nv_bfloat16 *dys = buf + (c & 1) * BUF, *xs = dys + WG_PIX * DS;
 #pragma unroll
         for (int e = tid; e < WG_PIX * (CO / 8); e += WG_THREADS) {
@@ -375,8 +415,10 @@ __device__ __forceinline__ void wgrad_layer(const LcWgradLayer &l, int H, int W,
                 copy_wait<0>();
             }
             __syncthreads();
-            if (tid < 256)
-                for (int px = tid / CO; px < WG_PIX; px += BS) bsum += __bfloat162float(dys[px * DS + tid % CO]);
+            if (tid < CO) {
+#pragma unroll 16
+                for (int px = 0; px < WG_PIX; ++px) bsum += __bfloat162float(dys[px * DS + tid]);
+            }
 #pragma unroll
             for (int ks = 0; ks < WG_PIX / 16; ++ks) {
                 // A[co][pixel] = dY[pixel][co]: rows of the staging are pixels (k), hence the transposition;
@@ -410,93 +452,78 @@ __device__ __forceinline__ void wgrad_layer(const LcWgradLayer &l, int H, int W,
             for (int h = 0; h < 2; ++h)
                 *reinterpret_cast<float2 *>(part + (size_t)(m * 16 + g + 8 * h) * CI + n * 8 + 2 * t) =
                     make_float2(acc[m][n][2 * h], acc[m][n][2 * h + 1]);
-    __syncthreads();
-    float *red = reinterpret_cast<float *>(smem);
-    if (tid < 256) red[tid] = bsum;
-    __syncthreads();
-    if (tid < CO) {
-        float b = 0.0f;
-        for (int k = 0; k < BS; ++k) b += red[k * CO + tid];
-        l.partb[(size_t)blockIdx.x * CO + tid] = b;
-    }
+    if (tid < CO) l.partb[(size_t)y * CO + tid] = bsum;
 }
 
-__global__ void __launch_bounds__(WG_THREADS) wgrad_kernel(const LcBackward p, int rows)
+__global__ void __launch_bounds__(WG_THREADS) wgrad_kernel(const LcBackward p)
 {
     __shared__ __align__(16) unsigned char smem[2 * (WG_PIX * (LC_HID + 8) + 3 * (WG_PIX + 2) * (LC_HID + 8)) * 2];
     pdl_wait();
     pdl_trigger();
     const LcWgradLayer &l = p.w[blockIdx.y];
-    if (blockIdx.y == 0) wgrad_layer<LC_CIN, LC_HID>(l, p.H, p.W, rows, smem);
-    else if (blockIdx.y < LC_LAYERS - 1) wgrad_layer<LC_HID, LC_HID>(l, p.H, p.W, rows, smem);
-    else wgrad_layer<LC_HID, LC_COUTP2>(l, p.H, p.W, rows, smem);
+    if (blockIdx.y == 0) wgrad_layer<LC_CIN, LC_HID>(l, p.W, smem);
+    else if (blockIdx.y < LC_LAYERS - 1) wgrad_layer<LC_HID, LC_HID>(l, p.W, smem);
+    else wgrad_layer<LC_HID, LC_COUTP2>(l, p.W, smem);
 }
 
-// The gradient of every parameter from the CTAs' partial sums (added in order) into g, in the master layout
+// The gradient of every parameter from the rows' partial sums (added in order) into g, in the master layout
 // (per layer W[co][ci][3][3], b[co]); with adam set, one Adam step (bias-corrected) on the FP32 master
 // weights and their BF16 copies: forward [COp][9][CIp] and backward data [CIp][9][COp2] (taps flipped,
 // channels swapped; the copies' padding channels stay zero).  Thread: one element of a layer's partial
-// sums [9][COp2][CIp] or one bias, and a quarter of the CTAs' partial sums; the quarters are added through
-// shared memory.  The last CTA adds the loss's partial sums.  (Per layer two reductions, a layout pass, a
-// copy, then Adam and a pass per layer over the copies: 26 launches, 110 us at 128 x 256.)
-constexpr int UPD_ELEMS = 64;
-__global__ void __launch_bounds__(4 * UPD_ELEMS) update_kernel(const LcBackward p, const LcAdam a, const double *lpart,
-                                                                int nl, double *loss)
+// sums [9][COp2][CIp], or one bias.  The last CTA adds the loss's partial sums.  (Per layer two
+// reductions, a layout pass, a copy, then Adam and a pass per layer over the copies: 26 launches,
+// 110 us at 128 x 256.)
+constexpr int UPD_THREADS = 128;
+__global__ void __launch_bounds__(UPD_THREADS) update_kernel(const LcBackward p, const LcAdam a, const double *lpart,
+                                                              int nl, double *loss)
 {
-    __shared__ double red[256];
     pdl_wait();
     pdl_trigger();
     if (blockIdx.x == gridDim.x - 1) {
+        __shared__ double red[UPD_THREADS];
         double s = 0.0;
-        for (int i = threadIdx.x; i < nl; i += 256) s += lpart[i];
+        for (int i = threadIdx.x; i < nl; i += UPD_THREADS) s += lpart[i];
         red[threadIdx.x] = s;
         __syncthreads();
-        for (int k = 128; k > 0; k >>= 1) {
+        for (int k = UPD_THREADS / 2; k > 0; k >>= 1) {
             if ((int)threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
             __syncthreads();
         }
         if (threadIdx.x == 0) *loss = red[0];
         return;
     }
-    int e = blockIdx.x * UPD_ELEMS + threadIdx.x % UPD_ELEMS, l = 0;
-    const int quarter = threadIdx.x / UPD_ELEMS, per = (p.ctas + 3) / 4;
-    for (; l < LC_LAYERS; ++l) {
-        const int total = 9 * p.w[l].cop2 * p.w[l].cip + p.w[l].cop2;
-        if (e < total) break;
-        e -= total;
-    }
-    const bool in = l < LC_LAYERS;
-    const LcWgradLayer &w = p.w[in ? l : 0];
-    const int n = 9 * w.cop2 * w.cip;
-    const bool bias = e >= n;
-    float s = 0.0f;
-    if (in) {
+    int e = blockIdx.x * UPD_THREADS + threadIdx.x;
+#pragma unroll 1
+    for (int l = 0; l < LC_LAYERS; ++l) {
+        const LcWgradLayer &w = p.w[l];
+        const int n = 9 * w.cop2 * w.cip, total = n + w.cop2;
+        if (e >= total) {
+            e -= total;
+            continue;
+        }
+        const bool bias = e >= n;
         const int stride = bias ? w.cop2 : n;
         const float *src = bias ? w.partb + (e - n) : w.part + e;
-        const int r1 = min((quarter + 1) * per, p.ctas);
-#pragma unroll 16
-        for (int r = quarter * per; r < r1; ++r) s += src[(size_t)r * stride];
+        float s = 0.0f;
+#pragma unroll 32
+        for (int r = 0; r < p.H; ++r) s += src[(size_t)r * stride];
+        const int ci = e % w.cip, co = bias ? e - n : (e / w.cip) % w.cop2, tap = e / (w.cip * w.cop2);
+        if (co >= w.co || (!bias && ci >= w.ci)) return;
+        const size_t i = bias ? w.boff + co : w.woff + ((size_t)co * w.ci + ci) * 9 + tap;
+        a.g[i] = s;
+        if (!a.step) return;
+        const float mi = a.b1 * a.m[i] + (1.0f - a.b1) * s;
+        const float vi = a.b2 * a.v[i] + (1.0f - a.b2) * s * s;
+        a.m[i] = mi;
+        a.v[i] = vi;
+        const float x = a.w[i] - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+        a.w[i] = x;
+        if (bias) return;
+        const __nv_bfloat16 h = __float2bfloat16(x);
+        w.wf[((size_t)co * 9 + tap) * w.cip + ci] = h;
+        if (w.wb) w.wb[((size_t)ci * 9 + 8 - tap) * w.cop2 + co] = h;
+        return;
     }
-    float *sum = reinterpret_cast<float *>(red);
-    sum[threadIdx.x] = s;
-    __syncthreads();
-    if (!in || quarter) return;
-    for (int k = 1; k < 4; ++k) s += sum[k * UPD_ELEMS + threadIdx.x];
-    const int ci = e % w.cip, co = bias ? e - n : (e / w.cip) % w.cop2, tap = e / (w.cip * w.cop2);
-    if (co >= w.co || (!bias && ci >= w.ci)) return;
-    const size_t i = bias ? w.boff + co : w.woff + ((size_t)co * w.ci + ci) * 9 + tap;
-    a.g[i] = s;
-    if (!a.step) return;
-    const float mi = a.b1 * a.m[i] + (1.0f - a.b1) * s;
-    const float vi = a.b2 * a.v[i] + (1.0f - a.b2) * s * s;
-    a.m[i] = mi;
-    a.v[i] = vi;
-    const float x = a.w[i] - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
-    a.w[i] = x;
-    if (bias) return;
-    const __nv_bfloat16 h = __float2bfloat16(x);
-    w.wf[((size_t)co * 9 + tap) * w.cip + ci] = h;
-    if (w.wb) w.wb[((size_t)ci * 9 + 8 - tap) * w.cop2 + co] = h;
 }
 
 // ---- elementwise pieces -------------------------------------------------------------
@@ -1186,21 +1213,23 @@ cudaError_t lc_prepare_conv()
 
 void lc_backward(const LcBackward &p, const LcAdam &adam, const double *loss_part, int nl, double *loss, cudaStream_t s)
 {
-    const dim3 grid = conv_grid(p.H, p.W);
+    const dim3 grid = conv_grid(p.H + 2, p.W + 2);
+    const int edge = 2 * p.W + 2 * (p.H - 2);
     for (int l = LC_LAYERS - 1; l > 0; --l) {
         const LcWgradLayer &w = p.w[l], &in = p.w[l - 1];
-        if (l == LC_LAYERS - 1) launch_after(true, conv_bwd_kernel<LC_COUTP2>, grid, CONV_THREADS, conv_smem<LC_COUTP2, LC_HID>(grid), s, w.dY, p.H, p.W, w.wb, w.act, in.dY);
-        else launch_after(true, conv_bwd_kernel<LC_HID>, grid, CONV_THREADS, conv_smem<LC_HID, LC_HID>(grid), s, w.dY, p.H, p.W, w.wb, w.act, in.dY);
+        if (l == LC_LAYERS - 1)
+            launch_after(true, conv_bwd_kernel<LC_COUTP2>, grid, CONV_THREADS, conv_smem<LC_COUTP2, LC_HID>(grid), s, w.dY,
+                         p.H, p.W, w.wb, w.act, in.dY, p.dXp);
+        else
+            launch_after(true, conv_bwd_kernel<LC_HID>, grid, CONV_THREADS, conv_smem<LC_HID, LC_HID>(grid), s, w.dY, p.H,
+                         p.W, w.wb, w.act, in.dY, p.dXp);
+        launch_after(true, fold_edge_kernel, (edge + 7) / 8, dim3(LC_HID, 8), 0, s, p.dXp, p.H, p.W, w.act, in.dY);
     }
-    launch_after(true, wgrad_kernel, dim3(p.ctas, LC_LAYERS), WG_THREADS, 0, s, p, lc_wgrad_rows(p.H));
+    launch_after(true, wgrad_kernel, dim3(p.H, LC_LAYERS), WG_THREADS, 0, s, p);
     int n = 0;
     for (int l = 0; l < LC_LAYERS; ++l) n += 9 * p.w[l].cop2 * p.w[l].cip + p.w[l].cop2;
-    launch_after(true, update_kernel, (n + UPD_ELEMS - 1) / UPD_ELEMS + 1, 4 * UPD_ELEMS, 0, s, p, adam, loss_part, nl, loss);
+    launch_after(true, update_kernel, (n + UPD_THREADS - 1) / UPD_THREADS + 1, UPD_THREADS, 0, s, p, adam, loss_part, nl, loss);
 }
-
-// output rows per CTA of the weight gradients, and the CTAs per layer
-int lc_wgrad_rows(int H) { return (LC_LAYERS * H + 303) / 304; }
-int lc_wgrad_ctas(int H) { return (H + lc_wgrad_rows(H) - 1) / lc_wgrad_rows(H); }
 
 int lc_loss_parts(int H, int W) { return (H * W + 255) / 256; }
 

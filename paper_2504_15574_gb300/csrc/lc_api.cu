@@ -28,11 +28,11 @@ struct vlbm_lc {
     __nv_bfloat16 *d_wf[LC_LAYERS] = {}, *d_wb[LC_LAYERS] = {};
     double *d_sin = nullptr, *d_cos = nullptr, *d_in = nullptr, *d_tg = nullptr, *d_out = nullptr, *d_part = nullptr, *d_scal = nullptr;
     __nv_bfloat16 *d_xp[LC_LAYERS] = {}, *d_z[LC_LAYERS] = {};
-    float *d_y = nullptr, *d_dy = nullptr;
+    float *d_y = nullptr, *d_dy = nullptr, *d_dxp = nullptr;
     float *d_dev = nullptr;      // the network's moment deviations (rho - 1, u^theta, u^phi, T - 1) [4][H][W]
     double *d_cpart = nullptr;   // direct-form correction: the last layer's per-CTA sums of sin(theta) output 0
     __nv_bfloat16 *d_dpre[LC_LAYERS] = {};   // gradients at the pre-activations [H][W][cop2]
-    float *d_wpart[LC_LAYERS] = {}, *d_bpart[LC_LAYERS] = {};   // their weight gradients' partial sums per CTA
+    float *d_wpart[LC_LAYERS] = {}, *d_bpart[LC_LAYERS] = {};   // their weight and bias gradients' sums per row
     double wsum = 0.0;
     float in_scale[LC_NSCALE] = {1e-3f, 1e-2f, 1e-2f, 1e-3f, 1e-6f, 1e-6f, 1e-5f, 1e-5f, 1e-5f,
                                  1e-5f, 1e-5f, 1e-5f, 1e-5f, 1e-5f};
@@ -175,7 +175,7 @@ int backward(vlbm_lc_t *n, float lr = 0.0f)
     LcBackward p;
     p.H = H;
     p.W = W;
-    p.ctas = lc_wgrad_ctas(H);
+    p.dXp = n->d_dxp;
     for (int l = 0; l < LC_LAYERS; ++l)
         p.w[l] = LcWgradLayer{n->d_dpre[l], n->d_xp[l], l ? n->d_z[l - 1] : nullptr, n->d_wf[l],
                               l ? n->d_wb[l] : nullptr, n->d_wpart[l], n->d_bpart[l], n->ci[l], n->co[l], n->cip[l],
@@ -308,8 +308,8 @@ int vlbm_lc_create(int n_theta, int n_phi, unsigned long long seed, vlbm_lc_t **
         A(&n->d_xp[l], HWp * n->cip[l]);
         A(&n->d_z[l], HW * LC_HID);
         A(&n->d_dpre[l], HW * n->cop2[l]);
-        A(&n->d_wpart[l], (size_t)lc_wgrad_ctas(n_theta) * 9 * n->cop2[l] * n->cip[l]);
-        A(&n->d_bpart[l], (size_t)lc_wgrad_ctas(n_theta) * n->cop2[l]);
+        A(&n->d_wpart[l], (size_t)n_theta * 9 * n->cop2[l] * n->cip[l]);
+        A(&n->d_bpart[l], (size_t)n_theta * n->cop2[l]);
     }
     A(&n->d_sin, (size_t)n_theta);
     A(&n->d_cos, (size_t)n_theta);
@@ -322,6 +322,7 @@ int vlbm_lc_create(int n_theta, int n_phi, unsigned long long seed, vlbm_lc_t **
     A(&n->d_scal, 4);
     A(&n->d_y, HW * LC_COUT);
     A(&n->d_dy, HW * LC_COUT);
+    A(&n->d_dxp, HWp * LC_HID);
     A(&n->d_gv, 2 * HW);
     const size_t M = (size_t)n_phi / 2 + 1;
     A(&n->d_ptabs, lc_poisson_table_floats(n_theta, n_phi));

@@ -37,7 +37,7 @@ int lc_conv_ctas(int H, int W);
 // One layer of the backward pass: its gradient dY at the pre-activation [H][W][cop2] (BF16), its padded
 // input Xp [H+2][W+2][cip], the activations act [H][W][32] that its input was (the ReLU mask of the layer
 // below; NULL for layer 0), BF16 weights (forward wf, backward data wb; NULL for layer 0), partial sums of
-// its weight and bias gradients per CTA, channel counts and master offsets.
+// its weight and bias gradients per row, channel counts and master offsets.
 struct LcWgradLayer {
     __nv_bfloat16 *dY;
     const __nv_bfloat16 *Xp, *act;
@@ -47,7 +47,8 @@ struct LcWgradLayer {
     size_t woff, boff;
 };
 struct LcBackward {
-    int H, W, ctas;   // ctas: lc_wgrad_ctas(H)
+    int H, W;
+    float *dXp;   // scratch [H+2][W+2][32]: the edge of a layer's input gradient
     LcWgradLayer w[LC_LAYERS];
 };
 // Gradient output g and, with step set, the Adam step of the master weights w (m, v: moments; c1, c2: bias
@@ -57,8 +58,6 @@ struct LcAdam {
     float *g, *w, *m, *v;
     float lr, b1, b2, eps, c1, c2;
 };
-int lc_wgrad_rows(int H);
-int lc_wgrad_ctas(int H);
 // The backward pass from the last layer's dY, the update, and the loss from its nl partial sums.
 void lc_backward(const LcBackward &p, const LcAdam &adam, const double *loss_part, int nl, double *loss,
                  cudaStream_t s);
