@@ -171,6 +171,16 @@ int dalloc(vlbm_t *h, void **p, size_t bytes)
     return VLBM_OK;
 }
 
+// Doubles of the diagnostics' read-back: six sums, the FP64 budget, one spare, and (FP32) the pole sums
+size_t diag_doubles(const vlbm_t *h)
+{
+    return 8 + (h->prec == VLBM_FP32 ? 2 * (size_t)((h->np + F32_TILE_COLS - 1) / F32_TILE_COLS) : 0);
+}
+
+// Largest moment fields (doubles of all four) that the moment kernels write to host memory themselves: up to
+// 256 KB a call is latency (three copies: 42 us for 40 x 100), above it the copy engine is faster
+constexpr size_t SMALL_MOMENTS = 32768;
+
 // FP32 tables that depend on rho_ref: packed velocity constants, per-face sine forms,
 // per-row constants and the per-row tendency of the reference state (times sin(theta)).
 int build_f32_tables(vlbm_t *h)
@@ -564,8 +574,7 @@ int after_reset(vlbm_t *h)
 {
     if (h->prec == VLBM_FP64) launch_fill_ghosts_f64((double *)h->F, h->L, h->stream);
     else launch_fill_ghosts_f32((float2 *)h->F, h->L, h->vd.q, h->stream);
-    CK(h, cudaMemsetAsync(h->d_budget, 0, sizeof(double), h->stream));
-    if (h->d_pole_part) CK(h, cudaMemsetAsync(h->d_pole_part, 0, sizeof(double) * 2 * h->run.tiles_x, h->stream));
+    CK(h, cudaMemsetAsync(h->d_budget, 0, sizeof(double) * (diag_doubles(h) - 6), h->stream));
     CK(h, cudaMemsetAsync(h->d_flags, 0, sizeof(unsigned) * 4, h->stream));
     CK(h, cudaGetLastError());
     h->steps = 0;
@@ -770,12 +779,13 @@ int vlbm_create(int n_theta, int n_phi, int velocity_set, double tau, double dt,
         }
     }
     if ((rc = dalloc(h, (void **)&h->d_pole, sizeof(double) * 3 * 2 * NK * (size_t)n_phi)) ||
-        (rc = dalloc(h, (void **)&h->d_budget, sizeof(double) * 8)) ||
         (rc = dalloc(h, (void **)&h->d_mom, sizeof(double) * 4 * (size_t)n_theta * n_phi)) ||
         (rc = dalloc(h, (void **)&h->d_part, sizeof(double) * diag_partials(h->L))) ||
-        (rc = dalloc(h, (void **)&h->d_diag, sizeof(double) * 8)) ||
-        (rc = dalloc(h, (void **)&h->d_flags, sizeof(unsigned) * 4)))
+        (rc = dalloc(h, (void **)&h->d_diag, sizeof(double) * diag_doubles(h))))
         return bail(rc);
+    // (the budget and the FP32 pole sums lie behind the sums: one copy reads all back)
+    h->d_budget = h->d_diag + 6;
+    if (h->prec == VLBM_FP32) h->d_pole_part = h->d_diag + 8;
     if (h->prec == VLBM_FP32) {
         // FP32 diagnostics: cos and sin of the column angles; the stage kernels' pole partials
         std::vector<double> cph(n_phi), sph(n_phi);
@@ -784,17 +794,22 @@ int vlbm_create(int n_theta, int n_phi, int velocity_set, double tau, double dt,
             cph[j] = std::cos((j + 0.5) * dph);
             sph[j] = std::sin((j + 0.5) * dph);
         }
-        const int ntx = (n_phi + F32_TILE_COLS - 1) / F32_TILE_COLS;
         if ((rc = upload(h, &h->d_cph, cph.data(), cph.size())) || (rc = upload(h, &h->d_sph, sph.data(), sph.size())) ||
-            (rc = dalloc(h, (void **)&h->d_pole_part, sizeof(double) * 2 * (size_t)ntx)) ||
             (rc = dalloc(h, (void **)&h->d_ctr, sizeof(unsigned) * 6)) ||
             (rc = dalloc(h, (void **)&h->d_scalar, sizeof(double) * 8)))
             return bail(rc);
     }
-    if (cudaMallocHost((void **)&h->h_flags, sizeof(unsigned) * 4) != cudaSuccess) {
-        h->err = "cudaMallocHost failed";
+    // pinned host memory that the device addresses too: the error flags (which kernels touch only on an
+    // error, so that a sync needs no copy), the diagnostics' read-back and small moments
+    if (cudaHostAlloc((void **)&h->h_flags, sizeof(unsigned) * 4, cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostAlloc((void **)&h->h_diag, sizeof(double) * diag_doubles(h), cudaHostAllocMapped) != cudaSuccess ||
+        (4 * (size_t)n_theta * n_phi <= SMALL_MOMENTS &&
+         cudaHostAlloc((void **)&h->h_mom, sizeof(double) * 4 * (size_t)n_theta * n_phi, cudaHostAllocMapped) != cudaSuccess)) {
+        h->err = "cudaHostAlloc failed";
         return bail(VLBM_ERR_CUDA);
     }
+    memset(h->h_flags, 0, sizeof(unsigned) * 4);
+    h->d_flags = h->h_flags;   // (unified addressing: the same pointer on the device)
     for (int q = 0; q < 4; ++q)
         if (cudaEventCreate(&h->ev[q]) != cudaSuccess) {
             h->err = "cudaEventCreate failed";
@@ -910,7 +925,6 @@ int vlbm_step_async(vlbm_t *h, int n)
 int vlbm_sync(vlbm_t *h)
 {
     if (!h) return fail(h, VLBM_ERR_ARG, "NULL handle");
-    CK(h, cudaMemcpyAsync(h->h_flags, h->d_flags, sizeof(unsigned) * 4, cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     CK(h, cudaGetLastError());
     if (h->h_flags[0] & 1u) return fail(h, VLBM_ERR_TIMEOUT, "a tile load did not complete within its time limit");
@@ -934,13 +948,21 @@ int vlbm_moments(vlbm_t *h, double *rho, double *u_theta, double *u_phi, double 
 {
     if (!h || !rho || !u_theta || !u_phi) return fail(h, VLBM_ERR_ARG, "NULL argument");
     const size_t n = (size_t)h->nt * h->np;
-    double *d = h->d_mom;
+    double *d = h->h_mom ? h->h_mom : h->d_mom;   // (small fields: straight to the host, without three copies)
     if (h->prec == VLBM_FP64)
         launch_moments_f64((const double *)h->F, h->L, d, d + n, d + 2 * n, T ? d + 3 * n : nullptr, h->vd, h->stream);
     else
         launch_moments_f32((const float2 *)h->F, h->L, d, d + n, d + 2 * n, T ? d + 3 * n : nullptr, h->vd,
                            h->rho_ref, h->d_ikss, h->stream);
     CK(h, cudaGetLastError());
+    if (h->h_mom) {
+        CK(h, cudaStreamSynchronize(h->stream));
+        memcpy(rho, d, n * sizeof(double));
+        memcpy(u_theta, d + n, n * sizeof(double));
+        memcpy(u_phi, d + 2 * n, n * sizeof(double));
+        if (T) memcpy(T, d + 3 * n, n * sizeof(double));
+        return VLBM_OK;
+    }
     CK(h, cudaMemcpyAsync(rho, d, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaMemcpyAsync(u_theta, d + n, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaMemcpyAsync(u_phi, d + 2 * n, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
@@ -960,24 +982,19 @@ int vlbm_diagnostics(vlbm_t *h, vlbm_diag *out)
         launch_diagnostics_f32((const float2 *)h->F, h->L, h->d_sin_t, h->d_cos_t, h->d_cph, h->d_sph, h->vd, area,
                                h->rho_ref, h->kscale, h->d_part, h->d_diag, h->stream);
     CK(h, cudaGetLastError());
-    double v[8];
-    CK(h, cudaMemcpyAsync(v, h->d_diag, 6 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaMemcpyAsync(v + 6, h->d_budget, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    std::vector<double> pole;
-    if (h->prec == VLBM_FP32 && h->run.pole_part) {
-        pole.resize(2 * (size_t)h->run.tiles_x);
-        CK(h, cudaMemcpyAsync(pole.data(), h->d_pole_part, sizeof(double) * pole.size(), cudaMemcpyDeviceToHost,
-                              h->stream));
-    }
+    const double *v = h->h_diag;
+    CK(h, cudaMemcpyAsync(h->h_diag, h->d_diag, sizeof(double) * diag_doubles(h), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
-    if (!pole.empty()) {
+    double pole_flux = v[6];
+    if (h->prec == VLBM_FP32 && h->run.pole_part) {
         // -dt R dphi times the stage-weighted flux out of the south minus the north pole: the deviations'
         // sums, and the reference state's constant flux of every step taken
+        const double *pole = v + 8;
         double sum[2] = {0.0, 0.0};
         for (int k = 0; k < 2; ++k)
             for (int b = 0; b < h->run.tiles_x; ++b) sum[k] += pole[(size_t)k * h->run.tiles_x + b];
         const double dev = (sum[1] - sum[0]) / h->kscale, ref = (h->pole_ref[1] - h->pole_ref[0]) * (double)h->steps;
-        v[6] = -h->dt * h->R * (2.0 * M_PI / h->np) * (dev + ref);
+        pole_flux = -h->dt * h->R * (2.0 * M_PI / h->np) * (dev + ref);
     }
     out->time = (double)h->steps * h->dt;
     out->steps = h->steps;
@@ -987,7 +1004,7 @@ int vlbm_diagnostics(vlbm_t *h, vlbm_diag *out)
     out->momentum[2] = v[3];
     out->energy = v[4];
     out->nonfinite = v[5] > 0.0 ? 1 : 0;
-    out->pole_flux = v[6];
+    out->pole_flux = pole_flux;
     out->mass0 = h->mass0;
     return VLBM_OK;
 }
@@ -1058,12 +1075,12 @@ void vlbm_destroy(vlbm_t *h)
     void *bufs[] = {h->F, h->A, h->B, h->d_sin_ext, h->d_rowd, h->d_sin_t, h->d_cos_t, h->d_sin_f, h->d_isp,
                     h->d_sfc, h->d_ft, h->d_fp,
                     h->d_rref, h->d_dsin, h->d_d2sin, h->d_tabs, h->d_kss, h->d_ikss, h->d_cph, h->d_sph,
-                    h->d_pole_part, h->d_scalar, h->d_ctr,
-                    h->d_row, h->d_frows, h->d_fblocks, h->d_pole, h->d_budget, h->d_mom, h->d_dense,
-                    h->d_part, h->d_diag, h->d_flags};
+                    h->d_scalar, h->d_ctr,
+                    h->d_row, h->d_frows, h->d_fblocks, h->d_pole, h->d_mom, h->d_dense, h->d_part, h->d_diag};
     for (void *p : bufs)
         if (p) cudaFree(p);
-    if (h->h_flags) cudaFreeHost(h->h_flags);
+    for (void *p : {(void *)h->h_flags, (void *)h->h_diag, (void *)h->h_mom})
+        if (p) cudaFreeHost(p);
     for (int q = 0; q < 4; ++q)
         if (h->ev[q]) cudaEventDestroy(h->ev[q]);
     for (cudaEvent_t e : h->evs)
@@ -1351,13 +1368,13 @@ int vlbm_batch_create(int nruns, const int *n_theta, const int *n_phi, const dou
     bool wide = false;
     for (const vlbm_t *h : b->runs) wide = wide || h->nfrows > 0;
     for (vlbm_t *h : b->runs) h->ring_in_stage = wide;
-    if (cudaMalloc(&b->d_flags, 4 * sizeof(unsigned)) != cudaSuccess ||
-        cudaMemset(b->d_flags, 0, 4 * sizeof(unsigned)) != cudaSuccess ||
-        cudaMallocHost(&b->h_flags, 4 * sizeof(unsigned)) != cudaSuccess ||
+    if (cudaHostAlloc(&b->h_flags, 4 * sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess ||
         cudaEventCreate(&b->ev[0]) != cudaSuccess || cudaEventCreate(&b->ev[1]) != cudaSuccess) {
         vlbm_batch_destroy(b);
         return bfail(nullptr, VLBM_ERR_CUDA, "batch allocation failed");
     }
+    memset(b->h_flags, 0, 4 * sizeof(unsigned));
+    b->d_flags = b->h_flags;   // (as a solver's)
     *out = b;
     return VLBM_OK;
 }
@@ -1416,7 +1433,6 @@ int vlbm_batch_step_async(vlbm_batch_t *b, int n)
 int vlbm_batch_sync(vlbm_batch_t *b)
 {
     if (!b) return bfail(b, VLBM_ERR_ARG, "NULL batch");
-    BCK(b, cudaMemcpyAsync(b->h_flags, b->d_flags, 4 * sizeof(unsigned), cudaMemcpyDeviceToHost, b->stream));
     BCK(b, cudaStreamSynchronize(b->stream));
     BCK(b, cudaGetLastError());
     if (b->h_flags[0] & 1u) return bfail(b, VLBM_ERR_TIMEOUT, "a tile load did not complete within its time limit");
@@ -1531,7 +1547,6 @@ void vlbm_batch_destroy(vlbm_batch_t *b)
     if (b->d_tms) cudaFree(b->d_tms);
     if (b->d_work) cudaFree(b->d_work);
     if (b->d_fitems) cudaFree(b->d_fitems);
-    if (b->d_flags) cudaFree(b->d_flags);
     if (b->h_flags) cudaFreeHost(b->h_flags);
     for (int q = 0; q < 2; ++q)
         if (b->ev[q]) cudaEventDestroy(b->ev[q]);

@@ -48,7 +48,8 @@ struct vlbm {
     // diagnostics, budget, I/O scratch
     double *d_pole = nullptr, *d_budget = nullptr, *d_mom = nullptr, *d_dense = nullptr;
     double *d_part = nullptr, *d_diag = nullptr;
-    unsigned *d_flags = nullptr, *h_flags = nullptr;
+    unsigned *d_flags = nullptr, *h_flags = nullptr;   // error flags: pinned host memory, one address on both sides
+    double *h_diag = nullptr, *h_mom = nullptr;        // pinned: the diagnostics' read-back; moments of small grids
     CUtensorMap tmF{}, tmA{}, tmB{};      // FP32 path: box maps (stage inputs)
     CUtensorMap tmFc{}, tmAc{}, tmBc{};   // FP32 path: tile-core maps (stage outputs, F prefetch)
     cudaGraphExec_t g1 = nullptr, g16 = nullptr;
