@@ -120,6 +120,33 @@ F64I double mul_int_zz(double a, double b)
 // a^2, a may be zero
 F64I double sq_int(double a) { return mul_int_z(a, a); }
 
+// a + b, neither negative, either may be zero.  The smaller significand is shifted right to the larger's
+// exponent, with ten spare bits below (what falls out of them only sets the last one), added, and
+// rounded as in mul_int; shifts of 64 bits and more leave the larger value as it is.
+F64I double add_pos(double a, double b)
+{
+    uint32_t ah, al, bh, bl;
+    f64_split(a, ah, al);
+    f64_split(b, bh, bl);
+    const bool less = ah < bh;   // (equal high words have the same exponent: either order will do)
+    const uint32_t xh = less ? bh : ah, xl = less ? bl : al, yh = less ? ah : bh, yl = less ? al : bl;
+    const uint32_t d = (xh >> 20) - (yh >> 20);
+    // significands above ten spare bits: [2^62, 2^63), zero for a zero
+    const uint64_t x = (((uint64_t)((xh & 0xfffffu) | 0x100000u) << 32) | xl) << 10;
+    const uint64_t y0 = (((uint64_t)((yh & 0xfffffu) | 0x100000u) << 32) | yl) << 10;
+    const uint64_t y = (d > 63u || (yh | yl) == 0) ? 0 : y0 >> d;
+    const uint64_t lost = (d > 63u || d == 0u || (yh | yl) == 0) ? 0 : y0 << (64u - d);
+    const uint64_t sum = x + y;
+    const uint32_t n = (uint32_t)(sum >> 63), sh = 10u + n;
+    const uint64_t m = sum >> sh;
+    const uint32_t rest = ((uint32_t)sum << (32u - sh)) | (lost != 0 ? 1u : 0u);
+    const uint32_t inc = rest + ((uint32_t)m & 1u) > 0x80000000u ? 1u : 0u;
+    const uint64_t r = m + inc;
+    const uint32_t h = (uint32_t)(r >> 32) + (xh & 0x7ff00000u) - 0x100000u + (n << 20);
+    const bool zero = (xh | xl) == 0;
+    return f64_of(zero ? 0u : h, zero ? 0u : (uint32_t)r);
+}
+
 // x N for a small odd N (3, 5, 7 or 11); x may be zero
 template <int N>
 F64I double mul_small(double x)

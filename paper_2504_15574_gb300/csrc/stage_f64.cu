@@ -98,7 +98,7 @@ __device__ __noinline__ double weno5_plain(double a, double b, double c, double 
 // expression order, and gives its flux to store(f, flux), v times the interface value (store_r: the
 // value itself, for the Komissarov factor).  The forms of one column (13/12 times the squared second
 // difference, and 5 y) are shared by the three candidate stencils centred on it, which changes no
-// bit.  34 FP64 instructions a face: with every value zero or in [2^-400, 2^100), differences are
+// bit.  28 FP64 instructions a face: with every value zero or in [2^-400, 2^100), differences are
 // zero or multiples of the smallest ulp, so no product leaves the normal range.
 template <class Load, class Store>
 __device__ __forceinline__ void weno5_walk(int n, bool plain, double eps, double v, const DivC &six, Load load,
@@ -124,16 +124,16 @@ __device__ __forceinline__ void weno5_walk(int n, bool plain, double eps, double
         const double d1b = a - scale2<2>(b) + c3;
         const double d2b = b - d;
         const double d3b = c3 - scale2<2>(d) + e;
-        const double s1 = k1 + scale2<-2>(sq_int(d1b)) + eps;
-        const double s2 = k2 + scale2<-2>(sq_int(d2b)) + eps;
-        const double s3 = k3 + scale2<-2>(sq_int(d3b)) + eps;
+        const double s1 = add_pos(add_pos(k1, scale2<-2>(sq_int(d1b))), eps);
+        const double s2 = add_pos(add_pos(k2, scale2<-2>(sq_int(d2b))), eps);
+        const double s3 = add_pos(add_pos(k3, scale2<-2>(sq_int(d3b))), eps);
         const double w1 = div_pos(0.1, mul_int(s1, s1)), w2 = div_pos(0.6, mul_int(s2, s2)),
                      w3 = div_pos(0.3, mul_int(s3, s3));
         const double p1 = div_const_int(scale2<1>(a) - mul_small<7>(b) + mul_small<11>(c), six);
         const double p2 = div_const_int(c5 - b + scale2<1>(d), six);
         const double p3 = div_const_int(scale2<1>(c) + d5 - e, six);
         const double num = mul_int_z(p1, w1) + mul_int_z(p2, w2) + mul_int_z(p3, w3);
-        const double r = div_pos(num, w1 + w2 + w3);
+        const double r = div_pos(num, add_pos(add_pos(w1, w2), w3));
         double flux = mul_int_zz(r, v);   // (v = 0: a D2Q9 population at rest along the axis)
         if (plain || out > 0 || !f64_within<500, 500>(num)) flux = weno5_plain(a, b, c, d, e, eps, v);
         store(f, flux);

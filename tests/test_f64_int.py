@@ -35,6 +35,10 @@ int main()
         bad += mul_int_zz(a, b) != p || (p != 0.0 && f64_bits(mul_int_zz(a, b)) != f64_bits(p));
         if (b != 0.0) bad += mul_int_z(a, b) != p;
         bad += sq_int(a) != a * a;
+        {   // sums of values that are not negative: near, far and equal exponents
+            const double u = std::fabs(a), v = t % 3 ? std::fabs(b) : std::ldexp(std::fabs(b) == 0.0 ? 0.0 : 1.0 + std::fabs(std::fmod(b, 1.0)), std::ilogb(u == 0.0 ? 1.0 : u) - (int)(g() % 70));
+            bad += add_pos(u, v) != u + v || add_pos(v, u) != u + v;
+        }
         bad += mul_small<3>(a) != 3.0 * a || mul_small<5>(a) != 5.0 * a || mul_small<7>(a) != 7.0 * a ||
                mul_small<11>(a) != 11.0 * a;
         bad += scale2<1>(a) != 2.0 * a || scale2<2>(a) != 4.0 * a || scale2<-1>(a) != 0.5 * a ||
