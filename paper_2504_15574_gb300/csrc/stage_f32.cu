@@ -168,6 +168,14 @@ __device__ __forceinline__ FF ff_add(FF a, FF b)
     return FF{hi, lo};
 }
 
+// a + b of two plain values (ff_add of zero low parts, whose renormalisation changes nothing)
+__device__ __forceinline__ FF ff_leaf(f2 a, f2 b)
+{
+    FF r;
+    two_sum(a, b, r.hi, r.lo);
+    return r;
+}
+
 __device__ __forceinline__ FF ff_shfl_xor(FF a, int m, unsigned mask = 0xffffffffu)
 {
     FF r;
@@ -224,8 +232,10 @@ __device__ __forceinline__ void ring_means(const FF (&a)[N], f2 (&out)[N], int b
             if constexpr (M > 1) {
                 keep.lo = pick(up, a[k].lo, a[k + N / 2].lo);
                 got.lo = shfl(pick(up, a[k + N / 2].lo, a[k].lo), M);
+                h[k] = up ? ff_add(got, keep) : ff_add(keep, got);
+            } else {
+                h[k] = up ? ff_leaf(got.hi, keep.hi) : ff_leaf(keep.hi, got.hi);
             }
-            h[k] = up ? ff_add(got, keep) : ff_add(keep, got);
         }
         ring_means<N / 2, 2 * M>(h, r, b, mask);
 #pragma unroll
@@ -235,6 +245,23 @@ __device__ __forceinline__ void ring_means(const FF (&a)[N], f2 (&out)[N], int b
             out[k + N / 2] = pick(up, other, r[k]);
         }
     }
+}
+
+// The polar ring filter of one cell's pairs on their way out, x[k stride], k < NO, in shared memory (every
+// lane its own cell's; 2 to 8 of them are summed as NR = 4 or 8).  Behind a call: inlined into the cell
+// phase its registers cost spills there (U3 + Komissarov at 1024 x 2048: 246 against 233 us a step),
+// and few rows come here.
+template <int NO>
+__device__ __noinline__ void ring_cell(f2 *x, int stride, int b, unsigned mask)
+{
+    constexpr int NR = NO <= 4 ? 4 : 8;
+    FF v[NR];
+    f2 m[NR];
+#pragma unroll
+    for (int q = 0; q < NR; ++q) v[q] = FF{q < NO ? x[q * stride] : make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+    ring_means<NR, 1>(v, m, b, mask);
+#pragma unroll
+    for (int q = 0; q < NO; ++q) x[q * stride] = m[q];
 }
 
 __device__ __forceinline__ float rcp_approx(float x)
@@ -730,7 +757,11 @@ __device__ __forceinline__ void load_cell_g(const Sm &S, int b, f2 *G)
 // of F when this begins.  Threads of cells outside the grid return early.
 // WIDE: two threads per cell, the warps of its row in the two halves of the CTA, each of which updates
 // the pairs of one k_theta half (both form the moments).
-template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false, class Sm>
+// RING: rows of narrow ring blocks are filtered here.  false: the run has none, and the compiler's schedule of
+// the rest is better without that path in the batch kernel (64 runs: 1.98 ms a step against 2.01) and in the
+// D2Q9 kernel (1024 x 2048: 200.6 us against 202.5); the persistent kernel (U3, Komissarov, 512 x 1024) takes
+// 70.3 us a step without it and 72.3 with it.
+template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false, bool RING = true, class Sm>
 __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q>::type &c, int stage, float dte,
                                            const CUtensorMap *tmo, int bx, int by, Sm &S, int b, int tb,
                                            const f2 *Gin)
@@ -923,22 +954,14 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
     // the output tile is staged in shared memory and leaves with one TMA store; the issuing
     // thread waits until the store has read it
     const bool core = (i0 >= GR && i0 + TY <= L.nt - GR && q0 >= GC && q0 + TX <= L.np - GC);
-    if (rc.ring > 1) {   // polar ring filter of this row (a row is a warp: uniform)
-        const int nv = L.np - q0;
-        const unsigned mask = nv >= 32 ? 0xffffffffu : (1u << nv) - 1u;
-        constexpr int NR = WIDE ? 4 : 8;
-        FF v[NR];
-        f2 m[NR];
+    const bool ring = RING && rc.ring > 1;   // polar ring filter of this row (a row is a warp: uniform)
+    f2 *ob = &S.ob[0][0][0], *own = ob + (oq * TY + cy) * TX + cx;
+    if (core || ring) {
 #pragma unroll
-        for (int q = 0; q < NR; ++q) v[q] = FF{q < NO ? o[q < NO ? q : 0] : splat(0.0f), splat(0.0f)};
-        ring_means<NR, 1>(v, m, rc.ring, mask);
-#pragma unroll
-        for (int q = 0; q < NO; ++q) o[q] = m[q];
+        for (int q = 0; q < NO; ++q) own[q * TY * TX] = o[q];
     }
+    if (ring) ring_cell<NO>(own, TY * TX, rc.ring, L.np - q0 >= 32 ? 0xffffffffu : (1u << (L.np - q0)) - 1u);
     if (core) {
-        f2 *ob = &S.ob[0][0][0];
-#pragma unroll
-        for (int q = 0; q < NO; ++q) ob[((oq + q) * TY + cy) * TX + cx] = o[q];
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
         if (tid == 0) {
@@ -952,7 +975,10 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
         return;
     }
     const bool plain = (i >= GR && i < L.nt - GR && j >= GC && j < L.np - GC);
-    if (plain) {
+    if (ring) {
+#pragma unroll 1
+        for (int q = 0; q < NO; ++q) store_images(out, L, Q, oq + q, i, j, own[q * TY * TX]);
+    } else if (plain) {
 #pragma unroll
         for (int q = 0; q < NO; ++q) out[L.at(oq + q, i, j)] = o[q];
     } else {
@@ -971,7 +997,7 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
 // LIN: the upwind schemes U1-U3 (Eq. fluxes_U1-3, optionally with the Komissarov theta flux)
 // instead of WENO-5.
 // Q: the velocity set (4: D2Q16, 3: D2Q9 in five pairs).
-template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false>
+template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false, bool RING = true>
 __device__ __forceinline__ bool stage_tile(const RunF &R, const typename VelOf<Q>::type &c, int stage,
                                            const CUtensorMap *tm, const CUtensorMap *tmo, const CUtensorMap *tmf,
                                            int bx, int by, SmemT<TY, (Q == 3 ? 5 : NP2), 1, 1, WIDE> &S, unsigned parity,
@@ -1024,7 +1050,7 @@ __device__ __forceinline__ bool stage_tile(const RunF &R, const typename VelOf<Q
     __syncthreads();
     f2 G[NPQ];
     load_cell_g<TY, NPQ>(S, 0, G);
-    tile_cells<TY, LIN, Q, KW, WIDE>(R, c, stage, dte, tmo, bx, by, S, 0, 0, G);
+    tile_cells<TY, LIN, Q, KW, WIDE, RING>(R, c, stage, dte, tmo, bx, by, S, 0, 0, G);
     return true;
 }
 
@@ -1036,7 +1062,7 @@ __device__ __forceinline__ bool stage_tile(const RunF &R, const typename VelOf<Q
 // 64 registers fit where three of 80 do, and beside another launch too (the polar part of the split
 // schedule: 256 x 512 with the filter 48.4 against 44.0).  The same operations on every value, so the
 // same bits.
-template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false>
+template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false, bool RING = true>
 __global__ void __launch_bounds__(TY * (WIDE ? 64 : 32), WIDE ? 2 : (Q == 3 ? 32 : 24) / TY) stage_f32_kernel(const __grid_constant__ CUtensorMap tm,
                                                                       const __grid_constant__ CUtensorMap tmo,
                                                                       const __grid_constant__ CUtensorMap tmf,
@@ -1052,7 +1078,7 @@ __global__ void __launch_bounds__(TY * (WIDE ? 64 : 32), WIDE ? 2 : (Q == 3 ? 32
     }
     __syncthreads();   // no thread may poll the barrier before its initialisation is visible
     const int by = rows.first + (int)blockIdx.y + ((int)blockIdx.y >= rows.split ? rows.skip : 0);
-    stage_tile<TY, LIN, Q, KW, WIDE>(R, c, stage, &tm, &tmo, &tmf, blockIdx.x, by, S, 0u, err);
+    stage_tile<TY, LIN, Q, KW, WIDE, RING>(R, c, stage, &tm, &tmo, &tmf, blockIdx.x, by, S, 0u, err);
 }
 
 // Persistent stage kernel (8 tile rows, three CTAs per SM): CTA b takes the launch's tiles
@@ -1064,7 +1090,7 @@ __global__ void __launch_bounds__(TY * (WIDE ? 64 : 32), WIDE ? 2 : (Q == 3 ? 32
 // soon as this tile's output has left the staging buffer.  tabs holds this stage's tables of every
 // tile row of the grid.  A copy that does not arrive within the run's wait limit sets *err; the
 // CTA then waits (bounded, 1 s) for its other copies in flight and leaves.
-template <bool LIN, int Q>
+template <bool LIN, int Q, bool RING = true>
 __global__ void __launch_bounds__(256, 3)
     stage_f32_persist_kernel(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUtensorMap tmo,
                              const __grid_constant__ CUtensorMap tmf, const RunF R,
@@ -1163,7 +1189,7 @@ __global__ void __launch_bounds__(256, 3)
             }
             if (stage != 1) ok = __syncthreads_and(wait_phase(&S.barF, par, R.wait_ns));
             if (ok) {
-                tile_cells<TY, LIN, Q>(R, c, stage, dte, &tmo, bx, by, S, 0, tb, Gc);
+                tile_cells<TY, LIN, Q, false, false, RING>(R, c, stage, dte, &tmo, bx, by, S, 0, tb, Gc);
                 __syncthreads();   // this tile's tables and the staging buffer are free; next_tile is set
                 t = next_tile;
                 if (tid == 0 && stage != 1 && t < total) issue_f(t);
@@ -1195,7 +1221,7 @@ __global__ void __launch_bounds__(256, 3)
 // is (run, tile index within the run).  The run's parameters are copied into
 // shared memory per item.  tms holds 6 maps per run: the box maps of F, A, B, then
 // the tile-core maps of F, A, B.
-template <int TY, bool LIN, int Q>
+template <int TY, bool LIN, int Q, bool RING>
 __global__ void __launch_bounds__(TY * 32, 24 / TY) batch_stage_f32_kernel(const RunF *runs, const CUtensorMap *tms,
                                                                             const int2 *work, int ntiles,
                                                                             const typename VelOf<Q>::type c,
@@ -1219,7 +1245,7 @@ __global__ void __launch_bounds__(TY * 32, 24 / TY) batch_stage_f32_kernel(const
         __syncthreads();
         const int tx = S.run.tiles_x;
         const CUtensorMap *tr = tms + 6 * w.x;
-        if (!stage_tile<TY, LIN, Q>(S.run, c, stage, tr + (stage - 1), tr + 3 + stage % 3, tr + 3, w.y % tx,
+        if (!stage_tile<TY, LIN, Q, false, false, RING>(S.run, c, stage, tr + (stage - 1), tr + 3 + stage % 3, tr + 3, w.y % tx,
                                     w.y / tx, S, parity, err))
             return;
         parity ^= 1u;
@@ -1410,7 +1436,7 @@ __device__ __forceinline__ void store_ghosts(f2 *f, const Layout &L, int vq, int
 template <int B>
 __device__ __forceinline__ FF ff_tree(const f2 (&v)[FILT_COLS], int j0)
 {
-    if constexpr (B == 1) return FF{v[j0], splat(0.0f)};
+    if constexpr (B == 2) return ff_leaf(v[j0], v[j0 + 1]);
     else return ff_add(ff_tree<B / 2>(v, j0), ff_tree<B / 2>(v, j0 + B / 2));
 }
 
@@ -1691,8 +1717,11 @@ static int persist_grid()
 template <bool LIN, int Q>
 static cudaError_t prepare_persist()
 {
-    const cudaError_t e = cudaFuncSetAttribute(stage_f32_persist_kernel<LIN, Q>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)persist_smem<Q>());
+    cudaError_t e = cudaFuncSetAttribute(stage_f32_persist_kernel<LIN, Q>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)persist_smem<Q>());
+    if (!e && LIN)
+        e = cudaFuncSetAttribute(stage_f32_persist_kernel<true, Q, false>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)persist_smem<Q>());
     if (e) return e;
     return persist_grid<LIN, Q>() > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
@@ -1721,11 +1750,16 @@ cudaError_t prepare_one()
                                  (int)smem_bytes<TY, 3>());
         if (e) return e;
     }
-    e = cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_bytes<TY, 3>());
-    if (e) return e;
-    return cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_bytes<TY>());
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if (TY == 8 && !LIN) {
+        e = cudaFuncSetAttribute(stage_f32_kernel<8, false, 3, false, false, false>, at, (int)smem_bytes<8, 3>());
+        if (e) return e;
+    }
+    if ((e = cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 3, true>, at, (int)smem_bytes<TY, 3>())) ||
+        (e = cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 3, false>, at, (int)smem_bytes<TY, 3>())) ||
+        (e = cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 4, true>, at, (int)smem_bytes<TY>())))
+        return e;
+    return cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 4, false>, at, (int)smem_bytes<TY>());
 }
 
 cudaError_t prepare_stage_f32()
@@ -1789,11 +1823,11 @@ int stage_f32_max_ctas_per_sm(int ty, int q)
 {
     int n = 0;
     if (q == 3) {
-        if (ty == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<4, false, 3>, 128, smem_bytes<4, 3>());
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<8, false, 3>, 256, smem_bytes<8, 3>());
+        if (ty == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<4, false, 3, true>, 128, smem_bytes<4, 3>());
+        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<8, false, 3, true>, 256, smem_bytes<8, 3>());
     } else {
-        if (ty == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<4, false, 4>, 128, smem_bytes<4>());
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<8, false, 4>, 256, smem_bytes<8>());
+        if (ty == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<4, false, 4, true>, 128, smem_bytes<4>());
+        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<8, false, 4, true>, 256, smem_bytes<8>());
     }
     return n;
 }
@@ -1814,7 +1848,8 @@ static void launch_persist_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out
     const size_t smem = persist_smem<Q>();
     if (lin) {
         const int grid = std::min(total, persist_grid<true, Q>());
-        launch_after(early, stage_f32_persist_kernel<true, Q>, grid, 256, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
+        if (!run.rings) launch_after(early, stage_f32_persist_kernel<true, Q, false>, grid, 256, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
+        else launch_after(early, stage_f32_persist_kernel<true, Q>, grid, 256, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
     } else {
         const int grid = std::min(total, persist_grid<false, Q>());
         launch_after(early, stage_f32_persist_kernel<false, Q>, grid, 256, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
@@ -1865,6 +1900,8 @@ static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, 
         else launch_after(early, stage_f32_kernel<4, false, Q>, grid, 128, smem_bytes<4, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
     } else {
         if (lin) launch_after(early, stage_f32_kernel<8, true, Q>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+        else if (Q == 3 && !run.rings)   // (Q == 4 keeps the one form: 336 us at 1024 x 2048, 340 without the path)
+            launch_after(early, stage_f32_kernel<8, false, Q, false, false, Q == 4>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
         else launch_after(early, stage_f32_kernel<8, false, Q>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
     }
 }
@@ -1882,30 +1919,33 @@ void launch_stage_f32_q3(const CUtensorMap &tm_in, const CUtensorMap &tm_out, co
     launch_stage_q<3>(tm_in, tm_out, tm_f, run, c, stage, ty, lin, rows, err, s);
 }
 
-template <int Q>
+template <int Q, bool RING>
 static void launch_batch_q(const RunF *runs, const CUtensorMap *tms, const int2 *work, int ntiles,
                            const typename VelOf<Q>::type &c, int stage, int ty, bool lin, int ctas, unsigned *err,
                            cudaStream_t s)
 {
     if (ty == 4) {
-        if (lin) launch_after(true, batch_stage_f32_kernel<4, true, Q>, ctas, 128, smem_bytes<4, Q>(), s, runs, tms, work, ntiles, c, stage, err);
-        else launch_after(true, batch_stage_f32_kernel<4, false, Q>, ctas, 128, smem_bytes<4, Q>(), s, runs, tms, work, ntiles, c, stage, err);
+        if (lin) launch_after(true, batch_stage_f32_kernel<4, true, Q, RING>, ctas, 128, smem_bytes<4, Q>(), s, runs, tms, work, ntiles, c, stage, err);
+        else launch_after(true, batch_stage_f32_kernel<4, false, Q, RING>, ctas, 128, smem_bytes<4, Q>(), s, runs, tms, work, ntiles, c, stage, err);
     } else {
-        if (lin) launch_after(true, batch_stage_f32_kernel<8, true, Q>, ctas, 256, smem_bytes<8, Q>(), s, runs, tms, work, ntiles, c, stage, err);
-        else launch_after(true, batch_stage_f32_kernel<8, false, Q>, ctas, 256, smem_bytes<8, Q>(), s, runs, tms, work, ntiles, c, stage, err);
+        if (lin) launch_after(true, batch_stage_f32_kernel<8, true, Q, RING>, ctas, 256, smem_bytes<8, Q>(), s, runs, tms, work, ntiles, c, stage, err);
+        else launch_after(true, batch_stage_f32_kernel<8, false, Q, RING>, ctas, 256, smem_bytes<8, Q>(), s, runs, tms, work, ntiles, c, stage, err);
     }
 }
 
 void launch_batch_stage_f32(const RunF *runs, const CUtensorMap *tms, const int2 *work, int ntiles, const VelC &c,
-                            int stage, int ty, bool lin, int ctas, unsigned *err, cudaStream_t s)
+                            int stage, int ty, bool lin, bool rings, int ctas, unsigned *err, cudaStream_t s)
 {
-    launch_batch_q<4>(runs, tms, work, ntiles, c, stage, ty, lin, ctas, err, s);
+    if (rings) launch_batch_q<4, true>(runs, tms, work, ntiles, c, stage, ty, lin, ctas, err, s);
+    else launch_batch_q<4, false>(runs, tms, work, ntiles, c, stage, ty, lin, ctas, err, s);
 }
 
 void launch_batch_stage_f32_q3(const RunF *runs, const CUtensorMap *tms, const int2 *work, int ntiles,
-                               const VelC3 &c, int stage, int ty, bool lin, int ctas, unsigned *err, cudaStream_t s)
+                               const VelC3 &c, int stage, int ty, bool lin, bool rings, int ctas, unsigned *err,
+                               cudaStream_t s)
 {
-    launch_batch_q<3>(runs, tms, work, ntiles, c, stage, ty, lin, ctas, err, s);
+    if (rings) launch_batch_q<3, true>(runs, tms, work, ntiles, c, stage, ty, lin, ctas, err, s);
+    else launch_batch_q<3, false>(runs, tms, work, ntiles, c, stage, ty, lin, ctas, err, s);
 }
 
 double f32_state_scale(double eps)

@@ -298,6 +298,7 @@ int build_f32_tables(vlbm_t *h)
         }
     h->pole_ref[0] *= h->np;
     h->pole_ref[1] *= h->np;
+    run.rings = 0;
     std::vector<RowF> row(nt);
     std::vector<float2> rref((size_t)nt * npq);
     std::vector<float> kss(nt), ikss(nt);
@@ -317,6 +318,7 @@ int build_f32_tables(vlbm_t *h)
         const int block = h->filter ? filter_block(nt, h->np, s) : 1;
         rc.ring = (h->ring_in_stage && block <= F32_RING_MAX) ? block : 0;
         rc.pad = 0;
+        if (rc.ring > 1) run.rings = 1;
         row[i] = rc;
         double rk[NK];
         for (int k = 0; k < q * q; ++k) {
@@ -741,10 +743,12 @@ int vlbm_create(int n_theta, int n_phi, int velocity_set, double tau, double dt,
         return bail(rc);
     // polar filter rows
     if (h->filter) {
+        // FP32: the stage kernels filter the rows of narrow blocks themselves
         std::vector<int> rows, blocks;
+        h->ring_in_stage = h->prec == VLBM_FP32;
         for (int i = 0; i < n_theta; ++i) {
             const int b = filter_block(n_theta, n_phi, h->sin_t[i]);
-            if (b > (h->prec == VLBM_FP32 ? F32_RING_MAX : 1)) {
+            if (b > (h->ring_in_stage ? F32_RING_MAX : 1)) {
                 rows.push_back(i);
                 blocks.push_back(b);
             }
@@ -1212,11 +1216,12 @@ void batch_enqueue_step(vlbm_batch_t *b)
     const int ctas = batch_ctas(b);
     for (int st = 1; st <= 3; ++st) {
         const bool lin = b->runs.front()->scheme != VLBM_WENO5;
+        const bool rings = std::any_of(b->runs.begin(), b->runs.end(), [](const vlbm_t *h) { return h->run.rings != 0; });
         if (b->q == 3)
-            launch_batch_stage_f32_q3(b->d_runs, b->d_tms, b->d_work, b->ntiles, b->vc3, st, b->ty, lin, ctas,
+            launch_batch_stage_f32_q3(b->d_runs, b->d_tms, b->d_work, b->ntiles, b->vc3, st, b->ty, lin, rings, ctas,
                                       b->d_flags, b->stream);
         else
-            launch_batch_stage_f32(b->d_runs, b->d_tms, b->d_work, b->ntiles, b->vc, st, b->ty, lin, ctas,
+            launch_batch_stage_f32(b->d_runs, b->d_tms, b->d_work, b->ntiles, b->vc, st, b->ty, lin, rings, ctas,
                                    b->d_flags, b->stream);
         // one polar-filter launch over the filtered rows of every run
         launch_batch_filter_f32(b->d_runs, b->d_fitems, b->nfitems, b->q, st, b->stream);
@@ -1367,7 +1372,7 @@ int vlbm_batch_create(int nruns, const int *n_theta, const int *n_phi, const dou
     // blocks too wide for a tile; a batch without such rows keeps all of it in that launch
     bool wide = false;
     for (const vlbm_t *h : b->runs) wide = wide || h->nfrows > 0;
-    for (vlbm_t *h : b->runs) h->ring_in_stage = wide;
+    for (vlbm_t *h : b->runs) h->ring_in_stage = h->ring_in_stage && wide;
     if (cudaHostAlloc(&b->h_flags, 4 * sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess ||
         cudaEventCreate(&b->ev[0]) != cudaSuccess || cudaEventCreate(&b->ev[1]) != cudaSuccess) {
         vlbm_batch_destroy(b);

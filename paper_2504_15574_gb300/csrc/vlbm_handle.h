@@ -44,7 +44,7 @@ struct vlbm {
     // polar filter
     int *d_frows = nullptr, *d_fblocks = nullptr;
     int nfrows = 0;         // rows of the filter kernel (FP32: those the stage kernels do not filter themselves)
-    bool ring_in_stage = true;   // FP32: the stage kernels filter rows of blocks up to F32_RING_MAX
+    bool ring_in_stage = false;  // FP32: the stage kernels filter rows of blocks up to F32_RING_MAX
     // diagnostics, budget, I/O scratch
     double *d_pole = nullptr, *d_budget = nullptr, *d_mom = nullptr, *d_dense = nullptr;
     double *d_part = nullptr, *d_diag = nullptr;
@@ -79,7 +79,7 @@ struct vlbm {
 };
 
 // Library-internal entry points on a solver (vlbm_api.cu), for the other host units.
-// Enqueues one RK3 step of h on its stream (stages, polar filters, pole budget).
+// Enqueues one RK3 step of h on its stream (stages, whose kernels add the pole sums, and polar filters).
 void solver_enqueue_step(vlbm_t *h);
 // Adds n steps to h's step counter (steps enqueued outside vlbm_step).
 void solver_count_steps(vlbm_t *h, int n);

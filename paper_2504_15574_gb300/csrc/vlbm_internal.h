@@ -130,7 +130,8 @@ struct RunF {
     int tiles_x;               // tiles per row of this run for the launch's tile shape
     // upwind schemes U1-U3 (Eq. fluxes_U1-3): interface value = lin0 x_up2 + lin1 x_up + lin2 x_down
     float lin0, lin1, lin2;
-    int komissarov;            // theta flux in the Komissarov form (upwind schemes)
+    short komissarov;          // theta flux in the Komissarov form (upwind schemes)
+    short rings;               // 1: some rows are filtered by the stage kernel (RowF.ring)
     const float *isp;          // [nt + 2GR + 8] 1/sin at padded row pr (negative at ghost rows)
     const float *sfc;          // [nt + 1 + 8] sin(fi dtheta) of theta interface fi (0 at both poles)
     // pole mass-flux budget (NULL: not recorded): per pole (north, south) and tile column, [2][tiles_x],
@@ -232,10 +233,11 @@ void launch_stage_f32_q3(const CUtensorMap &tm_in, const CUtensorMap &tm_out, co
 // (run, tile) over the run table `runs` (device) and tensor maps `tms` (device, [run][6]: the box
 // maps of F, A, B, then the tile-core maps of F, A, B).
 void launch_batch_stage_f32(const RunF *runs, const CUtensorMap *tms, const int2 *work, int ntiles, const VelC &c,
-                            int stage, int ty, bool lin, int ctas, unsigned *err, cudaStream_t s);
+                            int stage, int ty, bool lin, bool rings, int ctas, unsigned *err, cudaStream_t s);
 // The same for D2Q9 members (five pair planes).
 void launch_batch_stage_f32_q3(const RunF *runs, const CUtensorMap *tms, const int2 *work, int ntiles,
-                               const VelC3 &c, int stage, int ty, bool lin, int ctas, unsigned *err, cudaStream_t s);
+                               const VelC3 &c, int stage, int ty, bool lin, bool rings, int ctas, unsigned *err,
+                               cudaStream_t s);
 // Resident CTAs per SM of the batch stage kernel for tile rows ty and velocity set order q.
 int stage_f32_max_ctas_per_sm(int ty, int q = 4);
 // The persistent stage kernel (8 tile rows, one CTA per resident slot, the next tile's copies in
