@@ -760,7 +760,7 @@ __device__ __forceinline__ void load_cell_g(const Sm &S, int b, f2 *G)
 // RING: rows of narrow ring blocks are filtered here.  false: the run has none, and the compiler's schedule of
 // the rest is better without that path in the batch kernel (64 runs: 1.98 ms a step against 2.01) and in the
 // D2Q9 kernel (1024 x 2048: 200.6 us against 202.5); the persistent kernel (U3, Komissarov, 512 x 1024) takes
-// 70.3 us a step without it and 72.3 with it.
+// 70.3 us a step without it and 72.3 with it; the 512-thread form (128 x 256) 17.7 and 18.0.
 template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false, bool RING = true, class Sm>
 __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q>::type &c, int stage, float dte,
                                            const CUtensorMap *tmo, int bx, int by, Sm &S, int b, int tb,
@@ -1729,6 +1729,11 @@ static cudaError_t prepare_persist()
 template <bool LIN, bool KW>
 static cudaError_t prepare_wide()
 {
+    if constexpr (!LIN && !KW) {
+        const cudaError_t e = cudaFuncSetAttribute(stage_f32_kernel<8, LIN, 4, KW, true, false>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, SPREAD_SMEM);
+        if (e) return e;
+    }
     return cudaFuncSetAttribute(stage_f32_kernel<8, LIN, 4, KW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 SPREAD_SMEM);
 }
@@ -1886,7 +1891,8 @@ static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, 
             const size_t smem = spread_smem((long long)grid.x * grid.y, wide_smem());
             if (lin) launch_after(early, stage_f32_kernel<8, true, 4, false, true>, grid, 512, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
             else if (run.komissarov) launch_after(early, stage_f32_kernel<8, false, 4, true, true>, grid, 512, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
-            else launch_after(early, stage_f32_kernel<8, false, 4, false, true>, grid, 512, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+            else if (run.rings) launch_after(early, stage_f32_kernel<8, false, 4, false, true>, grid, 512, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+            else launch_after(early, stage_f32_kernel<8, false, 4, false, true, false>, grid, 512, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
             return;
         }
     }
