@@ -8,6 +8,7 @@
 // qualifiers, so that the same code is checked on the host against the hardware's products.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -164,5 +165,36 @@ F64I double mul_small(double x)
     const uint32_t h = ((uint32_t)(r >> 32) + ((hi & 0x7ff00000u) - 0x100000u) + (sh << 20)) | (hi & 0x80000000u);
     return f64_of(zero ? hi : h, zero ? lo : (uint32_t)r);
 }
+
+// ---- division by a constant -----------------------------------------------------------
+// 1/d as h + l, h = 1/d rounded toward zero, l > 0 the remainder: x / d is RN(x h + RN(x l)), a product
+// and one fused operation.
+struct DivC { double h, l; };
+
+// Where 1/d is a double, l = h 2^-120: x h is then exact and what l adds is far below half its ulp, while
+// x l stays a normal number for the x of the integer form (a subnormal l is no operand of mul_int); a
+// positive l also keeps an infinite x infinite.
+inline DivC div_const_of(double d)
+{
+    double y = 1.0 / d, r = fma(-y, d, 1.0);
+    if (r < 0.0) {
+        y = nextafter(y, 0.0);
+        r = fma(-y, d, 1.0);
+    }
+    const double l = r > 0.0 ? r / d : y * 0x1p-120;
+    return DivC{y, l > 0.0 ? l : 4.9406564584124654e-324};
+}
+
+F64I double fma_rn(double a, double b, double c)
+{
+#if defined(__CUDA_ARCH__)
+    return __fma_rn(a, b, c);
+#else
+    return fma(a, b, c);
+#endif
+}
+
+// x / d with the product by l on the integer pipe; x zero or well inside the normal range.
+F64I double div_const_int(double x, const DivC &d) { return fma_rn(x, d.h, mul_int_z(x, d.l)); }
 
 }  // namespace vk

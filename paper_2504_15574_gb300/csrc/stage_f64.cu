@@ -14,7 +14,6 @@
 // kernel updates the cells.  It is not the throughput path (that is stage_f32.cu);
 // it shares the ghost-row layout so that all reads are plain loads.
 #include "vlbm_internal.h"
-#include "f64_int.cuh"
 
 namespace vk {
 
@@ -36,12 +35,6 @@ namespace {
 // rounded quotient only where x / d is within 2^-105 of a boundary.  h is rounded toward zero and l
 // positive, so infinities pass through.
 __device__ __forceinline__ double div_const(double x, const DivC &d) { return __fma_rn(x, d.h, __dmul_rn(x, d.l)); }
-
-// The same with the product by l on the integer pipe; x zero or well inside the normal range.
-__device__ __forceinline__ double div_const_int(double x, const DivC &d)
-{
-    return __fma_rn(x, d.h, mul_int_z(x, d.l));
-}
 
 // 1 / b to 2^-44 for a positive b in [2^-500, 2^500]: the leading 24 bits of b's significand through
 // the hardware's FP32 reciprocal, one error term with the remaining bits, assembled into a double by

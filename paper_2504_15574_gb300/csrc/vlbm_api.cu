@@ -126,20 +126,6 @@ double sin_padded(const std::vector<double> &s, int nt, int pr)
     return s[r];
 }
 
-// 1/d as h + l: h = 1/d rounded toward zero, l > 0 the remainder (a division x / d is then
-// RN(x h + RN(x l)), stage_f64.cu; where 1/d is a double, the smallest positive l, so that an
-// infinite x stays infinite).
-DivC div_const_of(double d)
-{
-    double y = 1.0 / d, r = std::fma(-y, d, 1.0);
-    if (r < 0.0) {
-        y = std::nextafter(y, 0.0);
-        r = std::fma(-y, d, 1.0);
-    }
-    const double l = r / d;
-    return DivC{y, l > 0.0 ? l : 4.9406564584124654e-324};
-}
-
 // Polar ring filter block size (not in the paper): smallest power of two b with
 // b sin(theta) dphi >= dtheta / 4, dividing n_phi.
 int filter_block(int nt, int np, double sin_i)

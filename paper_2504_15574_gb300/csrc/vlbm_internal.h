@@ -20,6 +20,7 @@
 #include <stdint.h>
 
 #include "../../include/vlbm.h"
+#include "f64_int.cuh"
 
 namespace vk {
 
@@ -76,9 +77,6 @@ struct Layout {
 struct VelD { double v[4], w[4], K[16], Kt[16]; int q; };
 
 // ---- FP64 stage (parity path) -------------------------------------------------
-// 1/d to 106 bits: h = 1/d rounded toward zero, l the remainder (positive), for divisions by d in two
-// operations (stage_f64.cu)
-struct DivC { double h, l; };
 // per interior row: cot(theta) / R, and the divisors R sin(theta) dtheta (with the Komissarov flux
 // R (cos theta_{i-1/2} - cos theta_{i+1/2})) and R sin(theta) dphi
 struct RowD { double cotR; DivC th, ph; };

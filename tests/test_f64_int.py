@@ -60,3 +60,45 @@ def test_integer_products_equal_the_hardware_products(tmp_path):
     subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-I",
                     os.path.join(ROOT, "paper_2504_15574_gb300", "csrc"), str(src), "-o", str(exe)], check=True)
     assert int(subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout) == 0
+
+
+CONSTANT_DIVISION = r"""
+#include "f64_int.cuh"
+#include <cmath>
+#include <cstdio>
+#include <random>
+using namespace vk;
+int main()
+{
+    std::mt19937_64 g(5);
+    std::uniform_real_distribution<double> u(1.0, 2.0);
+    long bad = 0;
+    for (int k = 0; k < 200; ++k) {
+        const double fixed[] = {1.0, 0.5, 0.25, 0x1p-6, 0x1p-10, 2.0, 0x1p-99, 0x1p99, 3.0, 6.0, 0.02, 5e-3, 1e-30, 1e30};
+        const double d = k < 14 ? fixed[k] : std::ldexp(u(g), (int)(g() % 190) - 95);
+        const DivC c = div_const_of(d);
+        for (int t = 0; t < 20000; ++t) {
+            double x = std::ldexp(u(g), (int)(g() % 500) - 400) * (g() & 1 ? 1.0 : -1.0);
+            if (t % 50 == 0) x = 0.0;
+            if (t % 50 == 1) x = std::ldexp(1.0, (int)(g() % 500) - 400);
+            bad += div_const_int(x, c) != x / d;
+        }
+    }
+    std::printf("%ld\n", bad);
+}
+"""
+
+
+def _run(tmp_path, source):
+    src = tmp_path / "harness.cpp"
+    src.write_text(source)
+    exe = tmp_path / "harness"
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-I",
+                    os.path.join(ROOT, "paper_2504_15574_gb300", "csrc"), str(src), "-o", str(exe)], check=True)
+    return subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout
+
+
+def test_constant_divisions_equal_the_hardware_quotients(tmp_path):
+    """x / d as a product and a fused operation, for divisors with an exact reciprocal (tau = 1, 1/2, 1/64, ...)
+    and without one, over zero, powers of two and both signs."""
+    assert int(_run(tmp_path, CONSTANT_DIVISION)) == 0

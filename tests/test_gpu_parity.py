@@ -573,3 +573,15 @@ def test_fp32_two_threads_per_cell_equal_four_row_tiles(V, nt, np_, scheme, komi
     else:
         assert np.array_equal(out[0][0], out[1][0])
         assert out[0][1] == out[1][1]
+
+
+@pytest.mark.parametrize("velocity_set", ["d2q16", "d2q9"])
+@pytest.mark.parametrize("tau", [1.0, 0.5, 2.0**-6])
+def test_fp64_relaxation_times_with_an_exact_reciprocal_match_oracle(V, velocity_set, tau):
+    """The BGK quotient by a power of two: the remainder of its reciprocal is zero."""
+    nt, np_ = 13, 20
+    o, g = run_pair(V, nt, np_, tau, 0.25 * clamped_dt(nt, np_, tau), inputs.gaussian_vortices(nt, np_, 3), 5,
+                    velocity_set=velocity_set)
+    fo, fg = o.get_populations(), g.get_populations()
+    assert np.abs(fg - fo).max() <= FP64_TOL * np.abs(fo).max()
+    g.close()
