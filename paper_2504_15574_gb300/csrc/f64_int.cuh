@@ -168,8 +168,8 @@ F64I double mul_small(double x)
 
 // ---- division by a constant -----------------------------------------------------------
 // 1/d as h + l, h = 1/d rounded toward zero, l > 0 the remainder: x / d is RN(x h + RN(x l)), a product
-// and one fused operation.
-struct DivC { double h, l; };
+// and one fused operation.  d itself serves the plain forms, which divide (1/d need not be a normal number there).
+struct DivC { double h, l, d; };
 
 // Where 1/d is a double, l = h 2^-120: x h is then exact and what l adds is far below half its ulp, while
 // x l stays a normal number for the x of the integer form (a subnormal l is no operand of mul_int); a
@@ -182,7 +182,7 @@ inline DivC div_const_of(double d)
         r = fma(-y, d, 1.0);
     }
     const double l = r > 0.0 ? r / d : y * 0x1p-120;
-    return DivC{y, l > 0.0 ? l : 4.9406564584124654e-324};
+    return DivC{y, l > 0.0 ? l : 4.9406564584124654e-324, d};
 }
 
 F64I double fma_rn(double a, double b, double c)

@@ -244,14 +244,16 @@ __global__ void __launch_bounds__(128) faces_f64_kernel(const StageD p, int nb_p
 }
 
 // One population's update of one cell.  FAST: products on the integer pipe, for populations that are
-// zero or in [2^-40, 2^100) and a positive density (then every product here is zero or normal).
+// zero or in [2^-40, 2^100) and a positive density (then every product here is zero or normal).  Otherwise, and
+// for options outside the fast forms' range (StageD.plain), plain products and divisions.
 template <bool FAST, int CELLS>
 __device__ __forceinline__ void cell_update(const StageD &p, const Layout &L, const RowD &rd,
                                             const double (*gs)[CELLS], int lane, int i, int j, int k, double n,
                                             double ut, double up, double u2, double u23)
 {
     auto mul = [](double a, double b) { return FAST ? mul_int_zz(a, b) : a * b; };
-    auto divc = [](double a, const DivC &d) { return FAST ? div_const_int(a, d) : div_const(a, d); };
+    auto divc = [](double a, const DivC &d) { return FAST ? div_const_int(a, d) : a / d.d; };
+    auto divf = [](double a, const DivC &d) { return FAST ? div_const(a, d) : a / d.d; };   // (a of any size)
     const int q = p.c.q, a = k / q, b = k % q;
     const double va = p.c.v[a], vb = p.c.v[b];
     const double gk = gs[k][lane];
@@ -276,14 +278,14 @@ __device__ __forceinline__ void cell_update(const StageD &p, const Layout &L, co
         ktg += mul(p.c.Kt[b * q + m], gs[q * a + m][lane]);
     }
     const double force = mul(rd.cotR, mul(p.vb2[b], kg) - mul(va, ktg));
-    const double adv_t = -div_const(fs - fn, rd.th);
-    const double adv_p = -div_const(fe - fw, rd.ph);
+    const double adv_t = -divf(fs - fn, rd.th);
+    const double adv_p = -divf(fe - fw, rd.ph);
     const double Lk = adv_t + adv_p - force - divc(gk - feq, p.tau_div);
 
     double outv;
     if (p.stage == 1) outv = gk + p.dt * Lk;
     else if (p.stage == 2) outv = 0.75 * f0 + (FAST ? scale2<-2>(gk) : 0.25 * gk) + p.dt_stage * Lk;
-    else outv = div_const(f0, p.three) + mul(2.0 / 3.0, gk) + p.dt_stage * Lk;
+    else outv = divf(f0, p.three) + mul(2.0 / 3.0, gk) + p.dt_stage * Lk;
     store_with_images(p.out, L, k, i, j, outv);
 }
 

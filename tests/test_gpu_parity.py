@@ -585,3 +585,12 @@ def test_fp64_relaxation_times_with_an_exact_reciprocal_match_oracle(V, velocity
     fo, fg = o.get_populations(), g.get_populations()
     assert np.abs(fg - fo).max() <= FP64_TOL * np.abs(fo).max()
     g.close()
+
+
+def test_fp64_relaxation_time_without_a_normal_reciprocal_matches_oracle(V):
+    """tau below 2^-1024: the plain forms divide by it."""
+    nt, np_ = 8, 10
+    o, g = run_pair(V, nt, np_, 1e-310, 1e-312, inputs.gaussian_vortices(nt, np_, 3), 2)
+    fo, fg = o.get_populations(), g.get_populations()
+    assert np.isfinite(fo).all() and np.abs(fg - fo).max() <= FP64_TOL * np.abs(fo).max()
+    g.close()
