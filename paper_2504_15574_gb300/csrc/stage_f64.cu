@@ -28,47 +28,9 @@ namespace {
 // to the integer pipe (f64_int.cuh; issue slots were 11 % used), scalings by powers of two become
 // exponent additions, and reciprocal seeds come from the FP32 pipe.
 
-// x / d with 1/d = h + l held to 106 bits (DivC, built on the host): RN(x h + RN(x l)), the two-
-// operation multiplication by an arbitrary-precision constant of Brisebarre and Muller ("Correctly
-// rounded multiplication by arbitrary precision constants", 2005).  Exact for d = 6 and d = 3 (no
-// quotient comes within 1/6 ulp of a rounding boundary); for a general d it differs from the
-// rounded quotient only where x / d is within 2^-105 of a boundary.  h is rounded toward zero and l
-// positive, so infinities pass through.
-__device__ __forceinline__ double div_const(double x, const DivC &d) { return __fma_rn(x, d.h, __dmul_rn(x, d.l)); }
-
-// 1 / b to 2^-44 for a positive b in [2^-500, 2^500]: the leading 24 bits of b's significand through
-// the hardware's FP32 reciprocal, one error term with the remaining bits, assembled into a double by
-// integer operations.
-__device__ __forceinline__ double recip_seed(double b)
-{
-    const int hi = __double2hiint(b), lo = __double2loint(b);
-    const float bh = __int_as_float(0x3f800000 | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29));
-    const float bl = (float)(lo & 0x1fffffff) * 0x1p-52f;
-    float r0;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(bh));
-    r0 = fmaxf(fminf(r0, 0.99999994f), 0.5f);   // inside one binade: the error term is added to its bits
-    float e = __fmaf_rn(-bh, r0, 1.0f);
-    e = __fmaf_rn(-bl, r0, e);
-    const float r1 = __fmul_rn(r0, __fmaf_rn(e, e, e));
-    const int u = __float_as_int(r0), i1 = __float2int_rn(__fmul_rn(r1, 0x1p53f));
-    long long bits = ((long long)((u >> 3) + ((1023 - 127) << 20)) << 32) | (unsigned)(u << 29);
-    bits += i1;
-    bits -= (long long)((hi >> 20) - 1023) << 52;
-    return __longlong_as_double(bits);
-}
-
-// a / b for such a b: the product with the seed on the integer pipe (a zero or well inside the normal
-// range), then one residual correction in two FP64 operations (Markstein 1990).  The corrected
-// value is within 2^-88 of a / b before its rounding, so it is the rounded quotient but for a chance
-// of about 2^-35 per division (none in 4e8 random ones).
-__device__ __forceinline__ double div_pos(double a, double b)
-{
-    const double r = recip_seed(b), q = mul_int_z(a, r);
-    return __fma_rn(__fma_rn(-b, q, a), r, q);
-}
-
 // Interface flux v r of a stencil with values outside the fast forms' range (beyond [2^-400, 2^100)
-// and not zero, or not finite), with the interface value r as the oracle writes it.
+// and not zero, or not finite) or with a quotient that a fast division missed, with the interface value r as
+// the oracle writes it.
 __device__ __noinline__ double weno5_plain(double a, double b, double c, double d, double e, double eps, double v)
 {
     double p1 = (2.0 * a - 7.0 * b + 11.0 * c) / 6.0;
@@ -91,7 +53,7 @@ __device__ __noinline__ double weno5_plain(double a, double b, double c, double 
 // expression order, and gives its flux to store(f, flux), v times the interface value (store_r: the
 // value itself, for the Komissarov factor).  The forms of one column (13/12 times the squared second
 // difference, and 5 y) are shared by the three candidate stencils centred on it, which changes no
-// bit.  28 FP64 instructions a face: with every value zero or in [2^-400, 2^100), differences are
+// bit.  30 FP64 instructions a face (four of them check the quotients): with every value zero or in [2^-400, 2^100), differences are
 // zero or multiples of the smallest ulp, so no product leaves the normal range.
 template <class Load, class Store>
 __device__ __forceinline__ void weno5_walk(int n, bool plain, double eps, double v, const DivC &six, Load load,
@@ -120,15 +82,16 @@ __device__ __forceinline__ void weno5_walk(int n, bool plain, double eps, double
         const double s1 = add_pos(add_pos(k1, scale2<-2>(sq_int(d1b))), eps);
         const double s2 = add_pos(add_pos(k2, scale2<-2>(sq_int(d2b))), eps);
         const double s3 = add_pos(add_pos(k3, scale2<-2>(sq_int(d3b))), eps);
-        const double w1 = div_pos(0.1, mul_int(s1, s1)), w2 = div_pos(0.6, mul_int(s2, s2)),
-                     w3 = div_pos(0.3, mul_int(s3, s3));
+        bool miss = plain || out > 0;
+        const double w1 = div_pos(0.1, mul_int(s1, s1), miss), w2 = div_pos(0.6, mul_int(s2, s2), miss),
+                     w3 = div_pos(0.3, mul_int(s3, s3), miss);
         const double p1 = div_const_int(scale2<1>(a) - mul_small<7>(b) + mul_small<11>(c), six);
         const double p2 = div_const_int(c5 - b + scale2<1>(d), six);
         const double p3 = div_const_int(scale2<1>(c) + d5 - e, six);
         const double num = mul_int_z(p1, w1) + mul_int_z(p2, w2) + mul_int_z(p3, w3);
-        const double r = div_pos(num, add_pos(add_pos(w1, w2), w3));
+        const double r = div_pos(num, add_pos(add_pos(w1, w2), w3), miss);
         double flux = mul_int_zz(r, v);   // (v = 0: a D2Q9 population at rest along the axis)
-        if (plain || out > 0 || !f64_within<500, 500>(num)) flux = weno5_plain(a, b, c, d, e, eps, v);
+        if (miss || !f64_within<500, 500>(num)) flux = weno5_plain(a, b, c, d, e, eps, v);
         store(f, flux);
         --out;
         a = b;
@@ -244,16 +207,17 @@ __global__ void __launch_bounds__(128) faces_f64_kernel(const StageD p, int nb_p
 }
 
 // One population's update of one cell.  FAST: products on the integer pipe, for populations that are
-// zero or in [2^-40, 2^100) and a positive density (then every product here is zero or normal).  Otherwise, and
-// for options outside the fast forms' range (StageD.plain), plain products and divisions.
-template <bool FAST, int CELLS>
+// zero or in [2^-40, 2^100) and a positive density (then every product here is zero or normal).  PLAIN: real
+// divisions, for a run whose constants are no numbers of ordinary size (in a kernel of its own: the code of
+// these divisions beside the other forms cost 2.5 %, 256 x 512).
+template <bool FAST, bool PLAIN, int CELLS>
 __device__ __forceinline__ void cell_update(const StageD &p, const Layout &L, const RowD &rd,
                                             const double (*gs)[CELLS], int lane, int i, int j, int k, double n,
                                             double ut, double up, double u2, double u23)
 {
     auto mul = [](double a, double b) { return FAST ? mul_int_zz(a, b) : a * b; };
-    auto divc = [](double a, const DivC &d) { return FAST ? div_const_int(a, d) : a / d.d; };
-    auto divf = [](double a, const DivC &d) { return FAST ? div_const(a, d) : a / d.d; };   // (a of any size)
+    auto div = [](double a, const DivC &d) { return PLAIN ? a / d.d : div_const(a, d); };   // (a of any size)
+    auto divc = [=](double a, const DivC &d) { return FAST ? div_const_int(a, d) : div(a, d); };
     const int q = p.c.q, a = k / q, b = k % q;
     const double va = p.c.v[a], vb = p.c.v[b];
     const double gk = gs[k][lane];
@@ -278,14 +242,14 @@ __device__ __forceinline__ void cell_update(const StageD &p, const Layout &L, co
         ktg += mul(p.c.Kt[b * q + m], gs[q * a + m][lane]);
     }
     const double force = mul(rd.cotR, mul(p.vb2[b], kg) - mul(va, ktg));
-    const double adv_t = -divf(fs - fn, rd.th);
-    const double adv_p = -divf(fe - fw, rd.ph);
+    const double adv_t = -div(fs - fn, rd.th);
+    const double adv_p = -div(fe - fw, rd.ph);
     const double Lk = adv_t + adv_p - force - divc(gk - feq, p.tau_div);
 
     double outv;
     if (p.stage == 1) outv = gk + p.dt * Lk;
     else if (p.stage == 2) outv = 0.75 * f0 + (FAST ? scale2<-2>(gk) : 0.25 * gk) + p.dt_stage * Lk;
-    else outv = divf(f0, p.three) + mul(2.0 / 3.0, gk) + p.dt_stage * Lk;
+    else outv = div(f0, p.three) + mul(2.0 / 3.0, gk) + p.dt_stage * Lk;
     store_with_images(p.out, L, k, i, j, outv);
 }
 
@@ -326,7 +290,7 @@ __device__ __forceinline__ void pole_budget_f64(const StageD &p)
 // on large grids: the FP64 pipe (37 instructions per population, from 105).  16 cells per CTA where
 // 32 would leave SMs without one.  In stage 3 one more CTA adds the step's pole budget (a launch
 // of its own was 3-10 us a step).
-template <int CELLS>
+template <int CELLS, bool PLAIN>
 __global__ void __launch_bounds__(256) cells_f64_kernel(const StageD p, int nblocks)
 {
     constexpr int SLOTS = 256 / CELLS;
@@ -342,7 +306,7 @@ __global__ void __launch_bounds__(256) cells_f64_kernel(const StageD p, int nblo
     const long long cell = (long long)blockIdx.x * CELLS + c;
     const bool in = cell < cells;
     const int i = in ? (int)(cell / L.np) : 0, j = in ? (int)(cell - (long long)i * L.np) : 0;
-    bool out = p.plain;
+    bool out = PLAIN;
     for (int k = slot; k < nk; k += SLOTS) {
         const double g = p.in[L.at(k, i, j)];
         out |= !f64_within<40, 100>(g);
@@ -361,7 +325,13 @@ __global__ void __launch_bounds__(256) cells_f64_kernel(const StageD p, int nblo
     // (a density that is not positive takes the plain forms: its velocities may be of any size)
     const double n = mom[0][c];
     const bool slow = plain || !(n > 0.0) || !f64_within<110, 110>(n);
-    if (slot == 1 || slot == 2) vel[slot - 1][c] = slow ? mom[slot][c] / n : div_pos(mom[slot][c], n);
+    if (slot == 1 || slot == 2) {
+        const double m = mom[slot][c];
+        bool miss = slow;
+        double u = div_pos(m, n, miss);
+        if (miss) u = f64_zero(m) && !slow ? m : m / n;
+        vel[slot - 1][c] = u;
+    }
     __syncthreads();
     if (slot == 0) {
         const double ut = vel[0][c], up = vel[1][c];
@@ -375,8 +345,8 @@ __global__ void __launch_bounds__(256) cells_f64_kernel(const StageD p, int nblo
     const RowD rd = p.row[i];
 #pragma unroll 1
     for (int k = slot; k < nk; k += SLOTS) {
-        if (slow) cell_update<false, CELLS>(p, L, rd, gs, c, i, j, k, n, ut, up, u2, u23);
-        else cell_update<true, CELLS>(p, L, rd, gs, c, i, j, k, n, ut, up, u2, u23);
+        if (PLAIN || slow) cell_update<false, PLAIN, CELLS>(p, L, rd, gs, c, i, j, k, n, ut, up, u2, u23);
+        else cell_update<true, false, CELLS>(p, L, rd, gs, c, i, j, k, n, ut, up, u2, u23);
     }
 }
 
@@ -488,13 +458,13 @@ void launch_stage_f64(const StageD &p, cudaStream_t s)
     faces_f64_kernel<<<dim3(nb + nt, L.nk), 128, 0, s>>>(p, nb, S);
     const long long cells = (long long)p.L.nt * p.L.np;
     const int extra = (p.stage == 3 && p.budget) ? 1 : 0;
-    if (cells <= 32LL * 152 * 2) {   // 32 cells per CTA: fewer than two CTAs per SM
-        const unsigned nb = (unsigned)((cells + 15) / 16);
-        cells_f64_kernel<16><<<nb + extra, 256, 0, s>>>(p, (int)nb);
-    } else {
-        const unsigned nb = (unsigned)((cells + 31) / 32);
-        cells_f64_kernel<32><<<nb + extra, 256, 0, s>>>(p, (int)nb);
-    }
+    auto launch = [&](auto *kernel, int per) {
+        const unsigned nb = (unsigned)((cells + per - 1) / per);
+        kernel<<<nb + extra, 256, 0, s>>>(p, (int)nb);
+    };
+    if (p.plain) launch(cells_f64_kernel<32, true>, 32);
+    else if (cells <= 32LL * 152 * 2) launch(cells_f64_kernel<16, false>, 16);   // 32: fewer than two CTAs per SM
+    else launch(cells_f64_kernel<32, false>, 32);
 }
 
 void launch_init_f64(double *f, const Layout &L, const double *rho, const double *ut, const double *up,

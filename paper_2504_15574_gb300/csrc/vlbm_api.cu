@@ -499,11 +499,11 @@ void enqueue_step(vlbm_t *h, int stage_only = 0, int part = 0)
             p.dt = h->dt;
             p.dt_stage = (st == 1) ? h->dt : (st == 2) ? 0.25 * h->dt : 2.0 / 3.0 * h->dt;
             p.eps = h->eps;
-            p.tau_div = div_const_of(h->tau);
+            p.tau_div = h->tau_div;
             // the fast forms bound every factor by the populations' range: options far outside take plain ones
             p.plain = !(h->eps > 1e-60 && h->eps < 1e30 && h->tau > 1e-30 && h->tau < 1e30 && h->R > 1e-30 && h->R < 1e30);
-            p.six = div_const_of(6.0);
-            p.three = div_const_of(3.0);
+            p.six = h->six;
+            p.three = h->three;
             p.stage = st;
             p.c = h->vd;
             for (int k = 0; k < h->vd.q * h->vd.q; ++k) p.wk[k] = h->vd.w[k / h->vd.q] * h->vd.w[k % h->vd.q];
@@ -713,6 +713,9 @@ int vlbm_create(int n_theta, int n_phi, int velocity_set, double tau, double dt,
     if ((rc = upload(h, &h->d_sin_f, h->sin_f.data(), h->sin_f.size()))) return bail(rc);
     if (h->prec == VLBM_FP64) {
         // FP64 stage: the row constants in the oracle's evaluation order
+        h->tau_div = div_const_of(tau);
+        h->six = div_const_of(6.0);
+        h->three = div_const_of(3.0);
         std::vector<RowD> rowd(n_theta);
         const double dth = M_PI / n_theta, dph = 2.0 * M_PI / n_phi;
         for (int i = 0; i < n_theta; ++i) {
