@@ -12,6 +12,7 @@
 
 #include "../../include/vlbm.h"
 #include "lc_internal.h"
+#include "lc_rollout.h"
 #include "vlbm_handle.h"
 
 using namespace vk;
@@ -51,18 +52,18 @@ struct vlbm_lc {
     // launches of consecutive steps overlap; between graphs they do not)
     cudaGraphExec_t g_exec = nullptr, g_many = nullptr;
     vlbm_t *g_solver = nullptr;
-    unsigned long long g_gen = 0;       // the solver's step generation when g_exec was captured
+    unsigned long long g_gen = 0;       // the solver's step generation that the graphs are of
+    long long g_steps = 0;              // steps that they have taken
 };
 
 namespace {
-
-constexpr int ROLL_STEPS = 8;
 
 void drop_rollout(vlbm_lc_t *n)
 {
     if (n->g_exec) cudaGraphExecDestroy(n->g_exec);
     if (n->g_many) cudaGraphExecDestroy(n->g_many);
     n->g_exec = n->g_many = nullptr;
+    n->g_steps = 0;
 }
 
 int lfail(vlbm_lc_t *n, int code, const std::string &m)
@@ -472,14 +473,15 @@ int vlbm_lc_rollout(vlbm_lc_t *n, vlbm_t *h, int steps)
     if (!h->d_row) return lfail(n, VLBM_ERR_ARG, "FP32 state not initialised");
     // the captured step holds the solver's launch parameters (its FP32 reference density among
     // them): rebuild for another solver or once the solver has renewed them
-    if (n->g_exec && (n->g_solver != h || n->g_gen != h->step_gen)) drop_rollout(n);
-    if (!n->g_exec && (rc = capture_rollout(n, h, 1, &n->g_exec))) return rc;
-    if (steps >= ROLL_STEPS && !n->g_many && (rc = capture_rollout(n, h, ROLL_STEPS, &n->g_many))) return rc;
+    if (n->g_solver != h || n->g_gen != h->step_gen) drop_rollout(n);
     n->g_solver = h;
     n->g_gen = h->step_gen;
-    int left = steps;
-    for (; left >= ROLL_STEPS; left -= ROLL_STEPS) LCK(n, cudaGraphLaunch(n->g_many, h->stream));
-    for (; left > 0; --left) LCK(n, cudaGraphLaunch(n->g_exec, h->stream));
+    const RolloutPlan plan = rollout_plan(steps, n->g_steps, n->g_exec != nullptr, n->g_many != nullptr);
+    if (plan.capture_one && (rc = capture_rollout(n, h, 1, &n->g_exec))) return rc;
+    if (plan.capture_many && (rc = capture_rollout(n, h, ROLL_STEPS, &n->g_many))) return rc;
+    n->g_steps += steps;
+    for (int q = 0; q < plan.many; ++q) LCK(n, cudaGraphLaunch(n->g_many, h->stream));
+    for (int q = 0; q < plan.ones; ++q) LCK(n, cudaGraphLaunch(n->g_exec, h->stream));
     solver_count_steps(h, steps);
     if ((rc = vlbm_sync(h))) return lfail(n, rc, vlbm_last_error(h));
     return VLBM_OK;
