@@ -1382,13 +1382,13 @@ void lc_outputs(const float *Y, int CO, int H, int W, float3 scale, const double
 }
 
 void lc_moments(const float2 *f, const Layout &L, const VelD &c, double rho_ref, const float *inv_ks_s, float *dev,
-                cudaStream_t s)
+                cudaStream_t s, bool early)
 {
     VelM cm;
     for (int a = 0; a < 4; ++a) cm.v[a] = (float)c.v[a];
     cm.rho_ref = (float)rho_ref;
     cm.drho_ref = (float)(rho_ref - 1.0);
-    launch_after(true, lc_moments_kernel, dim3((L.np + 127) / 128, L.nt), 128, 0, s, f, L, cm, inv_ks_s, dev);
+    launch_after(early, lc_moments_kernel, dim3((L.np + 127) / 128, L.nt), 128, 0, s, f, L, cm, inv_ks_s, dev);
 }
 
 void lc_nudge(float2 *f, const Layout &L, const float *dev, const double *delta, const double *mean, double wsum,

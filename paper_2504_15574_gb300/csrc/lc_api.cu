@@ -204,7 +204,9 @@ int check_solver(vlbm_lc_t *n, vlbm_t *h)
 // cell's ghost images).
 int enqueue_correction(vlbm_lc_t *n, vlbm_t *h, cudaStream_t s)
 {
-    lc_moments((const float2 *)h->F, h->L, h->vd, h->rho_ref, h->d_ikss, n->d_dev, s);
+    // (a step on the split filter schedule ends with a join of two streams: a plain edge after it, as before
+    // the step's own launches there)
+    lc_moments((const float2 *)h->F, h->L, h->vd, h->rho_ref, h->d_ikss, n->d_dev, s, !solver_splits(h));
     int rc;
     if (n->form == VLBM_LC_DIRECT) {
         // the output scaling and the area mean of drho ride on the last convolution and the nudge

@@ -77,8 +77,9 @@ void lc_features(const float *dev, int H, int W, const double *sin_t, const doub
 void lc_dev_of_moments(const double *in4, int H, int W, float *dev, cudaStream_t s);
 // The deviations (rho - 1, u^theta, u^phi, T - 1) [4][H][W] of a solver's FP32 state (inv_ks_s: its
 // 1 / (k sin theta) per row), FP32 arithmetic on the stored deviations.
+// (early: launch_after's.)
 void lc_moments(const float2 *f, const Layout &L, const VelD &c, double rho_ref, const float *inv_ks_s, float *dev,
-                cudaStream_t s);
+                cudaStream_t s, bool early);
 void lc_outputs(const float *Y, int CO, int H, int W, float3 scale, const double *sin_t, double *out, double *part,
                 double *mean, cudaStream_t s);
 void lc_nudge(float2 *f, const Layout &L, const float *dev, const double *delta, const double *mean, double wsum,

@@ -473,7 +473,7 @@ void enqueue_split_step(vlbm_t *h)
 // its polar filter alone (part 0: both).
 void enqueue_step(vlbm_t *h, int stage_only = 0, int part = 0)
 {
-    if (h->prec == VLBM_FP32 && !stage_only && h->band_hi > h->band_lo) {
+    if (h->prec == VLBM_FP32 && !stage_only && solver_splits(h)) {
         enqueue_split_step(h);
         return;
     }
@@ -525,7 +525,7 @@ void enqueue_step(vlbm_t *h, int stage_only = 0, int part = 0)
 
 int kernels_per_step(const vlbm_t *h)
 {
-    int n = 3 + (h->nfrows ? 3 : 0) + (h->band_hi > h->band_lo ? 3 : 0);
+    int n = 3 + (h->nfrows ? 3 : 0) + (solver_splits(h) ? 3 : 0);
     if (h->prec == VLBM_FP64) n += 3;   // a face kernel per stage
     return n;
 }

@@ -82,5 +82,7 @@ struct vlbm {
 // Library-internal entry points on a solver (vlbm_api.cu), for the other host units.
 // Enqueues one RK3 step of h on its stream (stages, whose kernels add the pole sums, and polar filters).
 void solver_enqueue_step(vlbm_t *h);
+// Whether h's steps run on two streams (the split filter schedule).
+inline bool solver_splits(const vlbm_t *h) { return h->band_hi > h->band_lo; }
 // Adds n steps to h's step counter (steps enqueued outside vlbm_step).
 void solver_count_steps(vlbm_t *h, int n);

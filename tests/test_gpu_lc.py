@@ -450,3 +450,26 @@ def test_network_at_the_edges_of_its_tiles(V, H, W):
     assert np.array_equal(a.get_populations(), b.get_populations())
     a.close()
     b.close()
+
+
+def test_rollout_after_the_split_filter_schedule_equals_stepping_and_applying_bitwise(V):
+    """A grid with filter blocks wider than a tile: the step ends with a join of two streams, and the correction
+    follows it; steps in graphs of one and (from 96 steps on) of eight."""
+    H, W = 64, 512
+    net = V.LearnedCorrection(H, W, seed=7, in_scale=_in_scale(H, W), out_scale=OUT_SCALE)
+    p = net.get_weights().astype(np.float64)
+    p[-3:] = [0.3, -0.2, 0.1]
+    net.set_weights(p)
+    a, b = (V.Solver(H, W, 2e-3, 1e-5, precision="fp32", guard=False, polar_filter=True) for _ in range(2))
+    for s in (a, b):
+        s.init_moments(*inputs.gaussian_vortices(H, W, run=6))
+    done = 0
+    for steps in (3, 10, 90):
+        net.rollout(a, steps)
+        for _ in range(steps):
+            b.step(1)
+            net.apply(b)
+        done += steps
+        assert np.array_equal(a.get_populations(), b.get_populations()), done
+    a.close()
+    b.close()
