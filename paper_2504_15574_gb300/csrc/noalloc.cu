@@ -127,13 +127,14 @@ __global__ void __launch_bounds__(NOALLOC_THREADS) noalloc_sums_kernel(const dou
         double sb = bs[warp], cb = bc[warp];
         if (ch >= (int)(gridDim.x * (NOALLOC_THREADS / 32))) sincospi(64.0 * ch / np, &sb, &cb);
         const double sph = fma(sb, lc[lane], cb * ls[lane]), cph = fma(cb, lc[lane], -(sb * ls[lane]));
-        // sum |v|^2 f = v3^2 (so + sp) + v2^2 (si + the populations of |v_phi| = v[2])
-        const double mass = so + si;
+        // sum |v|^2 f = v3^2 (so + sp) + v2^2 (si + the populations of |v_phi| = v[2]: the others of the mass;
+        // an infinite sp is in so or si as well, and infinities of both signs meet there)
+        const double mass = so + si, rest = isinf(sp) ? 0.0 : mass - sp;
         acc[0] += mass;
         acc[1] += fma(a, cph, -(b * sph));
         acc[2] += fma(a, sph, b * cph);
         acc[3] -= z;
-        acc[4] += fma(c.v3 * c.v3, so + sp, c.v2 * c.v2 * (si + (mass - sp)));
+        acc[4] += fma(c.v3 * c.v3, so + sp, c.v2 * c.v2 * (si + rest));
     }
     acc[5] = bad;
     // warps by a butterfly whose first steps also halve the sums that a lane carries (9 additions, not 30):

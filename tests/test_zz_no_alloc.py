@@ -106,3 +106,25 @@ def test_noalloc_sums_match_numpy(nt, np_):
     torch.cuda.synchronize()
     # FP64 sums in another order: rounding of sums of positive terms; momenta cancel, so on the mass's scale
     np.testing.assert_allclose(out.cpu().numpy(), ref, rtol=1e-12, atol=1e-12 * ref[0])
+
+
+@pytest.mark.parametrize("k", [0, 1, 5, 6, 15])
+@pytest.mark.parametrize("value", [np.inf, -np.inf])
+def test_noalloc_energy_of_an_infinite_population(k, value):
+    """One infinite population: the sums of positive weights (mass, energy) are that infinity, whichever
+    velocity it belongs to, and one cell is counted."""
+    require_gpu()
+    import torch
+
+    from paper_2504_15574_gb300 import vlbm
+    vlbm.load()
+    nt, np_ = 20, 70
+    f = np.full((16, nt, np_), 0.0625)
+    f[k, 7, 33] = value
+    out = torch.zeros(6, dtype=torch.float64, device="cuda")
+    f_dev = torch.from_numpy(f).to("cuda")
+    vlbm.vlbm_diagnostics_noalloc(f_dev.data_ptr(), nt, np_, 1.0, out.data_ptr(),
+                                  torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    o = out.cpu().numpy()
+    assert o[0] == value and o[4] == value and o[5] == 1.0
