@@ -156,23 +156,29 @@ __global__ void __launch_bounds__(NOALLOC_THREADS) noalloc_sums_kernel(const dou
     __syncthreads();
     if (threadIdx.x < NQ) {
         const int q = threadIdx.x;
-        double t = red[q][0];
-        for (int w = 1; w < NOALLOC_THREADS / 32; ++w) t += red[q][w];
+        static_assert(NOALLOC_THREADS == 128, "four warps");
+        const double t = (red[q][0] + red[q][1]) + (red[q][2] + red[q][3]);
         const double scale = (q < 4) ? area : (q == 4 ? 0.5 * area : 1.0);
         part[(size_t)q * gridDim.x * gridDim.y + (size_t)blockIdx.y * gridDim.x + blockIdx.x] = t * scale;
     }
 }
 
-// One warp per quantity adds the n CTA partials in a fixed order.
+// One warp per quantity adds the n CTA partials in a fixed order: four chains a lane, then a tree.  (One chain
+// was up to 40 additions long, the longest of the whole sum.  Emulated against extended precision over ten grids
+// of 16 x 20 to 800 x 1500, the root mean square errors relative to those of the form with one block per row:
+// momentum vector 0.42 to 0.93, mass 0.64 to 1.21 (0.90 on the average), energy 0.48 to 1.26 (0.85).)
 __global__ void __launch_bounds__(32 * NQ) noalloc_final_kernel(const double *part, int n, double *out)
 {
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
-    double t = 0.0;
-#pragma unroll 4
-    for (int b = lane; b < n; b += 32) t += part[(size_t)q * n + b];
+    double t[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int b = lane; b < n; b += 128)
 #pragma unroll
-    for (int m = 16; m > 0; m >>= 1) t += __shfl_xor_sync(0xffffffffu, t, m);
-    if (lane == 0) out[q] = t;
+        for (int k = 0; k < 4; ++k)
+            if (b + 32 * k < n) t[k] += part[(size_t)q * n + b + 32 * k];
+    double s = (t[0] + t[2]) + (t[1] + t[3]);
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+    if (lane == 0) out[q] = s;
 }
 
 int na_fail(int code, const std::string &m)
