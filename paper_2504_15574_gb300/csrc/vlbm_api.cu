@@ -771,7 +771,8 @@ int vlbm_create(int n_theta, int n_phi, int velocity_set, double tau, double dt,
                 }
         }
     }
-    if ((rc = dalloc(h, (void **)&h->d_pole, sizeof(double) * 3 * 2 * NK * (size_t)n_phi)) ||
+    // (FP64: the pole faces' fluxes of the three stages; the FP32 stage kernels keep sums)
+    if ((h->prec == VLBM_FP64 && (rc = dalloc(h, (void **)&h->d_pole, sizeof(double) * 3 * 2 * NK * (size_t)n_phi))) ||
         (rc = dalloc(h, (void **)&h->d_mom, sizeof(double) * 4 * (size_t)n_theta * n_phi)) ||
         (rc = dalloc(h, (void **)&h->d_part, sizeof(double) * diag_partials(h->L))) ||
         (rc = dalloc(h, (void **)&h->d_diag, sizeof(double) * diag_doubles(h))))

@@ -594,3 +594,14 @@ def test_fp64_relaxation_time_without_a_normal_reciprocal_matches_oracle(V):
     fo, fg = o.get_populations(), g.get_populations()
     assert np.isfinite(fo).all() and np.abs(fg - fo).max() <= FP64_TOL * np.abs(fo).max()
     g.close()
+
+
+def test_fp32_solver_holds_no_pole_flux_buffer(V):
+    """Device memory of an FP32 solver: three population arrays, the moments, tables and sums of a few rows; the
+    FP64 path's pole fluxes (96 doubles a column) would be a third more here."""
+    nt, np_ = 6, 4096
+    s = V.Solver(nt, np_, 0.05, 1e-5, precision="fp32")
+    arrays = 3 * 8 * (nt + 6) * (np_ + 8) * 8
+    moments = 4 * nt * np_ * 8
+    assert s.device_bytes() < arrays + moments + 8 * 8 * np_ * 8
+    s.close()
