@@ -160,7 +160,7 @@ int dalloc(vlbm_t *h, void **p, size_t bytes)
 // Doubles of the diagnostics' read-back: six sums, the FP64 budget, one spare, and (FP32) the pole sums
 size_t diag_doubles(const vlbm_t *h)
 {
-    return 8 + (h->prec == VLBM_FP32 ? 2 * (size_t)((h->np + F32_TILE_COLS - 1) / F32_TILE_COLS) : 0);
+    return 8 + (h->prec == VLBM_FP32 ? 6 * (size_t)((h->np + F32_TILE_COLS - 1) / F32_TILE_COLS) : 0);
 }
 
 // Largest moment fields (doubles of all four) that the moment kernels write to host memory themselves: up to
@@ -983,10 +983,13 @@ int vlbm_diagnostics(vlbm_t *h, vlbm_diag *out)
     if (h->prec == VLBM_FP32 && h->run.pole_part) {
         // -dt R dphi times the stage-weighted flux out of the south minus the north pole: the deviations'
         // sums, and the reference state's constant flux of every step taken
-        const double *pole = v + 8;
+        const double *pole = v + 8, weight[3] = {1.0 / 6.0, 1.0 / 6.0, 2.0 / 3.0};
         double sum[2] = {0.0, 0.0};
-        for (int k = 0; k < 2; ++k)
-            for (int b = 0; b < h->run.tiles_x; ++b) sum[k] += pole[(size_t)k * h->run.tiles_x + b];
+        for (int k = 0; k < 6; ++k) {
+            double t = 0.0;
+            for (int b = 0; b < h->run.tiles_x; ++b) t += pole[(size_t)k * h->run.tiles_x + b];
+            sum[k % 2] += weight[k / 2] * t;
+        }
         const double dev = (sum[1] - sum[0]) / h->kscale, ref = (h->pole_ref[1] - h->pole_ref[0]) * (double)h->steps;
         pole_flux = -h->dt * h->R * (2.0 * M_PI / h->np) * (dev + ref);
     }

@@ -132,10 +132,10 @@ struct RunF {
     short rings;               // 1: some rows are filtered by the stage kernel (RowF.ring)
     const float *isp;          // [nt + 2GR + 8] 1/sin at padded row pr (negative at ghost rows)
     const float *sfc;          // [nt + 1 + 8] sin(fi dtheta) of theta interface fi (0 at both poles)
-    // pole mass-flux budget (NULL: not recorded): per pole (north, south) and tile column, [2][tiles_x],
-    // the sum over the stages run, each by its weight in the step (1/6, 1/6, 2/3), and over the tile's
-    // columns and populations of v_theta times the theta-face value of dg on the pole face.  Every
-    // element is added to by one CTA per stage launch, so the sums need no launch of their own.
+    // pole mass-flux budget (NULL: not recorded): per stage, pole (north, south) and tile column, [3][2][tiles_x],
+    // the sum over the steps run and over the tile's columns and populations of v_theta times the
+    // theta-face value of dg on the pole face.  Every element is added to by one CTA per stage launch, so
+    // the sums need no launch of their own.
     double *pole_part;
     // limit of the stage kernels' first wait for a tile's copies (ns; the second, after which
     // the CTA leaves, is always 1 s)
