@@ -1760,8 +1760,9 @@ cudaError_t prepare_one()
     }
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
     if (TY == 8 && !LIN) {
-        e = cudaFuncSetAttribute(stage_f32_kernel<8, false, 3, false, false, false>, at, (int)smem_bytes<8, 3>());
-        if (e) return e;
+        if ((e = cudaFuncSetAttribute(stage_f32_kernel<8, false, 3, false, false, false>, at, (int)smem_bytes<8, 3>())) ||
+            (e = cudaFuncSetAttribute(stage_f32_kernel<8, false, 3, true, false, false>, at, (int)smem_bytes<8, 3>())))
+            return e;
     }
     if ((e = cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 3, true>, at, (int)smem_bytes<TY, 3>())) ||
         (e = cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 3, false>, at, (int)smem_bytes<TY, 3>())) ||
@@ -1899,6 +1900,16 @@ static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, 
             return;
         }
     }
+    if constexpr (Q == 3) {
+        // runs without filtered rows of their own take the forms without that path: 1024 x 2048 201 against
+        // 203 us a step (launches one by one), with the Komissarov flux 207 against 214, 209 before the path was
+        // there.  (Q == 4 keeps the one form: 336 us at 1024 x 2048, 340 without the path.)
+        if (ty == 8 && !lin && !run.rings) {
+            if (run.komissarov) launch_after(early, stage_f32_kernel<8, false, 3, true, false, false>, grid, 256, smem_bytes<8, 3>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+            else launch_after(early, stage_f32_kernel<8, false, 3, false, false, false>, grid, 256, smem_bytes<8, 3>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+            return;
+        }
+    }
     if (!lin && run.komissarov) {   // WENO-5 with the Komissarov theta flux
         if (ty == 4) launch_after(early, stage_f32_kernel<4, false, Q, true>, grid, 128, smem_bytes<4, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
         else launch_after(early, stage_f32_kernel<8, false, Q, true>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
@@ -1909,8 +1920,6 @@ static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, 
         else launch_after(early, stage_f32_kernel<4, false, Q>, grid, 128, smem_bytes<4, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
     } else {
         if (lin) launch_after(early, stage_f32_kernel<8, true, Q>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
-        else if (Q == 3 && !run.rings)   // (Q == 4 keeps the one form: 336 us at 1024 x 2048, 340 without the path)
-            launch_after(early, stage_f32_kernel<8, false, Q, false, false, Q == 4>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
         else launch_after(early, stage_f32_kernel<8, false, Q>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
     }
 }
