@@ -174,9 +174,10 @@ VLBM_API int vlbm_max_stable_dt(int n_theta, int n_phi, int velocity_set, double
  * filter is off); ms_per_stage (6 doubles) may be NULL.  The steps give the same
  * state as vlbm_step's.  Returns in *launches (may be NULL) the launch count of one
  * vlbm_step step: 3 stage launches (FP64: and 3 launches of the interface fluxes), plus 3 filters
- * with the filter on (FP32: when some rows' blocks are wider than 32 columns; the stage kernels
- * average narrower ones), plus (FP32 with such filters, when some tile rows are clear of those rows) 3 more stage launches, the stage then being split into
- * polar and interior tile rows that run on two streams. */
+ * with the filter on (FP32: on grids with blocks wider than 32 columns; elsewhere the stage kernels
+ * average the rows themselves), plus (FP32 with such filters, when some tile rows are clear of the
+ * rows that the filters take) 3 more stage launches, the stage then being split into polar and
+ * interior tile rows that run on two streams. */
 VLBM_API int vlbm_profile_step(vlbm_t *h, int n, double *ms_per_stage, int *launches);
 
 /* Limit, in seconds (0 <= limit <= 10, default 1), of the FP32 stage kernels' first wait for a

@@ -138,6 +138,30 @@ int filter_block(int nt, int np, double sin_i)
     return b;
 }
 
+// Whether some rows' ring blocks are wider than a tile (grids of more than about 400 columns)
+bool has_wide_rings(const vlbm_t *h)
+{
+    if (!h->filter) return false;
+    for (int i = 0; i < h->nt; ++i)
+        if (filter_block(h->nt, h->np, h->sin_t[i]) > F32_RING_MAX) return true;
+    return false;
+}
+
+// Whether an FP32 solver's stage kernels filter the rows of blocks up to F32_RING_MAX themselves.  Always
+// where there are no wider ones: a step then has no filter launch.  Where there are, the filter launches and the
+// schedule on two streams stay for those rows, and averaging the others in the stage kernels pays only if the
+// polar tile rows' longer chain hides behind many others: D2Q16 with more than two waves (912 tiles of 8 rows at
+// three CTAs per SM), WENO-5 1024 x 2048 350 against 362 us a step, U3 384 x 768 55 against 59, U3 + Komissarov
+// 512 x 1024 87.0 against 88.7; below, U3 + Komissarov 256 x 512 44.5 against 40.3, 224 x 448 40.3 against 35.1.
+// D2Q9's lighter tiles never hide it: U3 + Komissarov 512 x 1024 68.3 against 63.6, WENO-5 256 x 512 41.8
+// against 38.5 (1024 x 2048 214.5 against 216.2, its only loss).
+bool filters_in_stage(const vlbm_t *h)
+{
+    if (h->prec != VLBM_FP32 || !h->filter) return false;
+    const long long tiles = (long long)((h->np + F32_TILE_COLS - 1) / F32_TILE_COLS) * ((h->nt + 7) / 8);
+    return !has_wide_rings(h) || (h->vd.q == 4 && tiles > 2 * 3 * 152);
+}
+
 template <typename T>
 int upload(vlbm_t *h, T **dst, const T *src, size_t n)
 {
@@ -732,9 +756,8 @@ int vlbm_create(int n_theta, int n_phi, int velocity_set, double tau, double dt,
         return bail(rc);
     // polar filter rows
     if (h->filter) {
-        // FP32: the stage kernels filter the rows of narrow blocks themselves
         std::vector<int> rows, blocks;
-        h->ring_in_stage = h->prec == VLBM_FP32;
+        h->ring_in_stage = filters_in_stage(h);
         for (int i = 0; i < n_theta; ++i) {
             const int b = filter_block(n_theta, n_phi, h->sin_t[i]);
             if (b > (h->ring_in_stage ? F32_RING_MAX : 1)) {
@@ -1364,8 +1387,8 @@ int vlbm_batch_create(int nruns, const int *n_theta, const int *n_phi, const dou
     // the members' polar filter: in the stage kernels, and one filter launch per stage for the rows with
     // blocks too wide for a tile; a batch without such rows keeps all of it in that launch
     bool wide = false;
-    for (const vlbm_t *h : b->runs) wide = wide || h->nfrows > 0;
-    for (vlbm_t *h : b->runs) h->ring_in_stage = h->ring_in_stage && wide;
+    for (const vlbm_t *h : b->runs) wide = wide || has_wide_rings(h);
+    for (vlbm_t *h : b->runs) h->ring_in_stage = h->filter && wide;
     if (cudaHostAlloc(&b->h_flags, 4 * sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess ||
         cudaEventCreate(&b->ev[0]) != cudaSuccess || cudaEventCreate(&b->ev[1]) != cudaSuccess) {
         vlbm_batch_destroy(b);

@@ -45,7 +45,7 @@ struct vlbm {
     // polar filter
     int *d_frows = nullptr, *d_fblocks = nullptr;
     int nfrows = 0;         // rows of the filter kernel (FP32: those the stage kernels do not filter themselves)
-    bool ring_in_stage = false;  // FP32: the stage kernels filter rows of blocks up to F32_RING_MAX
+    bool ring_in_stage = false;  // FP32: the stage kernels filter the rows of blocks up to F32_RING_MAX (filters_in_stage)
     // diagnostics, budget, I/O scratch
     double *d_pole = nullptr, *d_budget = nullptr, *d_mom = nullptr, *d_dense = nullptr;
     double *d_part = nullptr, *d_diag = nullptr;

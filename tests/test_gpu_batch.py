@@ -172,3 +172,27 @@ def test_ring_blocks_in_the_stage_kernels_equal_the_filter_kernel_bitwise(V, nt,
     assert np.array_equal(s.get_populations(), b.get_populations(0))
     s.close()
     b.close()
+
+
+@pytest.mark.parametrize("nt,np_,velocity_set,scheme", [
+    (64, 512, "d2q16", "weno5"), (64, 512, "d2q16", "u3"), (64, 512, "d2q9", "weno5"), (64, 512, "d2q9", "u3"),
+    (228, 1024, "d2q16", "weno5"), (232, 1024, "d2q16", "u3"), (120, 448, "d2q9", "weno5")])
+def test_filter_schedules_of_grids_with_wide_blocks_are_the_same_bits(V, nt, np_, velocity_set, scheme):
+    """Grids whose widest ring blocks exceed a tile: the narrower rows are averaged by the filter kernel (small
+    grids, D2Q9) or by the stage kernels (D2Q16 from 913 tiles on), in a solver on two streams, in a batch
+    on one, in profiled steps launch by launch."""
+    dt = 0.25 * V.vlbm_max_stable_dt(nt, np_, TAU, polar_filter=True)
+    ic = inputs.gaussian_vortices(nt, np_, 3, umax=0.08)
+    kw = dict(polar_filter=True, velocity_set=velocity_set, scheme=scheme)
+    s, p = (V.Solver(nt, np_, TAU, dt, precision="fp32", **kw) for _ in range(2))
+    b = V.Batch([(nt, np_)], TAU, dt, **kw)
+    for x in (s, p):
+        x.init_moments(*ic[:3])
+    b.init_moments(0, *ic[:3])
+    s.step(12)
+    p.profile_step(12)
+    b.step(12)
+    assert np.array_equal(s.get_populations(), b.get_populations(0))
+    assert np.array_equal(s.get_populations(), p.get_populations())
+    for x in (s, p, b):
+        x.close()
