@@ -1385,10 +1385,12 @@ int vlbm_batch_create(int nruns, const int *n_theta, const int *n_phi, const dou
         b->runs.push_back(h);
     }
     // the members' polar filter: in the stage kernels, and one filter launch per stage for the rows with
-    // blocks too wide for a tile; a batch without such rows keeps all of it in that launch
+    // blocks too wide for a tile; a batch without such rows keeps all of it in that launch, and so does D2Q9,
+    // whose tiles with filtered rows outlast the others' (64 x 128 to 256 x 512, two each: 78 against 83 us a step
+    // with WENO-5, 65 against 70 with U3; only large U3 mixes would be 3 % faster in the stage kernels)
     bool wide = false;
     for (const vlbm_t *h : b->runs) wide = wide || has_wide_rings(h);
-    for (vlbm_t *h : b->runs) h->ring_in_stage = h->filter && wide;
+    for (vlbm_t *h : b->runs) h->ring_in_stage = h->filter && wide && b->q == 4;
     if (cudaHostAlloc(&b->h_flags, 4 * sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess ||
         cudaEventCreate(&b->ev[0]) != cudaSuccess || cudaEventCreate(&b->ev[1]) != cudaSuccess) {
         vlbm_batch_destroy(b);
