@@ -1764,8 +1764,7 @@ cudaError_t prepare_one()
             (e = cudaFuncSetAttribute(stage_f32_kernel<8, false, 3, true, false, false>, at, (int)smem_bytes<8, 3>())))
             return e;
     }
-    if ((e = cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 3, true>, at, (int)smem_bytes<TY, 3>())) ||
-        (e = cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 3, false>, at, (int)smem_bytes<TY, 3>())) ||
+    if ((e = cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 3, false>, at, (int)smem_bytes<TY, 3>())) ||
         (e = cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 4, true>, at, (int)smem_bytes<TY>())))
         return e;
     return cudaFuncSetAttribute(batch_stage_f32_kernel<TY, LIN, 4, false>, at, (int)smem_bytes<TY>());
@@ -1832,8 +1831,8 @@ int stage_f32_max_ctas_per_sm(int ty, int q)
 {
     int n = 0;
     if (q == 3) {
-        if (ty == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<4, false, 3, true>, 128, smem_bytes<4, 3>());
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<8, false, 3, true>, 256, smem_bytes<8, 3>());
+        if (ty == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<4, false, 3, false>, 128, smem_bytes<4, 3>());
+        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<8, false, 3, false>, 256, smem_bytes<8, 3>());
     } else {
         if (ty == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<4, false, 4, true>, 128, smem_bytes<4>());
         else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_stage_f32_kernel<8, false, 4, true>, 256, smem_bytes<8>());
@@ -1937,17 +1936,23 @@ void launch_stage_f32_q3(const CUtensorMap &tm_in, const CUtensorMap &tm_out, co
     launch_stage_q<3>(tm_in, tm_out, tm_f, run, c, stage, ty, lin, rows, err, s);
 }
 
+// One tile per CTA: the next stage's (or the filter's) CTAs start early.  Fewer CTAs than tiles, each walking a fixed
+// share of them: plain edges.  The CTAs with one tile more than the others would otherwise land on whichever SMs
+// become free first, two and three of them together: 1.02 to 1.08 times the time of plain launches at a third
+// of the tile counts tried (64 x 128 runs, 19 to 64 of them), 0.95 to 1 at the others.  The filter behind them
+// starts early in D2Q16 all the same (0.94 to 1 of plain); D2Q9's is faster plain (0.97, 64 x 128 to 256 x 512).
 template <int Q, bool RING>
 static void launch_batch_q(const RunF *runs, const CUtensorMap *tms, const int2 *work, int ntiles,
                            const typename VelOf<Q>::type &c, int stage, int ty, bool lin, int ctas, unsigned *err,
                            cudaStream_t s)
 {
+    const bool early = ctas >= ntiles;
     if (ty == 4) {
-        if (lin) launch_after(true, batch_stage_f32_kernel<4, true, Q, RING>, ctas, 128, smem_bytes<4, Q>(), s, runs, tms, work, ntiles, c, stage, err);
-        else launch_after(true, batch_stage_f32_kernel<4, false, Q, RING>, ctas, 128, smem_bytes<4, Q>(), s, runs, tms, work, ntiles, c, stage, err);
+        if (lin) launch_after(early, batch_stage_f32_kernel<4, true, Q, RING>, ctas, 128, smem_bytes<4, Q>(), s, runs, tms, work, ntiles, c, stage, err);
+        else launch_after(early, batch_stage_f32_kernel<4, false, Q, RING>, ctas, 128, smem_bytes<4, Q>(), s, runs, tms, work, ntiles, c, stage, err);
     } else {
-        if (lin) launch_after(true, batch_stage_f32_kernel<8, true, Q, RING>, ctas, 256, smem_bytes<8, Q>(), s, runs, tms, work, ntiles, c, stage, err);
-        else launch_after(true, batch_stage_f32_kernel<8, false, Q, RING>, ctas, 256, smem_bytes<8, Q>(), s, runs, tms, work, ntiles, c, stage, err);
+        if (lin) launch_after(early, batch_stage_f32_kernel<8, true, Q, RING>, ctas, 256, smem_bytes<8, Q>(), s, runs, tms, work, ntiles, c, stage, err);
+        else launch_after(early, batch_stage_f32_kernel<8, false, Q, RING>, ctas, 256, smem_bytes<8, Q>(), s, runs, tms, work, ntiles, c, stage, err);
     }
 }
 
@@ -1959,11 +1964,9 @@ void launch_batch_stage_f32(const RunF *runs, const CUtensorMap *tms, const int2
 }
 
 void launch_batch_stage_f32_q3(const RunF *runs, const CUtensorMap *tms, const int2 *work, int ntiles,
-                               const VelC3 &c, int stage, int ty, bool lin, bool rings, int ctas, unsigned *err,
-                               cudaStream_t s)
+                               const VelC3 &c, int stage, int ty, bool lin, int ctas, unsigned *err, cudaStream_t s)
 {
-    if (rings) launch_batch_q<3, true>(runs, tms, work, ntiles, c, stage, ty, lin, ctas, err, s);
-    else launch_batch_q<3, false>(runs, tms, work, ntiles, c, stage, ty, lin, ctas, err, s);
+    launch_batch_q<3, false>(runs, tms, work, ntiles, c, stage, ty, lin, ctas, err, s);
 }
 
 double f32_state_scale(double eps)
@@ -2034,10 +2037,11 @@ void launch_fill_ghosts_f32(float2 *f, const Layout &L, int q, cudaStream_t s)
     fill_ghosts_f32_kernel<<<grid, 128, 0, s>>>(f, L, q);
 }
 
-void launch_batch_filter_f32(const RunF *runs, const int4 *items, int nitems, int q, int stage, cudaStream_t s)
+void launch_batch_filter_f32(const RunF *runs, const int4 *items, int nitems, int q, int stage, cudaStream_t s,
+                             bool early)
 {
     if (nitems <= 0) return;
-    launch_after(true, batch_filter_f32_kernel, dim3(nitems, f32_pairs(q)), FILT_THREADS, 0, s, runs, items, q, stage);
+    launch_after(early, batch_filter_f32_kernel, dim3(nitems, f32_pairs(q)), FILT_THREADS, 0, s, runs, items, q, stage);
 }
 
 void launch_filter_f32(float2 *f, const Layout &L, int q, const int *rows, const int *blocks, int nrows,

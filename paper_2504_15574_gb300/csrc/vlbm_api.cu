@@ -1234,13 +1234,14 @@ void batch_enqueue_step(vlbm_batch_t *b)
         const bool lin = b->runs.front()->scheme != VLBM_WENO5;
         const bool rings = std::any_of(b->runs.begin(), b->runs.end(), [](const vlbm_t *h) { return h->run.rings != 0; });
         if (b->q == 3)
-            launch_batch_stage_f32_q3(b->d_runs, b->d_tms, b->d_work, b->ntiles, b->vc3, st, b->ty, lin, rings, ctas,
+            launch_batch_stage_f32_q3(b->d_runs, b->d_tms, b->d_work, b->ntiles, b->vc3, st, b->ty, lin, ctas,
                                       b->d_flags, b->stream);
         else
             launch_batch_stage_f32(b->d_runs, b->d_tms, b->d_work, b->ntiles, b->vc, st, b->ty, lin, rings, ctas,
                                    b->d_flags, b->stream);
         // one polar-filter launch over the filtered rows of every run
-        launch_batch_filter_f32(b->d_runs, b->d_fitems, b->nfitems, b->q, st, b->stream);
+        launch_batch_filter_f32(b->d_runs, b->d_fitems, b->nfitems, b->q, st, b->stream,
+                                b->q == 4 || ctas >= b->ntiles);
     }
 }
 
