@@ -147,19 +147,26 @@ bool has_wide_rings(const vlbm_t *h)
     return false;
 }
 
+// Fewest tiles (of 8 rows, one more than two waves at three CTAs per SM) beside which the polar tile rows' longer
+// chain hides when the stage kernels average ring rows on grids that keep the filter launches too
+constexpr long long RING_TILES = 2 * 3 * 152 + 1;
+
+long long tiles_of_8_rows(const vlbm_t *h)
+{
+    return (long long)((h->np + F32_TILE_COLS - 1) / F32_TILE_COLS) * ((h->nt + 7) / 8);
+}
+
 // Whether an FP32 solver's stage kernels filter the rows of blocks up to F32_RING_MAX themselves.  Always
 // where there are no wider ones: a step then has no filter launch.  Where there are, the filter launches and the
 // schedule on two streams stay for those rows, and averaging the others in the stage kernels pays only if the
-// polar tile rows' longer chain hides behind many others: D2Q16 with more than two waves (912 tiles of 8 rows at
-// three CTAs per SM), WENO-5 1024 x 2048 350 against 362 us a step, U3 384 x 768 55 against 59, U3 + Komissarov
+// polar tile rows' longer chain hides behind many others: D2Q16 from RING_TILES on, WENO-5 1024 x 2048 350 against 362 us a step, U3 384 x 768 55 against 59, U3 + Komissarov
 // 512 x 1024 87.0 against 88.7; below, U3 + Komissarov 256 x 512 44.5 against 40.3, 224 x 448 40.3 against 35.1.
 // D2Q9's lighter tiles never hide it: U3 + Komissarov 512 x 1024 68.3 against 63.6, WENO-5 256 x 512 41.8
 // against 38.5 (1024 x 2048 214.5 against 216.2, its only loss).
 bool filters_in_stage(const vlbm_t *h)
 {
     if (h->prec != VLBM_FP32 || !h->filter) return false;
-    const long long tiles = (long long)((h->np + F32_TILE_COLS - 1) / F32_TILE_COLS) * ((h->nt + 7) / 8);
-    return !has_wide_rings(h) || (h->vd.q == 4 && tiles > 2 * 3 * 152);
+    return !has_wide_rings(h) || (h->vd.q == 4 && tiles_of_8_rows(h) >= RING_TILES);
 }
 
 template <typename T>
@@ -1388,10 +1395,15 @@ int vlbm_batch_create(int nruns, const int *n_theta, const int *n_phi, const dou
     // the members' polar filter: in the stage kernels, and one filter launch per stage for the rows with
     // blocks too wide for a tile; a batch without such rows keeps all of it in that launch, and so does D2Q9,
     // whose tiles with filtered rows outlast the others' (64 x 128 to 256 x 512, two each: 78 against 83 us a step
-    // with WENO-5, 65 against 70 with U3; only large U3 mixes would be 3 % faster in the stage kernels)
+    // with WENO-5, 65 against 70 with U3; only large U3 mixes would be 3 % faster in the stage kernels), and so
+    // does a small D2Q16 mix (one run each of these grids: 62.4 against 64.3, 50.9 against 53.2)
     bool wide = false;
-    for (const vlbm_t *h : b->runs) wide = wide || has_wide_rings(h);
-    for (vlbm_t *h : b->runs) h->ring_in_stage = h->filter && wide && b->q == 4;
+    long long tiles = 0;
+    for (const vlbm_t *h : b->runs) {
+        wide = wide || has_wide_rings(h);
+        tiles += tiles_of_8_rows(h);
+    }
+    for (vlbm_t *h : b->runs) h->ring_in_stage = h->filter && wide && b->q == 4 && tiles >= RING_TILES;
     if (cudaHostAlloc(&b->h_flags, 4 * sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess ||
         cudaEventCreate(&b->ev[0]) != cudaSuccess || cudaEventCreate(&b->ev[1]) != cudaSuccess) {
         vlbm_batch_destroy(b);

@@ -196,3 +196,25 @@ def test_filter_schedules_of_grids_with_wide_blocks_are_the_same_bits(V, nt, np_
     assert np.array_equal(s.get_populations(), p.get_populations())
     for x in (s, p, b):
         x.close()
+
+
+@pytest.mark.parametrize("runs", [1, 8])
+def test_batch_filter_schedules_are_the_same_bits(V, runs):
+    """Small D2Q16 mixes leave every filtered row to the filter kernel, larger ones (913 tiles) the narrower rows to
+    the stage kernels: both the solver's bits, in a schedule of one tile per CTA and of fewer CTAs."""
+    nt, np_ = 64, 512
+    dt = 0.25 * V.vlbm_max_stable_dt(nt, np_, TAU, polar_filter=True)
+    ic = inputs.gaussian_vortices(nt, np_, 3, umax=0.08)
+    s = V.Solver(nt, np_, TAU, dt, precision="fp32", polar_filter=True)
+    s.init_moments(*ic[:3])
+    s.step(12)
+    for schedule in ((8, -1), (8, 0), (4, 0)):
+        b = V.Batch([(nt, np_)] * runs, TAU, dt, polar_filter=True)
+        for r in range(runs):
+            b.init_moments(r, *ic[:3])
+        b.set_schedule(*schedule)
+        b.step(12)
+        for r in (0, runs - 1):
+            assert np.array_equal(s.get_populations(), b.get_populations(r)), (schedule, r)
+        b.close()
+    s.close()
