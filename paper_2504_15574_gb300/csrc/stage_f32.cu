@@ -1885,10 +1885,14 @@ static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, 
                            const RunF &run, const typename VelOf<Q>::type &c, int stage, int ty, bool lin,
                            TileRows rows, unsigned *err, cudaStream_t s)
 {
-    const bool early = rows.count < 0;   // (as launch_persist_q)
+    bool early = rows.count < 0;   // (as launch_persist_q)
     if (rows.count < 0) rows = TileRows{0, (run.L.nt + ty - 1) / ty, 1 << 30, 0};
     if (rows.count == 0) return;
     const dim3 grid((run.L.np + TX - 1) / TX, rows.count);
+    // D2Q9, four CTAs per SM: three tiles per SM would land as up to four on those that become free first
+    // (288 x 384 with the Komissarov flux 20.9 us a step, 19.3 with plain edges; two and four per SM gain 5 to 10 %)
+    const long long tiles = (long long)grid.x * grid.y;
+    if (Q == 3 && ty == 8 && tiles > 2 * 152 && tiles <= 3 * 152) early = false;
     if constexpr (Q == 4) {
         if (ty == 8 && early && stage_f32_wide(run.L)) {
             const size_t smem = spread_smem((long long)grid.x * grid.y, wide_smem());
