@@ -1883,7 +1883,7 @@ bool stage_f32_wide(const Layout &L) { return (long long)((L.np + TX - 1) / TX) 
 template <int Q>
 static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f,
                            const RunF &run, const typename VelOf<Q>::type &c, int stage, int ty, bool lin,
-                           TileRows rows, unsigned *err, cudaStream_t s)
+                           TileRows rows, StageForm form, unsigned *err, cudaStream_t s)
 {
     bool early = rows.count < 0;   // (as launch_persist_q)
     if (rows.count < 0) rows = TileRows{0, (run.L.nt + ty - 1) / ty, 1 << 30, 0};
@@ -1894,8 +1894,8 @@ static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, 
     const long long tiles = (long long)grid.x * grid.y;
     if (Q == 3 && ty == 8 && tiles > 2 * 152 && tiles <= 3 * 152) early = false;
     if constexpr (Q == 4) {
-        if (ty == 8 && early && stage_f32_wide(run.L)) {
-            const size_t smem = spread_smem((long long)grid.x * grid.y, wide_smem());
+        if (ty == 8 && early && form != STAGE_CROWDED && stage_f32_wide(run.L)) {
+            const size_t smem = form == STAGE_ALONE ? spread_smem(tiles, wide_smem()) : wide_smem();
             if (lin) launch_after(early, stage_f32_kernel<8, true, 4, false, true>, grid, 512, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
             else if (run.komissarov) launch_after(early, stage_f32_kernel<8, false, 4, true, true>, grid, 512, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
             else if (run.rings) launch_after(early, stage_f32_kernel<8, false, 4, false, true>, grid, 512, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
@@ -1928,16 +1928,17 @@ static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, 
 }
 
 void launch_stage_f32(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f, const RunF &run,
-                      const VelC &c, int stage, int ty, bool lin, unsigned *err, cudaStream_t s, TileRows rows)
+                      const VelC &c, int stage, int ty, bool lin, unsigned *err, cudaStream_t s, TileRows rows,
+                      StageForm form)
 {
-    launch_stage_q<4>(tm_in, tm_out, tm_f, run, c, stage, ty, lin, rows, err, s);
+    launch_stage_q<4>(tm_in, tm_out, tm_f, run, c, stage, ty, lin, rows, form, err, s);
 }
 
 void launch_stage_f32_q3(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f,
                          const RunF &run, const VelC3 &c, int stage, int ty, bool lin, unsigned *err, cudaStream_t s,
                          TileRows rows)
 {
-    launch_stage_q<3>(tm_in, tm_out, tm_f, run, c, stage, ty, lin, rows, err, s);
+    launch_stage_q<3>(tm_in, tm_out, tm_f, run, c, stage, ty, lin, rows, STAGE_ALONE, err, s);
 }
 
 // One tile per CTA: the next stage's (or the filter's) CTAs start early.  Fewer CTAs than tiles, each walking a fixed

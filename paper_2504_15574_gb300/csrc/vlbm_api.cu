@@ -151,11 +151,6 @@ bool has_wide_rings(const vlbm_t *h)
 // chain hides when the stage kernels average ring rows on grids that keep the filter launches too
 constexpr long long RING_TILES = 2 * 3 * 152 + 1;
 
-long long tiles_of_8_rows(const vlbm_t *h)
-{
-    return (long long)((h->np + F32_TILE_COLS - 1) / F32_TILE_COLS) * ((h->nt + 7) / 8);
-}
-
 // Whether an FP32 solver's stage kernels filter the rows of blocks up to F32_RING_MAX themselves.  Always
 // where there are no wider ones: a step then has no filter launch.  Where there are, the filter launches and the
 // schedule on two streams stay for those rows, and averaging the others in the stage kernels pays only if the
@@ -166,7 +161,7 @@ long long tiles_of_8_rows(const vlbm_t *h)
 bool filters_in_stage(const vlbm_t *h)
 {
     if (h->prec != VLBM_FP32 || !h->filter) return false;
-    return !has_wide_rings(h) || (h->vd.q == 4 && tiles_of_8_rows(h) >= RING_TILES);
+    return !has_wide_rings(h) || (h->vd.q == 4 && solver_tiles(h) >= RING_TILES);
 }
 
 template <typename T>
@@ -178,6 +173,14 @@ int upload(vlbm_t *h, T **dst, const T *src, size_t n)
     }
     CK(h, cudaMemcpy(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice));
     return VLBM_OK;
+}
+
+// Waits for everything enqueued on h's stream
+cudaError_t wait_stream(vlbm_t *h)
+{
+    const cudaError_t e = cudaStreamSynchronize(h->stream);
+    h->in_flight.leave();
+    return e;
 }
 
 int dalloc(vlbm_t *h, void **p, size_t bytes)
@@ -452,7 +455,7 @@ void launch_stage_f32_any(vlbm_t *h, int st, cudaStream_t s, TileRows rows = Til
     const CUtensorMap &tm = (st == 1) ? h->tmF : (st == 2) ? h->tmA : h->tmB;
     const CUtensorMap &tmo = (st == 1) ? h->tmAc : (st == 2) ? h->tmBc : h->tmFc;
     const bool lin = h->scheme != VLBM_WENO5;
-    const bool wide = h->vd.q == 4 && rows.count < 0 && stage_f32_wide(h->L);
+    const bool wide = h->vd.q == 4 && rows.count < 0 && h->form != STAGE_CROWDED && stage_f32_wide(h->L);
     if (h->ty == 8 && lin && !wide) {
         // the upwind schemes: the persistent kernel, whose next tile's copies are in flight during
         // the cell phase (their lighter faces leave the one-tile kernel's loads exposed; for WENO-5
@@ -466,7 +469,7 @@ void launch_stage_f32_any(vlbm_t *h, int st, cudaStream_t s, TileRows rows = Til
         return;
     }
     if (h->vd.q == 3) launch_stage_f32_q3(tm, tmo, h->tmFc, h->run, h->vc3, st, h->ty, lin, h->d_flags, s, rows);
-    else launch_stage_f32(tm, tmo, h->tmFc, h->run, h->vc, st, h->ty, lin, h->d_flags, s, rows);
+    else launch_stage_f32(tm, tmo, h->tmFc, h->run, h->vc, st, h->ty, lin, h->d_flags, s, rows, h->form);
 }
 
 // One FP32 RK3 step with the polar filter.  The tile rows touching a filtered row and the filter
@@ -561,11 +564,13 @@ int kernels_per_step(const vlbm_t *h)
     return n;
 }
 
-int build_graph(vlbm_t *h, int nsteps, cudaGraphExec_t *exec)
+int build_graph(vlbm_t *h, int nsteps, StageForm form, cudaGraphExec_t *exec)
 {
     cudaGraph_t g = nullptr;
     CK(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
+    h->form = form;
     for (int q = 0; q < nsteps; ++q) enqueue_step(h);
+    h->form = STAGE_ALONE;
     cudaError_t e = cudaStreamEndCapture(h->stream, &g);
     if (e != cudaSuccess) return fail(h, VLBM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
     // (node priorities: the kernels captured from the high-priority stream keep it)
@@ -582,9 +587,11 @@ std::atomic<unsigned long long> g_step_generation{0};
 
 void drop_graphs(vlbm_t *h)
 {
-    if (h->g1) cudaGraphExecDestroy(h->g1);
-    if (h->g16) cudaGraphExecDestroy(h->g16);
-    h->g1 = h->g16 = nullptr;
+    for (int f = 0; f < STAGE_FORMS; ++f) {
+        if (h->g1[f]) cudaGraphExecDestroy(h->g1[f]);
+        if (h->g16[f]) cudaGraphExecDestroy(h->g16[f]);
+        h->g1[f] = h->g16[f] = nullptr;
+    }
     h->step_gen = ++g_step_generation;
 }
 
@@ -617,7 +624,7 @@ int choose_rho_ref(vlbm_t *h, const double *d_rho)
     CK(h, cudaGetLastError());
     double v = 0.0;
     CK(h, cudaMemcpyAsync(&v, h->d_scalar, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
+    CK(h, wait_stream(h));
     h->rho_ref = v;
     return VLBM_OK;
 }
@@ -924,7 +931,7 @@ int vlbm_get_populations(vlbm_t *h, double *f)
     else launch_pack_f32((const float2 *)h->F, h->L, h->d_dense, h->vd, h->rho_ref, h->d_sin_t, h->kscale, h->stream);
     CK(h, cudaGetLastError());
     CK(h, cudaMemcpyAsync(f, h->d_dense, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
+    CK(h, wait_stream(h));
     return VLBM_OK;
 }
 
@@ -933,15 +940,19 @@ int vlbm_step_async(vlbm_t *h, int n)
     if (!h || n < 0) return fail(h, VLBM_ERR_ARG, "bad handle or step count");
     if (h->prec == VLBM_FP32 && !h->d_row) return fail(h, VLBM_ERR_ARG, "FP32 state not initialised");
     if (n == 0) return VLBM_OK;
+    const long long tiles = solver_tiles(h), others = h->in_flight.enter(tiles);
+    // (one form only: grids of more than two tiles per SM, 4-row tiles, D2Q9, FP64)
+    const bool forms = h->prec == VLBM_FP32 && h->vd.q == 4 && h->ty == 8 && !solver_splits(h) && stage_f32_wide(h->L);
+    const StageForm f = forms ? stage_form(tiles, others) : STAGE_ALONE;
     int rc;
-    if (!h->g1 && (rc = build_graph(h, 1, &h->g1))) return rc;
-    if (n >= 16 && !h->g16 && (rc = build_graph(h, 16, &h->g16))) return rc;
+    if (!h->g1[f] && (rc = build_graph(h, 1, f, &h->g1[f]))) return rc;
+    if (n >= 16 && !h->g16[f] && (rc = build_graph(h, 16, f, &h->g16[f]))) return rc;
     int left = n;
     while (left >= 16) {
-        CK(h, cudaGraphLaunch(h->g16, h->stream));
+        CK(h, cudaGraphLaunch(h->g16[f], h->stream));
         left -= 16;
     }
-    while (left-- > 0) CK(h, cudaGraphLaunch(h->g1, h->stream));
+    while (left-- > 0) CK(h, cudaGraphLaunch(h->g1[f], h->stream));
     h->steps += n;
     return VLBM_OK;
 }
@@ -949,7 +960,7 @@ int vlbm_step_async(vlbm_t *h, int n)
 int vlbm_sync(vlbm_t *h)
 {
     if (!h) return fail(h, VLBM_ERR_ARG, "NULL handle");
-    CK(h, cudaStreamSynchronize(h->stream));
+    CK(h, wait_stream(h));
     CK(h, cudaGetLastError());
     if (h->h_flags[0] & 1u) return fail(h, VLBM_ERR_TIMEOUT, "a tile load did not complete within its time limit");
     if (h->h_flags[1]) return fail(h, VLBM_ERR_NONFINITE, "non-finite population found by the guard");
@@ -980,7 +991,7 @@ int vlbm_moments(vlbm_t *h, double *rho, double *u_theta, double *u_phi, double 
                            h->rho_ref, h->d_ikss, h->stream);
     CK(h, cudaGetLastError());
     if (h->h_mom) {
-        CK(h, cudaStreamSynchronize(h->stream));
+        CK(h, wait_stream(h));
         memcpy(rho, d, n * sizeof(double));
         memcpy(u_theta, d + n, n * sizeof(double));
         memcpy(u_phi, d + 2 * n, n * sizeof(double));
@@ -991,7 +1002,7 @@ int vlbm_moments(vlbm_t *h, double *rho, double *u_theta, double *u_phi, double 
     CK(h, cudaMemcpyAsync(u_theta, d + n, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaMemcpyAsync(u_phi, d + 2 * n, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     if (T) CK(h, cudaMemcpyAsync(T, d + 3 * n, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
+    CK(h, wait_stream(h));
     return VLBM_OK;
 }
 
@@ -1008,7 +1019,7 @@ int vlbm_diagnostics(vlbm_t *h, vlbm_diag *out)
     CK(h, cudaGetLastError());
     const double *v = h->h_diag;
     CK(h, cudaMemcpyAsync(h->h_diag, h->d_diag, sizeof(double) * diag_doubles(h), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
+    CK(h, wait_stream(h));
     double pole_flux = v[6];
     if (h->prec == VLBM_FP32 && h->run.pole_part) {
         // -dt R dphi times the stage-weighted flux out of the south minus the north pole: the deviations'
@@ -1097,7 +1108,7 @@ const char *vlbm_last_error(const vlbm_t *h) { return h ? h->err.c_str() : g_cre
 void vlbm_destroy(vlbm_t *h)
 {
     if (!h) return;
-    if (h->stream) cudaStreamSynchronize(h->stream);
+    if (h->stream) wait_stream(h);
     drop_graphs(h);
     void *bufs[] = {h->F, h->A, h->B, h->d_sin_ext, h->d_rowd, h->d_sin_t, h->d_cos_t, h->d_sin_f, h->d_isp,
                     h->d_sfc, h->d_ft, h->d_fp,
@@ -1140,6 +1151,7 @@ struct vlbm_batch {
     cudaEvent_t ev[2] = {nullptr, nullptr};
     std::string err;
     long long steps = 0;
+    InFlight in_flight;
 };
 
 namespace {
@@ -1172,6 +1184,14 @@ void batch_drop_graphs(vlbm_batch_t *b)
     if (b->g1) cudaGraphExecDestroy(b->g1);
     if (b->g16) cudaGraphExecDestroy(b->g16);
     b->g1 = b->g16 = nullptr;
+}
+
+// Waits for everything enqueued on b's stream
+cudaError_t batch_wait(vlbm_batch_t *b)
+{
+    const cudaError_t e = cudaStreamSynchronize(b->stream);
+    b->in_flight.leave();
+    return e;
 }
 
 // Uploads the run table, tensor maps (for the current tile rows) and work list.
@@ -1401,7 +1421,7 @@ int vlbm_batch_create(int nruns, const int *n_theta, const int *n_phi, const dou
     long long tiles = 0;
     for (const vlbm_t *h : b->runs) {
         wide = wide || has_wide_rings(h);
-        tiles += tiles_of_8_rows(h);
+        tiles += solver_tiles(h);
     }
     for (vlbm_t *h : b->runs) h->ring_in_stage = h->filter && wide && b->q == 4 && tiles >= RING_TILES;
     if (cudaHostAlloc(&b->h_flags, 4 * sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess ||
@@ -1429,7 +1449,7 @@ int vlbm_batch_init_moments(vlbm_batch_t *b, int run, const double *rho, const d
 int vlbm_batch_get_populations(vlbm_batch_t *b, int run, double *f)
 {
     if (!b || run < 0 || run >= (int)b->runs.size()) return bfail(b, VLBM_ERR_ARG, "bad batch or run index");
-    BCK(b, cudaStreamSynchronize(b->stream));
+    BCK(b, batch_wait(b));
     int rc = vlbm_get_populations(b->runs[run], f);
     if (rc) return bfail(b, rc, b->runs[run]->err);
     return VLBM_OK;
@@ -1453,6 +1473,7 @@ int vlbm_batch_step_async(vlbm_batch_t *b, int n)
     if (n == 0) return VLBM_OK;
     int rc;
     if ((rc = batch_refresh(b))) return rc;
+    b->in_flight.enter(b->ntiles);
     if (!b->g1 && (rc = batch_build_graph(b, 1, &b->g1))) return rc;
     if (n >= 16 && !b->g16 && (rc = batch_build_graph(b, 16, &b->g16))) return rc;
     int left = n;
@@ -1469,7 +1490,7 @@ int vlbm_batch_step_async(vlbm_batch_t *b, int n)
 int vlbm_batch_sync(vlbm_batch_t *b)
 {
     if (!b) return bfail(b, VLBM_ERR_ARG, "NULL batch");
-    BCK(b, cudaStreamSynchronize(b->stream));
+    BCK(b, batch_wait(b));
     BCK(b, cudaGetLastError());
     if (b->h_flags[0] & 1u) return bfail(b, VLBM_ERR_TIMEOUT, "a tile load did not complete within its time limit");
     if (b->h_flags[1]) return bfail(b, VLBM_ERR_NONFINITE, "non-finite population found by the guard");
@@ -1490,7 +1511,7 @@ int vlbm_batch_step(vlbm_batch_t *b, int n)
 int vlbm_batch_moments(vlbm_batch_t *b, int run, double *rho, double *u_theta, double *u_phi, double *T)
 {
     if (!b || run < 0 || run >= (int)b->runs.size()) return bfail(b, VLBM_ERR_ARG, "bad batch or run index");
-    BCK(b, cudaStreamSynchronize(b->stream));
+    BCK(b, batch_wait(b));
     int rc = vlbm_moments(b->runs[run], rho, u_theta, u_phi, T);
     if (rc) return bfail(b, rc, b->runs[run]->err);
     return VLBM_OK;
@@ -1551,7 +1572,7 @@ int vlbm_batch_tune(vlbm_batch_t *b, const char *cache_path, int *tile_rows, int
             BCK(b, cudaMemcpyAsync(h->F, backup[r], h->arr_bytes, cudaMemcpyDeviceToDevice, b->stream));
             h->steps = 0;
         }
-        BCK(b, cudaStreamSynchronize(b->stream));
+        BCK(b, batch_wait(b));
         for (void *p : backup) cudaFree(p);
         b->steps = 0;
         cache_store(cache_path, key, best_ty, best_c, best);
@@ -1576,7 +1597,7 @@ const char *vlbm_batch_last_error(const vlbm_batch_t *b) { return b ? b->err.c_s
 void vlbm_batch_destroy(vlbm_batch_t *b)
 {
     if (!b) return;
-    if (b->stream) cudaStreamSynchronize(b->stream);
+    if (b->stream) batch_wait(b);
     batch_drop_graphs(b);
     for (vlbm_t *h : b->runs) vlbm_destroy(h);
     if (b->d_runs) cudaFree(b->d_runs);

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/vlbm.h"
+#include "stage_form.h"
 #include "vlbm_internal.h"
 
 struct vlbm {
@@ -53,7 +54,9 @@ struct vlbm {
     double *h_diag = nullptr, *h_mom = nullptr;        // pinned: the diagnostics' read-back; moments of small grids
     CUtensorMap tmF{}, tmA{}, tmB{};      // FP32 path: box maps (stage inputs)
     CUtensorMap tmFc{}, tmAc{}, tmBc{};   // FP32 path: tile-core maps (stage outputs, F prefetch)
-    cudaGraphExec_t g1 = nullptr, g16 = nullptr;
+    cudaGraphExec_t g1[vk::STAGE_FORMS] = {}, g16[vk::STAGE_FORMS] = {};   // one and 16 steps, per stage form
+    vk::StageForm form = vk::STAGE_ALONE;   // of the launches being captured
+    vk::InFlight in_flight;
     // generation of the step's launch parameters: renewed whenever g1 / g16 are dropped (new FP32
     // reference density, wait limit), so graphs captured elsewhere from this step know to rebuild
     unsigned long long step_gen = 0;
@@ -84,5 +87,10 @@ struct vlbm {
 void solver_enqueue_step(vlbm_t *h);
 // Whether h's steps run on two streams (the split filter schedule).
 inline bool solver_splits(const vlbm_t *h) { return h->band_hi > h->band_lo; }
+// Tiles of 8 rows of a launch over h's grid.
+inline long long solver_tiles(const vlbm_t *h)
+{
+    return (long long)((h->np + vk::F32_TILE_COLS - 1) / vk::F32_TILE_COLS) * ((h->nt + 7) / 8);
+}
 // Adds n steps to h's step counter (steps enqueued outside vlbm_step).
 void solver_count_steps(vlbm_t *h, int n);

@@ -21,6 +21,7 @@
 
 #include "../../include/vlbm.h"
 #include "f64_int.cuh"
+#include "stage_form.h"
 
 namespace vk {
 
@@ -219,8 +220,8 @@ cudaError_t prepare_stage_f32();   // sets the kernels' dynamic shared-memory li
 // `skip` tile rows after the first `split` of them (count < 0: every tile row of the grid).
 struct TileRows { int first, count, split, skip; };
 void launch_stage_f32(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f, const RunF &run,
-                      const VelC &c, int stage, int ty, bool lin, unsigned *err, cudaStream_t s,
-                      TileRows rows = TileRows{0, -1, 0, 0});
+                      const VelC &c, int stage, int ty, bool lin, unsigned *err, cudaStream_t s, TileRows rows,
+                      StageForm form);
 // Whether a D2Q16 launch of all 8-row tiles of a grid takes the stage kernel's 512-thread form.
 bool stage_f32_wide(const Layout &L);
 // The same for D2Q9 (five pair planes; tensor maps of depth 5).

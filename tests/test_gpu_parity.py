@@ -605,3 +605,35 @@ def test_fp32_solver_holds_no_pole_flux_buffer(V):
     moments = 4 * nt * np_ * 8
     assert s.device_bytes() < arrays + moments + 8 * 8 * np_ * 8
     s.close()
+
+
+@pytest.mark.parametrize("scheme,komissarov", [("weno5", False), ("u3", True)])
+def test_fp32_solvers_in_flight_together_give_the_bits_of_one_alone(V, scheme, komissarov):
+    """Beside other solvers' steps a small grid's take other forms of the stage kernel (two solvers: one, seven: the
+    other): the same bits, and the form of a solver alone again afterwards."""
+    nt, np_ = 93, 250   # 96 tiles
+    dt = clamped_dt(nt, np_, 0.02)
+    starts = [inputs.gaussian_vortices(nt, np_, 3 + r, umax=0.08) for r in range(7)]
+
+    def solver(ic):
+        s = V.Solver(nt, np_, 0.02, dt, precision="fp32", scheme=scheme, komissarov=komissarov)
+        s.init_moments(*ic)
+        return s
+    alone = []
+    for ic in starts:
+        s = solver(ic)
+        s.step(37)
+        alone.append(s.get_populations())
+        s.close()
+    for n in (2, 7):
+        together = [solver(ic) for ic in starts[:n]]
+        for steps in (16, 3):
+            for s in together:
+                s.step_async(steps)
+        for s in together:
+            s.sync()
+        for s in together:
+            s.step(18)
+        for s, f in zip(together, alone):
+            assert np.array_equal(s.get_populations(), f)
+            s.close()
