@@ -176,13 +176,13 @@ __device__ __forceinline__ FF ff_leaf(f2 a, f2 b)
     return r;
 }
 
-__device__ __forceinline__ FF ff_shfl_xor(FF a, int m, unsigned mask = 0xffffffffu)
+__device__ __forceinline__ FF ff_shfl_xor(FF a, int m)
 {
     FF r;
-    r.hi.x = __shfl_xor_sync(mask, a.hi.x, m);
-    r.hi.y = __shfl_xor_sync(mask, a.hi.y, m);
-    r.lo.x = __shfl_xor_sync(mask, a.lo.x, m);
-    r.lo.y = __shfl_xor_sync(mask, a.lo.y, m);
+    r.hi.x = __shfl_xor_sync(0xffffffffu, a.hi.x, m);
+    r.hi.y = __shfl_xor_sync(0xffffffffu, a.hi.y, m);
+    r.lo.x = __shfl_xor_sync(0xffffffffu, a.lo.x, m);
+    r.lo.y = __shfl_xor_sync(0xffffffffu, a.lo.y, m);
     return r;
 }
 
@@ -758,9 +758,10 @@ __device__ __forceinline__ void load_cell_g(const Sm &S, int b, f2 *G)
 // WIDE: two threads per cell, the warps of its row in the two halves of the CTA, each of which updates
 // the pairs of one k_theta half (both form the moments).
 // RING: rows of narrow ring blocks are filtered here.  false: the run has none, and the compiler's schedule of
-// the rest is better without that path in the batch kernel (64 runs: 1.98 ms a step against 2.01) and in the
-// D2Q9 kernel (1024 x 2048: 200.6 us against 202.5); the persistent kernel (U3, Komissarov, 512 x 1024) takes
-// 70.3 us a step without it and 72.3 with it; the 512-thread form (128 x 256) 17.7 and 18.0.
+// the rest is better without that path in the batch kernel (64 runs, WENO-5: 1.98 ms a step against 2.01; its 4-row
+// form 0.97 of the time, its upwind form 0.98 to 1) and in the D2Q9 kernel (1024 x 2048: 200.6 us against
+// 202.5); the persistent kernel (U3, Komissarov, 512 x 1024) takes 70.3 us a step without it and 72.3 with it;
+// the 512-thread form (128 x 256) 17.7 and 18.0.
 template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false, bool RING = true, class Sm>
 __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q>::type &c, int stage, float dte,
                                            const CUtensorMap *tmo, int bx, int by, Sm &S, int b, int tb,
@@ -1093,7 +1094,7 @@ __global__ void __launch_bounds__(TY * (WIDE ? 64 : 32), WIDE ? 2 : (Q == 3 ? 32
 // soon as this tile's output has left the staging buffer.  tabs holds this stage's tables of every
 // tile row of the grid.  A copy that does not arrive within the run's wait limit sets *err; the
 // CTA then waits (bounded, 1 s) for its other copies in flight and leaves.
-template <bool LIN, int Q, bool RING = true>
+template <int Q, bool RING>
 __global__ void __launch_bounds__(256, 3)
     stage_f32_persist_kernel(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUtensorMap tmo,
                              const __grid_constant__ CUtensorMap tmf, const RunF R,
@@ -1179,7 +1180,7 @@ __global__ void __launch_bounds__(256, 3)
         if (ok) {
             int bx, by;
             tile_xy(t, bx, by);
-            tile_faces<TY, LIN, Q>(R, c, dte, S, 0, tb, bx, by);
+            tile_faces<TY, true, Q>(R, c, dte, S, 0, tb, bx, by);
             __syncthreads();
             f2 Gc[NPQ];
             load_cell_g<TY, NPQ>(S, 0, Gc);
@@ -1192,7 +1193,7 @@ __global__ void __launch_bounds__(256, 3)
             }
             if (stage != 1) ok = __syncthreads_and(wait_phase(&S.barF, par, R.wait_ns));
             if (ok) {
-                tile_cells<TY, LIN, Q, false, false, RING>(R, c, stage, dte, &tmo, bx, by, S, 0, tb, Gc);
+                tile_cells<TY, true, Q, false, false, RING>(R, c, stage, dte, &tmo, bx, by, S, 0, tb, Gc);
                 __syncthreads();   // this tile's tables and the staging buffer are free; next_tile is set
                 t = next_tile;
                 if (tid == 0 && stage != 1 && t < total) issue_f(t);
@@ -1699,7 +1700,7 @@ static size_t persist_smem() { return sizeof(SmemT<8, (Q == 3 ? 5 : NP2), 1, 2>)
 
 // Resident CTAs of one persistent stage-kernel instance on the current device (CTAs per SM x SMs),
 // looked up once per device (first from prepare_stage_f32, outside any stream capture)
-template <bool LIN, int Q>
+template <int Q>
 static int persist_grid()
 {
     static int dev_cached = -1, grid = 0;
@@ -1707,7 +1708,7 @@ static int persist_grid()
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (dev != dev_cached) {
         int per = 0, nsm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, stage_f32_persist_kernel<LIN, Q>, 256,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, stage_f32_persist_kernel<Q, true>, 256,
                                                           persist_smem<Q>()) != cudaSuccess ||
             cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return 0;
@@ -1717,16 +1718,16 @@ static int persist_grid()
     return grid;
 }
 
-template <bool LIN, int Q>
+template <int Q>
 static cudaError_t prepare_persist()
 {
-    cudaError_t e = cudaFuncSetAttribute(stage_f32_persist_kernel<LIN, Q>,
+    cudaError_t e = cudaFuncSetAttribute(stage_f32_persist_kernel<Q, true>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)persist_smem<Q>());
-    if (!e && LIN)
-        e = cudaFuncSetAttribute(stage_f32_persist_kernel<true, Q, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)persist_smem<Q>());
+    if (!e)
+        e = cudaFuncSetAttribute(stage_f32_persist_kernel<Q, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)persist_smem<Q>());
     if (e) return e;
-    return persist_grid<LIN, Q>() > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
+    return persist_grid<Q>() > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
 template <bool LIN, bool KW>
@@ -1741,25 +1742,23 @@ static cudaError_t prepare_wide()
                                 SPREAD_SMEM);
 }
 
+// The one-tile kernels (the upwind schemes' 8-row tiles run in the persistent and 512-thread ones) and the batch's
 template <int TY, bool LIN>
 cudaError_t prepare_one()
 {
-    cudaError_t e = cudaFuncSetAttribute(stage_f32_kernel<TY, LIN, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_bytes<TY>());
-    if (e) return e;
-    e = cudaFuncSetAttribute(stage_f32_kernel<TY, LIN, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_bytes<TY, 3>());
-    if (e) return e;
-    if (!LIN) {   // WENO-5 with the Komissarov theta flux
-        e = cudaFuncSetAttribute(stage_f32_kernel<TY, false, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem_bytes<TY>());
-        if (e) return e;
-        e = cudaFuncSetAttribute(stage_f32_kernel<TY, false, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem_bytes<TY, 3>());
-        if (e) return e;
-    }
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if (TY == 8 && !LIN) {
+    cudaError_t e;
+    if constexpr (TY == 4 || !LIN) {
+        if ((e = cudaFuncSetAttribute(stage_f32_kernel<TY, LIN, 4>, at, (int)smem_bytes<TY>())) ||
+            (e = cudaFuncSetAttribute(stage_f32_kernel<TY, LIN, 3>, at, (int)smem_bytes<TY, 3>())))
+            return e;
+    }
+    if constexpr (!LIN) {   // WENO-5 with the Komissarov theta flux
+        if ((e = cudaFuncSetAttribute(stage_f32_kernel<TY, false, 4, true>, at, (int)smem_bytes<TY>())) ||
+            (e = cudaFuncSetAttribute(stage_f32_kernel<TY, false, 3, true>, at, (int)smem_bytes<TY, 3>())))
+            return e;
+    }
+    if constexpr (TY == 8 && !LIN) {
         if ((e = cudaFuncSetAttribute(stage_f32_kernel<8, false, 3, false, false, false>, at, (int)smem_bytes<8, 3>())) ||
             (e = cudaFuncSetAttribute(stage_f32_kernel<8, false, 3, true, false, false>, at, (int)smem_bytes<8, 3>())))
             return e;
@@ -1776,11 +1775,10 @@ cudaError_t prepare_stage_f32()
     if ((e = prepare_one<8, false>()) || (e = prepare_one<4, false>()) || (e = prepare_one<8, true>()) ||
         (e = prepare_one<4, true>()))
         return e;
-    if ((e = prepare_wide<false, false>()) || (e = prepare_wide<true, false>()) || (e = prepare_wide<false, true>()))
+    if ((e = prepare_wide<false, false>()) || (e = prepare_wide<true, false>()) || (e = prepare_wide<false, true>()) ||
+        (e = prepare_persist<4>()))
         return e;
-    if ((e = prepare_persist<false, 4>()) || (e = prepare_persist<true, 4>()) || (e = prepare_persist<false, 3>()))
-        return e;
-    return prepare_persist<true, 3>();
+    return prepare_persist<3>();
 }
 
 size_t f32_tile_table_bytes(int q) { return q == 3 ? sizeof(TabT<8, 5>) : sizeof(TabT<8, NP2>); }
@@ -1842,7 +1840,7 @@ int stage_f32_max_ctas_per_sm(int ty, int q)
 
 template <int Q>
 static void launch_persist_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f,
-                             const RunF &run, const typename VelOf<Q>::type &c, int stage, bool lin, TileRows rows,
+                             const RunF &run, const typename VelOf<Q>::type &c, int stage, TileRows rows,
                              const void *tabs, unsigned *err, unsigned *ctr, cudaStream_t s)
 {
     // a launch of some of the tile rows waits on two streams (enqueue_split_step): plain edges there
@@ -1854,28 +1852,23 @@ static void launch_persist_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out
     const Tab *tab = reinterpret_cast<const Tab *>(tabs) + (size_t)(stage - 1) * tiles_y;
     const int total = ((run.L.np + TX - 1) / TX) * rows.count;
     const size_t smem = persist_smem<Q>();
-    if (lin) {
-        const int grid = std::min(total, persist_grid<true, Q>());
-        if (!run.rings) launch_after(early, stage_f32_persist_kernel<true, Q, false>, grid, 256, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
-        else launch_after(early, stage_f32_persist_kernel<true, Q>, grid, 256, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
-    } else {
-        const int grid = std::min(total, persist_grid<false, Q>());
-        launch_after(early, stage_f32_persist_kernel<false, Q>, grid, 256, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
-    }
+    const int grid = std::min(total, persist_grid<Q>());
+    if (!run.rings) launch_after(early, stage_f32_persist_kernel<Q, false>, grid, 256, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
+    else launch_after(early, stage_f32_persist_kernel<Q, true>, grid, 256, smem, s, tm_in, tm_out, tm_f, run, c, stage, rows, tab, err, ctr);
 }
 
 void launch_stage_f32_persist(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f,
-                              const RunF &run, const VelC &c, int stage, bool lin, const void *tabs, unsigned *err,
+                              const RunF &run, const VelC &c, int stage, const void *tabs, unsigned *err,
                               unsigned *ctr, cudaStream_t s, TileRows rows)
 {
-    launch_persist_q<4>(tm_in, tm_out, tm_f, run, c, stage, lin, rows, tabs, err, ctr, s);
+    launch_persist_q<4>(tm_in, tm_out, tm_f, run, c, stage, rows, tabs, err, ctr, s);
 }
 
 void launch_stage_f32_persist_q3(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f,
-                                 const RunF &run, const VelC3 &c, int stage, bool lin, const void *tabs,
+                                 const RunF &run, const VelC3 &c, int stage, const void *tabs,
                                  unsigned *err, unsigned *ctr, cudaStream_t s, TileRows rows)
 {
-    launch_persist_q<3>(tm_in, tm_out, tm_f, run, c, stage, lin, rows, tabs, err, ctr, s);
+    launch_persist_q<3>(tm_in, tm_out, tm_f, run, c, stage, rows, tabs, err, ctr, s);
 }
 
 bool stage_f32_wide(const Layout &L) { return (long long)((L.np + TX - 1) / TX) * ((L.nt + 7) / 8) <= WIDE_TILES; }
@@ -1921,9 +1914,8 @@ static void launch_stage_q(const CUtensorMap &tm_in, const CUtensorMap &tm_out, 
     if (ty == 4) {
         if (lin) launch_after(early, stage_f32_kernel<4, true, Q>, grid, 128, smem_bytes<4, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
         else launch_after(early, stage_f32_kernel<4, false, Q>, grid, 128, smem_bytes<4, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
-    } else {
-        if (lin) launch_after(early, stage_f32_kernel<8, true, Q>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
-        else launch_after(early, stage_f32_kernel<8, false, Q>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
+    } else {   // (WENO-5: the upwind schemes' 8-row tiles are launch_stage_f32_persist's)
+        launch_after(early, stage_f32_kernel<8, false, Q>, grid, 256, smem_bytes<8, Q>(), s, tm_in, tm_out, tm_f, run, c, stage, rows, err);
     }
 }
 

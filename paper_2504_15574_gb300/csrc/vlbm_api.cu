@@ -462,10 +462,10 @@ void launch_stage_f32_any(vlbm_t *h, int st, cudaStream_t s, TileRows rows = Til
         // the one-tile kernel with three resident CTAs per SM measured faster)
         unsigned *ctr = h->d_ctr + 2 * slot;
         if (h->vd.q == 3)
-            launch_stage_f32_persist_q3(tm, tmo, h->tmFc, h->run, h->vc3, st, lin, h->d_tabs, h->d_flags, ctr, s,
+            launch_stage_f32_persist_q3(tm, tmo, h->tmFc, h->run, h->vc3, st, h->d_tabs, h->d_flags, ctr, s,
                                         rows);
         else
-            launch_stage_f32_persist(tm, tmo, h->tmFc, h->run, h->vc, st, lin, h->d_tabs, h->d_flags, ctr, s, rows);
+            launch_stage_f32_persist(tm, tmo, h->tmFc, h->run, h->vc, st, h->d_tabs, h->d_flags, ctr, s, rows);
         return;
     }
     if (h->vd.q == 3) launch_stage_f32_q3(tm, tmo, h->tmFc, h->run, h->vc3, st, h->ty, lin, h->d_flags, s, rows);

@@ -239,7 +239,7 @@ void launch_batch_stage_f32_q3(const RunF *runs, const CUtensorMap *tms, const i
                                cudaStream_t s);
 // Resident CTAs per SM of the batch stage kernel for tile rows ty and velocity set order q.
 int stage_f32_max_ctas_per_sm(int ty, int q = 4);
-// The persistent stage kernel (8 tile rows, one CTA per resident slot, the next tile's copies in
+// The persistent stage kernel of the upwind schemes (8 tile rows, one CTA per resident slot, the next tile's copies in
 // flight during the cell phase):
 // its per-tile-row tables [stage 1..3][tile row] (f32_tile_table_bytes(q) each) are built on
 // the host from the run's FP32 row arrays (ds, d2s, isp: padded rows; sfc: interfaces; row, rref:
@@ -250,10 +250,10 @@ void f32_fill_tile_tables(int q, int nt, float dt, const float *ds, const float 
 // ctr: two zeroed unsigned counters per launch slot (launches that may run at the same time need
 // different slots); the kernel leaves them zeroed.
 void launch_stage_f32_persist(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f,
-                              const RunF &run, const VelC &c, int stage, bool lin, const void *tabs, unsigned *err,
+                              const RunF &run, const VelC &c, int stage, const void *tabs, unsigned *err,
                               unsigned *ctr, cudaStream_t s, TileRows rows = TileRows{0, -1, 0, 0});
 void launch_stage_f32_persist_q3(const CUtensorMap &tm_in, const CUtensorMap &tm_out, const CUtensorMap &tm_f,
-                                 const RunF &run, const VelC3 &c, int stage, bool lin, const void *tabs,
+                                 const RunF &run, const VelC3 &c, int stage, const void *tabs,
                                  unsigned *err, unsigned *ctr, cudaStream_t s, TileRows rows = TileRows{0, -1, 0, 0});
 
 // State scale k of the FP32 storage for WENO regulariser eps: the power of two nearest
