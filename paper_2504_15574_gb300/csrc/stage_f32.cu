@@ -742,10 +742,10 @@ __device__ __forceinline__ void tile_faces(const RunF &R, const typename VelOf<Q
 }
 
 // The stage input of this thread's cell (warp = cell row, lane = column) from tile buffer b.
-template <int TY, int NPQ, class Sm>
+template <int TY, int NPQ, bool MASK = false, class Sm>
 __device__ __forceinline__ void load_cell_g(const Sm &S, int b, f2 *G)
 {
-    const int cy = (threadIdx.x >> 5) & (TY - 1), cx = threadIdx.x & 31;
+    const int cy = MASK ? (threadIdx.x >> 5) & (TY - 1) : threadIdx.x >> 5, cx = threadIdx.x & 31;
 #pragma unroll
     for (int q = 0; q < NPQ; ++q) G[q] = S.tile[b].v[q][cy + GR][cx + GC];
 }
@@ -788,7 +788,8 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
     const BoxT<TY, NPQ> &box = S.tile[b];
     const TabT<TY, NPQ> &tab = S.tab[tb];
     // the tile's pole-face partials (the face phase's per-pair sums, added in pair order)
-    if (R.pole_part != nullptr && tid == 0) {
+    auto add_pole = [&]() {
+        if (R.pole_part == nullptr || tid != 0) return;
         for (int pole = 0; pole < 2; ++pole) {
             if (pole == 0 ? i0 != 0 : i0 + TY < L.nt) continue;
             double sum = 0.0;
@@ -799,10 +800,17 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
             // 512 x 1024 86.8 against 84.7)
             atomicAdd(&R.pole_part[bx + (size_t)(2 * (stage - 1) + pole) * R.tiles_x], sum);
         }
-    }
+    };
+    // In the persistent kernel with the ring filter it comes after the core tiles have left (a tile at a pole is
+    // none): U3 + Komissarov with the filter 512 x 1024 82.0 against 83.9 us a step.  The other kernels are
+    // scheduled better with it here (WENO-5 256 x 512 36.8 against 37.1; 512 threads 128 x 256 16.7 against 17.1).
+    constexpr bool POLE_LATE = LIN && RING && !WIDE;
+    if constexpr (!POLE_LATE) add_pole();
     // ---- one cell per thread (WIDE: two): warp = cell row, lane = column
     constexpr int NO = WIDE ? NPQ / 2 : NPQ;   // pairs that a thread updates, from pair oq on
-    const int cy = warp & (TY - 1), cx = lane, oq = WIDE ? NO * (warp / TY) : 0;
+    // (the row index is masked where the compiler's schedule is the better for it: without, D2Q9 1024 x 2048 takes
+    // 212.7 us a step instead of 215.7, launches one by one, with the Komissarov flux 210.5 instead of 207)
+    const int cy = WIDE || KW ? warp & (TY - 1) : warp, cx = lane, oq = WIDE ? NO * (warp / TY) : 0;
     const int i = i0 + cy, j = q0 + cx;
     if (i >= L.nt || j >= L.np) return;
     // the step's start values of this cell (stages 2, 3; the slots this thread's output
@@ -978,6 +986,7 @@ __device__ __forceinline__ void tile_cells(const RunF &R, const typename VelOf<Q
         }
         return;
     }
+    if constexpr (POLE_LATE) add_pole();
     const bool plain = (i >= GR && i < L.nt - GR && j >= GC && j < L.np - GC);
     if (ring) {
 #pragma unroll 1
@@ -1053,7 +1062,7 @@ __device__ __forceinline__ bool stage_tile(const RunF &R, const typename VelOf<Q
     tile_faces<TY, LIN, Q, KW, WIDE>(R, c, dte, S, 0, 0, bx, by);
     __syncthreads();
     f2 G[NPQ];
-    load_cell_g<TY, NPQ>(S, 0, G);
+    load_cell_g<TY, NPQ, WIDE || KW>(S, 0, G);
     tile_cells<TY, LIN, Q, KW, WIDE, RING>(R, c, stage, dte, tmo, bx, by, S, 0, 0, G);
     return true;
 }
