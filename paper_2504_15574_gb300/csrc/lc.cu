@@ -19,7 +19,7 @@
 //   backward weight: dW[co][tap][ci] = sum_p dY[p][co] pad(X)[p + tap][ci].
 // At the sizes of a coarse grid every launch is bound by latency, not by the tensor
 // rate: the kernels are launched early (launch_after), fetch what no kernel before
-// them writes (weights) ahead of their wait, and a backward pass is twelve launches.
+// them writes (weights) ahead of their wait, and a backward pass is nine launches.
 // Every sum runs in a fixed order that does not depend on the launch shapes (products along the taps,
 // the ghosts of a pixel one after the other, rows in order): training is a chain of thousands of steps
 // through BF16 roundings, so another order of a sum gives another network in the end.

@@ -144,9 +144,10 @@ __device__ __forceinline__ f2 swap2(f2 a) { return make_float2(a.y, a.x); }
 // ---- polar ring filter: block means -------------------------------------------------
 // Block sums are compensated: every addition is Knuth's error-free TwoSum, so a partial sum is an
 // unevaluated pair hi + lo of floats that carries the exact sum of its inputs up to the rounding of the
-// small lo parts (relative error ~2^-46).  Every form adds the columns of a block along the same binary
+// small lo parts (relative error ~2^-46).  Every form adds up to 256 columns of a block along the same binary
 // tree (neighbours, pairs of neighbours, ..., the lower partial first), so the stage kernels' means
-// and the filter kernel's agree bit for bit.  The block mean is the pair scaled by the exact 1/b and
+// and the filter kernel's agree bit for bit; wider blocks, which only the filter kernel takes, add the
+// sums of 256 columns in order (up to 2,048 columns; beyond, every thread those 256 apart).  The block mean is the pair scaled by the exact 1/b and
 // rounded once to FP32, which is the value of an FP64 accumulation (to ~2^-46) at FP32-pipe cost:
 // GB300's FP64 rate is 1/64 of its FP32 rate.
 struct FF { f2 hi, lo; };   // a float-float pair per member
@@ -250,7 +251,8 @@ __device__ __forceinline__ void ring_means(const FF (&a)[N], f2 (&out)[N], int b
 // The polar ring filter of one cell's pairs on their way out, x[k stride], k < NO, in shared memory (every
 // lane its own cell's; 2 to 8 of them are summed as NR = 4 or 8).  Behind a call: inlined into the cell
 // phase its registers cost spills there (U3 + Komissarov at 1024 x 2048: 246 against 233 us a step),
-// and few rows come here.
+// and few rows come here.  (In the 512-thread form the call costs the rows that do: 181 x 384 with the
+// filter 30.5 us a step, inlined 29.6.)
 template <int NO>
 __device__ __noinline__ void ring_cell(f2 *x, int stride, int b, unsigned mask)
 {
@@ -1070,11 +1072,11 @@ __device__ __forceinline__ bool stage_tile(const RunF &R, const typename VelOf<Q
 // WIDE (D2Q16, TY = 8): 512 threads, the phi and theta faces on different warps and two threads per
 // cell, for grids of at most two tiles per SM: a tile alone on its SM is a chain of its warps' walks,
 // which this halves.  Measured per step against the 256-thread form (U3: the persistent kernel):
-// 128 x 256 17.1 against 18.0 us, 181 x 384 23.8 against 28.5; U3 + Komissarov 12.1 against 17.9 and
-// 16.5 against 24.6; at three tiles per SM it loses (216 x 400: 31.5 against 29.7), since two CTAs of
+// 128 x 256 16.7 against 17.7 us, 181 x 384 23.6 against 28.2 (24.8 with plain edges); U3 + Komissarov 12.1
+// against 17.0 and 16.4 against 23.3 (21.4); at three tiles per SM it loses (216 x 400: 31.5 against 29.7), since two CTAs of
 // 64 registers fit where three of 80 do, and beside another launch too (the polar part of the split
-// schedule: 256 x 512 with the filter 48.4 against 44.0).  The same operations on every value, so the
-// same bits.
+// schedule: 256 x 512 with the filter 48.4 against 44.0; other solvers: stage_form.h).  The same operations
+// on every value, so the same bits.
 template <int TY, bool LIN, int Q, bool KW = false, bool WIDE = false, bool RING = true>
 __global__ void __launch_bounds__(TY * (WIDE ? 64 : 32), WIDE ? 2 : (Q == 3 ? 32 : 24) / TY) stage_f32_kernel(const __grid_constant__ CUtensorMap tm,
                                                                       const __grid_constant__ CUtensorMap tmo,

@@ -1,6 +1,6 @@
 // stage_f64.cu -- FP64 kernels of the parity path (compiled with -fmad=false).
 //
-// One RK3 stage of arXiv 2504.15574 Sec. 3.7 fused into one kernel: moments
+// One RK3 stage of arXiv 2504.15574 Sec. 3.7 in two kernels (faces, cells): moments
 // (Eq. f_moments_sum), equilibrium (Eq. feq_Q=4), BGK (Sec. 3.2), geometric
 // force through K^H and Ktilde^H (Eq. df), WENO-5 fluxes in theta and phi
 // (Eqs. fluxes_W5, WENO5_delta, WENO5_sigma) in the flux form of
@@ -53,8 +53,9 @@ __device__ __noinline__ double weno5_plain(double a, double b, double c, double 
 // expression order, and gives its flux to store(f, flux), v times the interface value (store_r: the
 // value itself, for the Komissarov factor).  The forms of one column (13/12 times the squared second
 // difference, and 5 y) are shared by the three candidate stencils centred on it, which changes no
-// bit.  30 FP64 instructions a face (four of them check the quotients): with every value zero or in [2^-400, 2^100), differences are
-// zero or multiples of the smallest ulp, so no product leaves the normal range.
+// bit.  30 FP64 instructions a face, four of which check its quotients: with every value zero or in
+// [2^-400, 2^100), differences are zero or multiples of the smallest ulp, so no product leaves the
+// normal range.
 template <class Load, class Store>
 __device__ __forceinline__ void weno5_walk(int n, bool plain, double eps, double v, const DivC &six, Load load,
                                            Store store)
@@ -150,7 +151,9 @@ __device__ __forceinline__ void store_with_images(T *f, const Layout &L, int k, 
 // thread walks S columns of one row.  For a negative velocity the strip is walked backwards, which
 // puts its values in upwind order.  The first nb_phi CTAs take the phi faces, the others the theta
 // faces (one launch: on small grids either alone leaves schedulers idle).  The walk is a rolled
-// loop: unrolled, its 1,000 instructions a face would not stay in the instruction cache.
+// loop: unrolled, its 1,000 instructions a face would not stay in the instruction cache.  256 x 512: 298 us a
+// launch, the FP64 pipe 76 % and the integer pipe 69 % busy.  (82 registers, five CTAs per SM: held to 80 or
+// 72 for six or seven, a step took 1,479 and 1,422 us instead of 1,405.)
 __global__ void __launch_bounds__(128) faces_f64_kernel(const StageD p, int nb_phi, int S)
 {
     const Layout L = p.L;
@@ -289,7 +292,7 @@ __device__ __forceinline__ void pole_budget_f64(const StageD &p)
 // form, left a 32 x 64 grid with 64 warps of 1,700 serial FP64 operations (71 us a launch).  Bound
 // on large grids: the FP64 pipe (37 instructions per population, from 105).  16 cells per CTA where
 // 32 would leave SMs without one.  In stage 3 one more CTA adds the step's pole budget (a launch
-// of its own was 3-10 us a step).
+// of its own was 3-10 us a step).  256 x 512: 169 us a launch, the FP64 pipe 77 % busy.
 template <int CELLS, bool PLAIN>
 __global__ void __launch_bounds__(256) cells_f64_kernel(const StageD p, int nblocks)
 {
