@@ -78,14 +78,30 @@ int lfail(vlbm_lc_t *n, int code, const std::string &m)
         if (e_ != cudaSuccess) return lfail((n), VLBM_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
-template <typename T>
-int lalloc(vlbm_lc_t *n, T **p, size_t count)
-{
-    LCK(n, cudaMalloc((void **)p, count * sizeof(T)));
-    LCK(n, cudaMemset(*p, 0, count * sizeof(T)));
-    n->bufs.push_back(*p);
-    return VLBM_OK;
-}
+// Device buffers of a network, zeroed, in one allocation (51 of their own were half to three quarters of the time of
+// its creation: 16 x 32 590 against 255 us, 128 x 256 1,950 against 410)
+struct LcBuffers {
+    std::vector<std::pair<void **, size_t>> want;
+    template <typename T>
+    void add(T **p, size_t count)
+    {
+        want.emplace_back((void **)p, (count * sizeof(T) + 255) / 256 * 256);
+    }
+    int allocate(vlbm_lc_t *n)
+    {
+        size_t total = 0;
+        for (const auto &w : want) total += w.second;
+        char *base = nullptr;
+        LCK(n, cudaMalloc((void **)&base, total));
+        n->bufs.push_back(base);
+        LCK(n, cudaMemset(base, 0, total));
+        for (const auto &w : want) {
+            *w.first = base;
+            base += w.second;
+        }
+        return VLBM_OK;
+    }
+};
 
 // splitmix64 for the initial weights
 unsigned long long smix(unsigned long long &s)
@@ -297,10 +313,8 @@ int vlbm_lc_create(int n_theta, int n_phi, unsigned long long seed, vlbm_lc_t **
             w[n->woff[l] + q] = (float)(a * (2.0 * ((smix(s) >> 11) * (1.0 / 9007199254740992.0)) - 1.0));
     }
     const size_t HW = (size_t)n_theta * n_phi, HWp = (size_t)(n_theta + 2) * (n_phi + 2);
-    int rc = 0;
-    auto A = [&](auto **p, size_t c) {
-        if (!rc) rc = lalloc(n, p, c);
-    };
+    LcBuffers bufs;
+    auto A = [&](auto **p, size_t c) { bufs.add(p, c); };
     A(&n->d_w, off);
     A(&n->d_g, off);
     A(&n->d_m, off);
@@ -334,7 +348,7 @@ int vlbm_lc_create(int n_theta, int n_phi, unsigned long long seed, vlbm_lc_t **
     A(&n->d_psi, HW);
     A(&n->d_ppart, HW / 256 + 2);
     A(&n->d_psum, 1);
-    if (rc) {
+    if (int rc = bufs.allocate(n)) {
         vlbm_lc_destroy(n);
         return rc;
     }
